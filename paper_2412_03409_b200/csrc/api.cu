@@ -44,6 +44,21 @@ int ensure_dynamic_smem(const void *func, int bytes, bool *done_per_device)
     return PKV_OK;
 }
 
+int sm_count()
+{
+    static int count[64] = {};
+    int dev = 0, n = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && dev >= 0 && dev < 64 && count[dev] > 0) return count[dev];
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) {
+        set_cuda_error(e, "cudaDeviceGetAttribute(sm count)");
+        return 0;
+    }
+    if (dev >= 0 && dev < 64) count[dev] = n;
+    return n;
+}
+
 size_t decode_ws_bytes(const pkv_shape *s);
 
 template <typename T, int D>
@@ -57,6 +72,9 @@ int launch_score_tc(const pkv_shape *s, const void *q, pkv_strides qs, const voi
 bool score_tc_usable(const pkv_shape *s, const void *q, pkv_strides qs, const void *k, pkv_strides ks);
 
 size_t score_tc_ws_bytes(const pkv_shape *s);
+size_t score_split_ws_bytes(const pkv_shape *s);
+int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const float *k, pkv_strides ks,
+                       const float *scale, const float *lse, float *scores, void *ws, cudaStream_t st);
 int selftest_wait_score(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_stream(int32_t *dev_status, cudaStream_t st);
 
@@ -65,8 +83,9 @@ static size_t score_ws_bytes(const pkv_shape *s)
     // per-head column sums + per-query log-sum-exp, both [B, L, H, N] fp32; the tensor-core
     // path pads the second to whole 128-query tiles
     size_t per = (size_t)s->batch * s->layers * s->heads * s->prompt_len * sizeof(float);
-    size_t simt = round_up(2 * per, kWsAlign), tc = score_tc_ws_bytes(s);
-    return simt > tc ? simt : tc;
+    size_t simt = round_up(2 * per, kWsAlign), tc = score_tc_ws_bytes(s), split = score_split_ws_bytes(s);
+    size_t need = simt > tc ? simt : tc;
+    return need > split ? need : split;
 }
 
 // Gini coefficient from the descending cumulative sums.  The Lorenz curve over
@@ -140,9 +159,7 @@ extern "C" int prefixkv_score(const pkv_shape *shape, const void *q, pkv_strides
         return launch_score_simt<__nv_bfloat16, 128>(shape, q, qs, k, ks, layer_scale, lse, scores,
                                                      ws, stream);
     }
-    if (shape->head_dim == 64)
-        return launch_score_simt<float, 64>(shape, q, qs, k, ks, layer_scale, lse, scores, ws, stream);
-    return launch_score_simt<float, 128>(shape, q, qs, k, ks, layer_scale, lse, scores, ws, stream);
+    return launch_score_split(shape, (const float *)q, qs, (const float *)k, ks, layer_scale, lse, scores, ws, stream);
 }
 
 extern "C" int prefixkv_gini(const pkv_shape *shape, const uint64_t *cum, double *gini,

@@ -18,6 +18,9 @@ int check_launch(const char *where);
 // Raises a kernel's dynamic shared-memory limit once per device.
 int ensure_dynamic_smem(const void *func, int bytes, bool *done_per_device);
 
+// SMs of the current device; <= 0 (and the error recorded) when it cannot be asked.
+int sm_count();
+
 inline bool shape_ok(const pkv_shape *s)
 {
     return s && s->batch > 0 && s->layers > 0 && s->heads > 0 && s->prompt_len > 0 &&

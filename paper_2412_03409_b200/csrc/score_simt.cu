@@ -1,5 +1,5 @@
-// Importance score (Sec. 3.2), FP32-FMA path: used for fp32 inputs, where the
-// 1e-4 relative bar rules out reduced-precision tensor-core products.
+// Importance score (Sec. 3.2), FP32-FMA path: used for bf16 inputs whose strides no tensor map can
+// describe (a zero stride), and the head mean of every path.
 //
 //   pass 1: per query m, log2-sum-exp of the scaled causal logits (keys j <= m)
 //   pass 2: per key n, sum over queries m >= n of exp2(logit - lse[m])
@@ -216,8 +216,6 @@ int launch_score_simt(const pkv_shape *s, const void *q, pkv_strides qs, const v
     template int launch_score_simt<T, D>(const pkv_shape *, const void *, pkv_strides, const void *, \
                                          pkv_strides, const float *, const float *, float *, void *, \
                                          cudaStream_t);
-PKV_INST(float, 64)
-PKV_INST(float, 128)
 PKV_INST(__nv_bfloat16, 64)
 PKV_INST(__nv_bfloat16, 128)
 #undef PKV_INST

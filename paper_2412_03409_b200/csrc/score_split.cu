@@ -1,0 +1,555 @@
+// Importance score (Sec. 3.2) of fp32 inputs on the bf16 tensor cores, in fp32 precision.
+//
+// Every fp32 element is the exact sum of three bf16 numbers x = x0 + x1 + x2 (8 significant bits
+// each).  A logit is the sum of the six products that matter, smallest first,
+//   x0 y2 + x1 y1 + x2 y0 + x0 y1 + x1 y0 + x0 y0
+// (the dropped x1 y2, x2 y1, x2 y2 are below 2^-24 of the product), accumulated in fp32 by
+// tcgen05.mma.  The tensor core truncates a sum where an FMA rounds it, so a long chain drifts
+// towards zero; the large products of a logit are therefore spread over several accumulators
+// (D = 128: one for each 64 elements; D = 64: one for each 16) that are added in registers.
+// Measured against fp64 on N(0, 1) operands, D = 128: error of a logit 0.9e-6 rms, against 2.3e-6
+// for a chain of fp32 FMAs, which rounds 128 times.
+//
+// Passes, tiles and work items are those of score_tc.cu.  What differs is how operands get to
+// shared memory: eight loader warps read fp32 rows from global memory (a chunk of 128 rows x 64
+// elements at a time, the next chunk's loads in flight while the current one is converted), split
+// them and write the three bf16 tiles in the 128-byte swizzle that the tensor core reads.  One CTA
+// per SM, 13 warps.  A prompt of at most 128 tokens is one tile: both passes then run on it in one
+// launch (MODE 0), the second on the transposed product of the operands already in shared memory.
+//
+// Measured, 8 layers x 16 heads of 128, 777 tokens: 195 us for the whole call (1263 us with 64 x 64
+// tiles on FMA units), 100 us a pass.  A tile needs 48 MMAs of 64 clocks = 3072; it takes 6200: the
+// issuing warp waits 1800 of them for chunks, because a chunk costs a loader warp about 2300 clocks
+// (the latency of its loads, of which one chunk is in flight, and its share of the issue slots).
+// Sixteen loader warps leave 80 registers a thread and spill (211 us).  4 layers x 4 heads of 64,
+// 128 tokens (one tile each): 14.0 us for the call, 30.7 with three FMA kernels.
+#include "score_tiles.cuh"
+
+namespace pkv {
+
+namespace {
+
+constexpr int kReaders = 4;                  // accumulator reader warps (warps 0-3: one TMEM lane quarter each)
+constexpr int kLoaders = 8;                  // loader warps (warps 5-12; warp 4 issues the MMAs)
+constexpr int kVecs = TT / kLoaders / 2;     // float4 of a chunk per loader lane
+constexpr int kSplitThreads = (kReaders + 1 + kLoaders) * 32;
+constexpr int kRing = 2;                     // streamed chunks in shared memory
+static_assert(kRing == 2, "with two chunks a tile, chunk c of every tile goes through ring slot c");
+constexpr uint32_t kPart = TT * 128;         // bytes of one bf16 part of a chunk: 128 rows x 64 elements
+constexpr uint32_t kChunk = 3 * kPart;
+constexpr uint32_t kBuf = 256;               // tensor-memory columns of one of the two accumulator buffers
+constexpr int kQueue = 4;                    // item numbers in flight between the loaders and the other roles
+
+struct SplitArgs {
+    const float *q, *k;
+    pkv_strides qs, ks;
+    const float *layer_scale;
+    const float *lse_in;  // pass 2: [B*L*H][N] log-sum-exp; times lse_mul it is in the log2 domain
+    float lse_mul;
+    float *lse2;          // pass 1 out, same layout, log2 domain
+    float *partial;       // [B*L*H][N] per-head column sums
+    int32_t *abort_word;  // set when a bounded wait runs out: the head mean then writes NaN scores
+    int *next_item;       // work counter of this pass, zeroed before it; NULL: a CTA takes item blockIdx.x alone
+    int clear_abort;      // this launch is the call's first and nothing has zeroed the abort word
+    int L, H, N, tiles, nsh, group;
+};
+
+// One float into its three bf16 parts, two elements at a time (packed low, high).  The first part is
+// rounded towards zero so that the largest finite values do not become infinite.
+__device__ __forceinline__ void split2(float x, float y, uint32_t &p0, uint32_t &p1, uint32_t &p2)
+{
+    asm("cvt.rz.bf16x2.f32 %0, %1, %2;" : "=r"(p0) : "f"(y), "f"(x));
+    const float rx = x - __uint_as_float(p0 << 16), ry = y - __uint_as_float(p0 & 0xffff0000u);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p1) : "f"(ry), "f"(rx));
+    const float sx = rx - __uint_as_float(p1 << 16), sy = ry - __uint_as_float(p1 & 0xffff0000u);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p2) : "f"(sy), "f"(sx));
+}
+
+// Bounded wait of a whole warp: every lane learns when any lane's wait has run out.
+__device__ __forceinline__ void warp_wait(uint64_t *bar, uint32_t parity, bool &dead, int *abort_flag)
+{
+    bar_wait(bar, parity, dead, abort_flag);
+    dead = __any_sync(0xffffffffu, dead);
+}
+
+// An accumulator buffer holds one unit of a tile: UN columns, in NACC partial accumulators.
+template <int D> struct Unit {
+    static constexpr int UN = D == 128 ? 128 : 64;
+    static constexpr int NACC = (int)kBuf / UN;
+    static constexpr int PER_TILE = TT / UN;
+    static constexpr int BLOCKS = UN / 32;  // 32-column blocks of a unit
+};
+
+// Logits of 32 columns: the sum of the partial accumulators.
+template <int D> __device__ __forceinline__ void load_logits(uint32_t taddr, float (&v)[32])
+{
+    float w[32];
+    tmem_ld32(taddr, v);
+    tmem_ld32(taddr + Unit<D>::UN, w);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] += w[i];
+    if (Unit<D>::NACC == 4) {
+        float x[32];
+        tmem_ld32(taddr + 2 * Unit<D>::UN, w);
+        tmem_ld32(taddr + 3 * Unit<D>::UN, x);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] += w[i] + x[i];
+    }
+}
+
+// MODE 1: stationary = Q tile t, streamed = K tiles 0..t (log-sum-exp).  MODE 2: stationary = K tile
+// t, streamed = Q tiles t..tiles-1 (column sums).  MODE 0: one tile, Q stationary, both results.
+template <int MODE, int D>
+__global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const SplitArgs a)
+{
+    constexpr int KH = D / 64;
+    constexpr int PASS = MODE == 2 ? 2 : 1;
+    using U = Unit<D>;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *base = reinterpret_cast<unsigned char *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char *sA = base;                 // [KH] chunks
+    unsigned char *sB = base + KH * kChunk;   // [kRing] chunks
+    __shared__ __align__(8) uint64_t a_full[KH], a_empty[KH], b_full[kRing], b_empty[kRing], s_full[2], s_empty[2],
+        q_full[kQueue], q_empty[kQueue], lse_full[2], drained;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int s_abort;
+    __shared__ int q_item[kQueue];
+    __shared__ __align__(16) float s_lse[2][kReaders][TT];
+
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int nitems = a.nsh * a.tiles;
+
+    if (tid == 0) {
+        s_abort = 0;
+        for (int i = 0; i < KH; ++i) {
+            bar_init(a_full + i, kLoaders);
+            bar_init(a_empty + i, 1);
+        }
+        for (int i = 0; i < kRing; ++i) {
+            bar_init(b_full + i, kLoaders);
+            bar_init(b_empty + i, 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            bar_init(s_full + i, 1);
+            bar_init(s_empty + i, kReaders);
+            bar_init(lse_full + i, kReaders);
+        }
+        for (int i = 0; i < kQueue; ++i) {
+            bar_init(q_full + i, 1);
+            bar_init(q_empty + i, kReaders + 1 + kLoaders);
+        }
+        bar_init(&drained, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == kReaders) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_slot)),
+                     "r"(2 * kBuf)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem_base = tmem_slot;
+    dependent_entry();  // the set-up above overlapped the kernel before this one; its results are read from here on
+    if (a.clear_abort && blockIdx.x == 0 && tid == 0) *a.abort_word = 0;
+
+    if (warp > kReaders) {
+        // ---- loaders: fp32 rows -> three bf16 parts in shared memory --------------------------------
+        const int lw = warp - kReaders - 1;
+        const int r0 = lw * 2 * kVecs + (lane >> 4), c4 = lane & 15;  // rows r0, r0 + 2, ...; float4 c4 of the row
+        bool dead = false;
+        Ring2 rb{0, 0u}, rq{0, 0u}, rp{0, 0u};
+        uint32_t a_phase = 0;
+        // the chunk whose global loads come next
+        int w = -1, step = 0, nsteps = 0, t = 0;
+        const float *stat = nullptr, *strm = nullptr;
+        int64_t stat_n = 0, strm_n = 0;
+        // (only the announcing thread) the next item number, asked for one item ahead
+        int ahead = blockIdx.x;
+        if (a.next_item && lw == 0 && lane == 0) ahead = atomicAdd(a.next_item, 1);
+        auto announce = [&]() {  // publishes one item number, or -1 for the end
+            const int v = ahead < nitems ? ahead : -1;
+            if (v >= 0) ahead = a.next_item ? atomicAdd(a.next_item, 1) : nitems;
+            bar_wait(q_empty + rp.idx, rp.phase ^ 1u, dead, &s_abort);
+            if (dead) return;
+            q_item[rp.idx] = v;
+            bar_arrive(q_full + rp.idx);
+            rp.next(kQueue);
+        };
+        auto next_item = [&]() {
+            if (lw == 0 && lane == 0) announce();
+            warp_wait(q_full + rq.idx, rq.phase, dead, &s_abort);
+            w = dead ? -1 : *(volatile int *)(q_item + rq.idx);
+            __syncwarp();
+            if (lane == 0) bar_arrive(q_empty + rq.idx);
+            rq.next(kQueue);
+            if (w < 0) return;
+            int sh;
+            decode_item<PASS>(w, a.nsh, a.tiles, a.group, sh, t);
+            const int seg = sh / a.H, h = sh - seg * a.H, b = seg / a.L, l = seg - b * a.L;
+            const float *qb = a.q + b * a.qs.b + l * a.qs.l + h * a.qs.h;
+            const float *kb = a.k + b * a.ks.b + l * a.ks.l + h * a.ks.h;
+            stat = PASS == 1 ? qb : kb;
+            strm = PASS == 1 ? kb : qb;
+            stat_n = PASS == 1 ? a.qs.n : a.ks.n;
+            strm_n = PASS == 1 ? a.ks.n : a.qs.n;
+            step = 0;
+            nsteps = KH + KH * (PASS == 1 ? t + 1 : a.tiles - t);
+        };
+        // Step s of an item: the stationary chunk c and the first streamed tile's chunk c in turn, then
+        // the chunks of the other streamed tiles.
+        auto fetch = [&](float4 (&x)[kVecs], int &where) {
+            if (step == nsteps) next_item();
+            if (w < 0) {
+                where = -1;
+                return;
+            }
+            const bool head = step < 2 * KH;
+            const bool is_a = head && (step & 1) == 0;
+            const int u = head ? step >> 1 : step - KH;  // streamed chunk number (the stationary one: its own)
+            const int c = u % KH;
+            const int tile = is_a ? t : (PASS == 1 ? 0 : t) + u / KH;
+            const float *p = (is_a ? stat : strm) + c * 64 + c4 * 4;
+            const int64_t rn = is_a ? stat_n : strm_n;
+#pragma unroll
+            for (int i = 0; i < kVecs; ++i) {
+                const int row = tile * TT + r0 + 2 * i;
+                x[i] = row < a.N ? __ldg(reinterpret_cast<const float4 *>(p + row * rn)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            where = is_a ? c : KH;  // which stationary chunk, or KH: the ring
+            ++step;
+        };
+        auto store = [&](const float4 (&x)[kVecs], int where) {
+            unsigned char *dst;
+            uint64_t *full;
+            if (where < KH) {
+                warp_wait(a_empty + where, a_phase ^ 1u, dead, &s_abort);
+                dst = sA + where * kChunk;
+                full = a_full + where;
+                if (where == KH - 1) a_phase ^= 1u;
+            } else {
+                warp_wait(b_empty + rb.idx, rb.phase ^ 1u, dead, &s_abort);
+                dst = sB + rb.idx * kChunk;
+                full = b_full + rb.idx;
+                rb.next(kRing);
+            }
+            if (dead) return;
+#pragma unroll
+            for (int i = 0; i < kVecs; ++i) {
+                const int r = r0 + 2 * i;
+                uint2 p0, p1, p2;
+                split2(x[i].x, x[i].y, p0.x, p1.x, p2.x);
+                split2(x[i].z, x[i].w, p0.y, p1.y, p2.y);
+                unsigned char *d = dst + r * 128 + (((c4 >> 1) ^ (r & 7)) << 4) + (c4 & 1) * 8;
+                *reinterpret_cast<uint2 *>(d) = p0;
+                *reinterpret_cast<uint2 *>(d + kPart) = p1;
+                *reinterpret_cast<uint2 *>(d + 2 * kPart) = p2;
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) bar_arrive(full);
+        };
+        float4 x0[kVecs], x1[kVecs];
+        int w0, w1;
+        fetch(x0, w0);
+        while (w0 >= 0 && !dead) {
+            fetch(x1, w1);
+            store(x0, w0);
+            if (w1 < 0 || dead) break;
+            fetch(x0, w0);
+            store(x1, w1);
+        }
+    } else if (warp == kReaders) {
+        // ---- MMA issuer: the whole warp walks the stream, one elected lane issues.  (Every value that
+        // an MMA takes is then the same in all lanes and can be formed in uniform registers ahead of it;
+        // with a single lane in the loop each MMA waited for its operands to be moved there, and 128 x
+        // 128 x 16 took 94-108 clocks of its 64.) --------------------------------------------------------
+        bool dead = false;
+        uint32_t a_phase = 0;
+        Ring2 rb{0, 0u}, rs{0, 0u}, rq{0, 0u};
+        const uint64_t da = smem_desc(saddr(sA)), db = smem_desc(saddr(sB));
+        constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(U::UN >> 3) << 17) |
+                                   ((uint32_t)(TT >> 4) << 24);  // as kIdesc, N = UN
+        // One chunk's products, smallest first, into its accumulators of buffer d_tmem: D = 128
+        // accumulator c; D = 64 (one chunk) accumulator 0 up to the first large product, then one each.
+        // x, y describe part 0 of the operands.
+        auto issue = [&](uint32_t d_tmem, int c, uint64_t x, uint64_t y) {
+            constexpr int px[6] = {0, 1, 2, 0, 1, 0}, py[6] = {2, 1, 0, 1, 0, 0};
+#pragma unroll
+            for (int m = 0; m < 6; ++m)
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {
+                    const int acc = KH == 2 ? c : (m == 5 ? ks : 0);
+                    mma_bf16(d_tmem + acc * U::UN, desc_add(x, px[m] * kPart + ks * 32), desc_add(y, py[m] * kPart + ks * 32), idesc,
+                             KH == 2 ? ((m | ks) != 0) : (m != 5 ? ((m | ks) != 0) : ks == 0));
+                }
+        };
+        for (;;) {
+            warp_wait(q_full + rq.idx, rq.phase, dead, &s_abort);
+            if (dead) break;
+            const int w = __shfl_sync(0xffffffffu, *(volatile int *)(q_item + rq.idx), 0);
+            __syncwarp();
+            if (lane == 0) bar_arrive(q_empty + rq.idx);
+            rq.next(kQueue);
+            if (w < 0) break;
+            int sh, t;
+            decode_item<PASS>(w, a.nsh, a.tiles, a.group, sh, t);
+            const int count = PASS == 1 ? t + 1 : a.tiles - t;
+            for (int jj = 0; jj < count; ++jj) {
+                if (KH == 2) {  // one unit of 128 columns; its two chunks are the ring's two slots
+                    warp_wait(s_empty + rs.idx, rs.phase ^ 1u, dead, &s_abort);
+#pragma unroll
+                    for (int c = 0; c < KH; ++c) {
+                        if (jj == 0) warp_wait(a_full + c, a_phase, dead, &s_abort);
+                        warp_wait(b_full + c, rb.phase, dead, &s_abort);
+                        if (dead) break;
+                        fence_after();
+                        if (elect_one()) {
+                            issue(tmem_base + rs.idx * kBuf, c, desc_add(da, c * kChunk), desc_add(db, c * kChunk));
+                            if (MODE != 0) {
+                                mma_commit(b_empty + c);
+                                if (jj == count - 1) mma_commit(a_empty + c);
+                            }
+                            if (c == KH - 1) mma_commit(s_full + rs.idx);
+                        }
+                    }
+                    if (dead) break;
+                    rs.next(2);
+                    if (MODE == 0) {  // the transposed product: keys on the lanes
+                        warp_wait(s_empty + rs.idx, rs.phase ^ 1u, dead, &s_abort);
+                        if (dead) break;
+                        fence_after();
+                        if (elect_one()) {
+#pragma unroll
+                            for (int c = 0; c < KH; ++c) {
+                                issue(tmem_base + rs.idx * kBuf, c, desc_add(db, c * kChunk), desc_add(da, c * kChunk));
+                                mma_commit(b_empty + c);
+                                mma_commit(a_empty + c);
+                            }
+                            mma_commit(s_full + rs.idx);
+                        }
+                        rs.next(2);
+                    }
+                    rb.phase ^= 1u;
+                } else {  // two units of 64 columns each
+                    if (jj == 0) warp_wait(a_full, a_phase, dead, &s_abort);
+                    warp_wait(b_full + rb.idx, rb.phase, dead, &s_abort);
+                    const uint64_t dk = desc_add(db, rb.idx * kChunk);
+#pragma unroll
+                    for (int u = 0; u < (MODE == 0 ? 2 : 1) * U::PER_TILE; ++u) {
+                        warp_wait(s_empty + rs.idx, rs.phase ^ 1u, dead, &s_abort);
+                        if (dead) break;
+                        fence_after();
+                        const uint32_t rows = (u % U::PER_TILE) * (U::UN * 128);
+                        const bool swap = u >= U::PER_TILE;  // (MODE 0) the transposed product
+                        if (elect_one()) {
+                            issue(tmem_base + rs.idx * kBuf, 0, swap ? dk : da, desc_add(swap ? da : dk, rows));
+                            mma_commit(s_full + rs.idx);
+                            if (u == (MODE == 0 ? 2 : 1) * U::PER_TILE - 1) {
+                                mma_commit(b_empty + rb.idx);
+                                if (jj == count - 1) mma_commit(a_empty);
+                            }
+                        }
+                        rs.next(2);
+                    }
+                    if (dead) break;
+                    rb.next(kRing);
+                }
+            }
+            if (dead) break;
+            a_phase ^= 1u;
+        }
+        if (dead) {  // let the products in flight finish before the CTA can exit (bounded)
+            if (elect_one()) mma_commit(&drained);
+            for (uint32_t i = 0; i < kSpin; ++i)
+                if (bar_try(&drained, 0u)) break;
+        }
+    } else {
+        // ---- accumulator readers: one TMEM lane (tile row) per thread --------------------------------
+        const int row = warp * 32 + lane;
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(warp * 32) << 16);
+        bool dead = false;
+        Ring2 rs{0, 0u}, rq{0, 0u};
+        int flip = 0;
+        uint32_t lse_phase = 0;
+        auto release = [&]() {
+            fence_before();
+            __syncwarp();
+            if (lane == 0) bar_arrive(s_empty + rs.idx);
+            rs.next(2);
+        };
+        // Column sums of a tile; on the diagonal tile only the blocks from this warp's keys on count.
+        auto sum_tile = [&](const float *lse, bool diag, float sc, float &col_sum) {
+            for (int u = 0; u < U::PER_TILE; ++u) {
+                warp_wait(s_full + rs.idx, rs.phase, dead, &s_abort);
+                fence_after();
+#pragma unroll 1
+                for (int cb = max(diag ? warp : 0, u * U::BLOCKS); cb < (u + 1) * U::BLOCKS; ++cb) {
+                    float v[32];
+                    load_logits<D>(lane_addr + rs.idx * kBuf + (cb - u * U::BLOCKS) * 32, v);
+                    col_sum += colsum_block<32>(v, lse + cb * 32, sc, diag && cb == warp, lane);
+                }
+                release();
+            }
+        };
+        for (;;) {
+            warp_wait(q_full + rq.idx, rq.phase, dead, &s_abort);
+            if (dead) break;
+            const int w = *(volatile int *)(q_item + rq.idx);
+            __syncwarp();
+            if (lane == 0) bar_arrive(q_empty + rq.idx);
+            rq.next(kQueue);
+            if (w < 0) break;
+            int sh, t;
+            decode_item<PASS>(w, a.nsh, a.tiles, a.group, sh, t);
+            const float sc = a.layer_scale[(sh / a.H) % a.L] * kLog2eT;
+            const int grow = t * TT + row;  // query (pass 1) or key (pass 2) of this thread
+            float run_max = -INFINITY, run_sum = 0.f, col_sum = 0.f;
+            if (PASS == 1) {
+                for (int j = 0; j <= t; ++j) {
+                    // on the diagonal tile only the 32-column blocks up to this warp's rows count
+                    const int c_hi = j == t ? warp : TT / 32 - 1;
+                    for (int u = 0; u < U::PER_TILE; ++u) {
+                        warp_wait(s_full + rs.idx, rs.phase, dead, &s_abort);
+                        fence_after();
+#pragma unroll 1
+                        for (int cb = u * U::BLOCKS; cb < (u + 1) * U::BLOCKS && cb <= c_hi; ++cb) {
+                            float v[32];
+                            load_logits<D>(lane_addr + rs.idx * kBuf + (cb - u * U::BLOCKS) * 32, v);
+                            if (j == t && cb == warp) {  // the block the causal boundary crosses
+#pragma unroll
+                                for (int i = 0; i < 32; ++i) v[i] = i <= lane ? v[i] : -INFINITY;
+                            }
+                            lse_block<32>(v, sc, sc > 0.f, run_max, run_sum);
+                        }
+                        release();
+                    }
+                }
+                const float lse = run_max + log2f(run_sum);
+                if (MODE == 1) {
+                    if (grow < a.N) a.lse2[(size_t)sh * a.N + grow] = lse;
+                } else {
+                    // every reader warp needs all 128 normalisers (two buffers in turn, so that
+                    // no warp can write a buffer that another still reads)
+                    s_lse[flip][0][row] = grow < a.N ? lse : INFINITY;
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(lse_full + flip);
+                    warp_wait(lse_full + flip, lse_phase, dead, &s_abort);
+                    sum_tile(s_lse[flip][0], true, sc, col_sum);
+                    flip ^= 1;
+                    if (flip == 0) lse_phase ^= 1u;
+                    if (grow < a.N) a.partial[(size_t)sh * a.N + grow] = col_sum;
+                }
+            } else {
+                const float *lrow = a.lse_in + (size_t)sh * a.N;
+                // four of the tile's 128 query normalisers per lane, fetched a tile ahead; each warp keeps its own copy
+                float4 mine;
+                auto get = [&](int j) {
+                    const int m = j * TT + lane * 4;
+                    mine.x = m < a.N ? __ldg(lrow + m) * a.lse_mul : INFINITY;
+                    mine.y = m + 1 < a.N ? __ldg(lrow + m + 1) * a.lse_mul : INFINITY;
+                    mine.z = m + 2 < a.N ? __ldg(lrow + m + 2) * a.lse_mul : INFINITY;
+                    mine.w = m + 3 < a.N ? __ldg(lrow + m + 3) * a.lse_mul : INFINITY;
+                };
+                get(t);
+                for (int j = t; j < a.tiles; ++j) {
+                    __syncwarp();
+                    const int buf = j & 1;
+                    reinterpret_cast<float4 *>(s_lse[buf][warp])[lane] = mine;
+                    if (j + 1 < a.tiles) get(j + 1);
+                    __syncwarp();
+                    sum_tile(s_lse[buf][warp], j == t, sc, col_sum);
+                }
+                if (grow < a.N) a.partial[(size_t)sh * a.N + grow] = col_sum;
+            }
+        }
+    }
+
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (tid == 0 && s_abort) atomicExch(a.abort_word, (int)PKV_DEV_TIMEOUT);
+    if (warp == kReaders) {
+        __syncwarp();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * kBuf) : "memory");
+    }
+}
+
+template <int MODE, int D> int launch_split(const SplitArgs &a, int sms, cudaStream_t st)
+{
+    static bool done[64] = {};
+    const size_t smem = (size_t)(D / 64 + kRing) * kChunk + 1024;
+    int rc = ensure_dynamic_smem((const void *)score_split_kernel<MODE, D>, (int)smem, done);
+    if (rc != PKV_OK) return rc;
+    const int items = a.nsh * a.tiles;
+    cudaError_t e = launch_dependent(score_split_kernel<MODE, D>, dim3(items < sms ? items : sms), dim3(kSplitThreads), smem, st, a);
+    if (e != cudaSuccess) {
+        set_cuda_error(e, "score_split_kernel");
+        return PKV_ERR_CUDA;
+    }
+    return PKV_OK;
+}
+
+}  // namespace
+
+int launch_head_mean(const float *partial, int H, int N, size_t total, float *scores, const int32_t *abort_word,
+                     cudaStream_t st);
+
+// Workspace: partial [rows][N], lse2 [rows][N], then two work counters and the abort word.
+size_t score_split_ws_bytes(const pkv_shape *s)
+{
+    const size_t per = (size_t)s->batch * s->layers * s->heads * s->prompt_len * sizeof(float);
+    return round_up(2 * per, kWsAlign) + kWsAlign;
+}
+
+int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const float *k, pkv_strides ks,
+                       const float *scale, const float *lse, float *scores, void *ws, cudaStream_t st)
+{
+    const int B = s->batch, L = s->layers, H = s->heads, N = s->prompt_len;
+    const size_t per = (size_t)B * L * H * N;
+    SplitArgs a = {};
+    a.q = q; a.k = k; a.qs = qs; a.ks = ks;
+    a.layer_scale = scale;
+    a.partial = (float *)ws;
+    a.lse2 = a.partial + per;
+    int *words = (int *)((unsigned char *)ws + round_up(2 * per * sizeof(float), kWsAlign));
+    a.abort_word = words + 2;
+    a.L = L; a.H = H; a.N = N;
+    a.tiles = (N + TT - 1) / TT;
+    a.nsh = B * L * H;
+    a.group = head_group(a.nsh, N, s->head_dim, 4);
+    const int sms = sm_count();
+    if (sms <= 0) return PKV_ERR_CUDA;
+    // With an item for every CTA there is nothing to hand out: no counter, and so nothing to zero first.
+    const bool counted = a.nsh * a.tiles > sms;
+    if (counted) {
+        cudaError_t e = cudaMemsetAsync(words, 0, 4 * sizeof(int), st);
+        if (e != cudaSuccess) {
+            set_cuda_error(e, "cudaMemsetAsync(score work counters)");
+            return PKV_ERR_CUDA;
+        }
+    }
+    a.clear_abort = !counted;
+    const bool wide = s->head_dim == 128;
+    int rc = PKV_OK;
+    if (!lse && a.tiles == 1) {
+        a.next_item = counted ? words : nullptr;
+        rc = wide ? launch_split<0, 128>(a, sms, st) : launch_split<0, 64>(a, sms, st);
+    } else {
+        if (!lse) {
+            a.next_item = counted ? words : nullptr;
+            rc = wide ? launch_split<1, 128>(a, sms, st) : launch_split<1, 64>(a, sms, st);
+            if (rc != PKV_OK) return rc;
+            a.clear_abort = 0;
+        }
+        a.lse_in = lse ? lse : a.lse2;
+        a.lse_mul = lse ? kLog2eT : 1.f;
+        a.next_item = counted ? words + 1 : nullptr;
+        rc = wide ? launch_split<2, 128>(a, sms, st) : launch_split<2, 64>(a, sms, st);
+    }
+    if (rc != PKV_OK) return rc;
+    return launch_head_mean(a.partial, H, N, (size_t)B * L * N, scores, a.abort_word, st);
+}
+
+}  // namespace pkv

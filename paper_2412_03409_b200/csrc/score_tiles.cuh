@@ -1,0 +1,261 @@
+// Device helpers of the tensor-core scoring kernels (sm_100a): mbarriers with bounded waits, TMA,
+// tcgen05 descriptors, MMA issue and tensor-memory loads.  Tiles are 128 x 128 throughout.
+#pragma once
+#include <cuda.h>
+
+#include "common.cuh"
+
+namespace pkv {
+
+constexpr int TT = 128;                    // tile side
+constexpr uint32_t kSpin = 1u << 20;       // tries per wait; each may sleep up to kSuspendNs
+constexpr uint32_t kSuspendNs = 2000;      // suspend-time hint of one try: a waiting thread leaves the issue slots alone
+constexpr float kLog2eT = 1.4426950408889634f;
+
+__device__ __forceinline__ uint32_t saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void bar_init(uint64_t *bar, uint32_t count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(bar)), "r"(count));
+}
+__device__ __forceinline__ void bar_expect_tx(uint64_t *bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(bar)), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(bar)) : "memory");
+}
+__device__ __forceinline__ bool bar_try(uint64_t *bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(saddr(bar)), "r"(parity), "r"(kSuspendNs)
+        : "memory");
+    return ok != 0;
+}
+// Bounded wait.  `dead` latches for the calling thread once any wait in the CTA has run out.
+__device__ __forceinline__ void bar_wait(uint64_t *bar, uint32_t parity, bool &dead, int *abort_flag,
+                                         uint32_t limit = kSpin)
+{
+    if (dead) return;
+    for (uint32_t i = 0; i < limit; ++i) {
+        if (bar_try(bar, parity)) return;
+        if ((i & 255u) == 255u && *(volatile int *)abort_flag) break;
+    }
+    dead = true;
+    atomicExch(abort_flag, 1);
+}
+
+__device__ __forceinline__ void tma_load_5d(void *dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1,
+                                            int c2, int c3, int c4)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(saddr(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(saddr(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+        : "memory");
+}
+
+// Shared-memory matrix descriptor, K-major operand with the 128-byte swizzle: rows of 128 bytes,
+// eight-row groups 1024 bytes apart, tile base aligned to 1024 bytes.
+__device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);  // start address, bits [0,14)
+    d |= (uint64_t)1 << 16;                   // leading byte offset (not used by swizzled K-major)
+    d |= (uint64_t)(1024 >> 4) << 32;         // stride byte offset, bits [32,46)
+    d |= (uint64_t)1 << 46;                   // descriptor version for sm_100
+    d |= (uint64_t)2 << 61;                   // layout type: 128-byte swizzle
+    return d;
+}
+
+// The descriptor of an operand `bytes` further on (tiles end below 256 KiB, so the address field cannot carry).
+__device__ __forceinline__ uint64_t desc_add(uint64_t desc, uint32_t bytes)
+{
+    return (desc & 0xffffffff00000000ull) | ((uint32_t)desc + (bytes >> 4));
+}
+
+// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = N = 128.
+constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TT >> 3) << 17) |
+                            ((uint32_t)(TT >> 4) << 24);
+
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// True in one lane of a converged warp, always the same one.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+    return ok != 0;
+}
+__device__ __forceinline__ void mma_commit(uint64_t *bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(saddr(bar))
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
+{
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64])
+{
+    uint32_t r[64];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+}
+// Both halves of a 128-column accumulator row: two loads in flight, one wait.
+__device__ __forceinline__ void tmem_ld128(uint32_t taddr, float (&v)[128])
+{
+    uint32_t r[64], q[64];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+        : "r"(taddr));
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
+        : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]), "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15]), "=r"(q[16]), "=r"(q[17]), "=r"(q[18]), "=r"(q[19]), "=r"(q[20]), "=r"(q[21]), "=r"(q[22]), "=r"(q[23]), "=r"(q[24]), "=r"(q[25]), "=r"(q[26]), "=r"(q[27]), "=r"(q[28]), "=r"(q[29]), "=r"(q[30]), "=r"(q[31]), "=r"(q[32]), "=r"(q[33]), "=r"(q[34]), "=r"(q[35]), "=r"(q[36]), "=r"(q[37]), "=r"(q[38]), "=r"(q[39]), "=r"(q[40]), "=r"(q[41]), "=r"(q[42]), "=r"(q[43]), "=r"(q[44]), "=r"(q[45]), "=r"(q[46]), "=r"(q[47]), "=r"(q[48]), "=r"(q[49]), "=r"(q[50]), "=r"(q[51]), "=r"(q[52]), "=r"(q[53]), "=r"(q[54]), "=r"(q[55]), "=r"(q[56]), "=r"(q[57]), "=r"(q[58]), "=r"(q[59]), "=r"(q[60]), "=r"(q[61]), "=r"(q[62]), "=r"(q[63])
+        : "r"(taddr + 64));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 64; ++i) {
+        v[i] = __uint_as_float(r[i]);
+        v[64 + i] = __uint_as_float(q[i]);
+    }
+}
+// 2^x on the special-function unit, one instruction (inputs here are <= 0 or -inf; flushing
+// denormal results to zero is harmless for sums of probabilities).
+__device__ __forceinline__ float ex2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+
+struct Ring2 {
+    int idx;
+    uint32_t phase;
+    __device__ __forceinline__ void next(int n)
+    {
+        if (++idx == n) {
+            idx = 0;
+            phase ^= 1u;
+        }
+    }
+};
+
+// Pass 1 on NC consecutive logits of one query row: running maximum and sum in the log2
+// domain.  Four interleaved chains each for the maximum and the sum: with two reader warps per
+// scheduler a long dependent chain would leave it idle.  `fast` (scale > 0, the usual case):
+// the extreme of sc * x is sc * max x, so masked logits may stay -inf.
+template <int NC>
+__device__ __forceinline__ void lse_block(float (&v)[NC], float sc, bool fast, float &run_max, float &run_sum)
+{
+    if (!fast) {
+#pragma unroll
+        for (int i = 0; i < NC; ++i) v[i] = v[i] == -INFINITY ? -INFINITY : v[i] * sc;
+    }
+    // (three-input maximum: half the comparisons; the loop takes four values at a time, the last two come at the end)
+    float c2[2] = {v[0], v[1]};
+#pragma unroll
+    for (int i = 2; i + 2 < NC; i += 4) {
+        c2[0] = max3(c2[0], v[i], v[i + 1]);
+        c2[1] = max3(c2[1], v[i + 2], v[i + 3]);
+    }
+    const float cmax = max3(c2[0], c2[1], fmaxf(v[NC - 2], v[NC - 1]));
+    const float nm = fmaxf(run_max, fast ? cmax * sc : cmax);  // finite: column 0 is never masked
+    float p4[4] = {0.f, 0.f, 0.f, 0.f};
+    if (fast) {
+#pragma unroll
+        for (int i = 0; i < NC; ++i) p4[i & 3] += ex2(fmaf(v[i], sc, -nm));
+    } else {
+#pragma unroll
+        for (int i = 0; i < NC; ++i) p4[i & 3] += ex2(v[i] - nm);
+    }
+    run_sum = fmaf(run_sum, ex2(run_max - nm), (p4[0] + p4[1]) + (p4[2] + p4[3]));
+    run_max = nm;
+}
+
+// Pass 2 on the logits of NC consecutive queries against one key: sum of the probabilities,
+// lse = the queries' normalisers (shared memory, log2 domain).  On the block the causal boundary
+// crosses (`edge`) query i of the block counts only when i >= lane.
+template <int NC>
+__device__ __forceinline__ float colsum_block(const float (&v)[NC], const float *lse, float sc, bool edge, int lane)
+{
+    const float4 *lp = reinterpret_cast<const float4 *>(lse);
+    float p4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i4 = 0; i4 < NC / 4; ++i4) {
+        const float4 ls = lp[i4];
+        const float lv[4] = {ls.x, ls.y, ls.z, ls.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i4 * 4 + u;
+            const float p = ex2(fmaf(v[i], sc, -lv[u]));
+            p4[u] += (!edge || i >= lane) ? p : 0.f;
+        }
+    }
+    return (p4[0] + p4[1]) + (p4[2] + p4[3]);
+}
+
+// Work item w -> (segment-head sh, tile t).  CTAs take items in order from a counter.  Heads come in
+// groups whose Q and K stay in L2 (head_group), so that every operand byte comes from HBM once per
+// pass.  Within a group the longest items of all its heads come first (pass 1: the last query tiles,
+// pass 2: the first key tiles), so that what is left for the end of the pass is short.  Pass 2 walks
+// the groups backwards: it starts on what pass 1 touched last.
+template <int PASS> __device__ __forceinline__ void decode_item(int w, int nsh, int tiles, int group, int &sh, int &t)
+{
+    const int g = w / (group * tiles), r = w - g * group * tiles;
+    const int heads = min(group, nsh - g * group);
+    const int step = r / heads, first = g * group;
+    t = PASS == 1 ? tiles - 1 - step : step;
+    sh = first + (r - step * heads);
+    if (PASS == 2) sh = nsh - 1 - sh;
+}
+// Heads of a group: as many as 64 MB hold, half of the L2, evenly over the groups.
+inline int head_group(int nsh, int N, int D, size_t elem)
+{
+    const size_t fit = ((size_t)64 << 20) / (2 * (size_t)N * D * elem);
+    const int most = fit < 1 ? 1 : (fit < (size_t)nsh ? (int)fit : nsh);
+    const int groups = (nsh + most - 1) / most;
+    return (nsh + groups - 1) / groups;
+}
+
+}  // namespace pkv
