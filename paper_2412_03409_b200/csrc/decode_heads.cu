@@ -40,7 +40,7 @@
 #include <chrono>
 #include <mutex>
 
-#include "common.cuh"
+#include "decode_plan.cuh"
 
 namespace pkv {
 
@@ -161,44 +161,13 @@ __device__ __forceinline__ void hbulk_load(void *dst, const void *src, uint32_t 
                  : "memory");
 }
 
-template <typename T> struct HVec;
-template <> struct HVec<float> {
-    static constexpr int VE = 4;
-    __device__ static void unpack(const uint4 &r, float *x)
-    {
-        x[0] = __uint_as_float(r.x); x[1] = __uint_as_float(r.y);
-        x[2] = __uint_as_float(r.z); x[3] = __uint_as_float(r.w);
-    }
-    __device__ static uint4 pack(const float *x)
-    {
-        return make_uint4(__float_as_uint(x[0]), __float_as_uint(x[1]), __float_as_uint(x[2]), __float_as_uint(x[3]));
-    }
-};
-template <> struct HVec<__nv_bfloat16> {
-    static constexpr int VE = 8;
-    __device__ static void unpack(const uint4 &r, float *x)
-    {
-        x[0] = __uint_as_float(r.x << 16); x[1] = __uint_as_float(r.x & 0xffff0000u);
-        x[2] = __uint_as_float(r.y << 16); x[3] = __uint_as_float(r.y & 0xffff0000u);
-        x[4] = __uint_as_float(r.z << 16); x[5] = __uint_as_float(r.z & 0xffff0000u);
-        x[6] = __uint_as_float(r.w << 16); x[7] = __uint_as_float(r.w & 0xffff0000u);
-    }
-    __device__ static uint4 pack(const float *x)
-    {
-        __nv_bfloat162 a = __floats2bfloat162_rn(x[0], x[1]), b = __floats2bfloat162_rn(x[2], x[3]);
-        __nv_bfloat162 c = __floats2bfloat162_rn(x[4], x[5]), d = __floats2bfloat162_rn(x[6], x[7]);
-        return make_uint4(*reinterpret_cast<uint32_t *>(&a), *reinterpret_cast<uint32_t *>(&b),
-                          *reinterpret_cast<uint32_t *>(&c), *reinterpret_cast<uint32_t *>(&d));
-    }
-};
-
 // A head's slice of a row is D * sizeof(T) bytes = LPR 16-byte vectors: LPR lanes share a row, a
 // warp holds G = 32 / LPR rows at a time and a tile (8 KiB) is 16 such steps.
 template <typename T, int D>
 __global__ void __launch_bounds__((kHWarps + kHProducers) * 32, 1)
 decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 {
-    constexpr int VE = HVec<T>::VE;
+    constexpr int VE = RowVec<T>::VE;
     constexpr uint32_t SLICE = D * sizeof(T);
     constexpr int LPR = SLICE / 16;
     constexpr int G = 32 / LPR;
@@ -397,7 +366,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             float qf[VE];
             {
                 float x[VE];
-                HVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + c * 16), x);
+                RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + c * 16), x);
 #pragma unroll
                 for (int i = 0; i < VE; ++i) qf[i] = x[i] * m.sc;
             }
@@ -408,7 +377,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             for (int j = 0; j < 16; ++j) {
                 const int row = j * G + grp;
                 float x[VE], d0 = 0.f, d1 = 0.f;
-                HVec<T>::unpack(*reinterpret_cast<const uint4 *>(kt + (uint32_t)row * SLICE), x);
+                RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(kt + (uint32_t)row * SLICE), x);
 #pragma unroll
                 for (int i = 0; i < VE; i += 2) {
                     d0 = fmaf(qf[i], x[i], d0);
@@ -418,7 +387,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             }
             {
                 float x[VE], d0 = 0.f, d1 = 0.f;
-                HVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + SLICE + c * 16), x);
+                RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + SLICE + c * 16), x);
 #pragma unroll
                 for (int i = 0; i < VE; i += 2) {
                     d0 = fmaf(qf[i], x[i], d0);
@@ -455,7 +424,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
                 const float p = exp2f(s[j] - Mn);
                 lsum += p;
                 float x[VE];
-                HVec<T>::unpack(*reinterpret_cast<const uint4 *>(vt + (uint32_t)(j * G + grp) * SLICE), x);
+                RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(vt + (uint32_t)(j * G + grp) * SLICE), x);
 #pragma unroll
                 for (int i = 0; i < VE; ++i) acc[i] = fmaf(p, x[i], acc[i]);
             }
@@ -464,7 +433,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
                     const float p = exp2f(s[16] - Mn);
                     lsum += p;
                     float x[VE];
-                    HVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + 2 * SLICE + c * 16), x);
+                    RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + 2 * SLICE + c * 16), x);
 #pragma unroll
                     for (int i = 0; i < VE; ++i) acc[i] = fmaf(p, x[i], acc[i]);
                 }
@@ -540,7 +509,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 #pragma unroll
                     for (int i = 0; i < VE; ++i) x[i] = acc[i] * inv;
                     *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.out) + ((size_t)m.seg * H + m.h) * SLICE + c * 16) =
-                        HVec<T>::pack(x);
+                        RowVec<T>::pack(x);
                 }
             }
             M = -INFINITY;
@@ -642,18 +611,8 @@ int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const v
     const int H = s->heads, D = s->head_dim, nl = le - lb, nact = s->batch * nl;
     if (c->evict_distance != 0 || nact > kHMaxAct) return -1;
     if (D != 64 && D != 128) return -1;
-    static int sm_count[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int sms = (dev >= 0 && dev < 64) ? sm_count[dev] : 0;
-    if (!sms) {
-        cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) {
-            set_cuda_error(e, "cudaDeviceGetAttribute(sm count)");
-            return PKV_ERR_CUDA;
-        }
-        if (dev >= 0 && dev < 64) sm_count[dev] = sms;
-    }
+    int sms = sm_count();
+    if (sms <= 0) return PKV_ERR_CUDA;
     if (sms > kHMaxGrid) sms = kHMaxGrid;
     // Worth it while complete (segment, head) items balance over the SMs (at least four per SM)
     // and the segments are short.  Measured on 32 layers x 32 heads of 128, 128-256 rows per

@@ -1,0 +1,127 @@
+// What one decode step does to a segment, and 16-byte row vectors: shared by the decode kernels.
+#pragma once
+#include "common.cuh"
+
+namespace pkv {
+
+// 16 bytes of a cache row as floats.
+template <typename T> struct RowVec;
+template <> struct RowVec<float> {
+    static constexpr int VE = 4;
+    __device__ static void unpack(const uint4 &r, float *x)
+    {
+        x[0] = __uint_as_float(r.x); x[1] = __uint_as_float(r.y);
+        x[2] = __uint_as_float(r.z); x[3] = __uint_as_float(r.w);
+    }
+    __device__ static uint4 pack(const float *x)
+    {
+        return make_uint4(__float_as_uint(x[0]), __float_as_uint(x[1]), __float_as_uint(x[2]), __float_as_uint(x[3]));
+    }
+};
+template <> struct RowVec<__nv_bfloat16> {
+    static constexpr int VE = 8;
+    __device__ static void unpack(const uint4 &r, float *x)
+    {
+        x[0] = __uint_as_float(r.x << 16); x[1] = __uint_as_float(r.x & 0xffff0000u);
+        x[2] = __uint_as_float(r.y << 16); x[3] = __uint_as_float(r.y & 0xffff0000u);
+        x[4] = __uint_as_float(r.z << 16); x[5] = __uint_as_float(r.z & 0xffff0000u);
+        x[6] = __uint_as_float(r.w << 16); x[7] = __uint_as_float(r.w & 0xffff0000u);
+    }
+    __device__ static uint4 pack(const float *x)
+    {
+        __nv_bfloat162 a = __floats2bfloat162_rn(x[0], x[1]), b = __floats2bfloat162_rn(x[2], x[3]);
+        __nv_bfloat162 c = __floats2bfloat162_rn(x[4], x[5]), d = __floats2bfloat162_rn(x[6], x[7]);
+        return make_uint4(*reinterpret_cast<uint32_t *>(&a), *reinterpret_cast<uint32_t *>(&b),
+                          *reinterpret_cast<uint32_t *>(&c), *reinterpret_cast<uint32_t *>(&d));
+    }
+};
+
+struct DecodePlanArgs {
+    const int64_t *row_offset;
+    int32_t *len;
+    const int32_t *cap;
+    const int32_t *len0;  // [B*L] rows kept by compaction        } only with
+    int32_t *gen;         // [B*L] tokens decoded so far          } decode-time
+    int32_t *slot_ring;   // [B*L][distance + 1] rows of recent tokens } pruning
+    int64_t total_cap_rows;
+    int evict_distance, N, L, layer_begin, nl, nact;
+    bool append;
+};
+
+inline DecodePlanArgs decode_plan_args(const pkv_shape *s, const pkv_cache *c, bool append, int layer_begin, int nl)
+{
+    DecodePlanArgs a;
+    a.row_offset = c->row_offset; a.len = c->len; a.cap = c->cap;
+    a.len0 = c->len0; a.gen = c->gen; a.slot_ring = c->slot_ring;
+    a.total_cap_rows = c->total_cap_rows;
+    a.evict_distance = c->evict_distance;
+    a.N = s->prompt_len; a.L = s->layers;
+    a.layer_begin = layer_begin; a.nl = nl; a.nact = s->batch * nl;
+    a.append = append;
+    return a;
+}
+
+// What this step does to active segment si: the rows it attends over (the new row included),
+// or -1 when the segment cannot take the row (full, never compacted, or outside the cache);
+// the row the new token is written to; the length afterwards.  Without decode-time pruning
+// the new row is appended.  With it (Sec. 3.1: prune at a fixed distance to the latest token,
+// keep the layer's proportion): when generated token g would push the layer past
+// floor(len0 * (N + g + 1) / N) rows and token g - distance is still cached, the new row
+// takes that token's slot instead and the length stays.
+struct SegPlan {
+    int rows, dst, len_after;
+    bool evict;
+    int64_t off;
+};
+__device__ __forceinline__ SegPlan segment_plan(const DecodePlanArgs &a, int si)
+{
+    const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
+    const int ln = a.len[seg], cp = a.cap[seg];
+    SegPlan p;
+    p.off = a.row_offset[seg];
+    p.evict = false;
+    p.dst = ln;
+    bool ok = ln >= 1 && p.off >= 0 && p.off + cp <= a.total_cap_rows && ln <= cp;
+    if (!a.append) {  // nothing to append: attend over the rows that are there
+        p.dst = 0x3fffffff;
+        p.rows = ok ? ln : -1;
+        p.len_after = p.rows;
+        return p;
+    }
+    const int d = a.evict_distance;
+    if (ok && d > 0) {
+        const int g = a.gen[seg];
+        const int64_t target = ((int64_t)a.len0[seg] * ((int64_t)a.N + g + 1)) / a.N;
+        if ((int64_t)ln + 1 > target && g >= d) {
+            const int r = a.slot_ring[(size_t)seg * (d + 1) + (g - d) % (d + 1)];
+            if (r >= 0 && r < ln) {
+                p.evict = true;
+                p.dst = r;
+            }
+        }
+    }
+    if (!p.evict && ln >= cp) ok = false;  // appending needs head-room
+    p.rows = ok ? (p.evict ? ln : ln + 1) : -1;
+    p.len_after = p.rows;
+    return p;
+}
+// Writes what the step leaves for the next one: the length and, with pruning, the token's place.
+// (Only one thread of the call touches a segment's token count and slot ring.)
+__device__ __forceinline__ void segment_write(const DecodePlanArgs &a, int seg, int len_after, int dst, bool evict)
+{
+    a.len[seg] = len_after;
+    const int d = a.append ? a.evict_distance : 0;
+    if (d > 0) {
+        const int g = a.gen[seg];
+        int32_t *ring = a.slot_ring + (size_t)seg * (d + 1);
+        if (evict) ring[(g - d) % (d + 1)] = -1;  // the token d steps back gave up its slot
+        ring[g % (d + 1)] = dst;
+        a.gen[seg] = g + 1;
+    }
+}
+__device__ __forceinline__ void segment_advance(const DecodePlanArgs &a, int si, const SegPlan &sp)
+{
+    segment_write(a, (si / a.nl) * a.L + a.layer_begin + si % a.nl, sp.len_after, sp.dst, sp.evict);
+}
+
+}  // namespace pkv

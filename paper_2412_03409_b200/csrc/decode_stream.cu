@@ -18,7 +18,7 @@
 // (Merging inside the stream kernel instead, by the last CTA to arrive at a
 // counter, was measured slower: its fence, counter and loads wait behind the
 // other CTAs' bulk traffic, while the second kernel finds the memory system idle.)
-#include "common.cuh"
+#include "decode_plan.cuh"
 
 namespace pkv {
 
@@ -28,23 +28,15 @@ constexpr int kDynSmemMax = 226 * 1024;  // 227 KiB per CTA less the kernel's st
 constexpr uint32_t kSpinLimit = 1u << 22;
 constexpr float kLog2eD = 1.4426950408889634f;
 
-struct DecodeArgs {
+struct DecodeArgs : DecodePlanArgs {
     const void *q, *k_new, *v_new;
     void *ck, *cv, *out;
-    const int64_t *row_offset;
-    int32_t *len;
-    const int32_t *cap;
     const float *layer_scale;
     float *scratch;   // partial slots
     int *plan;        // [nact] int4 records written by the stream kernel for the merge kernel
     int32_t *dev_status;
-    const int32_t *len0;  // [B*L] rows kept by compaction        } only with
-    int32_t *gen;         // [B*L] tokens decoded so far          } decode-time
-    int32_t *slot_ring;   // [B*L][distance + 1] rows of recent tokens } pruning
-    int evict_distance, N;
-    int L, H, layer_begin, nl, nact, nseg_total, nstages, nwarps;
+    int H, nseg_total, nstages, nwarps;
     uint32_t row_bytes;
-    int64_t total_cap_rows;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p)
@@ -97,38 +89,6 @@ __device__ __forceinline__ void consumer_barrier(int nthreads)
     asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
 }
 
-template <typename T> struct Vec;
-template <> struct Vec<float> {
-    static constexpr int VE = 4;
-    __device__ static void unpack(const uint4 &r, float *x)
-    {
-        x[0] = __uint_as_float(r.x); x[1] = __uint_as_float(r.y);
-        x[2] = __uint_as_float(r.z); x[3] = __uint_as_float(r.w);
-    }
-    __device__ static uint4 pack(const float *x)
-    {
-        return make_uint4(__float_as_uint(x[0]), __float_as_uint(x[1]), __float_as_uint(x[2]),
-                          __float_as_uint(x[3]));
-    }
-};
-template <> struct Vec<__nv_bfloat16> {
-    static constexpr int VE = 8;
-    __device__ static void unpack(const uint4 &r, float *x)
-    {
-        x[0] = __uint_as_float(r.x << 16); x[1] = __uint_as_float(r.x & 0xffff0000u);
-        x[2] = __uint_as_float(r.y << 16); x[3] = __uint_as_float(r.y & 0xffff0000u);
-        x[4] = __uint_as_float(r.z << 16); x[5] = __uint_as_float(r.z & 0xffff0000u);
-        x[6] = __uint_as_float(r.w << 16); x[7] = __uint_as_float(r.w & 0xffff0000u);
-    }
-    __device__ static uint4 pack(const float *x)
-    {
-        __nv_bfloat162 a = __floats2bfloat162_rn(x[0], x[1]), b = __floats2bfloat162_rn(x[2], x[3]);
-        __nv_bfloat162 c = __floats2bfloat162_rn(x[4], x[5]), d = __floats2bfloat162_rn(x[6], x[7]);
-        return make_uint4(*reinterpret_cast<uint32_t *>(&a), *reinterpret_cast<uint32_t *>(&b),
-                          *reinterpret_cast<uint32_t *>(&c), *reinterpret_cast<uint32_t *>(&d));
-    }
-};
-
 // U units over G CTAs (G <= U): the first U % G CTAs take U / G + 1 units, the rest U / G.
 __device__ __forceinline__ int first_unit(int c, int q, int rem) { return c * q + min(c, rem); }
 __device__ __forceinline__ int unit_owner(int u, int q, int rem)
@@ -174,51 +134,6 @@ int selftest_wait_stream(int32_t *dev_status, cudaStream_t st)
     return check_launch("selftest_wait_stream_kernel");
 }
 
-// What this step does to active segment si: the rows it attends over (the new row included),
-// or -1 when the segment cannot take the row (full, never compacted, or outside the cache);
-// the row the new token is written to; the length afterwards.  Without decode-time pruning
-// the new row is appended.  With it (Sec. 3.1: prune at a fixed distance to the latest token,
-// keep the layer's proportion): when generated token g would push the layer past
-// floor(len0 * (N + g + 1) / N) rows and token g - distance is still cached, the new row
-// takes that token's slot instead and the length stays.
-struct SegPlan {
-    int rows, dst, len_after;
-    bool evict;
-    int64_t off;
-};
-__device__ __forceinline__ SegPlan segment_plan(const DecodeArgs &a, int si)
-{
-    const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
-    const int ln = a.len[seg], cp = a.cap[seg];
-    SegPlan p;
-    p.off = a.row_offset[seg];
-    p.evict = false;
-    p.dst = ln;
-    bool ok = ln >= 1 && p.off >= 0 && p.off + cp <= a.total_cap_rows && ln <= cp;
-    if (!a.k_new) {  // nothing to append: attend over the rows that are there
-        p.dst = 0x3fffffff;
-        p.rows = ok ? ln : -1;
-        p.len_after = p.rows;
-        return p;
-    }
-    const int d = a.evict_distance;
-    if (ok && d > 0) {
-        const int g = a.gen[seg];
-        const int64_t target = ((int64_t)a.len0[seg] * ((int64_t)a.N + g + 1)) / a.N;
-        if ((int64_t)ln + 1 > target && g >= d) {
-            const int r = a.slot_ring[(size_t)seg * (d + 1) + (g - d) % (d + 1)];
-            if (r >= 0 && r < ln) {
-                p.evict = true;
-                p.dst = r;
-            }
-        }
-    }
-    if (!p.evict && ln >= cp) ok = false;  // appending needs head-room
-    p.rows = ok ? (p.evict ? ln : ln + 1) : -1;
-    p.len_after = p.rows;
-    return p;
-}
-
 struct Ring {
     int slot, nstages;
     uint32_t phase;
@@ -236,7 +151,7 @@ struct Ring {
 template <typename T, int D, int LPR, int HPW, int UR, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) decode_stream_kernel(const DecodeArgs a)
 {
-    constexpr int VE = Vec<T>::VE;
+    constexpr int VE = RowVec<T>::VE;
     constexpr int NV = D / VE / LPR;  // vectors per lane
     constexpr int EPL = NV * VE;      // elements per lane
     constexpr int GPW = 32 / LPR;     // row groups per warp
@@ -452,7 +367,7 @@ __global__ void __launch_bounds__(MAXT, 1) decode_stream_kernel(const DecodeArgs
 #pragma unroll
                     for (int v = 0; v < NV; ++v) {
                         float x[VE];
-                        Vec<T>::unpack(*reinterpret_cast<const uint4 *>(qb + (size_t)h * D * sizeof(T) + (v * LPR + c) * 16), x);
+                        RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(qb + (size_t)h * D * sizeof(T) + (v * LPR + c) * 16), x);
 #pragma unroll
                         for (int i = 0; i < VE; ++i) {
                             if constexpr (!kQSmem) qf[hh][v * VE + i] = x[i] * sc;
@@ -490,7 +405,7 @@ __global__ void __launch_bounds__(MAXT, 1) decode_stream_kernel(const DecodeArgs
 #pragma unroll
                         for (int v = 0; v < NV; ++v) {
                             float x[VE];
-                            Vec<T>::unpack(*reinterpret_cast<const uint4 *>(q_held + hh * (int)(D * sizeof(T)) + v * LPR * 16), x);
+                            RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(q_held + hh * (int)(D * sizeof(T)) + v * LPR * 16), x);
 #pragma unroll
                             for (int i = 0; i < VE; ++i) qv[v * VE + i] = x[i] * q_scale;
                         }
@@ -502,7 +417,7 @@ __global__ void __launch_bounds__(MAXT, 1) decode_stream_kernel(const DecodeArgs
 #pragma unroll
                                 for (int v = 0; v < NV; ++v) {
                                     float x[VE];
-                                    Vec<T>::unpack(*reinterpret_cast<const uint4 *>(row + v * LPR * 16), x);
+                                    RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(row + v * LPR * 16), x);
 #pragma unroll
                                     for (int i = 0; i < VE; i += 2) {
                                         d0 = fmaf(qv[v * VE + i], x[i], d0);
@@ -524,7 +439,7 @@ __global__ void __launch_bounds__(MAXT, 1) decode_stream_kernel(const DecodeArgs
 #pragma unroll
                                 for (int v = 0; v < NV; ++v) {
                                     float x[VE];
-                                    Vec<T>::unpack(*reinterpret_cast<const uint4 *>(row + v * LPR * 16), x);
+                                    RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(row + v * LPR * 16), x);
 #pragma unroll
                                     for (int i = 0; i < VE; i += 2) {
                                         d0 = fmaf(qf[hh][v * VE + i], x[i], d0);
@@ -589,7 +504,7 @@ __global__ void __launch_bounds__(MAXT, 1) decode_stream_kernel(const DecodeArgs
 #pragma unroll
                             for (int v = 0; v < NV; ++v) {
                                 float x[VE];
-                                Vec<T>::unpack(*reinterpret_cast<const uint4 *>(row + v * LPR * 16), x);
+                                RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(row + v * LPR * 16), x);
 #pragma unroll
                                 for (int i = 0; i < VE; ++i)
                                     acc[hh][v * VE + i] = fmaf(pj, x[i], acc[hh][v * VE + i]);
@@ -645,7 +560,7 @@ __global__ void __launch_bounds__(MAXT, 1) decode_stream_kernel(const DecodeArgs
 #pragma unroll
                                 for (int i = 0; i < VE; ++i) x[i] = acc[hh][v * VE + i] * inv;
                                 *reinterpret_cast<uint4 *>(reinterpret_cast<T *>(a.out) + seg_vec +
-                                                           (size_t)h * D + (v * LPR + c) * VE) = Vec<T>::pack(x);
+                                                           (size_t)h * D + (v * LPR + c) * VE) = RowVec<T>::pack(x);
                             }
                         } else {
                             float *slot = a.scratch + ((size_t)(cta + si) * H + h) * kSlotStride;
@@ -747,15 +662,7 @@ __global__ void __launch_bounds__(kFinishWarps * 32) decode_finish_kernel(const 
         const int4 r = rec[si];
         if (r.x < 0) continue;  // could not take a row: reported and zero-filled by the stream kernel
         const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
-        a.len[seg] = r.x;
-        const int d = a.k_new ? a.evict_distance : 0;
-        if (d > 0) {  // only this thread touches the segment's token count and slot ring
-            const int g = a.gen[seg];
-            int32_t *ring = a.slot_ring + (size_t)seg * (d + 1);
-            if (r.w >> 30) ring[(g - d) % (d + 1)] = -1;  // the token d steps back gave up its slot
-            ring[g % (d + 1)] = r.w & 0x3fffffff;
-            a.gen[seg] = g + 1;
-        }
+        segment_write(a, seg, r.x, r.w & 0x3fffffff, (r.w >> 30) != 0);
     }
 
     const int groups = a.H / HG;
@@ -893,15 +800,7 @@ __global__ void __launch_bounds__(kFinishWarps * 32) decode_finish_small_kernel(
     // from here on r is the record as the finished stream kernel left it
     if (r.x < 0) return;  // could not take a row: reported and zero-filled by the stream kernel
     if (h == 0 && lane == 0) {
-        a.len[seg] = r.x;
-        const int d = a.k_new ? a.evict_distance : 0;
-        if (d > 0) {  // only this thread touches the segment's token count and slot ring
-            const int g = a.gen[seg];
-            int32_t *ring = a.slot_ring + (size_t)seg * (d + 1);
-            if (r.w >> 30) ring[(g - d) % (d + 1)] = -1;  // the token d steps back gave up its slot
-            ring[g % (d + 1)] = r.w & 0x3fffffff;
-            a.gen[seg] = g + 1;
-        }
+        segment_write(a, seg, r.x, r.w & 0x3fffffff, (r.w >> 30) != 0);
     }
     if (r.z <= 1) return;  // one CTA covered the segment and wrote its output
     const float inv = 1.f / z;
@@ -974,16 +873,15 @@ static int launch_variant(const DecodeArgs &a, int sms, cudaStream_t st)
     return PKV_OK;
 }
 
-// Returns PKV_OK, an error, or -1 when this shape is outside what the streaming kernel covers.
-int launch_decode_stream(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn,
-                         const void *vn, const float *scale, int lb, int le, void *out,
-                         int32_t *dev_status, void *ws, cudaStream_t st)
+// Rows per unit, ring stages, lanes per row and heads per warp for this call; false when the shape is
+// outside what the streaming kernel covers.
+static bool stream_variant(const pkv_shape *s, int nact, int &ur, int &nstages, int &lpr, int &hpw)
 {
-    const int H = s->heads, D = s->head_dim, nl = le - lb, nact = s->batch * nl;
-    if (nact > kMaxActive || H > 64) return -1;
+    const int H = s->heads, D = s->head_dim;
+    if (nact > kMaxActive || H > 64) return false;
     const size_t es = esize(s);
     const uint32_t row_bytes = (uint32_t)((size_t)H * D * es);
-    int ur = 0, nstages = 0;
+    ur = 0;
     for (int cand = 8; cand >= 2 && !ur; cand >>= 1) {  // rows per unit: as many as leave three ring stages
         int ns = kMaxStages;
         while (ns >= 3 && stream_smem_bytes(ns, cand, row_bytes, nact) > (size_t)kDynSmemMax) --ns;
@@ -992,44 +890,48 @@ int launch_decode_stream(const pkv_shape *s, pkv_cache *c, const void *q, const 
             nstages = ns;
         }
     }
-    if (!ur) return -1;
+    if (!ur) return false;
+    // (lanes per row, heads per warp): at most 17 warps, and few enough registers of per-head
+    // state that each SM sub-partition's register file holds its warps.
+    const int vec_per_head = D / (int)(16 / es);
+    lpr = 8;
+    hpw = H <= 16 ? 1 : (H <= 32 ? 2 : 4);
+    if (H > 16 && vec_per_head >= 16) lpr = 16;
+    return vec_per_head >= lpr && H % hpw == 0;
+}
 
-    static int sm_count[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int sms = (dev >= 0 && dev < 64) ? sm_count[dev] : 0;
-    if (!sms) {
-        cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) {
-            set_cuda_error(e, "cudaDeviceGetAttribute(sm count)");
-            return PKV_ERR_CUDA;
-        }
-        if (dev >= 0 && dev < 64) sm_count[dev] = sms;
-    }
+bool decode_stream_covers(const pkv_shape *s, int nact)
+{
+    int ur, nstages, lpr, hpw;
+    return stream_variant(s, nact, ur, nstages, lpr, hpw);
+}
+
+// Returns PKV_OK, an error, or -1 when this shape is outside what the streaming kernel covers.
+int launch_decode_stream(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn,
+                         const void *vn, const float *scale, int lb, int le, void *out,
+                         int32_t *dev_status, void *ws, cudaStream_t st)
+{
+    const int H = s->heads, D = s->head_dim, nl = le - lb, nact = s->batch * nl;
+    int ur = 0, nstages = 0, lpr = 0, hpw = 0;
+    if (!stream_variant(s, nact, ur, nstages, lpr, hpw)) return -1;
+    const uint32_t row_bytes = (uint32_t)((size_t)H * D * esize(s));
+
+    int sms = sm_count();
+    if (sms <= 0) return PKV_ERR_CUDA;
     if (sms > 256) sms = 256;
 
     DecodeArgs a;
+    static_cast<DecodePlanArgs &>(a) = decode_plan_args(s, c, kn != nullptr, lb, nl);
     a.q = q; a.k_new = kn; a.v_new = vn; a.ck = c->k; a.cv = c->v; a.out = out;
-    a.row_offset = c->row_offset; a.len = c->len; a.cap = c->cap;
     a.layer_scale = scale; a.dev_status = dev_status;
     a.plan = (int *)ws;
     a.scratch = (float *)((unsigned char *)ws + plan_bytes(nact));
-    a.L = s->layers; a.H = H; a.layer_begin = lb; a.nl = nl; a.nact = nact;
+    a.H = H;
     a.nseg_total = s->batch * s->layers; a.nstages = nstages; a.row_bytes = row_bytes;
-    a.total_cap_rows = c->total_cap_rows;
-    a.evict_distance = c->evict_distance;
-    a.len0 = c->len0; a.gen = c->gen; a.slot_ring = c->slot_ring;
-    a.N = s->prompt_len;
 
     const bool bf = s->dtype == PKV_BF16;
-    const int vec_per_head = D / (int)(16 / es);
-    // (lanes per row, heads per warp): at most 17 warps, and few enough registers of per-head
-    // state that each SM sub-partition's register file holds its warps.  (The last template
-    // argument is the block-size bound a variant is compiled for: 9, 12 or 17 warps, the smaller
-    // ones with room for more registers per thread.)
-    int lpr = 8, hpw = H <= 16 ? 1 : (H <= 32 ? 2 : 4);
-    if (H > 16 && vec_per_head >= 16) lpr = 16;
-    if (vec_per_head < lpr || H % hpw != 0) return -1;
+    // (The last template argument is the block-size bound a variant is compiled for: 9, 12 or 17 warps, the
+    // smaller ones with room for more registers per thread.)
     a.nwarps = H / hpw;
 #define PKV_V(T, DD, LPR, HPW, UR, MAXT)                                       \
     if (lpr == LPR && hpw == HPW && ur == UR && (a.nwarps + 1) * 32 <= MAXT) \

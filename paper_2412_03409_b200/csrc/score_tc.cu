@@ -435,18 +435,8 @@ int launch_score_tc(const pkv_shape *s, const void *q, pkv_strides qs, const voi
     a.nseg = B * L;
     a.group = head_group(B * L * H, N, s->head_dim, 2);
 
-    static int sm_count[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int sms = (dev >= 0 && dev < 64) ? sm_count[dev] : 0;
-    if (!sms) {
-        cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) {
-            set_cuda_error(e, "cudaDeviceGetAttribute(sm count)");
-            return PKV_ERR_CUDA;
-        }
-        if (dev >= 0 && dev < 64) sm_count[dev] = sms;
-    }
+    const int sms = sm_count();
+    if (sms <= 0) return PKV_ERR_CUDA;
     int rc;
     if (lse) {
         const size_t n = rows * a.Npad;

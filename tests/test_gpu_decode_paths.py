@@ -1,0 +1,127 @@
+"""Decode calls that take each of the library's kernels, against the oracle on the cache as it stands
+(needs a B200).  Few (segment, head) pairs: the cluster kernel; from four pairs per SM (592) the
+per-head kernel, the row-split kernel (long segments, pruning) or, above 64 heads, the two-kernel path."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import to_np32
+from paper_2412_03409_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+# fp32: sums of a few thousand terms; bf16: outputs are averages of N(0, 1) values, |out| < 4, so one
+# rounding to bf16 is at most 2^-9 * 4 = 8e-3
+TOL = {torch.float32: 2e-5, torch.bfloat16: 8e-3}
+
+CASES = [  # B, L, H, D, N, rows per layer, dtype, evict_distance
+    (1, 2, 1, 64, 40, 1, torch.bfloat16, 0),          # single cached row per layer
+    (1, 1, 32, 128, 300, 33, torch.bfloat16, 0),      # a row more than one round of a cluster's CTA
+    (2, 3, 5, 64, 300, 131, torch.float32, 0),
+    (1, 1, 3, 128, 3000, 2900, torch.float32, 0),     # eight CTAs of many rounds each
+    (3, 1, 7, 64, 2500, 1111, torch.bfloat16, 0),
+    (1, 4, 80, 64, 200, 50, torch.bfloat16, 0),       # above the row-split kernel's 64 heads
+    (2, 2, 4, 128, 64, 16, torch.bfloat16, 3),        # pruning: reused slots are skipped
+    (1, 3, 9, 64, 90, 30, torch.float32, 2),
+    (1, 20, 32, 128, 200, 60, torch.bfloat16, 3),     # 640 pairs with pruning: row-split kernel
+    (1, 20, 32, 64, 1100, 1050, torch.bfloat16, 0),   # 640 pairs, long segments: row-split kernel
+    (1, 9, 72, 64, 100, 20, torch.bfloat16, 0),       # 648 pairs, 72 heads: two-kernel path when segments are long
+    (1, 9, 72, 64, 1300, 1200, torch.bfloat16, 0),
+]
+
+
+def _ready(B, L, H, D, N, rows, dtype, d, T, seed=3):
+    from paper_2412_03409_b200.session import Session
+    g = torch.Generator(device="cuda").manual_seed(seed + N)
+    scale = np.full(L, 1.0 / np.sqrt(D), np.float32)
+    s = Session(B, L, H, D, N, dtype, scale, decode_cap=T, max_budget_rows=L * rows, evict_distance=d, poison=True)
+    scores = np.stack([wl.synthetic_scores(L, N, seed + b) for b in range(B)])
+    s.search(L * rows, scores=torch.from_numpy(scores).cuda())
+    k, v = (torch.randn(B, L, H, N, D, device="cuda", generator=g).to(dtype) for _ in range(2))
+    s.compact(k, v)
+    tok = [[torch.randn(B, L, H, D, device="cuda", generator=g).to(dtype) for _ in range(3)] for _ in range(T)]
+    return s, scale, tok
+
+
+@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d", CASES)
+def test_decode_steps_match_the_oracle(B, L, H, D, N, rows, dtype, d):
+    T = 8 if d else 2
+    s, scale, tok = _ready(B, L, H, D, N, rows, dtype, d, T)
+    ring = {i: np.full(d + 1, -1, np.int32) for i in range(B * L)}
+    len0 = s.cache.len.cpu().numpy()
+    off = s.cache.row_offset.cpu().numpy()
+    segs = range(B * L) if B * L * rows < 4000 else [0, B * L // 2, B * L - 1]
+    for t in range(T):
+        before = s.cache.len.cpu().numpy()
+        rows_k, rows_v = to_np32(s.cache.k), to_np32(s.cache.v)
+        q, kn, vn = tok[t]
+        got = to_np32(s.decode(q, kn, vn))
+        after = s.cache.len.cpu().numpy()
+        new_k, new_v = to_np32(s.cache.k), to_np32(s.cache.v)
+        for i in segs:
+            b, l, n, o = i // L, i % L, int(before[i]), int(off[i])
+            dst, n_after = n, n + 1
+            if d:
+                dst, _, n_after = oracle.decode_slot(int(len0[i]), N, t, n, d, ring[i])
+            want_k, want_v = rows_k[o:o + n_after].copy(), rows_v[o:o + n_after].copy()
+            want_k[dst], want_v[dst] = to_np32(kn[b, l]), to_np32(vn[b, l])
+            assert after[i] == n_after
+            np.testing.assert_array_equal(new_k[o:o + n_after], want_k)
+            np.testing.assert_array_equal(new_v[o:o + n_after], want_v)
+            ref = oracle.decode_attn(to_np32(q[b, l]), want_k, want_v, float(scale[l]))
+            assert np.abs(got[b, l] - ref).max() <= TOL[dtype], (t, i)
+    assert s.status.cpu().tolist() == [0] * B
+    # nothing appended: the same query over the rows that are there; lengths stay
+    if H <= 64:
+        q = tok[0][0]
+        n = s.cache.len.clone()
+        got = to_np32(s.decode(q, None, None))
+        assert torch.equal(n, s.cache.len)
+        for i in segs:
+            b, l, o = i // L, i % L, int(off[i])
+            ref = oracle.decode_attn(to_np32(q[b, l]), new_k[o:o + int(n[i])], new_v[o:o + int(n[i])], float(scale[l]))
+            assert np.abs(got[b, l] - ref).max() <= TOL[dtype]
+
+
+@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d", [CASES[4], CASES[6], CASES[8], CASES[9]])
+@pytest.mark.parametrize("byte", [0x7f, 0xff])
+def test_replay_and_stale_workspace(B, L, H, D, N, rows, dtype, d, byte):
+    """A captured call replayed token after token, over a workspace that holds anything, gives bit for
+    bit what separate calls give; a segment without rows is reported and zero."""
+    T = 6
+    a, _, tok = _ready(B, L, H, D, N, rows, dtype, d, T)
+    b, _, _ = _ready(B, L, H, D, N, rows, dtype, d, T)
+    warm, _, _ = _ready(B, L, H, D, N, rows, dtype, d, T)
+    buf = [x.clone() for x in tok[0]]
+    warm.decode(*buf)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        b.decode(*buf)
+    b.ws_decode.fill_(byte)
+    for t in range(T):
+        for x, y in zip(buf, tok[t]):
+            x.copy_(y)
+        if t == T - 1:
+            for s in (a, b):
+                s.cache.len[B * L - 1] = 0
+        graph.replay()
+        ref = a.decode(*tok[t])
+        torch.cuda.synchronize()
+        assert torch.equal(b.out, ref), t
+        assert torch.equal(a.cache.len, b.cache.len), t
+    from paper_2412_03409_b200 import api
+    assert a.status.cpu().tolist() == b.status.cpu().tolist() == [0] * (B - 1) + [api.DEV_CAPACITY]
+    assert (a.out[B - 1, L - 1] == 0).all() and int(a.cache.len[B * L - 1]) == 0
+
+
+def test_refused_calls_stay_refused():
+    """Pruning and attending without appending are for shapes within the row-split kernel's limits."""
+    from paper_2412_03409_b200 import api
+    s, _, tok = _ready(1, 1, 72, 64, 60, 20, torch.bfloat16, 2, 2)
+    with pytest.raises(api.PrefixKVError):
+        s.decode(*tok[0])
+    s, _, tok = _ready(1, 1, 72, 64, 60, 20, torch.bfloat16, 0, 2)
+    with pytest.raises(api.PrefixKVError):
+        s.decode(tok[0][0], None, None)
