@@ -65,13 +65,6 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t &p0, uint32_t 
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p2) : "f"(sy), "f"(sx));
 }
 
-// Bounded wait of a whole warp: every lane learns when any lane's wait has run out.
-__device__ __forceinline__ void warp_wait(uint64_t *bar, uint32_t parity, bool &dead, int *abort_flag)
-{
-    bar_wait(bar, parity, dead, abort_flag);
-    dead = __any_sync(0xffffffffu, dead);
-}
-
 // An accumulator buffer holds one unit of a tile: UN columns, in NACC partial accumulators.
 template <int D> struct Unit {
     static constexpr int UN = D == 128 ? 128 : 64;

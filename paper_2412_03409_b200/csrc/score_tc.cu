@@ -62,7 +62,7 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     __shared__ int q_item[kItemQ];  // the loader's announcements: an item number, or -1 for the end
     __shared__ __align__(16) float s_lse[2][4][TT];  // [accumulator][reader warp][query of the tile]
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const CUtensorMap *map_stat = PASS == 1 ? &map_q : &map_k;
     const CUtensorMap *map_strm = PASS == 1 ? &map_k : &map_q;
     const int nsh = a.nseg * a.H;
@@ -140,42 +140,46 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             }
         }
     } else if (warp == 1) {
-        // ---- MMA issuer -------------------------------------------------------------------------
-        if (lane == 0) {
-            bool dead = false;
-            uint32_t a_phase = 0;
-            Ring2 rb{0, 0u}, rs{0, 0u}, rq{0, 0u};
-            for (;;) {
-                bar_wait(q_full + rq.idx, rq.phase, dead, &s_abort);
+        // ---- MMA issuer: the whole warp walks the stream, one elected lane issues, so that the operands'
+        // descriptors are formed in uniform registers ahead of each instruction -----------------------------
+        bool dead = false;
+        uint32_t a_phase = 0;
+        Ring2 rb{0, 0u}, rs{0, 0u}, rq{0, 0u};
+        const uint64_t da = smem_desc(saddr(sA)), db = smem_desc(saddr(sB));
+        for (;;) {
+            warp_wait(q_full + rq.idx, rq.phase, dead, &s_abort);
+            if (dead) break;
+            const int w = __shfl_sync(0xffffffffu, *(volatile int *)(q_item + rq.idx), 0);
+            __syncwarp();
+            if (lane == 0) bar_arrive(q_empty + rq.idx);
+            rq.next(kItemQ);
+            if (w < 0) break;
+            int sh, t;
+            decode_item<PASS>(w, nsh, a.tiles, a.group, sh, t);
+            warp_wait(a_full, a_phase, dead, &s_abort);
+            a_phase ^= 1u;
+            const int count = PASS == 1 ? t + 1 : a.tiles - t;
+            for (int jj = 0; jj < count && !dead; ++jj) {
+                warp_wait(b_full + rb.idx, rb.phase, dead, &s_abort);
+                warp_wait(s_empty + rs.idx, rs.phase ^ 1u, dead, &s_abort);
                 if (dead) break;
-                const int w = q_item[rq.idx];
-                bar_arrive(q_empty + rq.idx);
-                rq.next(kItemQ);
-                if (w < 0) break;
-                int sh, t;
-                decode_item<PASS>(w, nsh, a.tiles, a.group, sh, t);
-                bar_wait(a_full, a_phase, dead, &s_abort);
-                a_phase ^= 1u;
-                const int count = PASS == 1 ? t + 1 : a.tiles - t;
-                for (int jj = 0; jj < count && !dead; ++jj) {
-                    bar_wait(b_full + rb.idx, rb.phase, dead, &s_abort);
-                    bar_wait(s_empty + rs.idx, rs.phase ^ 1u, dead, &s_abort);
-                    if (dead) break;
-                    fence_after();
-                    const uint32_t d_tmem = tmem_base + (uint32_t)rs.idx * TT;
-                    const uint32_t a_addr = saddr(sA), b_addr = saddr(sB + rb.idx * TILE);
+                fence_after();
+                const uint32_t d_tmem = tmem_base + (uint32_t)rs.idx * TT;
+                const uint64_t dk = desc_add(db, rb.idx * TILE);
+                if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < D / 16; ++k) {
                         const uint32_t off = (uint32_t)(k / 4) * HALF + (uint32_t)(k % 4) * 32;
-                        mma_bf16(d_tmem, smem_desc(a_addr + off), smem_desc(b_addr + off), kIdesc, k > 0 ? 1u : 0u);
+                        mma_bf16(d_tmem, desc_add(da, off), desc_add(dk, off), kIdesc, k > 0 ? 1u : 0u);
                     }
                     mma_commit(b_empty + rb.idx);  // the streamed stage is free once these MMAs retire
                     mma_commit(s_full + rs.idx);   // and the accumulator is ready to be read
-                    rb.next(kStagesB);
-                    rs.next(2);
+                    if (jj == count - 1) mma_commit(a_empty);  // the stationary tile may be replaced
                 }
-                if (!dead) mma_commit(a_empty);     // the stationary tile may be replaced
+                rb.next(kStagesB);
+                rs.next(2);
             }
+            if (dead) break;
         }
     } else {
         // ---- accumulator readers: one TMEM lane (tile row) per thread ----------------------------

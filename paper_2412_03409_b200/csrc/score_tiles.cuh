@@ -52,6 +52,13 @@ __device__ __forceinline__ void bar_wait(uint64_t *bar, uint32_t parity, bool &d
     atomicExch(abort_flag, 1);
 }
 
+// Bounded wait of a whole warp: every lane learns when any lane's wait has run out.
+__device__ __forceinline__ void warp_wait(uint64_t *bar, uint32_t parity, bool &dead, int *abort_flag)
+{
+    bar_wait(bar, parity, dead, abort_flag);
+    dead = __any_sync(0xffffffffu, dead);
+}
+
 __device__ __forceinline__ void tma_load_5d(void *dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1,
                                             int c2, int c3, int c4)
 {
@@ -160,6 +167,27 @@ __device__ __forceinline__ float ex2(float x)
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// Two fp32 operations in one instruction (same rounding as the scalar ones): half the issue slots.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, z, w;\n\t"
+        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
+        "fma.rn.f32x2 w, x, y, z;\n\tmov.b64 {%0, %1}, w;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, w;\n\t"
+        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+        "add.rn.f32x2 w, x, y;\n\tmov.b64 {%0, %1}, w;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
 __device__ __forceinline__ float max3(float a, float b, float c)
 {
     float d;
@@ -201,15 +229,14 @@ __device__ __forceinline__ void lse_block(float (&v)[NC], float sc, bool fast, f
     }
     const float cmax = max3(c2[0], c2[1], fmaxf(v[NC - 2], v[NC - 1]));
     const float nm = fmaxf(run_max, fast ? cmax * sc : cmax);  // finite: column 0 is never masked
-    float p4[4] = {0.f, 0.f, 0.f, 0.f};
-    if (fast) {
+    const float mul = fast ? sc : 1.f;  // (the other way v is scaled already)
+    float2 p[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-        for (int i = 0; i < NC; ++i) p4[i & 3] += ex2(fmaf(v[i], sc, -nm));
-    } else {
-#pragma unroll
-        for (int i = 0; i < NC; ++i) p4[i & 3] += ex2(v[i] - nm);
+    for (int i = 0; i < NC; i += 2) {
+        const float2 x = fma2(make_float2(v[i], v[i + 1]), make_float2(mul, mul), make_float2(-nm, -nm));
+        p[(i >> 1) & 1] = add2(p[(i >> 1) & 1], make_float2(ex2(x.x), ex2(x.y)));
     }
-    run_sum = fmaf(run_sum, ex2(run_max - nm), (p4[0] + p4[1]) + (p4[2] + p4[3]));
+    run_sum = fmaf(run_sum, ex2(run_max - nm), (p[0].x + p[0].y) + (p[1].x + p[1].y));
     run_max = nm;
 }
 
@@ -220,19 +247,22 @@ template <int NC>
 __device__ __forceinline__ float colsum_block(const float (&v)[NC], const float *lse, float sc, bool edge, int lane)
 {
     const float4 *lp = reinterpret_cast<const float4 *>(lse);
-    float p4[4] = {0.f, 0.f, 0.f, 0.f};
+    float2 p[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
     for (int i4 = 0; i4 < NC / 4; ++i4) {
         const float4 ls = lp[i4];
-        const float lv[4] = {ls.x, ls.y, ls.z, ls.w};
+        const int i = i4 * 4;
+        const float2 x = fma2(make_float2(v[i], v[i + 1]), make_float2(sc, sc), make_float2(-ls.x, -ls.y));
+        const float2 y = fma2(make_float2(v[i + 2], v[i + 3]), make_float2(sc, sc), make_float2(-ls.z, -ls.w));
+        float e[4] = {ex2(x.x), ex2(x.y), ex2(y.x), ex2(y.y)};
+        if (edge) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = i4 * 4 + u;
-            const float p = ex2(fmaf(v[i], sc, -lv[u]));
-            p4[u] += (!edge || i >= lane) ? p : 0.f;
+            for (int u = 0; u < 4; ++u) e[u] = i + u >= lane ? e[u] : 0.f;
         }
+        p[0] = add2(p[0], make_float2(e[0], e[1]));
+        p[1] = add2(p[1], make_float2(e[2], e[3]));
     }
-    return (p4[0] + p4[1]) + (p4[2] + p4[3]);
+    return (p[0].x + p[0].y) + (p[1].x + p[1].y);
 }
 
 // Work item w -> (segment-head sh, tile t).  CTAs take items in order from a counter.  Heads come in
