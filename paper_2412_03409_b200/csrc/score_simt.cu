@@ -169,7 +169,9 @@ __global__ void head_mean_kernel(const float *__restrict__ partial, int H, int N
     size_t seg = i / N;
     int n = (int)(i % N);
     float t = 0.f;
-    for (int h = 0; h < H; ++h) t += partial[(seg * H + h) * N + n];
+    const float *p = partial + seg * H * (size_t)N + n;
+#pragma unroll 16
+    for (int h = 0; h < H; ++h) t += __ldg(p + (size_t)h * N);
     scores[i] = t / (float)H;
 }
 

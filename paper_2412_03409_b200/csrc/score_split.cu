@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const Spl
                 for (int cb = max(diag ? warp : 0, u * U::BLOCKS); cb < (u + 1) * U::BLOCKS; ++cb) {
                     float v[32];
                     load_logits<D>(lane_addr + rs.idx * kBuf + (cb - u * U::BLOCKS) * 32, v);
-                    col_sum += colsum_block<32>(v, lse + cb * 32, sc, diag && cb == warp, lane);
+                    col_sum += colsum_block<32, 0>(v, lse + cb * 32, sc, diag && cb == warp, lane);
                 }
                 release();
             }
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const Spl
 #pragma unroll
                                 for (int i = 0; i < 32; ++i) v[i] = i <= lane ? v[i] : -INFINITY;
                             }
-                            lse_block<32>(v, sc, sc > 0.f, run_max, run_sum);
+                            lse_block<32, 0>(v, sc, sc > 0.f, run_max, run_sum);
                         }
                         release();
                     }

@@ -11,15 +11,27 @@
 // thread owns one query row and keeps its running max / sum in registers; keys in pass 2, so
 // a thread owns one key and its column sum needs no cross-thread reduction or atomics.
 //
-// Roles per CTA (192 threads): warp 0 lane 0 issues TMA, warp 1 owns tensor memory and its
-// lane 0 issues the MMAs, warps 2-5 read the accumulator (tcgen05.ld, one TMEM lane quarter
-// per warp) and do the exponentials.  Two accumulators alternate so that the MMAs of tile
-// j + 1 overlap the exponentials of tile j; two CTAs share an SM.  Work items (one stationary
-// tile and the tiles streamed against it) come from a device counter: the TMA thread takes the
-// next number and announces it to the other roles through a four-entry shared-memory queue,
-// so CTAs that run faster do more.  Every mbarrier wait is bounded: when one runs out the CTA
-// stops waiting, sets the call's abort word (the head mean then writes NaN for every score, which
-// the selection stage reports as PKV_DEV_BAD_SCORE) and still releases its tensor memory.
+// Roles per CTA (ten warps): warp 0 lane 0 issues TMA, warp 1 owns tensor memory and issues the MMAs,
+// warps 2-9 read the accumulators (tcgen05.ld, one TMEM lane quarter per warp) and do the
+// exponentials.  Two accumulators alternate, each read by a set of four warps, so that the MMAs of
+// tile j + 1 overlap the exponentials of tile j; the two sets' parts of an item's result meet in shared
+// memory.  Two CTAs share an SM.  Work items (one stationary tile and the tiles streamed against it)
+// come from a device counter, or by position where that serves as well: the TMA thread takes the
+// next number and announces it to the other roles through a four-entry shared-memory queue.  Every
+// mbarrier wait is bounded: when one runs out the CTA stops waiting, sets the call's abort word (the
+// head mean then writes NaN for every score, which the selection stage reports as
+// PKV_DEV_BAD_SCORE) and still releases its tensor memory.
+//
+// What bounds it: one exponential per logit per pass, 1024 clocks of the special-function unit for a
+// tile against 512 of the tensor pipe.  A quarter of them are therefore computed on the FMA pipe (a
+// degree-5 polynomial, add_exp2), and the arithmetic around them is packed two to an instruction.
+// Clocks a tile at 16384 tokens, 32 heads: 1340 with neither (issue slots 32 % used after packing), 1080
+// now (special-function unit 67-77 % busy, issue slots 54-60 %, FMA pipe 50 %).  Time of a pass pair, 64
+// heads of 16384 tokens / 1024 of 640: four reader warps and no polynomial 5168 / 191 us, a quarter
+// polynomial 4490 / 184; eight reader warps without it 4758 / 191, with an eighth 4465 / 187, a quarter
+// 4417 / 185, three eighths 4624 / 187.  A row read from tensor memory in quarters with the next on its
+// way 4650 / 191; one CTA per SM with sixteen reader warps, two stationary and four streamed stages
+// 4370 / 208.
 #include "score_tiles.cuh"
 
 namespace pkv {
@@ -27,22 +39,31 @@ namespace pkv {
 namespace {
 
 constexpr int kStagesB = 2;        // streamed-operand stages
+constexpr int kPoly1 = 2, kPoly2 = 2;  // pairs of exponentials in eight on the FMA pipe, pass 1 and 2
 
 struct ScoreArgs {
     const float *layer_scale;
-    float *lse2;     // [B*L*H][Npad] log2-sum-exp of scaled logits, +inf beyond N
+    float *lse2;         // pass 1 out: [B*L*H][Npad] log2-sum-exp of scaled logits, +inf beyond N
+    const float *lse_in; // pass 2: the caller's [B*L*H][N] natural-log sum-exp, or NULL (lse2 is taken)
     float *partial;  // [B*L*H][N] per-head column sums
     int32_t *abort_word;  // device word set when a bounded wait runs out: the head mean then writes NaN scores
     int *next_item;       // [2] work counters, one per pass; zeroed, with the abort word, before the first pass
     int L, H, N, Npad, tiles, nseg, group;
+    bool counted;      // items come from the counters; otherwise they are dealt out by position
+    bool clear_abort;  // this launch is the call's first and nothing has zeroed the abort word
 };
 
 constexpr int kItemQ = 4;  // item numbers in flight between the loader and the other roles
+constexpr int kReaders = 8;  // reader warps: two sets of four
+constexpr int kTileThreads = (2 + kReaders) * 32;
+// Items whose parts may be waiting for the other set's.  A set that is at item i + kItemQ + 1 knows, from the
+// queue's slot being free, that the other has taken item i + 1 and so is done with item i.
+constexpr int kPartSlots = kItemQ + 1;
 
 // PASS 1: stationary = Q tile t, streamed = K tiles 0..t.  PASS 2: stationary = K tile t,
 // streamed = Q tiles t..tiles-1.
 template <int PASS, int D>
-__global__ void __launch_bounds__(192, 2)
+__global__ void __launch_bounds__(kTileThreads, 2)
 score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                   const ScoreArgs a)
 {
@@ -60,7 +81,9 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(q_empty + kItemQ);
     __shared__ int s_abort;
     __shared__ int q_item[kItemQ];  // the loader's announcements: an item number, or -1 for the end
-    __shared__ __align__(16) float s_lse[2][4][TT];  // [accumulator][reader warp][query of the tile]
+    __shared__ __align__(16) float s_lse[2][4][TT];  // [reader set][lane quarter][query of the tile]
+    __shared__ float2 s_part[kPartSlots][2][4][32];  // an item's two parts: maximum and sum of every row
+    __shared__ int s_arrived[kPartSlots][4];
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const CUtensorMap *map_stat = PASS == 1 ? &map_q : &map_k;
@@ -82,8 +105,9 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         }
         for (int i = 0; i < kItemQ; ++i) {
             bar_init(q_full + i, 1);
-            bar_init(q_empty + i, 5);  // the MMA thread and the four reader warps
+            bar_init(q_empty + i, 1 + kReaders);  // the MMA warp and the reader warps
         }
+        for (int i = 0; i < kPartSlots * 4; ++i) s_arrived[i / 4][i % 4] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {  // two 128-column fp32 accumulators
@@ -99,6 +123,7 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     // Launched as a programmatic dependent: everything above (barriers, tensor memory) was set up
     // while the kernel before it drained; its results (Q, K, the normalisers) are read from here on.
     dependent_entry();
+    if (a.clear_abort && blockIdx.x == 0 && tid == 0) *a.abort_word = 0;
 
     if (warp == 0) {
         // ---- TMA producer ---------------------------------------------------------------------
@@ -106,11 +131,11 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             bool dead = false;
             uint32_t a_phase = 0;
             Ring2 rb{0, 0u}, rq{0, 0u};
-            int *ctr = a.next_item + (PASS - 1);
-            int next = atomicAdd(ctr, 1);  // asked for one item ahead: the answer takes a microsecond
+            int *ctr = a.counted ? a.next_item + (PASS - 1) : nullptr;
+            int next = ctr ? atomicAdd(ctr, 1) : blockIdx.x;  // asked for one item ahead: the answer takes a microsecond
             for (;;) {
                 const int w = next < nitems ? next : -1;
-                if (w >= 0) next = atomicAdd(ctr, 1);
+                if (w >= 0) next = ctr ? atomicAdd(ctr, 1) : next + (int)gridDim.x;
                 bar_wait(q_empty + rq.idx, rq.phase ^ 1u, dead, &s_abort);
                 if (dead) break;
                 q_item[rq.idx] = w;
@@ -182,15 +207,19 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             if (dead) break;
         }
     } else {
-        // ---- accumulator readers: one TMEM lane (tile row) per thread ----------------------------
-        const int quarter = warp & 3;
+        // ---- accumulator readers: one TMEM lane (tile row) per thread.  Tile c of the CTA's stream goes
+        // through accumulator c mod 2 to reader set c mod 2 ------------------------------------------------
+        const int set = (warp - 2) >> 2, quarter = warp & 3;
         const int row = quarter * 32 + lane;
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)set * TT;
+        float *my_lse = s_lse[set][quarter];
         bool dead = false;
-        Ring2 rs{0, 0u}, rq{0, 0u};
-        for (;;) {
-            bar_wait(q_full + rq.idx, rq.phase, dead, &s_abort);
+        uint32_t phase = 0, seq = 0, tile0 = 0;  // of the accumulator; number of the item; tiles before it
+        Ring2 rq{0, 0u};
+        for (;; ++seq) {
+            warp_wait(q_full + rq.idx, rq.phase, dead, &s_abort);
             if (dead) break;
-            const int w = q_item[rq.idx];
+            const int w = *(volatile int *)(q_item + rq.idx);
             __syncwarp();
             if (lane == 0) bar_arrive(q_empty + rq.idx);
             rq.next(kItemQ);
@@ -202,58 +231,58 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             const bool fast = sc > 0.f;     // the usual case: the extreme of sc * x is sc * max x
             const int grow = t * TT + row;  // query (pass 1) or key (pass 2) index of this thread
             const float *lse_row = a.lse2 + (size_t)sh * a.Npad;
-            float run_max = -INFINITY, run_sum = 0.f;  // pass 1
-            float col_sum = 0.f;                       // pass 2
-            const int j0 = PASS == 1 ? 0 : t, j1 = PASS == 1 ? t : a.tiles - 1;
+            float run_max = -INFINITY, run_sum = 0.f;  // pass 1 (pass 2: run_sum alone)
+            const int j0 = PASS == 1 ? 0 : t, count = PASS == 1 ? t + 1 : a.tiles - t;
+            const int odd = (set + tile0) & 1;  // this set's tiles of the item: j0 + odd, + 2, ...
+            tile0 += count;
             // pass 2: every thread needs the tile's 128 query normalisers.  Each warp keeps its own copy
             // in shared memory (four per lane, fetched a tile ahead so that the load's latency is not
             // in the way), so the reader warps never wait for one another.
             float4 lse_mine = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (PASS == 2) lse_mine = __ldg(reinterpret_cast<const float4 *>(lse_row + j0 * TT) + lane);
-            for (int j = j0; j <= j1; ++j) {
+            auto fetch_lse = [&](int j) {
+                if (a.lse_in == nullptr) {
+                    lse_mine = __ldg(reinterpret_cast<const float4 *>(lse_row + j * TT) + lane);
+                } else {  // (rows of N floats: no alignment to count on)
+                    const float *p = a.lse_in + (size_t)sh * a.N;
+                    const int m = j * TT + lane * 4;
+                    lse_mine.x = m < a.N ? __ldg(p + m) * kLog2eT : INFINITY;
+                    lse_mine.y = m + 1 < a.N ? __ldg(p + m + 1) * kLog2eT : INFINITY;
+                    lse_mine.z = m + 2 < a.N ? __ldg(p + m + 2) * kLog2eT : INFINITY;
+                    lse_mine.w = m + 3 < a.N ? __ldg(p + m + 3) * kLog2eT : INFINITY;
+                }
+            };
+            if (PASS == 2 && odd < count) fetch_lse(j0 + odd);
+            for (int jj = odd; jj < count; jj += 2) {
+                const int j = j0 + jj;
                 if (PASS == 2) {
-                    __syncwarp();  // the warp is done with the copy this one replaces (two tiles back)
-                    reinterpret_cast<float4 *>(s_lse[rs.idx][quarter])[lane] = lse_mine;
-                    if (j < j1) lse_mine = __ldg(reinterpret_cast<const float4 *>(lse_row + (j + 1) * TT) + lane);
+                    __syncwarp();  // the warp is done with the copy this one replaces
+                    reinterpret_cast<float4 *>(my_lse)[lane] = lse_mine;
+                    if (jj + 2 < count) fetch_lse(j + 2);
                     __syncwarp();
                 }
-                bar_wait(s_full + rs.idx, rs.phase, dead, &s_abort);
+                warp_wait(s_full + set, phase, dead, &s_abort);
+                phase ^= 1u;
                 fence_after();
-                const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)rs.idx * TT;
-                const bool diag = j == t;
-                // On the diagonal tile only the 32-column blocks that reach this warp's rows matter:
-                // blocks 0..quarter in pass 1 (keys <= query), quarter..3 in pass 2 (queries >= key).
-                const int c_lo = (PASS == 2 && diag) ? quarter : 0;
-                const int c_hi = (PASS == 1 && diag) ? quarter : TT / 32 - 1;
-                bool released = false;
-                if (!diag) {
-                    // a full tile: the whole row comes into registers at once and the accumulator goes
-                    // back to the MMA thread before the arithmetic starts
-                    if (PASS == 1) {
-                        float v[128];
-                        tmem_ld128(taddr, v);
-                        fence_before();
-                        __syncwarp();
-                        if (lane == 0) bar_arrive(s_empty + rs.idx);
-                        released = true;
-                        lse_block<128>(v, sc, fast, run_max, run_sum);
-                    } else {  // (pass 2 keeps more state: half a row at a time fits its registers)
+                auto release = [&]() {  // the accumulator's columns are all in registers: back to the MMA warp
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(s_empty + set);
+                };
+                if (j != t) {
+                    // a full tile, half a row at a time
 #pragma unroll 1
-                        for (int half = 0; half < 2; ++half) {
-                            float v[64];
-                            tmem_ld64(taddr + half * 64, v);
-                            if (half == 1) {
-                                fence_before();
-                                __syncwarp();
-                                if (lane == 0) bar_arrive(s_empty + rs.idx);
-                                released = true;
-                            }
-                            col_sum += colsum_block<64>(v, &s_lse[rs.idx][quarter][half * 64], sc, false, lane);
-                        }
+                    for (int half = 0; half < 2; ++half) {
+                        float v[64];
+                        tmem_ld64(taddr + half * 64, v);
+                        if (half == 1) release();
+                        if (PASS == 1) lse_block<64, kPoly1>(v, sc, fast, run_max, run_sum);
+                        else run_sum += colsum_block<64, kPoly2>(v, my_lse + half * 64, sc, false, lane);
                     }
                 } else {
+                    // On the diagonal tile only the 32-column blocks that reach this warp's rows matter:
+                    // blocks 0..quarter in pass 1 (keys <= query), quarter..3 in pass 2 (queries >= key).
 #pragma unroll 1
-                    for (int cblk = c_lo; cblk <= c_hi; ++cblk) {
+                    for (int cblk = PASS == 1 ? 0 : quarter; cblk <= (PASS == 1 ? quarter : TT / 32 - 1); ++cblk) {
                         float v[32];
                         tmem_ld32(taddr + cblk * 32, v);
                         const bool edge = cblk == quarter;  // the block the causal boundary crosses
@@ -262,23 +291,42 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
 #pragma unroll
                                 for (int i = 0; i < 32; ++i) v[i] = i <= lane ? v[i] : -INFINITY;
                             }
-                            lse_block<32>(v, sc, fast, run_max, run_sum);
+                            lse_block<32, 0>(v, sc, fast, run_max, run_sum);
                         } else {
-                            col_sum += colsum_block<32>(v, &s_lse[rs.idx][quarter][cblk * 32], sc, edge, lane);
+                            run_sum += colsum_block<32, 0>(v, my_lse + cblk * 32, sc, edge, lane);
                         }
                     }
+                    release();
                 }
-                if (!released) {
-                    fence_before();
-                    __syncwarp();
-                    if (lane == 0) bar_arrive(s_empty + rs.idx);
-                }
-                rs.next(2);
             }
-            if (PASS == 1) {
-                a.lse2[(size_t)sh * a.Npad + grow] = grow < a.N ? run_max + log2f(run_sum) : INFINITY;
-            } else if (grow < a.N) {
-                a.partial[(size_t)sh * a.N + grow] = col_sum;
+            // The item's result.  With two tiles or more both sets have a part of it, which they leave in
+            // shared memory: whichever warp is the second there adds the two (always the part with the
+            // first tile before the other, so that the sum does not depend on which warp it is).
+            bool writes = odd < count;
+            if (count > 1) {
+                float2 (*part)[4][32] = s_part[seq % kPartSlots];
+                int *arrived = s_arrived[seq % kPartSlots] + quarter;
+                part[odd][quarter][lane] = make_float2(run_max, run_sum);
+                __threadfence_block();
+                __syncwarp();
+                int before = 0;
+                if (lane == 0) before = atomicAdd(arrived, 1);
+                writes = __shfl_sync(0xffffffffu, before, 0) != 0;
+                if (writes) {
+                    __threadfence_block();
+                    const float2 p0 = part[0][quarter][lane], p1 = part[1][quarter][lane];
+                    if (PASS == 1) {
+                        run_max = fmaxf(p0.x, p1.x);
+                        run_sum = fmaf(p0.y, ex2(p0.x - run_max), p1.y * ex2(p1.x - run_max));
+                    } else {
+                        run_sum = p0.y + p1.y;
+                    }
+                    if (lane == 0) *(volatile int *)arrived = 0;
+                }
+            }
+            if (writes) {
+                if (PASS == 1) a.lse2[(size_t)sh * a.Npad + grow] = grow < a.N ? run_max + log2f(run_sum) : INFINITY;
+                else if (grow < a.N) a.partial[(size_t)sh * a.N + grow] = run_sum;
             }
         }
     }
@@ -312,17 +360,6 @@ __global__ void selftest_wait_kernel(int32_t *dev_status, uint32_t limit)
     __syncthreads();
     bar_wait(&bar, 0u, dead, &s_abort, limit);  // the other lanes see the flag and stop at once
     if (threadIdx.x == 0 && dead && s_abort) raise_status(dev_status, 0, PKV_DEV_TIMEOUT);
-}
-
-// Caller-supplied natural-log lse [B*L*H][N] -> padded log2 layout.
-__global__ void convert_lse_kernel(const float *__restrict__ lse, int N, int Npad, size_t rows,
-                                   float *__restrict__ lse2)
-{
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * Npad) return;
-    size_t r = i / Npad;
-    int n = (int)(i - r * Npad);
-    lse2[i] = n < N ? lse[r * N + n] * kLog2eT : INFINITY;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -376,11 +413,8 @@ int launch_pass(const CUtensorMap &mq, const CUtensorMap &mk, const ScoreArgs &a
     int rc = ensure_dynamic_smem((const void *)score_tile_kernel<PASS, D>, (int)smem, done);
     if (rc != PKV_OK) return rc;
     const int items = a.nseg * a.H * a.tiles;
-    // CTAs take items from a counter as they finish (long and short items mix in any case; with a
-    // fixed stride, 296 CTAs and 16 tiles per head left every CTA two tile indices only, and the
-    // slowest did 12 tiles per item against a mean of 8.5).
     const int grid = items < 2 * sms ? items : 2 * sms;
-    cudaError_t e = launch_dependent(score_tile_kernel<PASS, D>, dim3(grid), dim3(192), smem, st, mq, mk, a);
+    cudaError_t e = launch_dependent(score_tile_kernel<PASS, D>, dim3(grid), dim3(kTileThreads), smem, st, mq, mk, a);
     if (e != cudaSuccess) {
         set_cuda_error(e, PASS == 1 ? "score_tile_kernel<1>" : "score_tile_kernel<2>");
         return PKV_ERR_CUDA;
@@ -429,27 +463,29 @@ int launch_score_tc(const pkv_shape *s, const void *q, pkv_strides qs, const voi
     a.Npad = a.tiles * TT;
     a.next_item = (int *)((unsigned char *)a.lse2 + round_up(rows * a.Npad * sizeof(float), kWsAlign));
     a.abort_word = a.next_item + 2;
-    {
+    a.nseg = B * L;
+    a.group = head_group(B * L * H, N, s->head_dim, 2);
+
+    const int sms = sm_count();
+    if (sms <= 0) return PKV_ERR_CUDA;
+    // Items of nearly one length (a tile or two), or a few for each CTA: dealt out by position, which needs
+    // no counters and so no memset in front (32 x 32 heads of 100 tokens 42 -> 36 us, 2 x 32 of 640 38 ->
+    // 33.5, 128 x 32 of 200 193 -> 179).  Otherwise CTAs that run ahead take more (32 x 32 of 640 tokens
+    // 185 us, dealt 196; 2 x 32 of 16384 4.6 ms, dealt 5.0).
+    a.counted = a.tiles > 2 && rows * a.tiles > 8 * (size_t)sms;
+    if (a.counted) {
         cudaError_t e = cudaMemsetAsync(a.next_item, 0, 4 * sizeof(int), st);
         if (e != cudaSuccess) {
             set_cuda_error(e, "cudaMemsetAsync(score work counters)");
             return PKV_ERR_CUDA;
         }
     }
-    a.nseg = B * L;
-    a.group = head_group(B * L * H, N, s->head_dim, 2);
-
-    const int sms = sm_count();
-    if (sms <= 0) return PKV_ERR_CUDA;
-    int rc;
-    if (lse) {
-        const size_t n = rows * a.Npad;
-        convert_lse_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(lse, N, a.Npad, rows, a.lse2);
-        rc = check_launch("convert_lse_kernel");
-    } else {
-        rc = s->head_dim == 128 ? launch_pass<1, 128>(mq, mk, a, sms, st) : launch_pass<1, 64>(mq, mk, a, sms, st);
-    }
+    a.lse_in = lse;
+    int rc = PKV_OK;
+    a.clear_abort = !a.counted;
+    if (!lse) rc = s->head_dim == 128 ? launch_pass<1, 128>(mq, mk, a, sms, st) : launch_pass<1, 64>(mq, mk, a, sms, st);
     if (rc != PKV_OK) return rc;
+    a.clear_abort = !a.counted && lse;
     rc = s->head_dim == 128 ? launch_pass<2, 128>(mq, mk, a, sms, st) : launch_pass<2, 64>(mq, mk, a, sms, st);
     if (rc != PKV_OK) return rc;
     return launch_head_mean(a.partial, H, N, (size_t)B * L * N, scores, a.abort_word, st);

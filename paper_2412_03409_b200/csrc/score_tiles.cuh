@@ -188,6 +188,32 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b)
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return d;
 }
+// acc + 2^x on the FMA and integer pipes, two values at a time.  Rounding to the nearest integer n by
+// adding 1.5 * 2^23, a degree-5 polynomial in f = x - n (minimax in relative error on [-1/2, 1/2] with
+// p(0) = 1, fitted by Lawson's weighted least squares: 0.9e-7, 1.7e-7 with the rounding of Horner's rule;
+// ex2.approx is specified to 2^-22 = 2.4e-7), and 2^n put together in the exponent field.  x is held in
+// [-127, 128], where 2^n is 0 and infinity; NaN stays NaN.  UPPER: x may be above 128.
+template <bool UPPER> __device__ __forceinline__ float2 add_exp2(float2 acc, float2 x)
+{
+    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x.x));
+    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x.y));
+    if (UPPER) {
+        asm("min.NaN.f32 %0, %0, 0f43000000;" : "+f"(x.x));
+        asm("min.NaN.f32 %0, %0, 0f43000000;" : "+f"(x.y));
+    }
+    const float big = 12582912.f;
+    const float2 t = add2(x, make_float2(big, big));
+    const float2 n = add2(t, make_float2(-big, -big));
+    const float2 f = fma2(n, make_float2(-1.f, -1.f), x);
+    const float c[5] = {0x1.5bba14p-10f, 0x1.3cea88p-7f, 0x1.c6b752p-5f, 0x1.ebf9bcp-3f, 0x1.62e42ap-1f};
+    float2 p = make_float2(c[0], c[0]);
+#pragma unroll
+    for (int i = 1; i < 5; ++i) p = fma2(p, f, make_float2(c[i], c[i]));
+    p = fma2(p, f, make_float2(1.f, 1.f));
+    const float2 s = make_float2(__uint_as_float((__float_as_uint(t.x) << 23) + 0x3f800000u),
+                                 __uint_as_float((__float_as_uint(t.y) << 23) + 0x3f800000u));
+    return fma2(p, s, acc);
+}
 __device__ __forceinline__ float max3(float a, float b, float c)
 {
     float d;
@@ -209,11 +235,19 @@ struct Ring2 {
     }
 };
 
+// Whether pair i of a row goes to the FMA pipe: even pairs, POLY (0 to 4) of every eight, spread evenly.
+template <int POLY> __device__ __forceinline__ constexpr bool poly_pair(int i)
+{
+    return i % 2 == 0 && (i / 2 % 4) * POLY % 4 + POLY > 3;
+}
+
 // Pass 1 on NC consecutive logits of one query row: running maximum and sum in the log2
 // domain.  Four interleaved chains each for the maximum and the sum: with two reader warps per
 // scheduler a long dependent chain would leave it idle.  `fast` (scale > 0, the usual case):
 // the extreme of sc * x is sc * max x, so masked logits may stay -inf.
-template <int NC>
+// Of every eight pairs of exponentials POLY are computed on the FMA pipe, the others on the
+// special-function unit.
+template <int NC, int POLY>
 __device__ __forceinline__ void lse_block(float (&v)[NC], float sc, bool fast, float &run_max, float &run_sum)
 {
     if (!fast) {
@@ -234,7 +268,8 @@ __device__ __forceinline__ void lse_block(float (&v)[NC], float sc, bool fast, f
 #pragma unroll
     for (int i = 0; i < NC; i += 2) {
         const float2 x = fma2(make_float2(v[i], v[i + 1]), make_float2(mul, mul), make_float2(-nm, -nm));
-        p[(i >> 1) & 1] = add2(p[(i >> 1) & 1], make_float2(ex2(x.x), ex2(x.y)));
+        float2 &acc = p[(i >> 1) & 1];
+        acc = poly_pair<POLY>(i >> 1) ? add_exp2<false>(acc, x) : add2(acc, make_float2(ex2(x.x), ex2(x.y)));
     }
     run_sum = fmaf(run_sum, ex2(run_max - nm), (p[0].x + p[0].y) + (p[1].x + p[1].y));
     run_max = nm;
@@ -243,7 +278,7 @@ __device__ __forceinline__ void lse_block(float (&v)[NC], float sc, bool fast, f
 // Pass 2 on the logits of NC consecutive queries against one key: sum of the probabilities,
 // lse = the queries' normalisers (shared memory, log2 domain).  On the block the causal boundary
 // crosses (`edge`) query i of the block counts only when i >= lane.
-template <int NC>
+template <int NC, int POLY>
 __device__ __forceinline__ float colsum_block(const float (&v)[NC], const float *lse, float sc, bool edge, int lane)
 {
     const float4 *lp = reinterpret_cast<const float4 *>(lse);
@@ -254,6 +289,11 @@ __device__ __forceinline__ float colsum_block(const float (&v)[NC], const float 
         const int i = i4 * 4;
         const float2 x = fma2(make_float2(v[i], v[i + 1]), make_float2(sc, sc), make_float2(-ls.x, -ls.y));
         const float2 y = fma2(make_float2(v[i + 2], v[i + 3]), make_float2(sc, sc), make_float2(-ls.z, -ls.w));
+        if (!edge && poly_pair<POLY>(2 * i4)) {
+            p[0] = add_exp2<true>(p[0], x);
+            p[1] = add2(p[1], make_float2(ex2(y.x), ex2(y.y)));
+            continue;
+        }
         float e[4] = {ex2(x.x), ex2(x.y), ex2(y.x), ex2(y.y)};
         if (edge) {
 #pragma unroll

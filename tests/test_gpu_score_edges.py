@@ -1,4 +1,4 @@
-"""Scores of fp32 inputs at the edges of the 128-token tiles (needs a B200)."""
+"""Scores at the edges of the 128-token tiles, of both tensor-core kernels (needs a B200)."""
 import numpy as np
 import pytest
 import torch
@@ -12,25 +12,54 @@ pytestmark = pytest.mark.gpu
 TOL = 1e-5
 
 
-@pytest.mark.parametrize("B,L,H,D,N", [(1, 1, 1, 64, 1), (1, 2, 3, 128, 127), (1, 2, 2, 64, 128), (1, 1, 2, 128, 129),
-                                       (1, 2, 2, 64, 193), (1, 1, 2, 128, 257), (2, 1, 3, 64, 385),
-                                       (1, 10, 20, 64, 65), (1, 5, 40, 128, 40)])   # the last two: items > SMs
+SHAPES = [(1, 1, 1, 64, 1), (1, 2, 3, 128, 127), (1, 2, 2, 64, 128), (1, 1, 2, 128, 129), (1, 2, 2, 64, 193),
+          (1, 1, 2, 128, 257), (2, 1, 3, 64, 385), (1, 1, 2, 128, 1150),   # a set's turn comes round several times
+          (1, 10, 20, 64, 65), (1, 5, 40, 128, 40),                        # one-tile items, more than SMs
+          (1, 13, 20, 64, 600)]                                            # items from the counters
+
+
+@pytest.mark.parametrize("B,L,H,D,N", SHAPES)
 @pytest.mark.parametrize("given_lse", [False, True])
-def test_fp32_scores_at_tile_edges(B, L, H, D, N, given_lse):
+@pytest.mark.parametrize("dtype,sign", [(torch.float32, 1), (torch.bfloat16, 1), (torch.bfloat16, -1)])
+def test_scores_at_tile_edges(B, L, H, D, N, given_lse, dtype, sign):
     from paper_2412_03409_b200.session import Session
     g = torch.Generator(device="cuda").manual_seed(N * 7 + D)
     # token-major storage seen through [B, L, H, N, D] strides
-    q = torch.randn(B, L, N, H, D, device="cuda", generator=g).transpose(2, 3)
-    k = (torch.randn(B, L, N, H, D, device="cuda", generator=g) * 2).transpose(2, 3)
-    scale = np.full(L, 0.5 / np.sqrt(D), np.float32)
+    q = torch.randn(B, L, N, H, D, device="cuda", generator=g).to(dtype).transpose(2, 3)
+    k = (torch.randn(B, L, N, H, D, device="cuda", generator=g) * 2).to(dtype).transpose(2, 3)
+    scale = np.full(L, sign * 0.5 / np.sqrt(D), np.float32)
     lse = None
     if given_lse:
         x = torch.matmul(q.double(), k.double().transpose(-1, -2)) * float(scale[0])
         x.masked_fill_(torch.ones(N, N, dtype=torch.bool, device="cuda").triu(1), -float("inf"))
         lse = torch.logsumexp(x, -1).float().contiguous()
-    s = Session(B, L, H, D, N, torch.float32, scale, decode_cap=0, max_budget_rows=L)
+    s = Session(B, L, H, D, N, dtype, scale, decode_cap=0, max_budget_rows=L)
     s.scores.fill_(float("nan"))
     got = s.score(q, k, lse=lse).cpu().numpy()
-    for (b, l), ref in oracle_scores(q, k, scale).items():
+    segs = [(b, l) for b in range(B) for l in range(L)] if L < 13 else [(0, 0), (0, L - 1)]
+    for (b, l), ref in oracle_scores(q, k, scale, segs=segs).items():
         check_scores(got[b, l], ref, TOL)
     np.testing.assert_array_equal(got, s.score(q, k, lse=lse).cpu().numpy())   # bitwise reproducible
+
+
+@pytest.mark.parametrize("row", [3, 66, 130, 200])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_a_nan_is_not_lost(row, dtype):
+    """A NaN in a query reaches every key that the query attends to, whichever unit computes its exponential."""
+    from paper_2412_03409_b200.session import Session
+    q = torch.randn(1, 1, 2, 300, 64, device="cuda").to(dtype)
+    k = torch.randn(1, 1, 2, 300, 64, device="cuda").to(dtype)
+    q[0, 0, 1, row, 5] = float("nan")
+    s = Session(1, 1, 2, 64, 300, dtype, np.full(1, 0.125, np.float32), decode_cap=0, max_budget_rows=1)
+    got = s.score(q, k).cpu().numpy()[0, 0]
+    assert np.isnan(got[:row + 1]).all() and np.isfinite(got[row + 1:]).all()
+
+
+def test_exponents_out_of_range():
+    """A log-sum-exp far below (above) the logits makes infinite (zero) probabilities, never wrong finite ones."""
+    from paper_2412_03409_b200.session import Session
+    q = torch.zeros(1, 1, 1, 256, 64, device="cuda", dtype=torch.bfloat16)
+    s = Session(1, 1, 1, 64, 256, torch.bfloat16, np.full(1, 0.125, np.float32), decode_cap=0, max_budget_rows=1)
+    for value, want in [(-1000.0, np.inf), (1000.0, 0.0), (float("inf"), 0.0)]:
+        got = s.score(q, q, lse=torch.full((1, 1, 1, 256), value, device="cuda")).cpu().numpy()
+        assert (got == want).all()
