@@ -70,9 +70,10 @@ def measured_peaks():
         return FALLBACK_HBM_GBS, FALLBACK_BF16_TFLOPS, "fallback"
 
 
-# Which kernel a decode call takes: the library's rule (launch_decode_heads in csrc/decode_heads.cu)
+# Which kernel a decode call takes: the library's rules (launch_decode_cluster and launch_decode_heads)
 # restated, for the kernel's name, the launch count and the traffic figure below.
 DECODE_KERNELS = {
+    "cluster": ("decode_cluster_kernel", "decode_cluster.cu", "decode_cluster_kernel(const ClusterArgs a)", 1),
     "heads": ("decode_heads_kernel", "decode_heads.cu", "decode_heads_kernel(const __grid_constant__ HeadMaps maps", 1),
     "stream": ("decode_stream_kernel + its merge kernel", "decode_stream.cu", "decode_stream_kernel(const DecodeArgs a)", 2),
 }
@@ -80,8 +81,10 @@ DECODE_KERNELS = {
 
 def decode_path(w, sms):
     nact = w.B * w.L
+    if nact * w.H < 4 * sms:
+        return "cluster"
     cap_rows = w.B * (min(w.budget_rows(), w.L * w.N) + w.L * w.T)       # as Session sizes the cache
-    heads = w.D in (64, 128) and nact <= 256 and nact * w.H >= 4 * sms and cap_rows // nact <= 1024
+    heads = w.D in (64, 128) and nact <= 256 and cap_rows // nact <= 1024
     return "heads" if heads else "stream"
 
 
