@@ -397,11 +397,10 @@ static int launch_sort_items(const pkv_shape *s, const float *scores, int32_t *o
     const int N = s->prompt_len;
     const int threads = ((N + IPT - 1) / IPT + 31) / 32 * 32;
     const size_t smem = sort_smem_bytes(threads, IPT);
+    // (for every size: the default limit of 48 KiB is for the kernel's static variables and these together)
     static bool attr_done[64] = {};
-    if (smem > 48 * 1024) {
-        int rc = ensure_dynamic_smem((const void *)sort_scan_kernel<IPT>, (int)sort_smem_bytes(1024, IPT), attr_done);
-        if (rc != PKV_OK) return rc;
-    }
+    int rc = ensure_dynamic_smem((const void *)sort_scan_kernel<IPT>, (int)sort_smem_bytes(1024, IPT), attr_done);
+    if (rc != PKV_OK) return rc;
     cudaError_t e = launch_dependent(sort_scan_kernel<IPT>, dim3(s->batch * s->layers), dim3(threads), smem, st, scores, N,
                                      order, cum, seg_flags);
     if (e != cudaSuccess) {

@@ -1,4 +1,8 @@
 """Selection, bit for bit against the oracle, where the radix sort and the search change their ways (needs a B200)."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -57,3 +61,40 @@ def test_totals_out_of_range_are_reported():
         s.search(50, scores=x)
         assert s.status.item() == code, values[:2]
         assert int(s.len.min()) >= 1 and int(s.len.max()) <= 100
+
+
+def first_call(entry, N):
+    """One selection of N tokens as the first call of its process, bit for bit against the oracle."""
+    from paper_2412_03409_b200.session import Session
+    L, budget = 2, N
+    scores = np.stack([_scores("exp", L, N, N)])
+    s = Session(1, L, 2, 64, N, torch.float32, np.ones(L), decode_cap=0, max_budget_rows=L)
+    if entry == "search":
+        s.search(budget, scores=torch.from_numpy(scores).cuda())
+    else:
+        s.apply_lengths(torch.tensor([N // 3, N // 5]), scores=torch.from_numpy(scores).cuda())
+    (order, cum, res), = oracle_select(scores, [budget])
+    np.testing.assert_array_equal(s.order[0].cpu().numpy(), order)
+    np.testing.assert_array_equal(s.cum[0].cpu().numpy().view(np.uint64), cum)
+    np.testing.assert_array_equal(s.len[0].cpu().numpy(), res.len if entry == "search" else [N // 3, N // 5])
+    assert s.status.cpu().tolist() == [0]
+
+
+# Around 48 KiB of shared memory (four and eight scores a thread); the limit that an earlier, longer call raised
+# must not be what lets a launch through, so each length gets a process of its own.
+FIRST_CALLS = [("search", 3456), ("apply", 3585), ("search", 4608), ("search", 4609), ("apply", 4609), ("search", 4736),
+               ("search", 4864), ("apply", 4864), ("apply", 4865)]
+
+
+def test_first_call_of_a_process():
+    here = os.path.dirname(os.path.abspath(__file__))
+    path = os.pathsep.join([here, os.path.dirname(here)])
+    runs = [(c, subprocess.Popen([sys.executable, "-c", "import test_gpu_select_edges as t; t.first_call(%r, %d)" % c],
+                                 cwd=os.path.dirname(here), env=dict(os.environ, PYTHONPATH=path),
+                                 stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)) for c in FIRST_CALLS]
+    failed = []
+    for c, p in runs:
+        out, _ = p.communicate(timeout=300)
+        if p.returncode:
+            failed.append((c, out[-400:]))
+    assert not failed, failed
