@@ -150,7 +150,9 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
     const int skip = sp.evict ? sp.dst : -1;
     const int per = (cached + C - 1) / C;
     const int r0 = min(cached, rank * per), r1 = min(cached, r0 + per);
-    float qf[VE], acc[VE], M = -INFINITY, lsum = 0.f;
+    // M: the running maximum of the logits; Mz: the same, or 0 as long as all of them were -infinity or NaN, so
+    // that exp2f(s - Mz) is 0 for the one and stays NaN for the other.
+    float qf[VE], acc[VE], M = -INFINITY, Mz = 0.f, lsum = 0.f;
     RowVec<T>::unpack(qraw, qf);
 #pragma unroll
     for (int i = 0; i < VE; ++i) {
@@ -182,7 +184,8 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
 #pragma unroll
         for (int o = LPR; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         const float Mn = fmaxf(M, mx);
-        const float corr = M == -INFINITY ? 0.f : exp2f(M - Mn);
+        Mz = Mn == -INFINITY ? 0.f : Mn;
+        const float corr = exp2f(M - Mz);
         M = Mn;
         lsum *= corr;
 #pragma unroll
@@ -228,7 +231,7 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         for (int j = 0; j < kCU; ++j) {
             const int r = base + j * G + grp;
             if (r < r1 && r != skip)
-                add(M == -INFINITY ? 0.f : exp2f(s[j] - M), *reinterpret_cast<const uint4 *>(kt + kCRound + j * 512));
+                add(exp2f(s[j] - Mz), *reinterpret_cast<const uint4 *>(kt + kCRound + j * 512));
         }
         request(base + kCStages * kCWarps * STEP, stage);
         if (++stage == kCStages) stage = 0;
@@ -239,7 +242,7 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         rescale(s);
         if (grp == 0) {
-            add(exp2f(s - M), vnew);
+            add(exp2f(s - Mz), vnew);
             // the append: this head's slice of the new row goes to its place in the cache
             const size_t at = (size_t)(sp.off + sp.dst) * a.row_bytes + (size_t)h * SLICE + c * 16;
             *reinterpret_cast<uint4 *>(static_cast<unsigned char *>(a.ck) + at) = knew;
@@ -263,7 +266,8 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         s_ml[warp][1] = lsum;
     }
     __syncthreads();
-    // A state without rows has maximum -inf and weight 0 (at least one state of an item has rows).
+    // A state without rows has maximum -inf and weight 0 (at least one state of an item has rows); so has one whose
+    // only logits are NaN, and its sums, NaN, come through the product with 0.
     float z = 0.f, o = 0.f, m = -INFINITY;
 #pragma unroll
     for (int w = 0; w < kCWarps; ++w) m = fmaxf(m, s_ml[w][0]);

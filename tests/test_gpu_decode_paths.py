@@ -116,6 +116,23 @@ def test_replay_and_stale_workspace(B, L, H, D, N, rows, dtype, d, byte):
     assert (a.out[B - 1, L - 1] == 0).all() and int(a.cache.len[B * L - 1]) == 0
 
 
+@pytest.mark.parametrize("H,D,dtype", [(1, 64, torch.float32), (9, 128, torch.bfloat16), (72, 64, torch.bfloat16)])
+@pytest.mark.parametrize("rows", [1, 3, 19, 70])
+def test_a_nan_row_is_not_lost(H, D, dtype, rows):
+    """A NaN in one head's key makes that head's output NaN, whichever warp gets the row and whatever else it gets."""
+    s, _, tok = _ready(1, 1, H, D, 80, rows, dtype, 0, 1)
+    q, kn, vn = tok[0]
+    h, place, n = H // 2, int(s.cache.row_offset[0]), int(s.cache.len[0])
+    clean = s.cache.k.clone()
+    for row in range(n):
+        s.cache.k.copy_(clean)
+        s.cache.k[place + row, h, 3] = float("nan")
+        s.cache.len.fill_(n)
+        got = s.decode(q, kn, vn)[0, 0].cpu()
+        assert torch.isnan(got[h]).all(), row
+        assert torch.isfinite(got[torch.arange(H) != h]).all(), row
+
+
 def test_refused_calls_stay_refused():
     """Pruning and attending without appending are for shapes within the row-split kernel's limits."""
     from paper_2412_03409_b200 import api
