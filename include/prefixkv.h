@@ -319,6 +319,9 @@ int prefixkv_gini(const pkv_shape *shape, const uint64_t *cum, double *gini, voi
  * waiting, finishes in bounds and reports.  This call runs that give-up path alone: one warp
  * waits, with a limit of a few thousand tries (milliseconds), on a barrier that nothing
  * completes, and dev_status[0] is raised to PKV_DEV_TIMEOUT.  Nothing faults or hangs.
+ * which = 2: the wait of the decode kernels that write the lengths themselves for the flags of
+ * their CTAs; one block plays both parts, some flags not coming before the limit and then late,
+ * and raises the same code when every flag was left as a later call needs it.
  *   dev_status  [>= 1] int32, must hold PKV_DEV_OK on entry for the code to be recorded
  */
 int prefixkv_selftest_bounded_wait(int32_t which, int32_t *dev_status, void *cuda_stream);

@@ -10,7 +10,9 @@
 // in between.  The last CTA of a cluster also attends to the new row and appends it.
 // Lengths: every CTA reads its segment's length at the start and raises its flag (a per-call token
 // in the workspace); one extra cluster at the end of the grid, which has no rows, waits (bounded) for
-// all flags while the others work, and then writes the lengths of the next step.
+// all flags while the others work, and then writes the lengths of the next step.  However the wait
+// ends, all flags are zero once the launch is over: a call replayed from a CUDA graph comes with the
+// same token and must not find flags of its previous run.
 //
 // Measured, device time of calls replayed from a graph, against the row-split kernel and its merge
 // kernel (one layer, bf16, D = 128): 1 segment x 32 heads x 128 rows 4.5 us (10.0), 1024 rows 8.0
@@ -75,6 +77,36 @@ __device__ __forceinline__ void copy16(void *dst, const unsigned char *src)
     asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 
+// The give-up path in isolation: some CTAs' flags are raised, the wait for all of them runs out, the other flags
+// come late; all are zero after that, and a second run with the same token finds every flag it waits for.
+__global__ void selftest_flags_kernel(int32_t *dev_status, uint32_t limit)
+{
+    constexpr int n = 80, came = 50;
+    __shared__ unsigned long long flags[n];
+    const unsigned long long token = 0x9e3779b97f4a7c15ull;
+    const int i = threadIdx.x;
+    if (i < n) flags[i] = i % 3 ? 0ull : ~(unsigned long long)i;  // (left from anything)
+    __syncthreads();
+    bool ok = true;
+    if (i < came) ok = !raise_flag(flags + i, token);
+    __syncthreads();
+    ok = !settle_flags(flags, n, token, limit) && ok;
+    __syncthreads();
+    if (i >= came && i < n) {
+        const bool late = raise_flag(flags + i, token);
+        if (late) lower_flag(flags + i);
+        ok = ok && late;
+    }
+    __syncthreads();
+    if (i < n) ok = ok && flags[i] == 0ull;
+    if (i < n) ok = !raise_flag(flags + i, token) && ok;
+    __syncthreads();
+    ok = settle_flags(flags, n, token, limit) && ok;
+    __syncthreads();
+    if (i < n) ok = ok && flags[i] == 0ull;
+    if (__syncthreads_and(ok) && i == 0) raise_status(dev_status, 0, PKV_DEV_TIMEOUT);
+}
+
 // A head's slice of a row is D * sizeof(T) bytes: LPR lanes share a row, a warp reads G = 32 / LPR
 // rows per step.
 template <typename T, int D>
@@ -102,22 +134,10 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         // ---- the extra cluster: lengths of the next step, once every CTA has read this step's ----------
         if (C > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         if (rank != 0) return;
-        bool all_in = true;
-        for (int i = tid; i < nitems * C && all_in; i += kCWarps * 32) {
-            all_in = false;
-            for (uint32_t n = 0; n < kCSpinLimit; ++n)
-                if (*(volatile unsigned long long *)(a.flags + i) == a.token) {
-                    all_in = true;
-                    break;
-                }
-        }
-        if (!__syncthreads_and(all_in)) {
+        if (!settle_flags(a.flags, nitems * C, a.token, kCSpinLimit)) {
             if (tid == 0) raise_status(a.dev_status, 0, PKV_DEV_TIMEOUT);
             return;
         }
-        // (flags go back to zero, which no token is: a call replayed from a CUDA graph comes with the
-        // same token and must not find the flags of its previous run)
-        for (int i = tid; i < nitems * C; i += kCWarps * 32) a.flags[i] = 0ull;
         for (int si = tid; si < a.p.nact; si += kCWarps * 32) {
             const SegPlan sp = segment_plan(a.p, si);
             if (sp.rows < 0) raise_status(a.dev_status, si / a.p.nl, PKV_DEV_CAPACITY);
@@ -140,10 +160,8 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
     const float sc = a.layer_scale[a.p.layer_begin + si % a.p.nl] * kLog2eC;
     const SegPlan sp = segment_plan(a.p, si);
     __syncthreads();  // all of this CTA's reads of the lengths are done
-    if (tid == 0) {
-        __threadfence();
-        *(volatile unsigned long long *)(a.flags + blockIdx.x) = a.token;
-    }
+    bool late = false;
+    if (tid == 0) late = raise_flag(a.flags + blockIdx.x, a.token);
 
     // cached rows of the segment that are attended to: all of them, less the slot that the new row reuses
     const int cached = sp.rows < 0 ? 0 : (a.p.append ? (sp.evict ? sp.rows : sp.rows - 1) : sp.rows);
@@ -250,6 +268,8 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         }
     }
 
+    if (late) lower_flag(a.flags + blockIdx.x);
+
     // ---- merge: lane groups, warps, then the CTAs of the cluster ---------------------------------------
 #pragma unroll
     for (int o = LPR; o < 32; o <<= 1) {
@@ -329,6 +349,12 @@ template <typename T, int D> int launch_cluster(const ClusterArgs &a, int C, cud
 }
 
 }  // namespace
+
+int selftest_wait_cluster(int32_t *dev_status, cudaStream_t st)
+{
+    selftest_flags_kernel<<<1, 96, 0, st>>>(dev_status, 4096u);
+    return check_launch("selftest_flags_kernel");
+}
 
 size_t decode_cluster_ws_bytes() { return (size_t)kCMaxCtas * sizeof(unsigned long long); }
 

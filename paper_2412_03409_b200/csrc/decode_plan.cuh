@@ -1,4 +1,5 @@
-// What one decode step does to a segment, and 16-byte row vectors: shared by the decode kernels.
+// What one decode step does to a segment, 16-byte row vectors, and the flags that order the reads of the
+// lengths before their writes: shared by the decode kernels.
 #pragma once
 #include "common.cuh"
 
@@ -122,6 +123,40 @@ __device__ __forceinline__ void segment_write(const DecodePlanArgs &a, int seg, 
 __device__ __forceinline__ void segment_advance(const DecodePlanArgs &a, int si, const SegPlan &sp)
 {
     segment_write(a, (si / a.nl) * a.L + a.layer_begin + si % a.nl, sp.len_after, sp.dst, sp.evict);
+}
+
+// ---- flags: "this CTA has read the lengths" ----------------------------------------------------------
+// One per CTA in the workspace, which may hold anything before; raised with the call's token, an odd number.
+// A flag of kGone ^ token belongs to a CTA that is no longer waited for.
+constexpr unsigned long long kGone = 2;
+
+// One thread of a CTA: this CTA has read the lengths.  True when nobody waits for it any more; the flag is then
+// to be put to zero (lower_flag; later, so that the answer's latency is not in the way).
+__device__ __forceinline__ bool raise_flag(unsigned long long *flag, unsigned long long token)
+{
+    __threadfence();
+    return atomicExch(flag, token) == (token ^ kGone);
+}
+__device__ __forceinline__ void lower_flag(unsigned long long *flag) { *(volatile unsigned long long *)flag = 0ull; }
+
+// A whole CTA: waits for n flags and puts them back to zero.  False when the limit ran out: the flags
+// of those that have come are zero then, the others' get zero from their own CTAs when these come.
+__device__ __forceinline__ bool settle_flags(unsigned long long *flags, int n, unsigned long long token, uint32_t limit)
+{
+    bool all_in = true;
+    for (int i = threadIdx.x; i < n && all_in; i += blockDim.x) {
+        all_in = false;
+        for (uint32_t t = 0; t < limit; ++t)
+            if (*(volatile unsigned long long *)(flags + i) == token) {
+                all_in = true;
+                break;
+            }
+    }
+    __threadfence();  // what follows comes after the reads that the flags stand for
+    all_in = __syncthreads_and(all_in);
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        if (all_in || atomicExch(flags + i, token ^ kGone) == token) lower_flag(flags + i);
+    return all_in;
 }
 
 }  // namespace pkv

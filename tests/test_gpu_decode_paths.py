@@ -133,6 +133,15 @@ def test_a_nan_row_is_not_lost(H, D, dtype, rows):
         assert torch.isfinite(got[torch.arange(H) != h]).all(), row
 
 
+def test_a_wait_for_flags_that_runs_out():
+    """Flags that come late leave nothing that a replay with the same token could mistake for its own."""
+    from paper_2412_03409_b200 import api
+    status = torch.zeros(2, dtype=torch.int32, device="cuda")
+    api.prefixkv_selftest_bounded_wait(2, status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist() == [api.DEV_TIMEOUT, 0]
+
+
 def test_refused_calls_stay_refused():
     """Pruning and attending without appending are for shapes within the row-split kernel's limits."""
     from paper_2412_03409_b200 import api
