@@ -252,10 +252,8 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
     __syncthreads();
     // every length this CTA needs has been read: say so (the last CTA waits for all flags before it
     // writes the lengths of the next step)
-    if (tid == 0) {
-        __threadfence();
-        *(volatile unsigned long long *)(a.flags + blockIdx.x) = a.token;
-    }
+    bool late = false;
+    if (tid == 0 && append) late = raise_flag(a.flags + blockIdx.x, a.token);
 
     const int nitems = a.nact * H;
 
@@ -522,23 +520,14 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
         if (dead && lane == 0) raise_status(a.dev_status, 0, PKV_DEV_TIMEOUT);
     }
 
+    if (late) lower_flag(a.flags + blockIdx.x);
+
     // ---- the lengths of the next step, once every CTA has read this step's -------------------------
     if (blockIdx.x == gridDim.x - 1 && append) {
         __syncthreads();
-        bool all_in = true;
-        if (tid < (int)gridDim.x) {
-            all_in = false;
-            for (uint32_t i = 0; i < kHSpinLimit; ++i) {
-                if (*(volatile unsigned long long *)(a.flags + tid) == a.token) {
-                    all_in = true;
-                    break;
-                }
-            }
-        }
-        if (__syncthreads_and(all_in)) {
-            // (flags go back to zero, which no token is: a call replayed from a CUDA graph comes
-            // with the same token and must not find the flags of its previous run)
-            if (tid < (int)gridDim.x) a.flags[tid] = 0ull;
+        // (all flags are zero once the launch is over: a call replayed from a CUDA graph comes with the same
+        // token and must not find flags of its previous run)
+        if (settle_flags(a.flags, (int)gridDim.x, a.token, kHSpinLimit)) {
             for (int si = tid; si < a.nact; si += blockDim.x)
                 if (s_len[si] >= 0) a.len[(si / a.nl) * a.L + a.layer_begin + si % a.nl] = s_len[si] + 1;
         } else if (tid == 0) {
