@@ -262,16 +262,18 @@ __device__ __forceinline__ void lse_block(float (&v)[NC], float sc, bool fast, f
         c2[1] = max3(c2[1], v[i + 2], v[i + 3]);
     }
     const float cmax = max3(c2[0], c2[1], fmaxf(v[NC - 2], v[NC - 1]));
-    const float nm = fmaxf(run_max, fast ? cmax * sc : cmax);  // finite: column 0 is never masked
+    const float nm = fmaxf(run_max, fast ? cmax * sc : cmax);
+    // (the maximum is still -infinity when keys of infinite elements have masked all columns so far: sums of 0)
+    const float base = nm == -INFINITY ? 0.f : nm;
     const float mul = fast ? sc : 1.f;  // (the other way v is scaled already)
     float2 p[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
     for (int i = 0; i < NC; i += 2) {
-        const float2 x = fma2(make_float2(v[i], v[i + 1]), make_float2(mul, mul), make_float2(-nm, -nm));
+        const float2 x = fma2(make_float2(v[i], v[i + 1]), make_float2(mul, mul), make_float2(-base, -base));
         float2 &acc = p[(i >> 1) & 1];
         acc = poly_pair<POLY>(i >> 1) ? add_exp2<false>(acc, x) : add2(acc, make_float2(ex2(x.x), ex2(x.y)));
     }
-    run_sum = fmaf(run_sum, ex2(run_max - nm), (p[0].x + p[0].y) + (p[1].x + p[1].y));
+    run_sum = fmaf(run_sum, ex2(run_max - base), (p[0].x + p[0].y) + (p[1].x + p[1].y));
     run_max = nm;
 }
 

@@ -63,3 +63,24 @@ def test_exponents_out_of_range():
     for value, want in [(-1000.0, np.inf), (1000.0, 0.0), (float("inf"), 0.0)]:
         got = s.score(q, q, lse=torch.full((1, 1, 1, 256), value, device="cuda")).cpu().numpy()
         assert (got == want).all()
+
+
+@pytest.mark.parametrize("lo,hi", [(128, 192), (128, 256), (200, 300), (384, 448)])
+@pytest.mark.parametrize("D", [64, 128])
+def test_keys_masked_by_an_infinite_element(lo, hi, D):
+    """Keys with logits of -infinity (an infinite element against queries of one sign there) have score 0 and leave the
+    others' as they are without them, whole blocks of columns included."""
+    from paper_2412_03409_b200.session import Session
+    N = 512  # (no padding queries: zeros, whose logits against an infinite element are NaN)
+    g = torch.Generator(device="cuda").manual_seed(lo + D)
+    q = torch.randn(1, 1, 2, N, D, device="cuda", generator=g).bfloat16()
+    k = torch.randn(1, 1, 2, N, D, device="cuda", generator=g).bfloat16()
+    q[..., 0] = q[..., 0].abs() + 1
+    k[..., lo:hi, 0] = -float("inf")
+    s = Session(1, 1, 2, D, N, torch.bfloat16, np.full(1, D ** -0.5, np.float32), decode_cap=0, max_budget_rows=1)
+    got = s.score(q, k)[0, 0].double().cpu().numpy()
+    x = torch.matmul(q.double(), k.double().transpose(-1, -2))[0, 0] * float(np.float32(D ** -0.5))
+    x.masked_fill_(torch.ones(N, N, dtype=torch.bool, device="cuda").triu(1), -float("inf"))
+    ref = torch.softmax(x, -1).sum(1).mean(0).cpu().numpy()
+    check_scores(got, ref, TOL)
+    assert (got[lo:hi] == 0).all()
