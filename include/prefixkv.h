@@ -95,8 +95,9 @@ const char *prefixkv_last_cuda_error(void);
  *               NULL the library computes it in a first pass
  *   scores      [B,L,N] fp32, out
  * bf16 inputs use tensor cores with fp32 accumulation; fp32 inputs too, each element split exactly
- * into three bf16 numbers, with an error no larger than that of fp32 FMA (an infinite element makes
- * NaN scores); bf16 inputs whose strides no tensor map can describe, e.g. a zero stride, use FMA.
+ * into three bf16 numbers, with an error no larger than that of fp32 FMA (logits that an infinite
+ * element takes part in are formed by FMA); bf16 inputs whose strides no tensor map can describe,
+ * e.g. a zero stride, use FMA.
  * The workspace holds per-head partial sums and work counters: calls that share one must
  * not overlap on the GPU.  The call has no status argument: if a bounded wait inside the
  * tensor-core kernel runs out, every score of the call is written as NaN, which

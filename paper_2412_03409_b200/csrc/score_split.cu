@@ -90,10 +90,53 @@ template <int D> __device__ __forceinline__ void load_logits(uint32_t taddr, flo
     }
 }
 
+// What the parts cannot carry -- an infinite element, whose remainder is NaN, and products whose parts pass the
+// range where the product itself may not -- comes out as a NaN logit.  The thread that finds its sum turned
+// NaN by a block of 32 logits forms them again from the inputs with fp32 FMAs, so that NaN remains only
+// where the definition has one.  (A sum that is NaN already stays: nothing can change it.)
+template <int D> __device__ __forceinline__ float fma_logit(const float *x, const float *y)
+{
+    float s = 0.f;
+#pragma unroll 4
+    for (int d = 0; d < D; d += 4) {
+        const float4 u = __ldg(reinterpret_cast<const float4 *>(x + d)), v = __ldg(reinterpret_cast<const float4 *>(y + d));
+        s = fmaf(u.w, v.w, fmaf(u.z, v.z, fmaf(u.y, v.y, fmaf(u.x, v.x, s))));
+    }
+    return s;
+}
+__device__ __forceinline__ const float *head_rows(const float *p, const pkv_strides &st, const SplitArgs &a, int sh)
+{
+    const int seg = sh / a.H, h = sh - seg * a.H, b = seg / a.L, l = seg - b * a.L;
+    return p + b * st.b + l * st.l + h * st.h;
+}
+// Running maximum and sum of a query over the keys from key0 on, 32 at most.
+template <int D>
+__device__ __noinline__ float2 redo_lse(const SplitArgs &a, int sh, int query, int key0, float sc, float run_max, float run_sum)
+{
+    const float *q = head_rows(a.q, a.qs, a, sh) + query * a.qs.n, *k = head_rows(a.k, a.ks, a, sh);
+    for (int key = key0; key <= min(query, key0 + 31); ++key) {
+        const float x = fma_logit<D>(q, k + key * a.ks.n) * sc;
+        const float nm = fmaxf(run_max, x), base = nm == -INFINITY ? 0.f : nm;
+        run_sum = fmaf(run_sum, ex2(run_max - base), ex2(x - base));
+        run_max = nm;
+    }
+    return make_float2(run_max, run_sum);
+}
+// Probabilities that a key gets from the queries from query0 on, 32 at most; lse = their normalisers.
+template <int D>
+__device__ __noinline__ float redo_colsum(const SplitArgs &a, int sh, int key, int query0, const float *lse, float sc)
+{
+    const float *q = head_rows(a.q, a.qs, a, sh), *k = head_rows(a.k, a.ks, a, sh) + key * a.ks.n;
+    float sum = 0.f;
+    for (int m = max(key, query0); m < min(a.N, query0 + 32); ++m)
+        sum += ex2(fmaf(fma_logit<D>(q + m * a.qs.n, k), sc, -lse[m - query0]));
+    return sum;
+}
+
 // MODE 1: stationary = Q tile t, streamed = K tiles 0..t (log-sum-exp).  MODE 2: stationary = K tile
 // t, streamed = Q tiles t..tiles-1 (column sums).  MODE 0: one tile, Q stationary, both results.
 template <int MODE, int D>
-__global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const SplitArgs a)
+__global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __grid_constant__ SplitArgs a)
 {
     constexpr int KH = D / 64;
     constexpr int PASS = MODE == 2 ? 2 : 1;
@@ -373,7 +416,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const Spl
             rs.next(2);
         };
         // Column sums of a tile; on the diagonal tile only the blocks from this warp's keys on count.
-        auto sum_tile = [&](const float *lse, bool diag, float sc, float &col_sum) {
+        auto sum_tile = [&](const float *lse, int sh, int key, int tile, bool diag, float sc, float &col_sum) {
             for (int u = 0; u < U::PER_TILE; ++u) {
                 warp_wait(s_full + rs.idx, rs.phase, dead, &s_abort);
                 fence_after();
@@ -381,7 +424,13 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const Spl
                 for (int cb = max(diag ? warp : 0, u * U::BLOCKS); cb < (u + 1) * U::BLOCKS; ++cb) {
                     float v[32];
                     load_logits<D>(lane_addr + rs.idx * kBuf + (cb - u * U::BLOCKS) * 32, v);
-                    col_sum += colsum_block<32, 0>(v, lse + cb * 32, sc, diag && cb == warp, lane);
+                    float part = colsum_block<32, 0>(v, lse + cb * 32, sc, diag && cb == warp, lane);
+                    const bool redo = part != part && col_sum == col_sum && key < a.N;
+                    if (__any_sync(0xffffffffu, redo)) {
+                        if (redo) part = redo_colsum<D>(a, sh, key, tile * TT + cb * 32, lse + cb * 32, sc);
+                        __syncwarp();
+                    }
+                    col_sum += part;
                 }
                 release();
             }
@@ -414,7 +463,17 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const Spl
 #pragma unroll
                                 for (int i = 0; i < 32; ++i) v[i] = i <= lane ? v[i] : -INFINITY;
                             }
+                            const float old_max = run_max, old_sum = run_sum;
                             lse_block<32, 0>(v, sc, sc > 0.f, run_max, run_sum);
+                            const bool redo = run_sum != run_sum && old_sum == old_sum && grow < a.N;
+                            if (__any_sync(0xffffffffu, redo)) {
+                                if (redo) {
+                                    const float2 r = redo_lse<D>(a, sh, grow, j * TT + cb * 32, sc, old_max, old_sum);
+                                    run_max = r.x;
+                                    run_sum = r.y;
+                                }
+                                __syncwarp();
+                            }
                         }
                         release();
                     }
@@ -429,7 +488,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const Spl
                     __syncwarp();
                     if (lane == 0) bar_arrive(lse_full + flip);
                     warp_wait(lse_full + flip, lse_phase, dead, &s_abort);
-                    sum_tile(s_lse[flip][0], true, sc, col_sum);
+                    sum_tile(s_lse[flip][0], sh, grow, t, true, sc, col_sum);
                     flip ^= 1;
                     if (flip == 0) lse_phase ^= 1u;
                     if (grow < a.N) a.partial[(size_t)sh * a.N + grow] = col_sum;
@@ -452,7 +511,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const Spl
                     reinterpret_cast<float4 *>(s_lse[buf][warp])[lane] = mine;
                     if (j + 1 < a.tiles) get(j + 1);
                     __syncwarp();
-                    sum_tile(s_lse[buf][warp], j == t, sc, col_sum);
+                    sum_tile(s_lse[buf][warp], sh, grow, j, j == t, sc, col_sum);
                 }
                 if (grow < a.N) a.partial[(size_t)sh * a.N + grow] = col_sum;
             }

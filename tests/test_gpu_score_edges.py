@@ -84,3 +84,28 @@ def test_keys_masked_by_an_infinite_element(lo, hi, D):
     ref = torch.softmax(x, -1).sum(1).mean(0).cpu().numpy()
     check_scores(got, ref, TOL)
     assert (got[lo:hi] == 0).all()
+
+
+@pytest.mark.parametrize("N,lo,hi", [(512, 128, 256), (520, 200, 300), (777, 700, 770), (100, 1, 60), (128, 127, 128), (300, 0, 0)])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("given_lse", [False, True])
+def test_fp32_infinite_and_huge_elements(N, lo, hi, D, given_lse):
+    """As above in fp32, whose split cannot carry an infinite element, at every length; and an element next to the
+    largest float."""
+    from paper_2412_03409_b200.session import Session
+    g = torch.Generator(device="cuda").manual_seed(lo + D)
+    q = torch.randn(1, 1, 2, N, D, device="cuda", generator=g)
+    k = torch.randn(1, 1, 2, N, D, device="cuda", generator=g)
+    q[..., 0] = q[..., 0].abs() + 1
+    k[..., lo:hi, 0] = -float("inf")
+    huge = N // 2 if hi == 0 else 0
+    if huge:
+        q[..., 0] = 2.0 ** -122
+        k[..., huge, 0] = float(np.float32(3.4e38))   # above the largest bf16; a product of 64
+    s = Session(1, 1, 2, D, N, torch.float32, np.full(1, D ** -0.5, np.float32), decode_cap=0, max_budget_rows=1)
+    x = torch.matmul(q.double(), k.double().transpose(-1, -2))[0, 0] * float(np.float32(D ** -0.5))
+    x.masked_fill_(torch.ones(N, N, dtype=torch.bool, device="cuda").triu(1), -float("inf"))
+    lse = torch.logsumexp(x, -1).float()[None, None].contiguous() if given_lse else None
+    got = s.score(q, k, lse=lse)[0, 0].double().cpu().numpy()
+    check_scores(got, torch.softmax(x, -1).sum(1).mean(0).cpu().numpy(), TOL)
+    assert (got[lo:hi] == 0).all()
