@@ -1,10 +1,12 @@
 // Importance score (Sec. 3.2) of fp32 inputs on the bf16 tensor cores, in fp32 precision.
 //
-// Every fp32 element is the exact sum of three bf16 numbers x = x0 + x1 + x2 (8 significant bits
-// each).  A logit is the sum of the six products that matter, smallest first,
+// Every fp32 element of magnitude 2^-110 and above is the exact sum of three bf16 numbers x = x0 + x1 + x2
+// (8 significant bits each, rounded to nearest, so |x1| <= 2^-8 |x| and |x2| <= 2^-17 |x|; below that, what
+// is lost is less than 2^-133).  A logit is the sum of the six products that matter, smallest first,
 //   x0 y2 + x1 y1 + x2 y0 + x0 y1 + x1 y0 + x0 y0
-// (the dropped x1 y2, x2 y1, x2 y2 are below 2^-24 of the product), accumulated in fp32 by
-// tcgen05.mma.  The tensor core truncates a sum where an FMA rounds it, so a long chain drifts
+// (the dropped x1 y2 + x2 y1 + x2 y2 are at most 2^-24 of the product), accumulated in fp32 by
+// tcgen05.mma.  A single product that outweighs all others thus has an error of up to 2^-24 + 2^-23 (an FMA's
+// 2^-24), a sum of many terms less than a chain of FMAs.  The tensor core truncates a sum where an FMA rounds it, so a long chain drifts
 // towards zero; the large products of a logit are therefore spread over several accumulators
 // (D = 128: one for each 64 elements; D = 64: one for each 16) that are added in registers.
 // Measured against fp64 on N(0, 1) operands, D = 128: error of a logit 0.9e-6 rms, against 2.3e-6
@@ -54,11 +56,11 @@ struct SplitArgs {
     int L, H, N, tiles, nsh, group;
 };
 
-// One float into its three bf16 parts, two elements at a time (packed low, high).  The first part is
-// rounded towards zero so that the largest finite values do not become infinite.
+// One float into its three bf16 parts, two elements at a time (packed low, high).  (Above the largest bf16,
+// 2^128 - 2^120, the first part is infinite and the logit is formed by FMA, see below.)
 __device__ __forceinline__ void split2(float x, float y, uint32_t &p0, uint32_t &p1, uint32_t &p2)
 {
-    asm("cvt.rz.bf16x2.f32 %0, %1, %2;" : "=r"(p0) : "f"(y), "f"(x));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p0) : "f"(y), "f"(x));
     const float rx = x - __uint_as_float(p0 << 16), ry = y - __uint_as_float(p0 & 0xffff0000u);
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p1) : "f"(ry), "f"(rx));
     const float sx = rx - __uint_as_float(p1 << 16), sy = ry - __uint_as_float(p1 & 0xffff0000u);
@@ -90,7 +92,7 @@ template <int D> __device__ __forceinline__ void load_logits(uint32_t taddr, flo
     }
 }
 
-// What the parts cannot carry -- an infinite element, whose remainder is NaN, and products whose parts pass the
+// What the parts cannot carry -- an element whose first part is infinite, so that its remainder is NaN, and products whose parts pass the
 // range where the product itself may not -- comes out as a NaN logit.  The thread that finds its sum turned
 // NaN by a block of 32 logits forms them again from the inputs with fp32 FMAs, so that NaN remains only
 // where the definition has one.  (A sum that is NaN already stays: nothing can change it.)

@@ -109,3 +109,28 @@ def test_fp32_infinite_and_huge_elements(N, lo, hi, D, given_lse):
     got = s.score(q, k, lse=lse)[0, 0].double().cpu().numpy()
     check_scores(got, torch.softmax(x, -1).sum(1).mean(0).cpu().numpy(), TOL)
     assert (got[lo:hi] == 0).all()
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_fp32_single_products(D):
+    """Logits of one product each, prompts of one token: dropped parts of the split are at most 2^-24 of the product,
+    the last of the accumulations, which truncate, 2^-23, and those before it next to nothing."""
+    from paper_2412_03409_b200.session import Session
+    L = 4096
+    rng = np.random.default_rng(D)
+    x, y = (np.float32(1) + rng.integers(0, 1 << 23, (2, L)) * np.float32(2.0 ** -23)).astype(np.float32)
+    x[:2048] = y[:2048] = np.float32(1) + (0xfe80 + np.arange(2048) - 1024) * np.float32(2.0 ** -23)  # two large lower parts
+    scale = (64 / (x.astype(np.float64) * y)).astype(np.float32)
+    lse = (scale.astype(np.float64) * x * y).astype(np.float32)
+    q, k = (torch.zeros(1, L, 1, 1, D, device="cuda") for _ in range(2))
+    place = torch.arange(L, device="cuda") % D
+    q[0, torch.arange(L), 0, 0, place] = torch.from_numpy(x).cuda()
+    k[0, torch.arange(L), 0, 0, place] = torch.from_numpy(y).cuda()
+    s = Session(1, L, 1, D, 1, torch.float32, scale, decode_cap=0, max_budget_rows=L)
+    got = s.score(q, k, lse=torch.from_numpy(lse).cuda().view(1, L, 1, 1)).cpu().numpy().reshape(L).astype(np.float64)
+    log2e = np.float32(np.log2(np.e))
+    sc, l2 = (scale * log2e).astype(np.float64), (lse * log2e).astype(np.float64)   # rounded as the kernel rounds them
+    exact = sc * (x.astype(np.float64) * y)
+    error = (np.log2(got) + l2 - exact) / exact
+    # (log2 of a score near 1 has the rounding of the score and of the exponential, 2^-22, over an exponent of 92)
+    assert np.abs(error).max() <= 1.5 * 2.0 ** -23 + 2.0 ** -28
