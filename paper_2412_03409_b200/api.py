@@ -223,9 +223,9 @@ def prefixkv_compact(shape, k, v, order, length, cache: Cache, dev_status, ws, k
 def prefixkv_decode_attn(shape, cache: Cache, q, k_new, v_new, layer_scale, out, dev_status, ws,
                          layer_begin=0, layer_end=None):
     # (called once per layer and token: straight to the library, nothing else on the way)
-    rc = _decode_attn(ctypes.byref(shape), ctypes.byref(cache.c), q.data_ptr(), _ptr(k_new), _ptr(v_new),
-                      layer_scale.data_ptr(), int(layer_begin), shape.layers if layer_end is None else int(layer_end),
-                      out.data_ptr(), dev_status.data_ptr(), _ptr(ws), ws.numel() if ws is not None else 0, _stream())
+    rc = _decode_attn(ctypes.byref(shape), ctypes.byref(cache.c), _ptr(q), _ptr(k_new), _ptr(v_new),
+                      _ptr(layer_scale), int(layer_begin), shape.layers if layer_end is None else int(layer_end),
+                      _ptr(out), _ptr(dev_status), _ptr(ws), ws.numel() if ws is not None else 0, _stream())
     if rc:
         _check(rc, "prefixkv_decode_attn")
 

@@ -151,3 +151,14 @@ def test_refused_calls_stay_refused():
     s, _, tok = _ready(1, 1, 72, 64, 60, 20, torch.bfloat16, 0, 2)
     with pytest.raises(api.PrefixKVError):
         s.decode(tok[0][0], None, None)
+
+
+@pytest.mark.parametrize("missing", ["q", "k_new", "layer_scale", "out", "dev_status", "ws"])
+def test_a_missing_tensor_is_an_argument_error(missing):
+    from paper_2412_03409_b200 import api
+    s, _, tok = _ready(1, 1, 2, 64, 60, 20, torch.bfloat16, 0, 2)
+    args = dict(zip(("q", "k_new", "v_new"), tok[0]), layer_scale=s.layer_scale, out=s.out, dev_status=s.status,
+                ws=s.ws_decode)
+    args[missing] = None
+    with pytest.raises(api.PrefixKVError):
+        api.prefixkv_decode_attn(s.shape, s.cache, **args)
