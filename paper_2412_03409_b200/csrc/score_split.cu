@@ -400,8 +400,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
         }
         if (dead) {  // let the products in flight finish before the CTA can exit (bounded)
             if (elect_one()) mma_commit(&drained);
-            for (uint32_t i = 0; i < kSpin; ++i)
-                if (bar_try(&drained, 0u)) break;
+            drain(&drained, 0u);
         }
     } else {
         // ---- accumulator readers: one TMEM lane (tile row) per thread --------------------------------

@@ -79,6 +79,7 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
     uint64_t *s_full = b_empty + kStagesB, *s_empty = s_full + 2;
     uint64_t *q_full = s_empty + 2, *q_empty = q_full + kItemQ;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(q_empty + kItemQ);
+    __shared__ __align__(8) uint64_t drained;
     __shared__ int s_abort;
     __shared__ int q_item[kItemQ];  // the loader's announcements: an item number, or -1 for the end
     __shared__ __align__(16) float s_lse[2][4][TT];  // [reader set][lane quarter][query of the tile]
@@ -107,6 +108,7 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
             bar_init(q_full + i, 1);
             bar_init(q_empty + i, 1 + kReaders);  // the MMA warp and the reader warps
         }
+        bar_init(&drained, 1);
         for (int i = 0; i < kPartSlots * 4; ++i) s_arrived[i / 4][i % 4] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -129,7 +131,7 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
         // ---- TMA producer ---------------------------------------------------------------------
         if (lane == 0) {
             bool dead = false;
-            uint32_t a_phase = 0;
+            uint32_t a_phase = 0, a_loads = 0, b_loads = 0;  // loads issued
             Ring2 rb{0, 0u}, rq{0, 0u};
             int *ctr = a.counted ? a.next_item + (PASS - 1) : nullptr;
             int next = ctr ? atomicAdd(ctr, 1) : blockIdx.x;  // asked for one item ahead: the answer takes a microsecond
@@ -152,6 +154,7 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 for (int kh = 0; kh < KH; ++kh)
                     tma_load_5d(sA + kh * HALF, map_stat, a_full, kh * 64, t * TT, h, l, b);
                 a_phase ^= 1u;
+                ++a_loads;
                 const int j0 = PASS == 1 ? 0 : t, j1 = PASS == 1 ? t : a.tiles - 1;
                 for (int j = j0; j <= j1; ++j) {
                     bar_wait(b_empty + rb.idx, rb.phase ^ 1u, dead, &s_abort);
@@ -161,7 +164,13 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                     for (int kh = 0; kh < KH; ++kh)
                         tma_load_5d(sB + rb.idx * TILE + kh * HALF, map_strm, b_full + rb.idx, kh * 64, j * TT, h, l, b);
                     rb.next(kStagesB);
+                    ++b_loads;
                 }
+            }
+            if (dead) {  // let the loads on their way land before the CTA can exit (bounded)
+                if (a_loads > 0) drain(a_full, (a_loads - 1) & 1u);
+                for (uint32_t n = b_loads > kStagesB ? b_loads - kStagesB : 0; n < b_loads; ++n)
+                    drain(b_full + n % kStagesB, n / kStagesB & 1u);
             }
         }
     } else if (warp == 1) {
@@ -205,6 +214,10 @@ score_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_consta
                 rs.next(2);
             }
             if (dead) break;
+        }
+        if (dead) {  // and the products in flight finish before tensor memory is given back (bounded)
+            if (elect_one()) mma_commit(&drained);
+            drain(&drained, 0u);
         }
     } else {
         // ---- accumulator readers: one TMEM lane (tile row) per thread.  Tile c of the CTA's stream goes

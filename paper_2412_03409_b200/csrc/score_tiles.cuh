@@ -52,6 +52,12 @@ __device__ __forceinline__ void bar_wait(uint64_t *bar, uint32_t parity, bool &d
     atomicExch(abort_flag, 1);
 }
 
+// Bounded wait of a role that has given up for what it has in flight itself.
+__device__ __forceinline__ void drain(uint64_t *bar, uint32_t parity)
+{
+    for (uint32_t i = 0; i < kSpin && !bar_try(bar, parity); ++i) {}
+}
+
 // Bounded wait of a whole warp: every lane learns when any lane's wait has run out.
 __device__ __forceinline__ void warp_wait(uint64_t *bar, uint32_t parity, bool &dead, int *abort_flag)
 {
