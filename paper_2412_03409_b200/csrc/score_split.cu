@@ -94,7 +94,7 @@ template <int D> __device__ __forceinline__ void load_logits(uint32_t taddr, flo
 
 // What the parts cannot carry -- an element whose first part is infinite, so that its remainder is NaN, and products whose parts pass the
 // range where the product itself may not -- comes out as a NaN logit.  The thread that finds its sum turned
-// NaN by a block of 32 logits forms them again from the inputs with fp32 FMAs, so that NaN remains only
+// NaN by a tile forms that tile's logits again from the inputs with fp32 FMAs, so that NaN remains only
 // where the definition has one.  (A sum that is NaN already stays: nothing can change it.)
 template <int D> __device__ __forceinline__ float fma_logit(const float *x, const float *y)
 {
@@ -111,12 +111,12 @@ __device__ __forceinline__ const float *head_rows(const float *p, const pkv_stri
     const int seg = sh / a.H, h = sh - seg * a.H, b = seg / a.L, l = seg - b * a.L;
     return p + b * st.b + l * st.l + h * st.h;
 }
-// Running maximum and sum of a query over the keys from key0 on, 32 at most.
+// Running maximum and sum of a query over the keys of the tile from key0 on.
 template <int D>
 __device__ __noinline__ float2 redo_lse(const SplitArgs &a, int sh, int query, int key0, float sc, float run_max, float run_sum)
 {
     const float *q = head_rows(a.q, a.qs, a, sh) + query * a.qs.n, *k = head_rows(a.k, a.ks, a, sh);
-    for (int key = key0; key <= min(query, key0 + 31); ++key) {
+    for (int key = key0; key <= min(query, key0 + TT - 1); ++key) {
         const float x = fma_logit<D>(q, k + key * a.ks.n) * sc;
         const float nm = fmaxf(run_max, x), base = nm == -INFINITY ? 0.f : nm;
         run_sum = fmaf(run_sum, ex2(run_max - base), ex2(x - base));
@@ -124,13 +124,13 @@ __device__ __noinline__ float2 redo_lse(const SplitArgs &a, int sh, int query, i
     }
     return make_float2(run_max, run_sum);
 }
-// Probabilities that a key gets from the queries from query0 on, 32 at most; lse = their normalisers.
+// Probabilities that a key gets from the queries of the tile from query0 on; lse = their normalisers.
 template <int D>
 __device__ __noinline__ float redo_colsum(const SplitArgs &a, int sh, int key, int query0, const float *lse, float sc)
 {
     const float *q = head_rows(a.q, a.qs, a, sh), *k = head_rows(a.k, a.ks, a, sh) + key * a.ks.n;
     float sum = 0.f;
-    for (int m = max(key, query0); m < min(a.N, query0 + 32); ++m)
+    for (int m = max(key, query0); m < min(a.N, query0 + TT); ++m)
         sum += ex2(fmaf(fma_logit<D>(q + m * a.qs.n, k), sc, -lse[m - query0]));
     return sum;
 }
@@ -418,6 +418,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
         };
         // Column sums of a tile; on the diagonal tile only the blocks from this warp's keys on count.
         auto sum_tile = [&](const float *lse, int sh, int key, int tile, bool diag, float sc, float &col_sum) {
+            const float before = col_sum;
             for (int u = 0; u < U::PER_TILE; ++u) {
                 warp_wait(s_full + rs.idx, rs.phase, dead, &s_abort);
                 fence_after();
@@ -425,15 +426,14 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
                 for (int cb = max(diag ? warp : 0, u * U::BLOCKS); cb < (u + 1) * U::BLOCKS; ++cb) {
                     float v[32];
                     load_logits<D>(lane_addr + rs.idx * kBuf + (cb - u * U::BLOCKS) * 32, v);
-                    float part = colsum_block<32, 0>(v, lse + cb * 32, sc, diag && cb == warp, lane);
-                    const bool redo = part != part && col_sum == col_sum && key < a.N;
-                    if (__any_sync(0xffffffffu, redo)) {
-                        if (redo) part = redo_colsum<D>(a, sh, key, tile * TT + cb * 32, lse + cb * 32, sc);
-                        __syncwarp();
-                    }
-                    col_sum += part;
+                    col_sum += colsum_block<32, 0>(v, lse + cb * 32, sc, diag && cb == warp, lane);
                 }
                 release();
+            }
+            const bool redo = col_sum != col_sum && before == before && key < a.N;
+            if (__any_sync(0xffffffffu, redo)) {
+                if (redo) col_sum = before + redo_colsum<D>(a, sh, key, tile * TT, lse, sc);
+                __syncwarp();
             }
         };
         for (;;) {
@@ -453,6 +453,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
                 for (int j = 0; j <= t; ++j) {
                     // on the diagonal tile only the 32-column blocks up to this warp's rows count
                     const int c_hi = j == t ? warp : TT / 32 - 1;
+                    const float old_max = run_max, old_sum = run_sum;
                     for (int u = 0; u < U::PER_TILE; ++u) {
                         warp_wait(s_full + rs.idx, rs.phase, dead, &s_abort);
                         fence_after();
@@ -464,19 +465,18 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
 #pragma unroll
                                 for (int i = 0; i < 32; ++i) v[i] = i <= lane ? v[i] : -INFINITY;
                             }
-                            const float old_max = run_max, old_sum = run_sum;
                             lse_block<32, 0>(v, sc, sc > 0.f, run_max, run_sum);
-                            const bool redo = run_sum != run_sum && old_sum == old_sum && grow < a.N;
-                            if (__any_sync(0xffffffffu, redo)) {
-                                if (redo) {
-                                    const float2 r = redo_lse<D>(a, sh, grow, j * TT + cb * 32, sc, old_max, old_sum);
-                                    run_max = r.x;
-                                    run_sum = r.y;
-                                }
-                                __syncwarp();
-                            }
                         }
                         release();
+                    }
+                    const bool redo = run_sum != run_sum && old_sum == old_sum && grow < a.N;
+                    if (__any_sync(0xffffffffu, redo)) {
+                        if (redo) {
+                            const float2 r = redo_lse<D>(a, sh, grow, j * TT, sc, old_max, old_sum);
+                            run_max = r.x;
+                            run_sum = r.y;
+                        }
+                        __syncwarp();
                     }
                 }
                 const float lse = run_max + log2f(run_sum);
