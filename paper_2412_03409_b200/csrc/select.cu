@@ -18,9 +18,14 @@ namespace pkv {
 // shared memory), turns the table of the warps' counts into offsets with one scan in the order (digit,
 // warp), and moves keys and positions to their places in shared memory.
 //
+// Up to 256 scores, one a thread, there are no passes: an item's place is the number of items before it, counted.
+//
 // Bounded by the issue slots of the ranking (some 60 instructions an item and pass) and, after it, by the
-// scattered stores.  32 segments of 640 scores: 13.4 us with a bitonic network of 64-bit keys, 10.7 now;
-// 64 segments of 16384: 204 us, 75 now.
+// scattered stores; with few items by the barriers of the passes and, as each warp brings a table of 256 counts
+// to be scanned, by the number of warps.  64 segments of 16384: 204 us with a bitonic network of 64-bit keys,
+// 75 now.  Sort and search together, 32 segments, bitonic / one item a thread / as here: 64 scores 18.3 / 19.2 /
+// 17.3 us, 256 16.2 / 16.4 / 15.1, 640 28.6 / 25.9 / 24.2, 1024 34.9 / 37.1 / 31.5, 2048 44.5 / 38.2 (two items)
+// / 33.8; 512 segments of 1024 62.8 / 67.0 / 40.7.
 // ---------------------------------------------------------------------------
 // Fixed-point weight of a sort key (inverted score bits): round-half-even(score * 2^32).  In integers:
 // fp64 instructions are few per clock here, and two conversions and a product per key took a good part of
@@ -87,6 +92,31 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
             key[i] = ~bits;
         }
     }
+    if constexpr (IPT == 1) {
+        skey[tid] = key[0];
+        __syncthreads();
+        uint32_t place = 0;
+        const uint4 *four = reinterpret_cast<const uint4 *>(skey);
+        for (int i = 0; i < warp * 8; ++i) {  // equal keys of earlier places come first
+            const uint4 x = four[i];
+            place += (x.x <= key[0]) + (x.y <= key[0]) + (x.z <= key[0]) + (x.w <= key[0]);
+        }
+        for (int i = (warp + 1) * 8; i < nthr / 4; ++i) {
+            const uint4 x = four[i];
+            place += (x.x < key[0]) + (x.y < key[0]) + (x.z < key[0]) + (x.w < key[0]);
+        }
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i) {
+            const uint32_t x = __shfl_sync(0xffffffffu, key[0], i);
+            place += x < key[0] || (x == key[0] && i < lane);
+        }
+        __syncthreads();
+        skey[place] = key[0];
+        spos[place] = pos[0];
+        __syncthreads();
+        key[0] = skey[tid];
+        pos[0] = spos[tid];
+    } else
     for (int shift = 0; shift < 32; shift += 8) {
         for (int i = tid; i < kDigits * nwarp; i += nthr) count[i] = 0;
         __syncthreads();  // (and every item of the pass before is in registers)
@@ -410,13 +440,16 @@ static int launch_sort_items(const pkv_shape *s, const float *scores, int32_t *o
     return PKV_OK;
 }
 
-// As few items per thread as 1024 threads allow.
+// Up to 256 scores places are counted: the work grows with the square, 512 of them cost more than the passes.
+// Two items a thread beat four up to some 768 scores for one prompt (18.0 / 18.4 us with the search) and not for
+// 16 (42.8 / 37.6); beyond, four do throughout (1024: 19.8 / 19.2 and 47.9 / 40.7).  Above that as few as 1024
+// threads allow.
 static int launch_sort(const pkv_shape *s, const float *scores, int32_t *order, uint64_t *cum,
                        int32_t *seg_flags, cudaStream_t st)
 {
     const int N = s->prompt_len;
-    if (N <= 1024) return launch_sort_items<1>(s, scores, order, cum, seg_flags, st);
-    if (N <= 2048) return launch_sort_items<2>(s, scores, order, cum, seg_flags, st);
+    if (N <= 256) return launch_sort_items<1>(s, scores, order, cum, seg_flags, st);
+    if (N <= 768) return launch_sort_items<2>(s, scores, order, cum, seg_flags, st);
     if (N <= 4096) return launch_sort_items<4>(s, scores, order, cum, seg_flags, st);
     if (N <= 8192) return launch_sort_items<8>(s, scores, order, cum, seg_flags, st);
     return launch_sort_items<16>(s, scores, order, cum, seg_flags, st);

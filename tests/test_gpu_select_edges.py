@@ -29,6 +29,8 @@ def _scores(kind, L, N, seed):
 @pytest.mark.parametrize("B,L,N,kind,tol", [
     (1, 3, 1, "wide", 0.0), (2, 2, 31, "ties", 0.0), (1, 4, 33, "halves", 1e-6), (1, 5, 1023, "exp", 1e-15),
     (1, 33, 1024, "ties", 1e-6), (2, 65, 1025, "wide", 1e-6), (1, 3, 2049, "halves", 1e-17), (1, 130, 700, "exp", 0.0),
+    (1, 3, 64, "ties", 0.0), (2, 3, 255, "halves", 0.0), (1, 4, 256, "ties", 1e-6), (1, 4, 257, "ties", 1e-6),
+    (1, 3, 768, "wide", 0.0), (2, 3, 769, "ties", 1e-9), (1, 2, 3072, "halves", 0.0),
     (1, 2, 4097, "ties", 0.0), (1, 2, 8193, "wide", 1e-9), (1, 3, 16384, "exp", 0.25), (1, 2, 16383, "halves", 2.0),
 ])
 @pytest.mark.parametrize("ratio,max_iters", [(0.2, 2000), (0.7, 2000), (0.33, 3)])
