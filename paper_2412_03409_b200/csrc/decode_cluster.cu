@@ -17,7 +17,7 @@
 // Measured, device time of calls replayed from a graph, against the row-split kernel and its merge
 // kernel (one layer, bf16, D = 128): 1 segment x 32 heads x 128 rows 4.5 us (10.0), 1024 rows 8.0
 // (26.4); 4 x 32 x 128 rows 6.1 (12.1); 8 x 40 x 410 rows 17.4 (25.7; 10.3 us of bytes: SMs hold four
-// or five of the 642 CTAs); 16 x 32 x 2048 rows 89 (91).  A second wave of CTAs costs as much as the
+// or five of the 642 CTAs); 8 x 64 x 900 rows 50 (51).  A second wave of CTAs costs as much as the
 // first's latency, 4-5 us (C = 8 for 4 x 32 x 128 rows: 8.9 us), hence the choice of C below.  Loads to
 // registers instead of the rings, eight steps of K and V in flight: the same for one round of rows,
 // 20.5 us for 8 x 40 x 410.  Ring shapes (steps, rounds, CTAs per SM): 4, 2, 5 as here; 8, 2, 3 and
@@ -28,6 +28,8 @@
 #include "decode_plan.cuh"
 
 namespace pkv {
+
+bool decode_stream_covers(const pkv_shape *s, int nact);
 
 namespace {
 
@@ -368,9 +370,23 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     if ((int64_t)nact * H >= 4 * (int64_t)sms) return -1;  // (the per-head kernel's and the row-split kernel's calls)
     const int items = nact * H;
     const int64_t seg_rows = c->total_cap_rows / ((int64_t)s->batch * s->layers);
+    // Long segments are the row-split kernel's, where it covers the shape: eight CTAs of a pair keep 256 KiB in
+    // flight however long it is, and CTAs that come in waves read the slices of a row at different times.
+    // Measured, one layer, this kernel / row-split.  Few pairs, by a pair's bytes: 1 head of 128, bf16, 12000 rows
+    // (6.1 MB) 29 / 33 us, 16000 (8.2) 38 / 35, fp32 6000 rows 29 / 30, 8000 38 / 31, 16000 70 / 35; 8 heads
+    // fp32 8000 38 / 40, 12000 56 / 45.  From 24 pairs on the row-split kernel's merge costs more: 24 heads fp32
+    // 12000 rows (12.3 MB) 64 / 81, 32 pairs of 4 segments 72 / 73, 16000 rows 94 / 92.  Many pairs, by pairs x
+    // rows: 128 x 4000 rows 52 / 55, x 6000 73 / 73, x 12000 137 / 130; 512 x 1100 55 / 59, x 1800 89 / 83 (heads
+    // of 64: 34 / 36, 55 / 49); 576 x 1100 60 / 60, x 1800 96 / 90; and by bytes: 64 pairs of 8000 rows of fp32
+    // (524 MB) 90 / 90, 12000 134 / 126.
+    const int64_t pair_bytes = seg_rows * D * 2 * (int64_t)esize(s);
+    if ((pair_bytes > ((int64_t)(items < 24 ? 6 : 12) << 20) || items * seg_rows > (640 << 10) ||
+         items * pair_bytes > ((int64_t)512 << 20)) &&
+        decode_stream_covers(s, nact))
+        return -1;
     // As many CTAs as the SMs hold at a time, none of them with less than one round of rows (32) unless
     // the call is so small that SMs would be idle; further waves only for CTAs of 256 rows and more,
-    // whose bytes outweigh a wave's latency (16 x 32 x 2048 rows: C = 1 111 us, 6 89 us).
+    // whose bytes outweigh a wave's latency (16 x 32 x 2048 rows: C = 1 111 us, 6 89 us in one run, 99 in another).
     int C = 1;
     while (C < kCMaxCluster) {
         const int n = C + 1;
