@@ -97,8 +97,9 @@ const char *prefixkv_last_cuda_error(void);
  * bf16 inputs use tensor cores with fp32 accumulation; fp32 inputs too, each element split into
  * three bf16 numbers (exactly, from 2^-110 in magnitude up): a single product has an error of up to
  * 1.5 * 2^-23, a logit of many like terms one below that of fp32 FMA (logits that an infinite element
- * or one above the largest bf16 takes part in are formed by FMA); bf16 inputs whose strides no tensor map can describe,
- * e.g. a zero stride, use FMA.
+ * or one above the largest bf16 takes part in are formed by FMA).  bf16 inputs whose strides no
+ * tensor map can describe, e.g. a zero stride, use FMA, and so do fp32 prompts of up to 64 tokens
+ * with heads of 64 and the caller's lse.
  * The workspace holds per-head partial sums and work counters: calls that share one must
  * not overlap on the GPU.  The call has no status argument: if a bounded wait inside the
  * tensor-core kernel runs out, every score of the call is written as NaN, which

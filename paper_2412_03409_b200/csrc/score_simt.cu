@@ -1,5 +1,6 @@
 // Importance score (Sec. 3.2), FP32-FMA path: used for bf16 inputs whose strides no tensor map can
-// describe (a zero stride), and the head mean of every path.
+// describe (a zero stride), for short fp32 prompts with heads of 64 and the caller's log-sum-exp (one
+// tile of 64 x 64), and the head mean of every path.
 //
 //   pass 1: per query m, log2-sum-exp of the scaled causal logits (keys j <= m)
 //   pass 2: per key n, sum over queries m >= n of exp2(logit - lse[m])
@@ -218,6 +219,7 @@ int launch_score_simt(const pkv_shape *s, const void *q, pkv_strides qs, const v
     template int launch_score_simt<T, D>(const pkv_shape *, const void *, pkv_strides, const void *, \
                                          pkv_strides, const float *, const float *, float *, void *, \
                                          cudaStream_t);
+PKV_INST(float, 64)
 PKV_INST(__nv_bfloat16, 64)
 PKV_INST(__nv_bfloat16, 128)
 #undef PKV_INST

@@ -15,6 +15,7 @@ TOL = 1e-5
 SHAPES = [(1, 1, 1, 64, 1), (1, 2, 3, 128, 127), (1, 2, 2, 64, 128), (1, 1, 2, 128, 129), (1, 2, 2, 64, 193),
           (1, 1, 2, 128, 257), (2, 1, 3, 64, 385), (1, 1, 2, 128, 1150),   # a set's turn comes round several times
           (1, 10, 20, 64, 65), (1, 5, 40, 128, 40),                        # one-tile items, more than SMs
+          (1, 2, 3, 64, 63), (2, 2, 3, 64, 64),                            # fp32 with the caller's lse: FMA kernel
           (1, 13, 20, 64, 600)]                                            # items from the counters
 
 
@@ -113,21 +114,22 @@ def test_fp32_infinite_and_huge_elements(N, lo, hi, D, given_lse):
 
 @pytest.mark.parametrize("D", [64, 128])
 def test_fp32_single_products(D):
-    """Logits of one product each, prompts of one token: dropped parts of the split are at most 2^-24 of the product,
+    """Logits of one product each, of the last token with itself: dropped parts of the split are at most 2^-24 of the product,
     the last of the accumulations, which truncate, 2^-23, and those before it next to nothing."""
     from paper_2412_03409_b200.session import Session
-    L = 4096
+    L, N = 4096, 1 if D == 128 else 65  # (64 tokens and fewer of D = 64 go to the FMA kernel)
     rng = np.random.default_rng(D)
     x, y = (np.float32(1) + rng.integers(0, 1 << 23, (2, L)) * np.float32(2.0 ** -23)).astype(np.float32)
     x[:2048] = y[:2048] = np.float32(1) + (0xfe80 + np.arange(2048) - 1024) * np.float32(2.0 ** -23)  # two large lower parts
     scale = (64 / (x.astype(np.float64) * y)).astype(np.float32)
     lse = (scale.astype(np.float64) * x * y).astype(np.float32)
-    q, k = (torch.zeros(1, L, 1, 1, D, device="cuda") for _ in range(2))
+    q, k = (torch.zeros(1, L, 1, N, D, device="cuda") for _ in range(2))
     place = torch.arange(L, device="cuda") % D
-    q[0, torch.arange(L), 0, 0, place] = torch.from_numpy(x).cuda()
-    k[0, torch.arange(L), 0, 0, place] = torch.from_numpy(y).cuda()
-    s = Session(1, L, 1, D, 1, torch.float32, scale, decode_cap=0, max_budget_rows=L)
-    got = s.score(q, k, lse=torch.from_numpy(lse).cuda().view(1, L, 1, 1)).cpu().numpy().reshape(L).astype(np.float64)
+    q[0, torch.arange(L), 0, N - 1, place] = torch.from_numpy(x).cuda()
+    k[0, torch.arange(L), 0, N - 1, place] = torch.from_numpy(y).cuda()
+    given = torch.from_numpy(lse).cuda().view(1, L, 1, 1).expand(1, L, 1, N).contiguous()
+    s = Session(1, L, 1, D, N, torch.float32, scale, decode_cap=0, max_budget_rows=L)
+    got = s.score(q, k, lse=given)[0, :, N - 1].cpu().numpy().astype(np.float64)
     log2e = np.float32(np.log2(np.e))
     sc, l2 = (scale * log2e).astype(np.float64), (lse * log2e).astype(np.float64)   # rounded as the kernel rounds them
     exact = sc * (x.astype(np.float64) * y)
