@@ -42,6 +42,7 @@ constexpr int kCMaxCluster = 8;        // portable cluster size
 constexpr int kCMaxCtas = 8192;        // CTAs of a call (flags in the workspace)
 constexpr uint32_t kCSpinLimit = 1u << 22;
 constexpr float kLog2eC = 1.4426950408889634f;
+constexpr float kNoLogit = -3.402823466e38f;  // the lowest finite number
 
 struct ClusterArgs {
     DecodePlanArgs p;
@@ -90,18 +91,14 @@ __global__ void selftest_flags_kernel(int32_t *dev_status, uint32_t limit)
     if (i < n) flags[i] = i % 3 ? 0ull : ~(unsigned long long)i;  // (left from anything)
     __syncthreads();
     bool ok = true;
-    if (i < came) ok = !raise_flag(flags + i, token);
+    if (i < came) ok = !unraise_flag(flags + i, token, raise_flag(flags + i, token));
     __syncthreads();
     ok = !settle_flags(flags, n, token, limit) && ok;
     __syncthreads();
-    if (i >= came && i < n) {
-        const bool late = raise_flag(flags + i, token);
-        if (late) lower_flag(flags + i);
-        ok = ok && late;
-    }
+    if (i >= came && i < n) ok = unraise_flag(flags + i, token, raise_flag(flags + i, token)) && ok;
     __syncthreads();
     if (i < n) ok = ok && flags[i] == 0ull;
-    if (i < n) ok = !raise_flag(flags + i, token) && ok;
+    if (i < n) ok = !unraise_flag(flags + i, token, raise_flag(flags + i, token)) && ok;
     __syncthreads();
     ok = settle_flags(flags, n, token, limit) && ok;
     __syncthreads();
@@ -162,17 +159,17 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
     const float sc = a.layer_scale[a.p.layer_begin + si % a.p.nl] * kLog2eC;
     const SegPlan sp = segment_plan(a.p, si);
     __syncthreads();  // all of this CTA's reads of the lengths are done
-    bool late = false;
-    if (tid == 0) late = raise_flag(a.flags + blockIdx.x, a.token);
+    unsigned long long held = 0;
+    if (tid == 0) held = raise_flag(a.flags + blockIdx.x, a.token);
 
     // cached rows of the segment that are attended to: all of them, less the slot that the new row reuses
     const int cached = sp.rows < 0 ? 0 : (a.p.append ? (sp.evict ? sp.rows : sp.rows - 1) : sp.rows);
     const int skip = sp.evict ? sp.dst : -1;
     const int per = (cached + C - 1) / C;
     const int r0 = min(cached, rank * per), r1 = min(cached, r0 + per);
-    // M: the running maximum of the logits; Mz: the same, or 0 as long as all of them were -infinity or NaN, so
-    // that exp2f(s - Mz) is 0 for the one and stays NaN for the other.
-    float qf[VE], acc[VE], M = -INFINITY, Mz = 0.f, lsum = 0.f;
+    // M: the running maximum of the logits, from the lowest finite number on, so that exp2f(s - M) is 0 for a logit
+    // of -infinity and NaN for NaN whatever came before it.
+    float qf[VE], acc[VE], M = kNoLogit, lsum = 0.f;
     RowVec<T>::unpack(qraw, qf);
 #pragma unroll
     for (int i = 0; i < VE; ++i) {
@@ -204,8 +201,7 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
 #pragma unroll
         for (int o = LPR; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         const float Mn = fmaxf(M, mx);
-        Mz = Mn == -INFINITY ? 0.f : Mn;
-        const float corr = exp2f(M - Mz);
+        const float corr = exp2f(M - Mn);
         M = Mn;
         lsum *= corr;
 #pragma unroll
@@ -251,7 +247,7 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         for (int j = 0; j < kCU; ++j) {
             const int r = base + j * G + grp;
             if (r < r1 && r != skip)
-                add(exp2f(s[j] - Mz), *reinterpret_cast<const uint4 *>(kt + kCRound + j * 512));
+                add(exp2f(s[j] - M), *reinterpret_cast<const uint4 *>(kt + kCRound + j * 512));
         }
         request(base + kCStages * kCWarps * STEP, stage);
         if (++stage == kCStages) stage = 0;
@@ -262,15 +258,13 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         rescale(s);
         if (grp == 0) {
-            add(exp2f(s - Mz), vnew);
+            add(exp2f(s - M), vnew);
             // the append: this head's slice of the new row goes to its place in the cache
             const size_t at = (size_t)(sp.off + sp.dst) * a.row_bytes + (size_t)h * SLICE + c * 16;
             *reinterpret_cast<uint4 *>(static_cast<unsigned char *>(a.ck) + at) = knew;
             *reinterpret_cast<uint4 *>(static_cast<unsigned char *>(a.cv) + at) = vnew;
         }
     }
-
-    if (late) lower_flag(a.flags + blockIdx.x);
 
     // ---- merge: lane groups, warps, then the CTAs of the cluster ---------------------------------------
 #pragma unroll
@@ -288,14 +282,13 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         s_ml[warp][1] = lsum;
     }
     __syncthreads();
-    // A state without rows has maximum -inf and weight 0 (at least one state of an item has rows); so has one whose
-    // only logits are NaN, and its sums, NaN, come through the product with 0.
-    float z = 0.f, o = 0.f, m = -INFINITY;
+    // (a state without rows has sums of 0; one whose only logits are NaN has sums of NaN, whatever their factor)
+    float z = 0.f, o = 0.f, m = kNoLogit;
 #pragma unroll
     for (int w = 0; w < kCWarps; ++w) m = fmaxf(m, s_ml[w][0]);
 #pragma unroll
     for (int w = 0; w < kCWarps; ++w) {
-        const float f = s_ml[w][0] == -INFINITY ? 0.f : exp2f(s_ml[w][0] - m);
+        const float f = exp2f(s_ml[w][0] - m);
         z = fmaf(f, s_ml[w][1], z);
         if (tid < D) o = fmaf(f, s_acc[w][tid], o);
     }
@@ -307,20 +300,24 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
             store_first_cta(&c_ml[rank][1], z);
         }
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        if (rank != 0) return;  // (only the first CTA's memory is written, and it waits for everyone)
+        if (rank != 0) {  // (only the first CTA's memory is written, and it waits for everyone)
+            unraise_flag(a.flags + blockIdx.x, a.token, held);
+            return;
+        }
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        m = -INFINITY;
+        m = kNoLogit;
         for (int r = 0; r < C; ++r) m = fmaxf(m, c_ml[r][0]);
         z = 0.f;
         o = 0.f;
         for (int r = 0; r < C; ++r) {
-            const float f = c_ml[r][0] == -INFINITY ? 0.f : exp2f(c_ml[r][0] - m);
+            const float f = exp2f(c_ml[r][0] - m);
             z = fmaf(f, c_ml[r][1], z);
             if (tid < D) o = fmaf(f, c_acc[r][tid], o);
         }
     }
     if (tid < D)  // (a segment that cannot take the step is reported by the extra cluster; its output is zero)
         reinterpret_cast<T *>(static_cast<unsigned char *>(a.out) + hoff)[tid] = from_float<T>(sp.rows < 0 ? 0.f : o * (1.f / z));
+    unraise_flag(a.flags + blockIdx.x, a.token, held);
 }
 
 template <typename T, int D> int launch_cluster(const ClusterArgs &a, int C, cudaStream_t st)

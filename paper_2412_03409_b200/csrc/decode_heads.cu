@@ -252,8 +252,8 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
     __syncthreads();
     // every length this CTA needs has been read: say so (the last CTA waits for all flags before it
     // writes the lengths of the next step)
-    bool late = false;
-    if (tid == 0 && append) late = raise_flag(a.flags + blockIdx.x, a.token);
+    unsigned long long held = 0;
+    if (tid == 0 && append) held = raise_flag(a.flags + blockIdx.x, a.token);
 
     const int nitems = a.nact * H;
 
@@ -520,7 +520,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
         if (dead && lane == 0) raise_status(a.dev_status, 0, PKV_DEV_TIMEOUT);
     }
 
-    if (late) lower_flag(a.flags + blockIdx.x);
+    unraise_flag(a.flags + blockIdx.x, a.token, held);
 
     // ---- the lengths of the next step, once every CTA has read this step's -------------------------
     if (blockIdx.x == gridDim.x - 1 && append) {

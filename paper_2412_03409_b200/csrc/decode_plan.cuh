@@ -130,29 +130,50 @@ __device__ __forceinline__ void segment_advance(const DecodePlanArgs &a, int si,
 // A flag of kGone ^ token belongs to a CTA that is no longer waited for.
 constexpr unsigned long long kGone = 2;
 
-// One thread of a CTA: this CTA has read the lengths.  True when nobody waits for it any more; the flag is then
-// to be put to zero (lower_flag; later, so that the answer's latency is not in the way).
-__device__ __forceinline__ bool raise_flag(unsigned long long *flag, unsigned long long token)
+// One thread of a CTA: this CTA has read the lengths.  What the flag held goes to unraise_flag when the CTA's work
+// is done (and the answer has come): when nobody was waiting any more, it puts the flag to zero; true then.
+__device__ __forceinline__ unsigned long long raise_flag(unsigned long long *flag, unsigned long long token)
 {
-    __threadfence();
-    return atomicExch(flag, token) == (token ^ kGone);
+    unsigned long long held;
+    asm volatile("atom.release.gpu.exch.b64 %0, [%1], %2;" : "=l"(held) : "l"(flag), "l"(token) : "memory");
+    return held;
 }
 __device__ __forceinline__ void lower_flag(unsigned long long *flag) { *(volatile unsigned long long *)flag = 0ull; }
+__device__ __forceinline__ bool unraise_flag(unsigned long long *flag, unsigned long long token, unsigned long long held)
+{
+    const bool late = held == (token ^ kGone);
+    if (late) lower_flag(flag);
+    return late;
+}
+
+__device__ __forceinline__ unsigned long long load_flag(const unsigned long long *flag)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.u64 %0, [%1];" : "=l"(v) : "l"(flag) : "memory");
+    return v;
+}
 
 // A whole CTA: waits for n flags and puts them back to zero.  False when the limit ran out: the flags
 // of those that have come are zero then, the others' get zero from their own CTAs when these come.
 __device__ __forceinline__ bool settle_flags(unsigned long long *flags, int n, unsigned long long token, uint32_t limit)
 {
+    constexpr int kBatch = 8;  // flags of a thread asked for at once
     bool all_in = true;
-    for (int i = threadIdx.x; i < n && all_in; i += blockDim.x) {
-        all_in = false;
-        for (uint32_t t = 0; t < limit; ++t)
-            if (*(volatile unsigned long long *)(flags + i) == token) {
-                all_in = true;
-                break;
-            }
+    for (int i0 = threadIdx.x; i0 < n && all_in; i0 += kBatch * blockDim.x) {
+        unsigned long long v[kBatch];
+#pragma unroll
+        for (int e = 0; e < kBatch; ++e) {
+            const int i = i0 + e * (int)blockDim.x;
+            v[e] = i < n ? load_flag(flags + i) : token;
+        }
+#pragma unroll
+        for (int e = 0; e < kBatch; ++e)
+            for (uint32_t t = 0; v[e] != token && t < limit; ++t) v[e] = load_flag(flags + i0 + e * blockDim.x);
+#pragma unroll
+        for (int e = 0; e < kBatch; ++e) all_in = all_in && v[e] == token;
     }
-    __threadfence();  // what follows comes after the reads that the flags stand for
+    // (as raise_flag releases: what follows comes after the reads that the flags stand for)
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
     all_in = __syncthreads_and(all_in);
     for (int i = threadIdx.x; i < n; i += blockDim.x)
         if (all_in || atomicExch(flags + i, token ^ kGone) == token) lower_flag(flags + i);
