@@ -373,11 +373,11 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     // (6.1 MB) 29 / 33 us, 16000 (8.2) 38 / 35, fp32 6000 rows 29 / 30, 8000 38 / 31, 16000 70 / 35; 8 heads
     // fp32 8000 38 / 40, 12000 56 / 45.  From 24 pairs on the row-split kernel's merge costs more: 24 heads fp32
     // 12000 rows (12.3 MB) 64 / 81, 32 pairs of 4 segments 72 / 73, 16000 rows 94 / 92.  Many pairs, by pairs x
-    // rows: 128 x 4000 rows 52 / 55, x 6000 73 / 73, x 12000 137 / 130; 512 x 1100 55 / 59, x 1800 89 / 83 (heads
-    // of 64: 34 / 36, 55 / 49); 576 x 1100 60 / 60, x 1800 96 / 90; and by bytes: 64 pairs of 8000 rows of fp32
+    // rows: 128 x 6000 rows 73 / 73, x 12000 137 / 130; 320 x 1800 58 / 59, x 3200 86 / 92; 512 x 1100 55 / 59, x
+    // 1800 89 / 83 (heads of 64: 34 / 36, 55 / 49); 576 x 1100 60 / 60, x 1800 96 / 90; and by bytes: 64 pairs of 8000 rows of fp32
     // (524 MB) 90 / 90, 12000 134 / 126.
     const int64_t pair_bytes = seg_rows * D * 2 * (int64_t)esize(s);
-    if ((pair_bytes > ((int64_t)(items < 24 ? 6 : 12) << 20) || items * seg_rows > (640 << 10) ||
+    if ((pair_bytes > ((int64_t)(items < 24 ? 6 : 12) << 20) || items * seg_rows > (items <= 320 ? 1 << 20 : 704 << 10) ||
          items * pair_bytes > ((int64_t)512 << 20)) &&
         decode_stream_covers(s, nact))
         return -1;
