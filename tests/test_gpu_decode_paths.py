@@ -1,6 +1,7 @@
 """Decode calls that take each of the library's kernels, against the oracle on the cache as it stands
 (needs a B200).  Few (segment, head) pairs: the cluster kernel; from four pairs per SM (592) the
-per-head kernel, the row-split kernel (long segments, pruning) or, above 64 heads, the two-kernel path."""
+per-head kernel, the row-split kernel (long segments, more than 256 of them, pruning) or, above 64 heads, the
+two-kernel path."""
 import numpy as np
 import pytest
 import torch
@@ -28,6 +29,31 @@ CASES = [  # B, L, H, D, N, rows per layer, dtype, evict_distance
     (1, 20, 32, 64, 1100, 1050, torch.bfloat16, 0),   # 640 pairs, long segments: row-split kernel
     (1, 9, 72, 64, 100, 20, torch.bfloat16, 0),       # 648 pairs, 72 heads: two-kernel path when segments are long
     (1, 9, 72, 64, 1300, 1200, torch.bfloat16, 0),
+    # the row-split kernel: the (lanes per row, heads per warp, rows per unit, block size) that fewer than 900 segments
+    # choose, and one that more do.
+    # Rows of up to 8.9 KB go in units of eight, up to 16.5 KB of four, up to 28.9 KB of two; many segments leave
+    # less room for the ring.
+    (1, 38, 16, 128, 40, 12, torch.bfloat16, 3),      # 8, 1, 8
+    (1, 15, 40, 128, 40, 12, torch.bfloat16, 3),      # 16, 4, 4, 12 warps
+    (1, 10, 64, 128, 40, 12, torch.bfloat16, 3),      # 16, 4, 4, 17 warps
+    (4, 32, 64, 128, 24, 6, torch.bfloat16, 3),       # 16, 4, 2, 17 warps
+    (2, 19, 16, 64, 40, 12, torch.bfloat16, 3),       # 8, 1, 8
+    (2, 10, 32, 64, 40, 12, torch.bfloat16, 3),       # 8, 2, 8
+    (1, 15, 40, 64, 40, 12, torch.bfloat16, 3),       # 8, 4, 8, 12 warps
+    (1, 10, 64, 64, 40, 12, torch.bfloat16, 3),       # 8, 4, 8, 17 warps
+    (1, 38, 16, 128, 40, 12, torch.float32, 3),       # 8, 1, 8
+    (30, 32, 16, 128, 20, 4, torch.float32, 3),       # 8, 1, 4
+    (1, 20, 32, 128, 40, 12, torch.float32, 3),       # 16, 2, 4
+    (4, 32, 32, 128, 24, 6, torch.float32, 3),        # 16, 2, 2
+    (1, 15, 40, 128, 40, 12, torch.float32, 3),       # 16, 4, 2, 12 warps
+    (1, 11, 56, 128, 40, 12, torch.float32, 3),       # 16, 4, 2, 17 warps
+    (1, 38, 16, 64, 40, 12, torch.float32, 3),        # 8, 1, 8
+    (1, 20, 32, 64, 40, 12, torch.float32, 3),        # 16, 2, 8
+    (1, 15, 40, 64, 40, 12, torch.float32, 3),        # 16, 4, 4, 12 warps
+    (1, 10, 64, 64, 40, 12, torch.float32, 3),        # 16, 4, 4, 17 warps
+    (10, 32, 2, 128, 40, 9, torch.bfloat16, 0),       # 320 segments
+    (1, 1, 2, 128, 6600, 6500, torch.float32, 0),     # two pairs of 6.7 MB each: split over all SMs
+    (2, 12, 32, 128, 1100, 1040, torch.bfloat16, 0),  # segments split over a few CTAs each
 ]
 
 
@@ -84,7 +110,7 @@ def test_decode_steps_match_the_oracle(B, L, H, D, N, rows, dtype, d):
             assert np.abs(got[b, l] - ref).max() <= TOL[dtype]
 
 
-@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d", [CASES[4], CASES[6], CASES[8], CASES[9]])
+@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d", [CASES[4], CASES[6], CASES[8], CASES[9], CASES[-2], CASES[-1]])
 @pytest.mark.parametrize("byte", [0x7f, 0xff])
 def test_replay_and_stale_workspace(B, L, H, D, N, rows, dtype, d, byte):
     """A captured call replayed token after token, over a workspace that holds anything, gives bit for

@@ -270,10 +270,10 @@ def _decode_reference(w, s, k, v, ref_sel, steps, layer_scale):
     ("llava7b_b16", dict(B=3, L=2, H=4, N=97, T=4)),
     ("tiny", dict(D=128, H=2, T=3)),
     ("llava7b_b1", dict(L=2, H=5, D=64, N=130, T=3)),
-    ("tiny", dict(D=128, H=32, L=2, N=100, T=3)),           # fp32 rows of 16 KiB: four-row units
-    ("llava7b_b1", dict(L=2, H=64, N=90, T=2)),              # 64 heads: four heads per consumer warp
-    ("llava7b_b1", dict(L=2, H=72, D=64, N=90, T=2)),        # more heads than the streaming kernel takes: two-kernel path
-    ("llava7b_b16", dict(B=40, L=32, H=2, D=64, N=24, T=2)),  # 1280 segments: two layer chunks through the streaming kernel
+    ("tiny", dict(D=128, H=32, L=2, N=100, T=3)),           # fp32 rows of 16 KiB
+    ("llava7b_b1", dict(L=2, H=64, N=90, T=2)),              # 64 heads
+    ("llava7b_b1", dict(L=2, H=72, D=64, N=90, T=2)),        # more heads than the row-split kernel takes
+    ("llava7b_b16", dict(B=40, L=32, H=2, D=64, N=24, T=2)),  # 1280 segments: two layer chunks through the row-split kernel
     # few segments, many (segment, head) items: the per-head kernel (whole softmax rows per CTA)
     ("llava7b_b1", dict(L=20, H=32, N=100, T=3)),            # bf16, 256-byte head slices
     ("tiny", dict(L=16, H=40, N=70, T=3)),                   # fp32, D = 64
@@ -328,7 +328,7 @@ def test_decode_full_budget_is_dense_attention(api):
 
 
 @pytest.mark.parametrize("kw,step", [
-    (dict(L=4, H=4, N=80, T=2), 1),                 # a model calls one layer at a time (streaming kernel)
+    (dict(L=4, H=4, N=80, T=2), 1),                 # a model calls one layer at a time (cluster kernel)
     (dict(B=2, L=20, H=32, N=70, T=2), 10),         # two samples, ten layers per call: the per-head kernel on a sub-range
 ])
 def test_decode_layer_range(api, kw, step):
@@ -350,7 +350,7 @@ def test_decode_layer_range(api, kw, step):
     assert torch.equal(a.cache.len, b.cache.len)
 
 
-@pytest.mark.parametrize("kw", [dict(L=6, H=8, N=300, T=5),        # streaming kernel + merge kernel
+@pytest.mark.parametrize("kw", [dict(L=6, H=8, N=300, T=5),        # cluster kernel
                                 dict(L=20, H=32, N=100, T=5)])     # per-head kernel
 def test_decode_replayed_from_a_cuda_graph(api, kw):
     """One decode call captured in a CUDA graph and replayed token after token gives, bit for bit,
@@ -381,13 +381,12 @@ def test_decode_replayed_from_a_cuda_graph(api, kw):
     assert int(b.status.max()) == 0
 
 
-@pytest.mark.parametrize("kw", [dict(L=6, H=8, N=300, T=2),        # streaming kernel + merge kernel
+@pytest.mark.parametrize("kw", [dict(L=6, H=8, N=300, T=2),        # cluster kernel
                                 dict(L=20, H=32, N=120, T=2)])     # per-head kernel (its flags live in the workspace)
 @pytest.mark.parametrize("byte", [0x7f, 0xff, 0x00])
 def test_decode_with_stale_workspace(api, byte, kw):
     """The decode workspace may hold anything (another shape's partials, an earlier call's plan):
-    results do not depend on it.  (The merge kernel looks at its plan record early, before the record
-    is final, and must bound what it does with that copy.)"""
+    results do not depend on it.  (The cluster and the per-head kernel keep their CTAs' flags there.)"""
     w = wl.scaled(wl.WORKLOADS["llava7b_b1"], **kw)
     q, k, v = wl.make_prompt(w, "cuda")
     scale = wl.layer_scale(w)
@@ -409,7 +408,7 @@ def test_decode_with_stale_workspace(api, byte, kw):
     assert a.status.cpu().tolist() == b.status.cpu().tolist() == [0]
 
 
-@pytest.mark.parametrize("kw", [dict(H=4), dict(H=72, D=64),       # streaming kernel; two-kernel path (H > 64)
+@pytest.mark.parametrize("kw", [dict(H=4), dict(H=72, D=64),       # cluster kernel, also above 64 heads
                                 dict(H=32, L=10)])                 # per-head kernel
 def test_decode_empty_segment_is_reported(api, kw):
     """A segment with no rows (never compacted) cannot be attended over: the sample's status says
@@ -529,9 +528,9 @@ def test_score_token_major_layout(api, name, kw):
 
 
 @pytest.mark.parametrize("name,kw", [
-    ("llava7b_b1", dict(L=2, H=4, N=300)),           # bf16: tensor-core pass 2 on a converted lse
+    ("llava7b_b1", dict(L=2, H=4, N=300)),           # bf16: pass 2 alone, on the natural-log lse as it is
     ("llava7b_b16", dict(B=2, L=1, H=3, N=129, D=64)),
-    ("tiny", dict(N=150, H=3, L=2)),                 # fp32: FMA pass 2 with the natural-log lse
+    ("tiny", dict(N=150, H=3, L=2)),                 # fp32: likewise, split into bf16 parts
     ("tiny", dict(N=70, H=2, L=1, D=128)),
 ])
 def test_score_with_caller_lse(api, name, kw):
