@@ -161,15 +161,13 @@ __device__ __forceinline__ void hbulk_load(void *dst, const void *src, uint32_t 
                  : "memory");
 }
 
-template <typename T> using HVec = RowVec<T>;
-
 // A head's slice of a row is D * sizeof(T) bytes = LPR 16-byte vectors: LPR lanes share a row, a
 // warp holds G = 32 / LPR rows at a time and a tile (8 KiB) is 16 such steps.
 template <typename T, int D>
 __global__ void __launch_bounds__((kHWarps + kHProducers) * 32, 1)
 decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 {
-    constexpr int VE = HVec<T>::VE;
+    constexpr int VE = RowVec<T>::VE;
     constexpr uint32_t SLICE = D * sizeof(T);
     constexpr int LPR = SLICE / 16;
     constexpr int G = 32 / LPR;
@@ -366,7 +364,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             float qf[VE];
             {
                 float x[VE];
-                HVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + c * 16), x);
+                RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + c * 16), x);
 #pragma unroll
                 for (int i = 0; i < VE; ++i) qf[i] = x[i] * m.sc;
             }
@@ -377,7 +375,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             for (int j = 0; j < 16; ++j) {
                 const int row = j * G + grp;
                 float x[VE], d0 = 0.f, d1 = 0.f;
-                HVec<T>::unpack(*reinterpret_cast<const uint4 *>(kt + (uint32_t)row * SLICE), x);
+                RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(kt + (uint32_t)row * SLICE), x);
 #pragma unroll
                 for (int i = 0; i < VE; i += 2) {
                     d0 = fmaf(qf[i], x[i], d0);
@@ -387,7 +385,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             }
             {
                 float x[VE], d0 = 0.f, d1 = 0.f;
-                HVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + SLICE + c * 16), x);
+                RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + SLICE + c * 16), x);
 #pragma unroll
                 for (int i = 0; i < VE; i += 2) {
                     d0 = fmaf(qf[i], x[i], d0);
@@ -424,7 +422,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
                 const float p = exp2f(s[j] - Mn);
                 lsum += p;
                 float x[VE];
-                HVec<T>::unpack(*reinterpret_cast<const uint4 *>(vt + (uint32_t)(j * G + grp) * SLICE), x);
+                RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(vt + (uint32_t)(j * G + grp) * SLICE), x);
 #pragma unroll
                 for (int i = 0; i < VE; ++i) acc[i] = fmaf(p, x[i], acc[i]);
             }
@@ -433,7 +431,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
                     const float p = exp2f(s[16] - Mn);
                     lsum += p;
                     float x[VE];
-                    HVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + 2 * SLICE + c * 16), x);
+                    RowVec<T>::unpack(*reinterpret_cast<const uint4 *>(sb + 64 + 2 * SLICE + c * 16), x);
 #pragma unroll
                     for (int i = 0; i < VE; ++i) acc[i] = fmaf(p, x[i], acc[i]);
                 }
@@ -509,7 +507,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 #pragma unroll
                     for (int i = 0; i < VE; ++i) x[i] = acc[i] * inv;
                     *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.out) + ((size_t)m.seg * H + m.h) * SLICE + c * 16) =
-                        HVec<T>::pack(x);
+                        RowVec<T>::pack(x);
                 }
             }
             M = -INFINITY;
