@@ -19,12 +19,12 @@
 // per SM, 13 warps.  A prompt of at most 128 tokens is one tile: both passes then run on it in one
 // launch (MODE 0), the second on the transposed product of the operands already in shared memory.
 //
-// Measured, 8 layers x 16 heads of 128, 777 tokens: 195 us for the whole call (1263 us with 64 x 64
-// tiles on FMA units), 100 us a pass.  A tile needs 48 MMAs of 64 clocks = 3072; it takes 6200: the
+// Measured, 8 layers x 16 heads of 128, 777 tokens: 190 us for the whole call (1263 us with 64 x 64
+// tiles on FMA units), 94 and 98 us a pass.  A tile needs 48 MMAs of 64 clocks = 3072; it takes 6200: the
 // issuing warp waits 1800 of them for chunks, because a chunk costs a loader warp about 2300 clocks
 // (the latency of its loads, of which one chunk is in flight, and its share of the issue slots).
 // Sixteen loader warps leave 80 registers a thread and spill (211 us).  4 layers x 4 heads of 64,
-// 128 tokens (one tile each): 14.0 us for the call, 30.7 with three FMA kernels.
+// 128 tokens (one tile each): 12.3 us for the call, 30.7 with three FMA kernels.
 #include "score_tiles.cuh"
 
 namespace pkv {
