@@ -503,9 +503,10 @@ def run_ours(args):
 
 
 def LAUNCHES_PER_STEP(w, path):
-    # score: lse + column sums + head mean; search: sort/scan + bisection;
-    # compact: plan + gather; decode: one kernel per token, or stream + merge
-    return 3 + 2 + 2 + DECODE_KERNELS[path][3] * w.T
+    # score: one kernel for both sums, or two passes, + head mean (the rule of score_fused_covers, and fp32 one-tile
+    # prompts); search: sort/scan + bisection; compact: plan + gather; decode: one kernel per token, or stream + merge
+    one_kernel = w.N <= 128 if str(w.dtype) == "torch.float32" else w.N <= 512 or (w.N <= 640 and w.B * w.L * w.H >= 64)
+    return (2 if one_kernel else 3) + 2 + 2 + DECODE_KERNELS[path][3] * w.T
 
 
 def run_e2e(torch, api, w, s, q, k, v, pool, budget, dev, steps):

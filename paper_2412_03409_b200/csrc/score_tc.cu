@@ -1,4 +1,5 @@
-// Importance score (Sec. 3.2), tensor-core path for bf16 inputs.
+// Importance score (Sec. 3.2), tensor-core path for bf16 inputs (prompts of up to 640 tokens without the caller's
+// log-sum-exp: score_fused.cu).
 //
 //   pass 1: per query m, log2-sum-exp of the scaled causal logits over keys j <= m
 //   pass 2: per key n, sum over queries m >= n of exp2(logit - lse[m])
@@ -395,8 +396,10 @@ EncodeTiledFn encode_fn()
     return fn;
 }
 
-// [B, L, H, N, D] bf16 with element strides -> rank-5 map, box = 64 elements x 128 rows.
-bool make_map(CUtensorMap *map, const void *ptr, const pkv_shape *s, pkv_strides st)
+}  // namespace
+
+// [B, L, H, N, D] bf16 with element strides -> rank-5 map, box = 64 elements x box_rows rows.
+bool score_make_map(CUtensorMap *map, const void *ptr, const pkv_shape *s, pkv_strides st, int box_rows)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
@@ -410,13 +413,15 @@ bool make_map(CUtensorMap *map, const void *ptr, const pkv_shape *s, pkv_strides
         strides[i] = (cuuint64_t)v * 2;
         if (strides[i] % 16 != 0 || strides[i] >= ((cuuint64_t)1 << 40) || strides[i] == 0) return false;
     }
-    cuuint32_t box[5] = {64, TT, 1, 1, 1};
+    cuuint32_t box[5] = {64, (cuuint32_t)box_rows, 1, 1, 1};
     cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(ptr), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
+
+namespace {
 
 template <int PASS, int D>
 int launch_pass(const CUtensorMap &mq, const CUtensorMap &mk, const ScoreArgs &a, int sms, cudaStream_t st)
@@ -439,6 +444,9 @@ int launch_pass(const CUtensorMap &mq, const CUtensorMap &mk, const ScoreArgs &a
 
 int launch_head_mean(const float *partial, int H, int N, size_t total, float *scores, const int32_t *abort_word,
                      cudaStream_t st);
+bool score_fused_covers(const pkv_shape *s);
+int launch_score_fused(const pkv_shape *s, const void *q, pkv_strides qs, const void *k, pkv_strides ks, const float *scale,
+                       float *scores, float *partial, int32_t *abort_word, cudaStream_t st);
 
 int selftest_wait_score(int32_t *dev_status, cudaStream_t st)
 {
@@ -463,8 +471,6 @@ size_t score_tc_ws_bytes(const pkv_shape *s)
 int launch_score_tc(const pkv_shape *s, const void *q, pkv_strides qs, const void *k, pkv_strides ks,
                     const float *scale, const float *lse, float *scores, void *ws, cudaStream_t st)
 {
-    CUtensorMap mq, mk;
-    if (!make_map(&mq, q, s, qs) || !make_map(&mk, k, s, ks)) return -1;
     const int B = s->batch, L = s->layers, H = s->heads, N = s->prompt_len;
     const size_t rows = (size_t)B * L * H;
     ScoreArgs a;
@@ -478,7 +484,12 @@ int launch_score_tc(const pkv_shape *s, const void *q, pkv_strides qs, const voi
     a.abort_word = a.next_item + 2;
     a.nseg = B * L;
     a.group = head_group(B * L * H, N, s->head_dim, 2);
+    // (with the caller's log-sum-exp one pass is left, and the tile kernel is at least as fast: 32 x 32 heads of 640
+    // tokens 102 us, 101 in a form of the fused kernel for it, of 100 tokens 17 and 25)
+    if (!lse && score_fused_covers(s)) return launch_score_fused(s, q, qs, k, ks, scale, scores, a.partial, a.abort_word, st);
 
+    CUtensorMap mq, mk;
+    if (!score_make_map(&mq, q, s, qs, TT) || !score_make_map(&mk, k, s, ks, TT)) return -1;
     const int sms = sm_count();
     if (sms <= 0) return PKV_ERR_CUDA;
     // Items of nearly one length (a tile or two), or a few for each CTA: dealt out by position, which needs

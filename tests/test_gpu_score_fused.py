@@ -1,0 +1,66 @@
+"""Scores of short bf16 prompts, both sums in one kernel, at the edges of its key tiles and query strips (needs a B200)."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import check_scores
+
+pytestmark = pytest.mark.gpu
+
+
+def reference(q, k, scale):
+    """The scores of every layer in 64 bits, and its largest logit."""
+    B, L, _, N, _ = q.shape
+    ref, top = np.empty((B, L, N)), np.zeros(L)
+    mask = torch.ones(N, N, dtype=torch.bool, device="cuda").triu(1)
+    for b in range(B):
+        for l in range(L):
+            x = torch.matmul(q[b, l].double(), k[b, l].double().transpose(-1, -2)) * float(scale[l])
+            top[l] = max(top[l], float(x.abs().max()))
+            ref[b, l] = torch.softmax(x.masked_fill_(mask, -float("inf")), -1).sum(1).mean(0).cpu().numpy()
+    return ref, top
+
+
+# Up to five key tiles of 128 and ten strips of 64; more heads than SMs, and several for a CTA where tiles are few.
+@pytest.mark.parametrize("L,H,N", [(40, 30, 1), (40, 30, 63), (20, 30, 65), (10, 31, 128), (10, 31, 129), (8, 40, 191), (10, 31, 192),
+                                   (8, 20, 257), (8, 20, 320), (4, 40, 385), (4, 40, 511), (4, 39, 512), (4, 39, 513),
+                                   (2, 64, 576), (4, 80, 577), (4, 80, 640), (1, 63, 640), (1, 64, 640)])
+@pytest.mark.parametrize("D", [64, 128])
+def test_scores_of_short_prompts(L, H, N, D):
+    from paper_2412_03409_b200.session import Session
+    g = torch.Generator(device="cuda").manual_seed(N * 7 + D)
+    q = torch.randn(1, L, N, H, D, device="cuda", generator=g).bfloat16().transpose(2, 3)
+    k = (torch.randn(1, L, N, H, D, device="cuda", generator=g) * 2).bfloat16().transpose(2, 3)
+    # Layers in turn: ordinary logits, of either sign; logits so large that their exponentials overflow, and so small
+    # that they vanish, unless taken relative to the maximum.
+    scale = np.resize(np.array([0.5, -0.5, 6.0, -6.0], np.float32), L) / np.float32(np.sqrt(D))
+    k[:, 2::4, :, :, 0] = -300.0
+    q[:, 2::4, ::2, :, 0] = 1.0     # even heads: every logit near -150 (D = 128); odd heads: of either sign
+    ref, top = reference(q, k, scale)
+    s = Session(1, L, H, D, N, torch.bfloat16, scale, decode_cap=0, max_budget_rows=L)
+    s.scores.fill_(float("nan"))
+    got = s.score(q, k).cpu().numpy()
+    # A logit is a sum of D products rounded to 2^-24 of its partial sums, at most twice the largest logit, and
+    # multiplied by the scale: some 4 * 2^-24 of that is the relative error of its exponential.
+    for l in range(L):
+        check_scores(got[0, l], ref[0, l], max(1e-5, 8 * top[l] * 2.0 ** -24))
+    np.testing.assert_array_equal(got, s.score(q, k).cpu().numpy())
+
+
+@pytest.mark.parametrize("N", [100, 500])
+def test_one_head_out_of_range(N):
+    """Heads that need the maximum among heads that do not, on the same SM: neither changes the others' scores."""
+    from paper_2412_03409_b200.session import Session
+    g = torch.Generator(device="cuda").manual_seed(N)
+    q, k = (torch.randn(1, 700, 1, N, 64, device="cuda", generator=g).bfloat16() for _ in range(2))
+    scale = np.full(700, 0.125, np.float32)
+    s = Session(1, 700, 1, 64, N, torch.bfloat16, scale, decode_cap=0, max_budget_rows=700)
+    plain = s.score(q, k).clone()
+    big = [0, 1, 147, 148, 300, 699]
+    scale[big] = 40.0
+    s = Session(1, 700, 1, 64, N, torch.bfloat16, scale, decode_cap=0, max_budget_rows=700)
+    got = s.score(q, k)
+    rest = [l for l in range(700) if l not in big]
+    assert torch.equal(got[0, rest], plain[0, rest])
+    ref, top = reference(q[:, big], k[:, big], scale[big])
+    check_scores(got[:, big].cpu().numpy(), ref, 8 * top.max() * 2.0 ** -24)
