@@ -7,6 +7,8 @@ kernels.  There is no CPU fallback: a missing library raises at import.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -90,9 +92,6 @@ def _load():
 _lib = _load()
 
 
-_decode_attn = _lib.prefixkv_decode_attn
-
-
 def lib():
     return _lib
 
@@ -118,6 +117,25 @@ def _stream():
     if _raw_stream is None or _raw_device is None:
         return torch.cuda.current_stream().cuda_stream
     return _raw_stream(_raw_device())
+
+
+def _load_call():
+    """The decode call's own binding: of all calls it alone is made per layer and token."""
+    if not os.path.exists(_build.CALL_PATH):
+        raise ImportError("_decode_call.so is not built; run `python -m paper_2412_03409_b200.build`. "
+                          "There is no fallback path.")
+    loader = importlib.machinery.ExtensionFileLoader("_decode_call", _build.CALL_PATH)
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_decode_call", loader))
+    loader.exec_module(mod)
+    address = ctypes.cast(_lib.prefixkv_decode_attn, ctypes.c_void_p).value
+    if _raw_stream is None or _raw_device is None:
+        mod.bind(address, _stream, None)
+    else:
+        mod.bind(address, _raw_stream, _raw_device)
+    return mod.decode_attn
+
+
+_decode_attn = _load_call()
 
 
 def make_shape(B, L, H, D, N, dtype) -> Shape:
@@ -222,10 +240,8 @@ def prefixkv_compact(shape, k, v, order, length, cache: Cache, dev_status, ws, k
 
 def prefixkv_decode_attn(shape, cache: Cache, q, k_new, v_new, layer_scale, out, dev_status, ws,
                          layer_begin=0, layer_end=None):
-    # (called once per layer and token: straight to the library, nothing else on the way)
-    rc = _decode_attn(ctypes.byref(shape), ctypes.byref(cache.c), _ptr(q), _ptr(k_new), _ptr(v_new),
-                      _ptr(layer_scale), int(layer_begin), shape.layers if layer_end is None else int(layer_end),
-                      _ptr(out), _ptr(dev_status), _ptr(ws), ws.numel() if ws is not None else 0, _stream())
+    rc = _decode_attn(shape, cache.c, q, k_new, v_new, layer_scale, layer_begin,
+                      shape.layers if layer_end is None else layer_end, out, dev_status, ws)
     if rc:
         _check(rc, "prefixkv_decode_attn")
 

@@ -1,14 +1,17 @@
-"""Builds libprefixkv.so (sm_100a) next to this file with nvcc."""
+"""Builds, next to this file, libprefixkv.so (sm_100a, with nvcc) and the decode call's binding (with the C compiler)."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 LIB_PATH = os.path.join(_HERE, "libprefixkv.so")
+CALL_SRC = os.path.join(_HERE, "csrc", "decode_call.c")
+CALL_PATH = os.path.join(_HERE, "_decode_call.so")
 
 
 def _sources():
@@ -32,7 +35,18 @@ def is_stale() -> bool:
     return any(os.path.getmtime(f) > t for f in _sources() + _headers())
 
 
+def build_call(force: bool = False) -> str:
+    newest = max(os.path.getmtime(f) for f in (CALL_SRC, os.path.join(_ROOT, "include", "prefixkv.h")))
+    if force or not os.path.exists(CALL_PATH) or os.path.getmtime(CALL_PATH) < newest:
+        tmp = CALL_PATH + ".%d.tmp" % os.getpid()
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", os.path.join(_ROOT, "include"),
+                               "-I", sysconfig.get_paths()["include"], "-o", tmp, CALL_SRC])
+        os.replace(tmp, CALL_PATH)
+    return CALL_PATH
+
+
 def build_library(force: bool = False, verbose: bool = False) -> str:
+    build_call(force)
     if not force and not is_stale():
         return LIB_PATH
     obj_dir = os.path.join(_HERE, "_build")
