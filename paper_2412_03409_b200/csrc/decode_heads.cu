@@ -20,6 +20,12 @@
 // the workspace); the last CTA, when its own work is done, waits for all flags and only then writes the
 // new lengths, so no CTA can read a length of the next step.  Every wait is bounded.
 //
+// Long segments (SHARED): items dealt round-robin leave the CTAs with sums of tiles that differ by an item or more.  There a CTA
+// has all but the last rounds of items for its own, and the tiles of the others, the pool, are shared out as
+// consecutive ranges that make the sums alike; an item that a range cuts goes from CTA to CTA as a softmax state in
+// global memory.  A CTA takes its range from the end on and before its own items but the first, so that what the next CTA
+// waits for is there long before that is done.  Every CTA works the shares out for itself, from the lengths.
+//
 // Measured on the 32-layer, 32-head, 128-rows-per-layer case (22.3 us per call with this design),
 // each alone: one producer thread 24.1 us, five 22.9, ten 23.1; eight stages 22.4, twelve 21.9 (with
 // the prefetch below, against 21.95 for ten); two consumer warps per tile
@@ -57,6 +63,9 @@ static_assert(kHPrefetch * kHPrefetchItems <= 32, "one lane per prefetched tile"
 constexpr int kHSlots = 4;         // items whose partial results may be waiting for their last tile
 constexpr int kHMaxAct = 256;      // segments planned per call
 constexpr int kHMaxGrid = 256;
+// Mean capacity of a segment from which items are shared out by tiles (launch_decode_heads), and from which two rounds of
+// them besides the incomplete one are; one below.
+constexpr int64_t kHSharedRows = 256, kHTwoRoundsRows = 400;
 constexpr int64_t kHMaxSegRows = 1024;  // mean capacity of a segment above which calls go to the row-split kernel
 constexpr uint32_t kHTile = 8192;  // bytes of one K (or V) tile: 16 rows per row group of a warp
 constexpr int kHProducers = 2;     // issuing threads (one per warp): stage s is always filled by producer s mod kHProducers
@@ -64,13 +73,14 @@ static_assert(kHStages % kHProducers == 0, "a stage must keep its producer, whic
 constexpr uint32_t kHSpinLimit = 1u << 22;
 constexpr float kLog2eH = 1.4426950408889634f;
 
-enum { kFlagNew = 1, kFlagItemLast = 2, kFlagWarpLast = 4, kFlagEnd = 8 };
+// (kFlagItemLast: the last tile of an item, or of the CTA's piece of one)
+enum { kFlagNew = 1, kFlagItemLast = 2, kFlagWarpLast = 4, kFlagEnd = 8, kFlagBegun = 16, kFlagGoesOn = 32 };
 
 struct TileMeta {
     int item, seg, h, nrows, flags, tiles, first_warp, slot_parity;
     long long new_row;  // cache row the new token is written to
     float sc;           // layer scale * log2(e)
-    int pad2;
+    int start;          // (a pool item) tile of the pool the item begins with
 };
 
 // Tensor maps over K and V with boxes of one head's slice by 1/kHHeights ... kHHeights/kHHeights of a
@@ -87,9 +97,11 @@ struct HeadArgs {
     const int32_t *cap;
     const float *layer_scale;
     unsigned long long *flags;  // [grid] per-call tokens: "this CTA has read the lengths"
+    unsigned long long *sent;   // [grid] per-call tokens: "this CTA's part of an item is in `parts`"
+    float *parts;               // [grid][D + 4] state of the item that the next CTA goes on with: acc[D], max, sum
     unsigned long long token;
     int32_t *dev_status;
-    int L, H, layer_begin, nl, nact;
+    int L, H, layer_begin, nl, nact, pool_rounds;
     uint32_t row_bytes;
     int64_t total_cap_rows;
 };
@@ -163,7 +175,8 @@ __device__ __forceinline__ void hbulk_load(void *dst, const void *src, uint32_t 
 
 // A head's slice of a row is D * sizeof(T) bytes = LPR 16-byte vectors: LPR lanes share a row, a
 // warp holds G = 32 / LPR rows at a time and a tile (8 KiB) is 16 such steps.
-template <typename T, int D>
+// SHARED: the CTAs' sums of tiles are made alike, by sharing out the last items by tiles.
+template <typename T, int D, bool SHARED>
 __global__ void __launch_bounds__((kHWarps + kHProducers) * 32, 1)
 decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 {
@@ -188,6 +201,10 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
     int *s_len = reinterpret_cast<int *>(s_off + a.nact);                // [nact] cached rows, or -1 (cannot take the step)
     float *s_scale = reinterpret_cast<float *>(s_len + a.nact);          // [nact]
     __shared__ int s_abort;
+    // SHARED:
+    __shared__ int s_known, s_sum[2], s_scan[kHMaxGrid / 32];
+    __shared__ int s_start[SHARED ? kHMaxGrid + 1 : 1];                  // first tile of the pool of every CTA
+    __shared__ __align__(16) float s_own[SHARED ? PSTRIDE : 4];          // the CTA's part of the item that another began
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int H = a.H;
@@ -195,6 +212,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 
     if (tid == 0) {
         s_abort = 0;
+        if (SHARED) s_sum[0] = s_sum[1] = s_known = 0;
 #pragma unroll
         for (int i = 0; i < kHHeights; ++i) {
             prefetch_map(&maps.k[i]);
@@ -236,6 +254,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
+    if (SHARED && tid == 0) lower_flag(a.sent + blockIdx.x);  // (zero already, unless a wait ran out in an earlier launch)
     // ---- plan: what this step does to every active segment -------------------------------------
     for (int si = tid; si < a.nact; si += blockDim.x) {
         const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
@@ -254,6 +273,45 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
     if (tid == 0 && append) held = raise_flag(a.flags + blockIdx.x, a.token);
 
     const int nitems = a.nact * H;
+    // ---- (SHARED) shares: `rounds` items of a CTA's own, and of the others' tiles as many as make all CTAs' sums alike ----
+    const int ctas = (int)gridDim.x, rounds = SHARED ? max(0, nitems / ctas - a.pool_rounds) : 0;
+    const int pool = rounds * ctas;  // items from this one on are shared out by tiles
+    auto tiles_of = [&](int si) { return s_len[si] < 0 ? 0 : (s_len[si] + TILE_ROWS - 1) / TILE_ROWS; };
+    // Worked out by the consumers while the producers issue the CTA's first item.
+    auto share_out = [&]() {
+        int own = 0, both = 0;  // tiles of CTA tid's own items; of the pool
+        if (tid < ctas)
+            for (int r = 0; r < rounds; ++r) own += tiles_of((tid + r * ctas) / H);
+        for (int si = tid; si < a.nact; si += kHWarps * 32) both += tiles_of(si) * (H - min(H, max(0, pool - si * H)));
+        const int all = __reduce_add_sync(0xffffffffu, own + both);
+        both = __reduce_add_sync(0xffffffffu, both);
+        if (lane == 0) {
+            atomicAdd(&s_sum[0], all);
+            atomicAdd(&s_sum[1], both);
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kHWarps * 32) : "memory");
+        const int pool_tiles = s_sum[1], want = tid < ctas ? max(0, (s_sum[0] + ctas - 1) / ctas - own) : 0;
+        int incl = want;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += up;
+        }
+        if (lane == 31 && warp < kHMaxGrid / 32) s_scan[warp] = incl;
+        asm volatile("bar.sync 1, %0;" ::"n"(kHWarps * 32) : "memory");
+        if (tid < ctas) {
+            int sum = incl - want;
+            for (int w = 0; w < warp; ++w) sum += s_scan[w];
+            s_start[tid] = min(pool_tiles, sum);
+        }
+        if (tid == 0) s_start[ctas] = pool_tiles;
+        asm volatile("bar.sync 1, %0;" ::"n"(kHWarps * 32) : "memory");
+        if (tid == 0) {
+            __threadfence_block();
+            *(volatile int *)&s_known = 1;
+        }
+    };
+    static_assert(kHWarps * 32 >= kHMaxGrid, "a consumer thread for every CTA");
 
     if (warp >= kHWarps) {
         // ---- producers: every one walks the CTA's whole tile stream and issues the tiles that are its own ----
@@ -264,8 +322,59 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             int uses[kHSlots];
 #pragma unroll
             for (int i = 0; i < kHSlots; ++i) uses[i] = 0;
-            for (int it = blockIdx.x; it < nitems && !dead; it += gridDim.x) {
-                const int si = it / H, h = it - si * H;
+            // SHARED: first an item of the CTA's own (its first tiles are on their way to L2); then its share of the pool, from
+            // the end on, so that the item that the next CTA goes on with comes early and its part is there by the
+            // time that CTA is done; then its other items.
+            int it = blockIdx.x, x0 = 0, x1 = 0;   // next item; tiles of the pool still to come
+            int ps = 0, ph = 0, base = 0, pt = 0;  // place in the pool: segment, its first head there, that one's first tile,
+            bool known = !SHARED;                  // and tiles of a head
+            for (; (SHARED || it < nitems) && !dead; it += SHARED ? 0 : gridDim.x) {
+                int si, h, t0 = 0, t1 = -1, start = 0;
+                if (SHARED && (it != (int)blockIdx.x || rounds == 0) && !known) {
+                    known = true;
+                    for (uint32_t i = 0; *(volatile int *)&s_known == 0 && i < kHSpinLimit && *(volatile int *)&s_abort == 0; ++i) {}
+                    __threadfence_block();
+                    if (*(volatile int *)&s_known == 0) {
+                        dead = true;
+                        atomicExch(&s_abort, 1);
+                        break;
+                    }
+                    x0 = s_start[blockIdx.x];
+                    x1 = s_start[blockIdx.x + 1];
+                    ps = pool / H;
+                    ph = pool - ps * H;
+                    if (x0 < x1) {
+                        pt = tiles_of(ps);
+                        while (x1 > base + (H - ph) * pt) {
+                            base += (H - ph) * pt;
+                            ph = 0;
+                            pt = tiles_of(++ps);
+                        }
+                    }
+                }
+                if (SHARED && x0 < x1) {
+                    while (x1 <= base) {
+                        pt = tiles_of(--ps);
+                        ph = max(0, pool - ps * H);
+                        base -= (H - ph) * pt;
+                    }
+                    const int hh = (x1 - 1 - base) / pt;
+                    start = base + hh * pt;
+                    si = ps;
+                    h = ph + hh;
+                    t1 = x1 - start;
+                    x1 = max(x0, start);
+                    t0 = x1 - start;
+                } else {
+                    if (SHARED && it >= nitems) break;
+                    si = it / H;
+                    h = it - si * H;
+                    if (SHARED) {
+                        it += gridDim.x;
+                        // (items of the pool have been shared out; those that cannot take the step are in no share)
+                        if (it - (int)gridDim.x >= pool && s_len[si] >= 0) continue;
+                    }
+                }
                 const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
                 const int ln = s_len[si];
                 if (ln < 0) {
@@ -278,7 +387,9 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
                     continue;
                 }
                 const int64_t off = s_off[si];
-                const int tiles = (ln + TILE_ROWS - 1) / TILE_ROWS;
+                const int item_tiles = (ln + TILE_ROWS - 1) / TILE_ROWS;
+                if (!SHARED || t1 < 0) t1 = item_tiles;
+                const int tiles = SHARED ? t1 - t0 : item_tiles;  // of the CTA's piece
                 const int first_warp = g % kHWarps;
                 const int slot = item_seq % kHSlots;
                 int slot_parity = 0;
@@ -290,22 +401,26 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
                     slot_parity = uses[slot] & 1;  // the phase of the slot's barrier this item completes
                     ++uses[slot];
                 }
-                for (int t = 0; t < tiles && !dead; ++t, ++g) {
+                for (int t = t0; t < t1 && !dead; ++t, ++g) {
                     if (g % kHProducers != me) continue;
                     const int st = g % kHStages;
                     hbar_wait(empty + st, ((uint32_t)(g / kHStages) & 1u) ^ 1u, dead, &s_abort);
                     if (dead) break;
                     unsigned char *sb = stages + (size_t)st * STAGE;
                     TileMeta *m = reinterpret_cast<TileMeta *>(sb);
-                    const bool last = t == tiles - 1;
+                    const bool last = t == item_tiles - 1;
                     m->item = item_seq;
                     m->seg = seg;
                     m->h = h;
                     const int nrows = min(TILE_ROWS, ln - t * TILE_ROWS);
                     const int quarters = (nrows + TILE_ROWS / kHHeights - 1) / (TILE_ROWS / kHHeights);  // box height, in steps
                     m->nrows = nrows;
-                    m->flags = (last && append ? kFlagNew : 0) | (last ? kFlagItemLast : 0) |
-                               (t + kHWarps >= tiles ? kFlagWarpLast : 0);
+                    m->flags = (last && append ? kFlagNew : 0) | ((SHARED ? t == t1 - 1 : last) ? kFlagItemLast : 0) |
+                               (t + kHWarps >= t1 ? kFlagWarpLast : 0);
+                    if (SHARED) {
+                        m->flags |= (t0 > 0 ? kFlagBegun : 0) | (t1 < item_tiles ? kFlagGoesOn : 0);
+                        m->start = start;
+                    }
                     m->tiles = tiles;
                     m->first_warp = first_warp;
                     m->slot_parity = slot_parity;
@@ -351,9 +466,80 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
         // ---- consumers: warp w takes tiles w, w + kHWarps, ... of the CTA's stream, all through stage w ----
         const int grp = lane / LPR, c = lane % LPR;
         bool dead = false;
+        if (SHARED) share_out();
         float M = -INFINITY, lsum = 0.f, acc[VE];
 #pragma unroll
         for (int i = 0; i < VE; ++i) acc[i] = 0.f;
+        // Adds another part of the item to the state.
+        auto join = [&](float M2, float l2, const float4 *x) {
+            const float Mn2 = fmaxf(M, M2);
+            const float f1 = exp2f(M - Mn2), f2 = exp2f(M2 - Mn2);
+            lsum = lsum * f1 + l2 * f2;
+#pragma unroll
+            for (int i = 0; i < VE; i += 4) {
+                const float4 y = x[i / 4];
+                acc[i] = acc[i] * f1 + y.x * f2;
+                acc[i + 1] = acc[i + 1] * f1 + y.y * f2;
+                acc[i + 2] = acc[i + 2] * f1 + y.z * f2;
+                acc[i + 3] = acc[i + 3] * f1 + y.w * f2;
+            }
+            M = Mn2;
+        };
+        auto write_out = [&](int seg, int h) {
+            if (grp == 0) {
+                const float inv = 1.f / lsum;
+                float x[VE];
+#pragma unroll
+                for (int i = 0; i < VE; ++i) x[i] = acc[i] * inv;
+                *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.out) + ((size_t)seg * H + h) * SLICE + c * 16) =
+                    RowVec<T>::pack(x);
+            }
+        };
+        auto leave = [&](float *p) {  // the state, for another warp to join
+            if (grp == 0) {
+#pragma unroll
+                for (int i = 0; i < VE; i += 4)
+                    *reinterpret_cast<float4 *>(p + c * VE + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
+                if (c == 0) {
+                    p[D] = M;
+                    p[D + 1] = lsum;
+                }
+            }
+            __syncwarp();
+        };
+        // The parts of an item that begins at tile `start` of the pool, from the CTAs before this one, the nearest first: when
+        // all are there (`last`: all that come within the limit).  False when one is still to come.
+        auto collect = [&](int start, bool last) {
+            for (int b = (int)blockIdx.x - 1;; --b) {
+                if (s_start[b] < s_start[b + 1]) {
+                    unsigned long long v = load_flag(a.sent + b);
+                    for (uint32_t i = 0; last && v != a.token && i < kHSpinLimit; ++i) v = load_flag(a.sent + b);
+                    if (!__all_sync(0xffffffffu, v == a.token)) {
+                        if (!last) return false;
+                        dead = true;
+                    }
+                }
+                if (s_start[b] <= start) break;
+            }
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
+            for (int b = (int)blockIdx.x - 1;; --b) {
+                if (s_start[b] < s_start[b + 1]) {
+                    if (!dead) {
+                        const float *p = a.parts + (size_t)b * PSTRIDE;
+                        float4 x[VE / 4];
+#pragma unroll
+                        for (int i = 0; i < VE / 4; ++i) x[i] = __ldcg(reinterpret_cast<const float4 *>(p + c * VE) + i);
+                        join(__ldcg(p + D), __ldcg(p + D + 1), x);
+                    }
+                    // back to zero; one that has not come gets it from its own CTA
+                    if (lane == 0 && (!dead || atomicExch(a.sent + b, a.token ^ kGone) == a.token)) lower_flag(a.sent + b);
+                }
+                if (s_start[b] <= start) break;
+            }
+            return true;
+        };
+        int late_seg = -1, late_h = 0, late_start = 0;  // an item of this warp whose other parts are still to come
+        unsigned long long sent_held = 0;
         for (int g = warp;; g += kHWarps) {
             const int st = g % kHStages;
             hbar_wait(full + st, (uint32_t)(g / kHStages) & 1u, dead, &s_abort);
@@ -501,13 +687,16 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
                     __syncwarp();
                     if (lane == 0) hbar_arrive(slot_empty + slot);
                 }
-                if (grp == 0) {
-                    const float inv = 1.f / lsum;
-                    float x[VE];
-#pragma unroll
-                    for (int i = 0; i < VE; ++i) x[i] = acc[i] * inv;
-                    *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.out) + ((size_t)m.seg * H + m.h) * SLICE + c * 16) =
-                        RowVec<T>::pack(x);
+                if (SHARED && (m.flags & kFlagGoesOn)) {
+                    leave(a.parts + (size_t)blockIdx.x * PSTRIDE);
+                    if (lane == 0) sent_held = raise_flag(a.sent + blockIdx.x, a.token);
+                } else if (SHARED && (m.flags & kFlagBegun) && !collect(m.start, false)) {
+                    leave(s_own);
+                    late_seg = m.seg;
+                    late_h = m.h;
+                    late_start = m.start;
+                } else {
+                    write_out(m.seg, m.h);
                 }
             }
             M = -INFINITY;
@@ -515,6 +704,15 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 #pragma unroll
             for (int i = 0; i < VE; ++i) acc[i] = 0.f;
         }
+        if (SHARED && late_seg >= 0 && !dead) {
+            float4 x[VE / 4];
+#pragma unroll
+            for (int i = 0; i < VE / 4; ++i) x[i] = reinterpret_cast<const float4 *>(s_own + c * VE)[i];
+            join(s_own[D], s_own[D + 1], x);
+            collect(late_start, true);
+            write_out(late_seg, late_h);
+        }
+        if (SHARED && lane == 0) unraise_flag(a.sent + blockIdx.x, a.token, sent_held);
         if (dead && lane == 0) raise_status(a.dev_status, 0, PKV_DEV_TIMEOUT);
     }
 
@@ -569,7 +767,9 @@ bool make_cache_map(CUtensorMap *map, void *ptr, const pkv_shape *s, int64_t row
     return r == CUDA_SUCCESS;
 }
 
-template <typename T, int D>
+constexpr int kHMaxSmem = 224 * 1024;  // dynamic; there are up to 1.7 KiB of static variables beside it
+
+template <typename T, int D, bool SHARED>
 int launch_heads(const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t st)
 {
     static bool done[64] = {};
@@ -577,10 +777,10 @@ int launch_heads(const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t
     constexpr uint32_t HEAD = (64 + 3 * SLICE + 127) / 128 * 128;
     const size_t smem = (size_t)kHStages * (HEAD + 2 * kHTile) + (size_t)kHSlots * kHWarps * (D + 4) * sizeof(float) +
                         (2 * kHStages + 2 * kHSlots) * sizeof(uint64_t) + (size_t)a.nact * (sizeof(int64_t) + 2 * sizeof(int));
-    int rc = ensure_dynamic_smem((const void *)decode_heads_kernel<T, D>, 226 * 1024, done);
+    int rc = ensure_dynamic_smem((const void *)decode_heads_kernel<T, D, SHARED>, kHMaxSmem, done);
     if (rc != PKV_OK) return rc;
-    if (smem > 226 * 1024) return -1;
-    cudaError_t e = launch_dependent(decode_heads_kernel<T, D>, dim3(grid), dim3((kHWarps + kHProducers) * 32), smem, st, maps, a);
+    if (smem > kHMaxSmem) return -1;
+    cudaError_t e = launch_dependent(decode_heads_kernel<T, D, SHARED>, dim3(grid), dim3((kHWarps + kHProducers) * 32), smem, st, maps, a);
     if (e != cudaSuccess) {
         set_cuda_error(e, "decode_heads_kernel");
         return PKV_ERR_CUDA;
@@ -588,9 +788,16 @@ int launch_heads(const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t
     return PKV_OK;
 }
 
+template <typename T> int launch_heads(int D, bool shared, const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t st)
+{
+    if (D == 128) return shared ? launch_heads<T, 128, true>(maps, a, grid, st) : launch_heads<T, 128, false>(maps, a, grid, st);
+    return shared ? launch_heads<T, 64, true>(maps, a, grid, st) : launch_heads<T, 64, false>(maps, a, grid, st);
+}
+
 }  // namespace
 
-size_t decode_heads_ws_bytes() { return round_up((size_t)kHMaxGrid * sizeof(unsigned long long), kWsAlign); }
+// Flags of either kind, and a part of an item for every CTA.
+size_t decode_heads_ws_bytes() { return round_up((size_t)kHMaxGrid * (2 * sizeof(unsigned long long) + (128 + 4) * sizeof(float)), kWsAlign); }
 
 // Returns PKV_OK, an error, or -1 when this call is outside what the per-head kernel covers (the
 // caller then takes the row-split streaming kernel).
@@ -660,6 +867,8 @@ int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const v
     a.q = q; a.k_new = kn; a.v_new = vn; a.ck = c->k; a.cv = c->v; a.out = out;
     a.row_offset = c->row_offset; a.len = c->len; a.cap = c->cap; a.layer_scale = scale;
     a.flags = (unsigned long long *)ws;
+    a.sent = a.flags + kHMaxGrid;
+    a.parts = (float *)(a.sent + kHMaxGrid);
     a.token = g_token.fetch_add(0x9e3779b97f4a7c15ull) | 1ull;
     a.dev_status = dev_status;
     a.L = s->layers; a.H = H; a.layer_begin = lb; a.nl = nl; a.nact = nact;
@@ -667,12 +876,14 @@ int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const v
     a.total_cap_rows = c->total_cap_rows;
     const int items = nact * H;
     const int grid = items < sms ? items : sms;
-    if (s->dtype == PKV_BF16) {
-        if (D == 128) return launch_heads<__nv_bfloat16, 128>(maps, a, grid, st);
-        return launch_heads<__nv_bfloat16, 64>(maps, a, grid, st);
-    }
-    if (D == 128) return launch_heads<float, 128>(maps, a, grid, st);
-    return launch_heads<float, 64>(maps, a, grid, st);
+    // Segments of some hundred rows differ in length and an item is a good part of a CTA's work: CTAs' sums of tiles
+    // made alike.  It costs 2 us a call, the shares' arithmetic and the parts that pass through global memory:
+    // 32 x 32 heads, 128 rows of capacity 19.3 us a call without / 23.0 with; 256 31.5 / 31.5; 300 37.5 / 36.0 (two rounds shared
+    // out 38.8); 40 x 40 heads, 500 rows 77 / 77 (74); 800 rows of 32 x 32 heads 87 / 82 (77); 4 x 32 x 32 heads of 819 rows 296
+    // / 284 (279); fp32, 16 x 40 heads of 600 rows 81 / 67 (66).
+    const bool shared = seg_rows >= kHSharedRows;
+    a.pool_rounds = seg_rows >= kHTwoRoundsRows ? 2 : 1;
+    return s->dtype == PKV_BF16 ? launch_heads<__nv_bfloat16>(D, shared, maps, a, grid, st) : launch_heads<float>(D, shared, maps, a, grid, st);
 }
 
 }  // namespace pkv
