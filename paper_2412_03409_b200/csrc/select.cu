@@ -249,51 +249,65 @@ __device__ __forceinline__ int status_from_flags(int flags)
     return (flags & 1) ? (int)PKV_DEV_BAD_SCORE : ((flags & 2) ? (int)PKV_DEV_RANGE : (int)PKV_DEV_OK);
 }
 
-// ---------------------------------------------------------------------------
-// Length rule of Sec. 3.3 for one layer, evaluated by one warp: the number of
-// cumulative values below theta, found by a 32-way search (every lane probes
-// one pivot per round), plus one, clamped to [1, N].
-// ---------------------------------------------------------------------------
-// `pivot` is the lane's probe of the first round, c[(lane + 1) * chunk0 - 1] (or ~0 past the
-// end): it does not depend on theta, so a caller that searches one row many times loads it once.
-__device__ __forceinline__ int warp_length_for_theta(const uint64_t *__restrict__ c, int N,
-                                                     uint64_t theta, int lane, uint64_t pivot)
+// Number of cumulative values below theta, known to lie in [a, b]: a search by quarters, three loads at a time.
+__device__ __forceinline__ int count_below(const uint64_t *__restrict__ c, int a, int b, uint64_t theta)
 {
-    int a = 0, bnd = N;  // the count lies in [a, bnd]
-    {
-        const int chunk = (N + 31) >> 5;
-        const int k = __popc(__ballot_sync(0xffffffffu, pivot < theta));
-        a = k * chunk;
-        const int nb = (k + 1) * chunk - 1;
-        bnd = nb < N ? nb : N;
+    while (a < b) {
+        const int i1 = a + ((b - a) >> 2), i2 = a + ((b - a) >> 1), i3 = a + (3 * (b - a) >> 2);
+        const uint64_t x1 = c[i1], x2 = c[i2], x3 = c[i3];
+        if (x2 < theta) {
+            a = x3 < theta ? i3 + 1 : i2 + 1;
+            b = x3 < theta ? b : i3;
+        } else {
+            b = x1 < theta ? i2 : i1;
+            a = x1 < theta ? i1 + 1 : a;
+        }
     }
-    while (bnd > a) {
-        int chunk = (bnd - a + 31) >> 5;
-        int idx = a + (lane + 1) * chunk - 1;
-        bool below = (idx < bnd) ? (c[idx] < theta) : false;
-        int k = __popc(__ballot_sync(0xffffffffu, below));
-        int na = a + k * chunk;
-        int nb = a + (k + 1) * chunk - 1;
-        a = na;
-        bnd = nb < bnd ? nb : bnd;
-    }
-    int n = a + 1;
-    return n > N ? N : (n < 1 ? 1 : n);
+    return a;
 }
 
-// One CTA per sample.  Warps take layers round-robin; every thread tracks the
-// same (p1, p2) so control flow is uniform.  Two length buffers alternate so
-// that one barrier per midpoint is enough.
+// Length rule of Sec. 3.3 (a layer keeps one row more than there are cumulative values below p * total, at most N) and the
+// bisection on p that makes the lengths meet the budget.  One CTA per sample, warp per layer.
+//
+// A midpoint by itself is a chain of latencies -- a load or two, the sum over the layers, a barrier -- of some 1000
+// clocks.  So the tree of the next five bisections is evaluated at once, a lane to each of its 31 midpoints (formed by the
+// same additions and halvings that would lead there), and then walked: a round costs little more than a midpoint did, the
+// first one apart, whose searches cover whole rows; later ones lie between the counts at both ends of the interval.
+// Selection and compaction of one sample, a midpoint at a time / five levels at a time: 32 layers of 640 scores 58.2 / 52.0 us
+// (four levels 54.0), of 128 28.8 / 24.7, of 16384 274 / 266; 40 layers of 1024 109 / 98.
+constexpr int kTreeLevels = 5;
 __global__ void __launch_bounds__(1024)
 search_kernel(const uint64_t *__restrict__ cum, const int64_t *__restrict__ budget_rows, int L,
               int N, double tol, int max_iters, int64_t slack, int64_t slack_over, int32_t *__restrict__ len,
               double *__restrict__ p_out, int32_t *__restrict__ iters_out, int32_t *dev_status)
 {
-    extern __shared__ int s_len[];  // [2][L]
+    __shared__ int s_sum[3][32];  // total length at every midpoint of the tree; buffers in turn
     const int b = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const uint64_t *cb = cum + (size_t)b * L * N;
+    if (threadIdx.x < 96) s_sum[threadIdx.x / 32][lane] = 0;
     dependent_entry();  // the sort kernel's sums and flags are complete
+    // What a layer's searches need, kept in registers for the first kHoist layers of the warp: its total, the counts at both
+    // ends of the interval, and a pivot per lane, c[(lane + 1) * chunk - 1] (or ~0 past the end).
+    constexpr int kHoist = 4;
+    const int chunk = (N + 31) >> 5;
+    double tot[kHoist];
+    uint64_t pivot[kHoist];
+    int lo[kHoist], hi[kHoist], at[kHoist];
+#pragma unroll
+    for (int k = 0; k < kHoist; ++k) {
+        const int l = warp + k * nwarp;
+        tot[k] = 0.0;
+        pivot[k] = ~0ull;
+        lo[k] = at[k] = 0;
+        hi[k] = N;
+        if (l < L) {
+            const uint64_t *c = cb + (size_t)l * N;
+            const int idx = (lane + 1) * chunk - 1;
+            tot[k] = (double)c[N - 1];
+            if (idx < N) pivot[k] = c[idx];
+        }
+    }
     const int64_t budget = budget_rows[b];
     {
         int flags = 0;
@@ -303,92 +317,97 @@ search_kernel(const uint64_t *__restrict__ cum, const int64_t *__restrict__ budg
         if (threadIdx.x == 0) dev_status[b] = status_from_flags(flags);  // overwrites: this call's status starts here
     }
 
-    // What every midpoint needs of a layer's row and never changes: its total and this lane's
-    // first-round probe.  Kept in registers for the first kHoist layers of the warp.
-    constexpr int kHoist = 4;
-    const int chunk0 = (N + 31) >> 5;
-    double tot_r[kHoist];
-    uint64_t piv_r[kHoist];
-#pragma unroll
-    for (int k = 0; k < kHoist; ++k) {
-        const int l = warp + k * nwarp;
-        tot_r[k] = 0.0;
-        piv_r[k] = ~0ull;
-        if (l < L) {
-            const uint64_t *c = cb + (size_t)l * N;
-            const int idx = (lane + 1) * chunk0 - 1;
-            tot_r[k] = (double)c[N - 1];
-            if (idx < N) piv_r[k] = c[idx];
-        }
-    }
-
-    auto eval = [&](double p, int buf) -> int64_t {
-        int *dst = s_len + buf * L;
-#pragma unroll
-        for (int k = 0; k < kHoist; ++k) {
-            const int l = warp + k * nwarp;
-            if (l < L) {
-                int n = N;
-                if (p < 1.0) {
-                    const uint64_t theta = __double2ull_ru(__dmul_rn(p, tot_r[k]));
-                    n = warp_length_for_theta(cb + (size_t)l * N, N, theta, lane, piv_r[k]);
-                }
-                if (lane == 0) dst[l] = n;
-            }
-        }
-        for (int l = warp + kHoist * nwarp; l < L; l += nwarp) {
-            const uint64_t *c = cb + (size_t)l * N;
-            int n;
-            if (p >= 1.0) {
-                n = N;
-            } else {
-                const int idx = (lane + 1) * chunk0 - 1;
-                double total = (double)c[N - 1];
-                uint64_t theta = __double2ull_ru(__dmul_rn(p, total));
-                n = warp_length_for_theta(c, N, theta, lane, idx < N ? c[idx] : ~0ull);
-            }
-            if (lane == 0) dst[l] = n;
-        }
-        __syncthreads();
-        int64_t s = 0;
-        for (int l = lane; l < L; l += 32) s += dst[l];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        return s;
-    };
+    auto threshold = [](double p, double total) { return __double2ull_ru(__dmul_rn(p, total)); };
+    auto length_of = [&](int count) { return count + 1 > N ? N : count + 1; };
 
     double p_final = 0.0;
-    int iters = 0, buf = 0;
-    bool have = false;  // s_len[buf] already holds the lengths of p_final
+    int iters = 0, taken = -1;  // taken: the midpoint, of the last tree, that is p_final
     if (budget < (int64_t)L) {
         if (threadIdx.x == 0) raise_status(dev_status, b, PKV_DEV_BUDGET_TOO_SMALL);
     } else if ((int64_t)L * (int64_t)N <= budget) {
         p_final = 1.0;
     } else {
         double p1 = 0.0, p2 = 1.0;
-        for (;;) {
-            double p = (p1 + p2) * 0.5;
-            if (p == p1 || p == p2 || iters == max_iters || p2 - p1 <= tol) {
-                p_final = p1;
-                break;
+        bool done = false;
+        for (int round = 0; !done; ++round) {
+            // the lane's midpoint: node `lane` of the tree (root 1; the upper half of a node's interval is its odd child)
+            double a1 = p1, a2 = p2, p = (p1 + p2) * 0.5;
+            for (int bit = 30 - __clz(lane | 1); bit >= 0; --bit) {
+                if (lane >> bit & 1) a1 = p;
+                else a2 = p;
+                p = (a1 + a2) * 0.5;
             }
-            buf ^= 1;
-            int64_t S = eval(p, buf);
-            ++iters;
-            int64_t delta = S - budget;
-            if (delta >= -slack && delta <= slack_over) {  // within the threshold on delta (Sec. 3.3)
-                p_final = p;
-                have = true;
-                break;
+            int total = 0;
+#pragma unroll
+            for (int k = 0; k < kHoist; ++k) {
+                const int l = warp + k * nwarp;
+                if (l >= L) continue;
+                const uint64_t theta = threshold(p, tot[k]);
+                int x = lo[k], y = hi[k];
+                if (y - x > chunk) {  // (the first round: which 32nd of the row)
+                    int n = 0;
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1)
+                        n += __shfl_sync(0xffffffffu, pivot[k], n + step - 1) < theta ? step : 0;
+                    n += __shfl_sync(0xffffffffu, pivot[k], 31) < theta ? n == 31 : 0;
+                    x = max(x, n * chunk);
+                    y = min(y, (n + 1) * chunk - 1);
+                }
+                at[k] = p < 1.0 ? count_below(cb + (size_t)l * N, x, y, theta) : N;
+                total += length_of(at[k]);
             }
-            if (delta < 0) p1 = p; else p2 = p;
+            for (int l = warp + kHoist * nwarp; l < L; l += nwarp) {
+                const uint64_t *c = cb + (size_t)l * N;
+                total += length_of(p < 1.0 ? count_below(c, 0, N, threshold(p, (double)c[N - 1])) : N);
+            }
+            int *sums = s_sum[round % 3];
+            atomicAdd(sums + lane, total);
+            if (warp == 0) s_sum[(round + 1) % 3][lane] = 0;  // (read two rounds ago, before the last barrier)
+            __syncthreads();
+            int node = 1, at1 = -1, at2 = -1;  // nodes that became the ends of the interval
+            for (int level = 0; level < kTreeLevels; ++level) {
+                const double mid = (p1 + p2) * 0.5;
+                if (mid == p1 || mid == p2 || iters == max_iters || p2 - p1 <= tol) {
+                    p_final = p1;
+                    done = true;
+                    break;
+                }
+                ++iters;
+                const int64_t delta = (int64_t)sums[node] - budget;
+                if (delta >= -slack && delta <= slack_over) {  // within the threshold on delta (Sec. 3.3)
+                    p_final = mid;
+                    taken = node;
+                    done = true;
+                    break;
+                }
+                if (delta < 0) {
+                    p1 = mid;
+                    at1 = node;
+                } else {
+                    p2 = mid;
+                    at2 = node;
+                }
+                node = 2 * node + (delta < 0 ? 1 : 0);
+            }
+#pragma unroll
+            for (int k = 0; k < kHoist; ++k) {
+                const int n1 = __shfl_sync(0xffffffffu, at[k], at1 & 31), n2 = __shfl_sync(0xffffffffu, at[k], at2 & 31);
+                if (at1 >= 0) lo[k] = n1;
+                if (at2 >= 0) hi[k] = n2;
+            }
         }
     }
-    if (!have) {
-        buf ^= 1;
-        eval(p_final, buf);
+#pragma unroll
+    for (int k = 0; k < kHoist; ++k) {
+        const int l = warp + k * nwarp;
+        const int count = __shfl_sync(0xffffffffu, at[k], taken & 31);
+        if (l < L && lane == 0) len[(size_t)b * L + l] = p_final >= 1.0 ? N : length_of(taken >= 0 ? count : lo[k]);
     }
-    for (int l = threadIdx.x; l < L; l += blockDim.x) len[(size_t)b * L + l] = s_len[buf * L + l];
+    for (int l = warp + kHoist * nwarp; l < L; l += nwarp) {
+        const uint64_t *c = cb + (size_t)l * N;
+        const int count = p_final < 1.0 ? count_below(c, 0, N, threshold(p_final, (double)c[N - 1])) : N;
+        if (lane == 0) len[(size_t)b * L + l] = length_of(count);
+    }
     if (threadIdx.x == 0) {
         p_out[b] = p_final;
         iters_out[b] = iters;
@@ -475,7 +494,7 @@ extern "C" int prefixkv_search(const pkv_shape *shape, const float *scores,
     if ((size_t)2 * L * sizeof(int) > 40 * 1024) return PKV_ERR_UNSUPPORTED;
     int rc = launch_sort(shape, scores, order, cum, len, st);
     if (rc != PKV_OK) return rc;
-    cudaError_t e = launch_dependent(search_kernel, dim3(B), dim3(1024), 2 * L * sizeof(int), st,
+    cudaError_t e = launch_dependent(search_kernel, dim3(B), dim3(1024), 0, st,
                                      (const uint64_t *)cum, budget_rows, L, N, tol, (int)max_iters, slack_rows, slack_over_rows, len,
                                      p_out, iters_out, dev_status);
     if (e != cudaSuccess) {
