@@ -4,6 +4,8 @@
 // All arithmetic that decides an index is integer: the sort key is the fp32 bit
 // pattern (monotone for non-negative floats), cumulative sums are 2^-32 fixed
 // point in uint64, and only p and the threshold p*total are fp64.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace pkv {
@@ -47,29 +49,71 @@ __device__ __forceinline__ uint64_t weight_of_key(uint32_t key, bool &range_bad)
 }
 
 constexpr int kDigits = 256;
+constexpr int kSplitFour = 4096, kSplitTwo = 8192;  // scores above which a segment may be split over a cluster of so many
 
 // Shared memory: keys [items], counts [warps][kDigits] (a warp's lanes then meet in a bank by chance only; with
 // the warps of a digit side by side they always did), positions [items].
-static size_t sort_smem_bytes(int threads, int ipt)
+// SPLIT: also the sums [items], and room for the keys of another CTA where the counts are.
+static size_t sort_smem_bytes(int threads, int ipt, bool split)
 {
-    return (size_t)threads * ipt * (sizeof(uint32_t) + sizeof(uint16_t)) + (size_t)kDigits * (threads / 32) * sizeof(uint32_t);
+    const size_t items = (size_t)threads * ipt;
+    return items * (sizeof(uint32_t) + sizeof(uint16_t) + (split ? sizeof(uint64_t) : 0)) +
+           std::max((size_t)kDigits * (threads / 32), split ? items : 0) * sizeof(uint32_t);
 }
 
-template <int IPT>
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Address, in CTA `rank` of the cluster, of what `p` is in this one; and loads from there.
+__device__ __forceinline__ uint32_t in_cta(const void *p, uint32_t rank)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ uint4 load_there16(uint32_t a)
+{
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint64_t load_there8(uint32_t a)
+{
+    uint64_t v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// SPLIT: a cluster takes a segment.  Each of its CTAs sorts and sums a run of consecutive positions; an item's place is then its
+// own among them and, for every other CTA, the number of that one's items before it (a binary search over its keys,
+// copied next door), and its cumulative sum likewise.
+template <int IPT, bool SPLIT>
 __global__ void __launch_bounds__(1024)
 sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ order,
-                 uint64_t *__restrict__ cum, int32_t *__restrict__ seg_flags)
+                 uint64_t *__restrict__ cum, int32_t *__restrict__ seg_flags, int split)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nthr = blockDim.x, nwarp = nthr >> 5;
     uint32_t *skey = reinterpret_cast<uint32_t *>(smem_raw);                 // [nthr * IPT]
     uint32_t *count = skey + nthr * IPT;                                     // [nwarp][kDigits]
-    uint16_t *spos = reinterpret_cast<uint16_t *>(count + kDigits * nwarp);  // [nthr * IPT]
+    const int items = nthr * IPT;
+    uint16_t *spos = reinterpret_cast<uint16_t *>(count + (SPLIT ? max(kDigits * nwarp, items) : kDigits * nwarp));  // [nthr * IPT]
+    uint64_t *ssum = reinterpret_cast<uint64_t *>(spos + items);             // (SPLIT) [nthr * IPT]
     __shared__ uint32_t warp_sum[32];
     __shared__ uint64_t warp_tot[32], warp_high[32];
     __shared__ int s_flags;
+    __shared__ uint64_t s_total[2];  // (SPLIT) the CTA's sum, and that of high parts
 
-    const int seg = blockIdx.x;
+    const int rank = SPLIT ? (int)cluster_rank() : 0, ctas = SPLIT ? split : 1;
+    const int seg = SPLIT ? blockIdx.x / split : blockIdx.x, first = SPLIT ? rank * items : 0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t below = (1u << lane) - 1;
     const int base = warp * 32 * IPT + lane;  // place of the lane's item 0
@@ -82,7 +126,7 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
     uint16_t pos[IPT];
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
-        const int n = base + i * 32;
+        const int n = first + base + i * 32;
         key[i] = ~0u;  // padding: after every score, those of 0 included (it starts behind them)
         pos[i] = (uint16_t)n;
         if (n < N) {
@@ -197,7 +241,7 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
     uint64_t local = 0, high = 0;
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
-        const uint64_t w = base + i * 32 < N ? weight_of_key(key[i], range_bad) : 0;
+        const uint64_t w = first + base + i * 32 < N ? weight_of_key(key[i], range_bad) : 0;
         local += w;
         high += w >> 20;
     }
@@ -216,19 +260,25 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
     if (warp == nwarp - 1) {
         uint64_t h = 0;
         for (int w = 0; w < nwarp; ++w) h += warp_high[w];
+        if (SPLIT) {
+            s_total[0] = run + local;
+            s_total[1] = h;
+        }
         if (h >= (1ull << 34) || run + local >= (1ull << 53)) range_bad = true;
     }
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
         const int j = base + i * 32;
         bool dummy = false;
-        uint64_t incl = j < N ? weight_of_key(key[i], dummy) : 0;
+        uint64_t incl = first + j < N ? weight_of_key(key[i], dummy) : 0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint64_t up = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += up;
         }
-        if (j < N) {
+        if (SPLIT) {
+            ssum[j] = run + incl;
+        } else if (j < N) {
             order[(size_t)seg * N + j] = (int32_t)pos[i];
             if (cum) cum[(size_t)seg * N + j] = run + incl;
         }
@@ -236,6 +286,64 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
     }
     if (bad) atomicOr(&s_flags, 1);
     if (range_bad) atomicOr(&s_flags, 2);
+    if (SPLIT) {
+        cluster_sync();
+        int place[IPT];
+        uint64_t sum[IPT];
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) {
+            place[i] = base + i * 32;
+            sum[i] = ssum[place[i]];
+        }
+        for (int step = 1; step < ctas; ++step) {
+            const int other = (rank + step) % ctas;
+            const uint32_t there = in_cta(skey, other);
+            for (int i = tid; i < items / 4; i += nthr) reinterpret_cast<uint4 *>(count)[i] = load_there16(there + i * 16);
+            __syncthreads();
+            // (of equal keys those of earlier positions, another CTA's as a whole, come first)
+            int n[IPT];
+#pragma unroll
+            for (int i = 0; i < IPT; ++i) n[i] = 0;
+            for (int half = 1 << (31 - __clz(items)); half > 0; half >>= 1)
+#pragma unroll
+                for (int i = 0; i < IPT; ++i) {
+                    const int at = n[i] + half - 1;
+                    if (at < items) {
+                        const uint32_t x = count[at];
+                        if (other < rank ? x <= key[i] : x < key[i]) n[i] += half;
+                    }
+                }
+            const uint32_t sums = in_cta(ssum, other);
+#pragma unroll
+            for (int i = 0; i < IPT; ++i) {
+                place[i] += n[i];
+                if (n[i] > 0) sum[i] += load_there8(sums + (n[i] - 1) * 8);
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int i = 0; i < IPT; ++i)
+            if (first + base + i * 32 < N) {  // (paddings are a CTA's last)
+                order[(size_t)seg * N + place[i]] = (int32_t)pos[i];
+                if (cum) cum[(size_t)seg * N + place[i]] = sum[i];
+            }
+        if (rank == 0 && tid == 0) {
+            int flags = 0;
+            uint64_t total = 0, high = 0;
+            for (int r = 0; r < ctas; ++r) {
+                uint32_t f;
+                asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(f) : "r"(in_cta(&s_flags, r)) : "memory");
+                flags |= (int)f;
+                total += load_there8(in_cta(s_total, r));
+                high += load_there8(in_cta(s_total + 1, r));
+            }
+            if (high >= (1ull << 34) || total >= (1ull << 53)) flags |= 2;
+            seg_flags[seg] = flags;
+        }
+        __syncwarp();
+        cluster_sync();  // (the others' shared memory is read no more)
+        return;
+    }
     __syncthreads();
     // What was found goes to the segment's slot of the length array (bit 0: a bad score, bit 1:
     // the fixed-point range); the kernel that follows turns the flags of a sample's layers into
@@ -439,19 +547,31 @@ take_lengths_kernel(const int32_t *__restrict__ len_in, int per_sample, int L, i
     }
 }
 
-template <int IPT>
+template <int IPT, bool SPLIT = false>
 static int launch_sort_items(const pkv_shape *s, const float *scores, int32_t *order, uint64_t *cum,
-                             int32_t *seg_flags, cudaStream_t st)
+                             int32_t *seg_flags, cudaStream_t st, int split = 1)
 {
-    const int N = s->prompt_len;
-    const int threads = ((N + IPT - 1) / IPT + 31) / 32 * 32;
-    const size_t smem = sort_smem_bytes(threads, IPT);
+    const int N = s->prompt_len, share = (N + split - 1) / split;
+    const int threads = ((share + IPT - 1) / IPT + 31) / 32 * 32;
+    const size_t smem = sort_smem_bytes(threads, IPT, SPLIT);
     // (for every size: the default limit of 48 KiB is for the kernel's static variables and these together)
     static bool attr_done[64] = {};
-    int rc = ensure_dynamic_smem((const void *)sort_scan_kernel<IPT>, (int)sort_smem_bytes(1024, IPT), attr_done);
+    int rc = ensure_dynamic_smem((const void *)sort_scan_kernel<IPT, SPLIT>, (int)sort_smem_bytes(1024, IPT, SPLIT), attr_done);
     if (rc != PKV_OK) return rc;
-    cudaError_t e = launch_dependent(sort_scan_kernel<IPT>, dim3(s->batch * s->layers), dim3(threads), smem, st, scores, N,
-                                     order, cum, seg_flags);
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)split;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(s->batch * s->layers * split));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = SPLIT ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, sort_scan_kernel<IPT, SPLIT>, scores, N, order, cum, seg_flags, split);
     if (e != cudaSuccess) {
         set_cuda_error(e, "sort_scan_kernel");
         return PKV_ERR_CUDA;
@@ -462,11 +582,16 @@ static int launch_sort_items(const pkv_shape *s, const float *scores, int32_t *o
 // Up to 256 scores places are counted: the work grows with the square, 512 of them cost more than the passes.
 // Two items a thread beat four up to some 768 scores for one prompt (18.0 / 18.4 us with the search) and not for
 // 16 (42.8 / 37.6); beyond, four do throughout (1024: 19.8 / 19.2 and 47.9 / 40.7).  Above that as few as 1024
-// threads allow.
+// threads allow.  Long prompts whose segments leave SMs idle are split over clusters of four or two (with compaction, whole / split
+// over four: 32 segments of 4096 scores 127.9 / 125.9 us, of 4500 136.0 / 134.8, of 8192 226 / 219, of 16384 264 / 238; 64 segments, over
+// two: of 4500 230 / 235, 40 of 6000 252 / 253, 64 of 16384 431 / 421).
 static int launch_sort(const pkv_shape *s, const float *scores, int32_t *order, uint64_t *cum,
                        int32_t *seg_flags, cudaStream_t st)
 {
-    const int N = s->prompt_len;
+    const int N = s->prompt_len, sms = sm_count();
+    const int64_t segments = (int64_t)s->batch * s->layers;
+    if (N > kSplitFour && 4 * segments <= sms) return launch_sort_items<4, true>(s, scores, order, cum, seg_flags, st, 4);
+    if (N > kSplitTwo && 2 * segments <= sms) return launch_sort_items<8, true>(s, scores, order, cum, seg_flags, st, 2);
     if (N <= 256) return launch_sort_items<1>(s, scores, order, cum, seg_flags, st);
     if (N <= 768) return launch_sort_items<2>(s, scores, order, cum, seg_flags, st);
     if (N <= 4096) return launch_sort_items<4>(s, scores, order, cum, seg_flags, st);
