@@ -65,7 +65,7 @@ constexpr int kHMaxAct = 256;      // segments planned per call
 constexpr int kHMaxGrid = 256;
 // Mean capacity of a segment from which items are shared out by tiles (launch_decode_heads), and from which two rounds of
 // them besides the incomplete one are; one below.
-constexpr int64_t kHSharedRows = 256, kHTwoRoundsRows = 400;
+constexpr int64_t kHSharedRows = 288, kHTwoRoundsRows = 400;
 constexpr int64_t kHMaxSegRows = 1024;  // mean capacity of a segment above which calls go to the row-split kernel
 constexpr uint32_t kHTile = 8192;  // bytes of one K (or V) tile: 16 rows per row group of a warp
 constexpr int kHProducers = 2;     // issuing threads (one per warp): stage s is always filled by producer s mod kHProducers
@@ -878,7 +878,8 @@ int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const v
     const int grid = items < sms ? items : sms;
     // Segments of some hundred rows differ in length and an item is a good part of a CTA's work: CTAs' sums of tiles
     // made alike.  It costs 2 us a call, the shares' arithmetic and the parts that pass through global memory:
-    // 32 x 32 heads, 128 rows of capacity 19.3 us a call without / 23.0 with; 256 31.5 / 31.5; 300 37.5 / 36.0 (two rounds shared
+    // 32 x 32 heads, 128 rows 19.3 us a call without / 23.0 with; 256 31.5 / 31.5 (and caches are mostly below their
+    // capacity); 300 37.5 / 36.0 (two rounds shared
     // out 38.8); 40 x 40 heads, 500 rows 77 / 77 (74); 800 rows of 32 x 32 heads 87 / 82 (77); 4 x 32 x 32 heads of 819 rows 296
     // / 284 (279); fp32, 16 x 40 heads of 600 rows 81 / 67 (66).
     const bool shared = seg_rows >= kHSharedRows;
