@@ -189,7 +189,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         bar_init(drained + 1, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == kMmaWarp) {  // (one CTA per SM: its registers leave no room for another)
+    if (warp == kMmaWarp) {  // (one CTA per SM: its shared memory leaves no room for another)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_slot)),
                      "r"(512u)
                      : "memory");
