@@ -65,7 +65,7 @@ constexpr int kHMaxAct = 256;      // segments planned per call
 constexpr int kHMaxGrid = 256;
 // Mean capacity of a segment from which items are shared out by tiles (launch_decode_heads), and from which two rounds of
 // them besides the incomplete one are; one below.
-constexpr int64_t kHSharedRows = 288, kHTwoRoundsRows = 400;
+constexpr int64_t kHSharedRows = 288, kHSharedAlways = 512, kHTwoRoundsRows = 400;
 constexpr int64_t kHMaxSegRows = 1024;  // mean capacity of a segment above which calls go to the row-split kernel
 constexpr uint32_t kHTile = 8192;  // bytes of one K (or V) tile: 16 rows per row group of a warp
 constexpr int kHProducers = 2;     // issuing threads (one per warp): stage s is always filled by producer s mod kHProducers
@@ -882,7 +882,8 @@ int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const v
     // capacity); 300 37.5 / 36.0 (two rounds shared
     // out 38.8); 40 x 40 heads, 500 rows 77 / 77 (74); 800 rows of 32 x 32 heads 87 / 82 (77); 4 x 32 x 32 heads of 819 rows 296
     // / 284 (279); fp32, 16 x 40 heads of 600 rows 81 / 67 (66).
-    const bool shared = seg_rows >= kHSharedRows;
+    // With many rounds of items the sums are alike without it: 80 x 40 heads (21 rounds) of 361 rows 105 / 108, of 604 171 / 162.
+    const bool shared = seg_rows >= kHSharedAlways || (seg_rows >= kHSharedRows && items <= 12 * sms);
     a.pool_rounds = seg_rows >= kHTwoRoundsRows ? 2 : 1;
     return s->dtype == PKV_BF16 ? launch_heads<__nv_bfloat16>(D, shared, maps, a, grid, st) : launch_heads<float>(D, shared, maps, a, grid, st);
 }
