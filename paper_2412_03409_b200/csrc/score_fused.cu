@@ -176,7 +176,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         for (int i = 0; i < SM::kQ; ++i) {
             bar_init(q_full + i, 1);
-            bar_init(q_empty + i, 1);
+            bar_init(q_empty + i, 2);
         }
         for (int i = 0; i < kSlots; ++i) {
             bar_init(s_empty + i, kReadWarps / 2);
@@ -231,7 +231,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 if (!wanted(i, safe)) continue;
                 for (int s = S - 1; s >= 0 && !dead; --s) {
                     const int top = s >> 1;
-                    // (both warps wait for every strip: a barrier's phases must not pass by either unseen)
+                    // (both warps wait for every strip and both give its stage back, whoever multiplies it: the stage's next
+                    // phase then cannot end before either has seen this one, which a parity test would miss)
                     warp_wait_ready(q_full + ring_q.idx, ring_q.phase, dead, &s_abort);
                     if ((s & 1) == odd) {
                         const uint64_t db = desc_add(dq, ring_q.idx * SM::QTILE);
@@ -265,11 +266,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         // (the next tile of the warp's own lies beyond the other's strip, or is the next head's)
                         const int skip = s > 0 ? ((s - 1) >> 1) + 1 : ((S - 1) & 1) == odd ? 0 : ((S - 1) >> 1) + 1;
                         if (lane == 0) *(volatile int *)(s_next + odd) = (int)n + skip;
-                    } else if (s == S - 1 && odd) {  // no odd strip attends to the last tile
-                        warp_wait_ready(k_full + ring_k.idx, ring_k.phase, dead, &s_abort);
-                        if (lane == 0) {
-                            bar_arrive(k_empty + ring_k.idx);
-                            *(volatile int *)(s_next + odd) = (int)n_tile + top + 1;
+                    } else {
+                        if (lane == 0) bar_arrive(q_empty + ring_q.idx);
+                        if (s == S - 1 && odd) {  // no odd strip attends to the last tile
+                            warp_wait_ready(k_full + ring_k.idx, ring_k.phase, dead, &s_abort);
+                            if (lane == 0) {
+                                bar_arrive(k_empty + ring_k.idx);
+                                *(volatile int *)(s_next + odd) = (int)n_tile + top + 1;
+                            }
                         }
                     }
                     n_tile += (uint32_t)top + 1;
