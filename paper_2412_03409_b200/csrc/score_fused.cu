@@ -242,11 +242,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         for (int g = top; g >= 0; --g, ++n) {
                             if (s >= S - 2) warp_wait_ready(k_full + k.idx, k.phase, dead, &s_abort);
                             // the slot's last user must have been issued, so that the phase waited for is the next
-                            for (uint32_t t = 0; seen <= (int)n - kSlots && !dead; ++t) {
-                                seen = __shfl_sync(0xffffffffu, *(volatile int *)(s_next + !odd), 0);
-                                if (t > kSpin || *(volatile int *)&s_abort) dead = true;
-                                dead = __any_sync(0xffffffffu, dead);
-                            }
+                            count_wait(s_next + !odd, (int)n - kSlots, seen, dead, &s_abort);
                             warp_wait_ready(s_empty + n % kSlots, (n / kSlots & 1u) ^ 1u, dead, &s_abort);
                             if (dead) break;
                             fence_after();
@@ -551,6 +547,20 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     }
 }
 
+// The wait for a count that nothing raises gives up, latches `dead` and sets the abort word.
+__global__ void selftest_count_kernel(int32_t *dev_status, uint32_t limit)
+{
+    __shared__ int s_abort, s_count;
+    if (threadIdx.x == 0) s_abort = s_count = 0;
+    __syncthreads();
+    bool dead = false, past = false;
+    int seen = -1;
+    count_wait(&s_count, -1, seen, past, &s_abort, limit);  // (there already)
+    count_wait(&s_count, 0, seen, dead, &s_abort, limit);
+    __syncwarp();
+    if (threadIdx.x == 0 && dead && !past && s_abort) raise_status(dev_status, 0, PKV_DEV_TIMEOUT);
+}
+
 template <int D>
 int launch_fused(const CUtensorMap &mq, const CUtensorMap &mk, const FusedArgs &a, int sms, cudaStream_t st)
 {
@@ -568,6 +578,12 @@ int launch_fused(const CUtensorMap &mq, const CUtensorMap &mk, const FusedArgs &
 }
 
 }  // namespace
+
+int selftest_wait_fused(int32_t *dev_status, cudaStream_t st)
+{
+    selftest_count_kernel<<<1, 32, 0, st>>>(dev_status, 500u);
+    return check_launch("selftest_count_kernel");
+}
 
 // Prompts whose keys a CTA holds.  With five key tiles a head is 22 us of one CTA, and a few heads, spread over all SMs
 // by tiles, are faster in two passes: 8 heads of 640 tokens 23 us here, 18 there, 48 24 and 24 (heads of 64: 23 and

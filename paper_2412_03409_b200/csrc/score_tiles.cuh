@@ -65,6 +65,22 @@ __device__ __forceinline__ void warp_wait(uint64_t *bar, uint32_t parity, bool &
     dead = __any_sync(0xffffffffu, dead);
 }
 
+// Bounded wait of a whole warp for a count in shared memory, which another warp raises, to be above `n`; `seen` is what
+// was last read of it.  Read often at first, as it is seldom far behind; the limit is about as long as the other waits'.
+__device__ __forceinline__ void count_wait(const int *count, int n, int &seen, bool &dead, int *abort_flag, uint32_t limit = kSpin)
+{
+    for (uint32_t i = 0; seen <= n && !dead; ++i) {
+        seen = __shfl_sync(0xffffffffu, *(const volatile int *)count, 0);
+        if (seen > n) return;
+        if (i >= limit || *(volatile int *)abort_flag) {
+            dead = true;
+            atomicExch(abort_flag, 1);
+        }
+        dead = __any_sync(0xffffffffu, dead);
+        if (i >= 64) __nanosleep(i < 4096 ? 50 : kSuspendNs);
+    }
+}
+
 __device__ __forceinline__ void tma_load_5d(void *dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1,
                                             int c2, int c3, int c4)
 {

@@ -64,3 +64,11 @@ def test_one_head_out_of_range(N):
     assert torch.equal(got[0, rest], plain[0, rest])
     ref, top = reference(q[:, big], k[:, big], scale[big])
     check_scores(got[:, big].cpu().numpy(), ref, 8 * top.max() * 2.0 ** -24)
+
+
+def test_a_wait_for_the_other_warp_that_runs_out():
+    from paper_2412_03409_b200 import api
+    status = torch.zeros(2, dtype=torch.int32, device="cuda")
+    api.prefixkv_selftest_bounded_wait(3, status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist() == [api.DEV_TIMEOUT, 0]
