@@ -16,17 +16,23 @@
 // Strips go from the last to the first and a head's last key tile is loaded first: tiles of the five-tile ring become
 // free in the order of their loads, and the next head's come in while this one's last strips are still in work.
 //
-// The exponentials are of the logits themselves, without the maximum: within some 2^+-60 they are as exact, and the
-// maximum first would be a third walk over tensor memory with a barrier in it.  A strip with a sum out of that range
-// (or NaN) has its head done again, relative to the maximum, after the CTA's others.
+// The exponentials are of the logits themselves, without the maximum: that would be another walk over tensor memory with a
+// barrier in it.  A head whose first blocks show logits (log2) above 60, or a query with none above -45, is taken relative to
+// the maximum: in the later strips of such a head the four warps that share one exchange their maxima first; in the first strip
+// a warp that sees such logits takes its own, as the other three may not see any, and with the sums' exchange all are brought to one
+// scale.  A strip whose sum is out of 2^-80 ... 2^100 all the same (or NaN) has its head done again, after the CTA's others.
+// 1024 heads of 128, 640 tokens: 125 us; with all heads relative to the maximum 178 (two passes 182 to 207), with one in eight
+// 138.  With every such head done twice these took 118, 305 and 171; a look at every block instead of the first 144.
 //
-// What bounds it: the chain of short steps, not a unit.  A tile of 128 x 64 takes 990 clocks (of 385 to 430 in the
+// What bounds it: the chain of short steps, not a unit.  A tile of 128 x 64 takes some 1000 clocks (of 385 to 430 in the
 // tensor pipe and 512 in the special-function unit); the waits of an MMA warp and of a reader, 200 to 300 clocks each
-// although complete, and a strip's exchange are what the second MMA warp and the second team are for.  32 x 32 heads
-// of 128, 640 tokens: 186 us with the two passes, 118 here, and without exponentials still 109; 300 tokens 89 and 52,
-// 64 tokens 26 and 18.  One MMA warp 163; logits of a strip in registers (80 a thread) instead of exponentials put back
-// 160, weighing by eight warps of their own 163; three teams 138; halves of a block loaded ahead 145; an eighth, a
-// quarter of the exponentials on the FMA pipe 123, 126; two query stages 122; L2 prefetch of the next head 123.
+// although complete, and a strip's exchange are what the second MMA warp and the second team are for.  The readers' code is kept
+// short (one loop for both walks, one copy of the weighing): the same steps with the weighing unrolled over five tiles and a loop to
+// each walk took 134.  Scores of 32 x 32 heads of 128: 640 tokens 182 us with two passes, 125 here; 300 tokens 87 and 56;
+// 64 tokens 25 and 20.  Before the look at the first block 118, and of these without exponentials 109; one MMA warp 163; logits
+// of a strip in registers (80 a thread) instead of exponentials put back 160, weighing by eight warps of their own 163; three
+// teams 138; halves of a block loaded ahead 145; an eighth, a quarter of the exponentials on the FMA pipe 123, 126; two query
+// stages 122; L2 prefetch of the next head 123.
 //
 // Every wait is bounded: when one runs out the CTA stops waiting, sets the call's abort word (the head mean then
 // writes NaN for every score) and still releases its tensor memory.
@@ -47,9 +53,12 @@ constexpr int kReadWarps = 16;     // two teams x two halves of a strip x four l
 constexpr int kMmaWarp = 0, kLoadWarp = 2, kFlushWarp = 3, kFirstReader = 4;
 constexpr int kFThreads = (kFirstReader + kReadWarps) * 32;
 constexpr int kBadWords = 64;      // heads to be done again, a bit to each of the CTA's (modulo the bits there are)
-// Sums of exponentials of the logits themselves that are taken: what flushes to zero is below 2^-66 of them, and
+// Sums of exponentials of the logits themselves that are taken: what flushes to zero is below 2^-46 of them, and
 // neither they nor their reciprocals are near the ends of the range.
-constexpr float kLowSum = 0x1p-60f, kHighSum = 0x1p+100f;
+constexpr float kLowSum = 0x1p-80f, kHighSum = 0x1p+100f;
+// Logits (log2) of a head's first block within which its maxima are not formed: some way from where the sums go out of range.
+constexpr float kHighLogit = 60.f, kLowLogit = -45.f;
+constexpr float kLowest = -1e30f;  // scale of a sum of nothing
 constexpr uint32_t kIdescStrip = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(QS >> 3) << 17) | ((uint32_t)(TT >> 4) << 24);
 
 struct FusedArgs {
@@ -117,6 +126,19 @@ __device__ __forceinline__ void block_mask(Block &v, int d, float x)
         v[hf][i][rr].x = at < 0 ? x : v[hf][i][rr].x;
         v[hf][i][rr].y = at + 1 < 0 ? x : v[hf][i][rr].y;
     }
+}
+// Whether the thread's logits are within the range: every query's largest of the four keys, unless all of these are masked.
+__device__ __forceinline__ bool block_in_range(const Block &v, float sc)
+{
+    float up = 0.f, low = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float x = fmaxf(max3(v[0][i][0].x * sc, v[0][i][1].x * sc, v[1][i][0].x * sc), v[1][i][1].x * sc);
+        const float y = fmaxf(max3(v[0][i][0].y * sc, v[0][i][1].y * sc, v[1][i][0].y * sc), v[1][i][1].y * sc);
+        up = max3(up, x, y);
+        low = fminf(low, fminf(x == -INFINITY ? 0.f : x, y == -INFINITY ? 0.f : y));
+    }
+    return up <= kHighLogit && low >= kLowLogit;
 }
 __device__ __forceinline__ float2 shfl_xor2(float2 v, int o)
 {
@@ -370,13 +392,15 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                             // other, which everybody reaches only after reading this one
 #pragma unroll 1
         for (int round = 0; round < 2; ++round) {
-            const bool safe = round == 1;
-            if (safe && !another()) break;
+            if (round == 1 && !another()) break;
 #pragma unroll 1
             for (int i = 0; i < mine; ++i) {
-                if (!wanted(i, safe)) continue;
+                if (!wanted(i, round == 1)) continue;
+                bool safe = round == 1;
                 const int head = blockIdx.x + i * gridDim.x;
-                const float sc = a.layer_scale[head / a.H % a.L] * kLog2eT;
+                float sc = a.layer_scale[head / a.H % a.L] * kLog2eT;
+                if (sc == 0.f) sc = 0x1p-149f;  // (what is masked is infinite, and times 0 it would be NaN)
+                const float masked = sc > 0.f ? -INFINITY : INFINITY;
                 float acc[kMaxTiles] = {};
 #pragma unroll 1
                 for (int s = S - 1; s >= 0; --s) {
@@ -393,98 +417,123 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         fence_after();
                         return taddr + slot * QS;
                     };
+                    auto exchange = [&](const float2 (&v)[4]) {
+                        float *b = s_x + (part * 2 + (turn++ & 1u)) * 128;
+                        if (lane < 4) {
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) *reinterpret_cast<float2 *>(b + quarter * 32 + 8 * c + c2) = v[c];
+                        }
+                        asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");
+                        return (const float *)b;
+                    };
                     float2 base2[4], sum[4];
-                    float mul = sc;
-                    bool fast = true;
 #pragma unroll
                     for (int c = 0; c < 4; ++c) base2[c] = sum[c] = make_float2(0.f, 0.f);
-                    if (safe) {
-                        // The maximum of every query first.  With a scale above 0 the extreme of sc * x is sc * max x;
-                        // otherwise logits are scaled first (those of -infinity, masked, stay that).
-                        fast = sc > 0.f;
-                        mul = fast ? sc : 1.f;
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) base2[c] = make_float2(-INFINITY, -INFINITY);
+                    const bool mixed = round == 0 && s >= S - 2;  // the team's first strip of the head
+                    bool look = mixed;
+                    // Over the blocks: for the maximum of every query, where that is needed, and for the exponentials.
+#pragma unroll 1
+                    for (int walk = safe ? 0 : 1; walk < 2; ++walk) {
 #pragma unroll 1
                         for (int g = hi; g >= 0; --g) {
+                            const uint32_t at = wait_tile(g);
                             Block v;
-                            block_load(wait_tile(g), v);
-                            if (g == top && rel == 0) block_mask(v, c2 - r, -INFINITY);
+                            block_load(at, v);
+                            if (g == top && rel == 0) block_mask(v, c2 - r, masked);
+                            if (walk == 0) {
+#pragma unroll
+                                for (int x = 0; x < 16; ++x) {
+                                    const float2 t = v[x >> 3][x & 3][x >> 2 & 1];
+                                    float2 &m = base2[x & 3];
+                                    m = g == hi && x < 4 ? make_float2(t.x * sc, t.y * sc) : make_float2(fmaxf(m.x, t.x * sc), fmaxf(m.y, t.y * sc));
+                                }
+                                continue;
+                            }
+                            if (look) {
+                                // The first block shows whether the head's exponentials need a maximum: the warp's own here,
+                                // as the others may not need one.
+                                look = false;
+                                safe = !__all_sync(0xffffffffu, block_in_range(v, sc));
+                                if (safe) {
+                                    walk = -1;
+                                    break;
+                                }
+                            }
 #pragma unroll
                             for (int x = 0; x < 16; ++x) {
-                                float2 t = v[x >> 3][x & 3][x >> 2 & 1];
-                                if (!fast) {
-                                    t.x = t.x == -INFINITY ? -INFINITY : t.x * sc;
-                                    t.y = t.y == -INFINITY ? -INFINITY : t.y * sc;
-                                }
-                                base2[x & 3] = make_float2(fmaxf(base2[x & 3].x, t.x), fmaxf(base2[x & 3].y, t.y));
+                                float2 &t = v[x >> 3][x & 3][x >> 2 & 1];
+                                t = fma2(t, make_float2(sc, sc), make_float2(-base2[x & 3].x, -base2[x & 3].y));
+                                t = make_float2(ex2(t.x), ex2(t.y));
                             }
+                            block_store(at, v);
+#pragma unroll
+                            for (int x = 0; x < 16; ++x) sum[x & 3] = add2(sum[x & 3], v[x >> 3][x & 3][x >> 2 & 1]);
                         }
-                        float *mx = s_x + (part * 2 + (turn++ & 1u)) * 128;
+                        if (walk != 0) continue;
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
+                            if (hi < 0) base2[c] = make_float2(-INFINITY, -INFINITY);
 #pragma unroll
                             for (int o = 4; o < 32; o <<= 1) {
                                 const float2 t = shfl_xor2(base2[c], o);
                                 base2[c] = make_float2(fmaxf(base2[c].x, t.x), fmaxf(base2[c].y, t.y));
                             }
-                            if (lane < 4) *reinterpret_cast<float2 *>(mx + quarter * 32 + 8 * c + c2) = base2[c];
                         }
-                        asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");
+                        if (!mixed) {
+                            const float *mx = exchange(base2);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
+                            for (int c = 0; c < 4; ++c)
 #pragma unroll
-                            for (int p = 0; p < 4; ++p) {
-                                const float2 t = *reinterpret_cast<const float2 *>(mx + p * 32 + 8 * c + c2);
-                                base2[c] = make_float2(fmaxf(base2[c].x, t.x), fmaxf(base2[c].y, t.y));
-                            }
-                            // (-infinity when infinite elements mask every key: sums of 0)
-                            base2[c].x = base2[c].x == -INFINITY ? 0.f : base2[c].x * mul;
-                            base2[c].y = base2[c].y == -INFINITY ? 0.f : base2[c].y * mul;
+                                for (int p = 0; p < 4; ++p) {
+                                    const float2 t = *reinterpret_cast<const float2 *>(mx + p * 32 + 8 * c + c2);
+                                    base2[c] = make_float2(fmaxf(base2[c].x, t.x), fmaxf(base2[c].y, t.y));
+                                }
                         }
-                    }
-#pragma unroll 1
-                    for (int g = hi; g >= 0; --g) {
-                        const uint32_t at = wait_tile(g);
-                        Block v;
-                        block_load(at, v);
-                        if (!fast) {
+                        // (-infinity when infinite elements mask every key: sums of 0)
 #pragma unroll
-                            for (int x = 0; x < 16; ++x) {
-                                float2 &t = v[x >> 3][x & 3][x >> 2 & 1];
-                                t.x = t.x == -INFINITY ? -INFINITY : t.x * sc;
-                                t.y = t.y == -INFINITY ? -INFINITY : t.y * sc;
-                            }
-                        }
-#pragma unroll
-                        for (int x = 0; x < 16; ++x) {
-                            float2 &t = v[x >> 3][x & 3][x >> 2 & 1];
-                            t = fma2(t, make_float2(mul, mul), make_float2(-base2[x & 3].x, -base2[x & 3].y));
-                            t = make_float2(ex2(t.x), ex2(t.y));
-                        }
-                        if (g == top && rel == 0) block_mask(v, c2 - r, 0.f);
-                        block_store(at, v);
-#pragma unroll
-                        for (int x = 0; x < 16; ++x) sum[x & 3] = add2(sum[x & 3], v[x >> 3][x & 3][x >> 2 & 1]);
+                        for (int c = 0; c < 4; ++c)
+                            base2[c] = make_float2(base2[c].x == -INFINITY ? 0.f : base2[c].x, base2[c].y == -INFINITY ? 0.f : base2[c].y);
                     }
                     // The lanes' and then the four quarters' parts of a query's sum; its weight goes to a lane.
 #pragma unroll
                     for (int o = 4; o < 32; o <<= 1)
 #pragma unroll
                         for (int c = 0; c < 4; ++c) sum[c] = add2(sum[c], shfl_xor2(sum[c], o));
-                    float *xb = s_x + (part * 2 + (turn++ & 1u)) * 128;
-                    if (lane < 4) {
+                    const float *x;
+                    float factor = 1.f;  // from the warp's scale to the strip's, for the lane's query
+                    if (!mixed) {
+                        x = exchange(sum);
+                    } else {
+                        float2 y[4];
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) *reinterpret_cast<float2 *>(xb + quarter * 32 + 8 * c + c2) = sum[c];
+                        for (int c = 0; c < 4; ++c) y[c] = safe ? make_float2(-1.f, -1.f) : sum[c];
+                        x = exchange(y);  // (a sign shows all four that scales differ)
+                        if (__any_sync(0xffffffffu, fminf(fminf(x[lane], x[32 + lane]), fminf(x[64 + lane], x[96 + lane])) < 0.f)) {
+                            safe = true;
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) y[c] = hi < 0 ? make_float2(kLowest, kLowest) : base2[c];
+                            x = exchange(y);
+                            factor = ex2(x[quarter * 32 + lane] - fmaxf(fmaxf(x[lane], x[32 + lane]), fmaxf(x[64 + lane], x[96 + lane])));
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                float2 n = y[c];
+#pragma unroll
+                                for (int p = 0; p < 4; ++p) {
+                                    const float2 t = *reinterpret_cast<const float2 *>(x + p * 32 + 8 * c + c2);
+                                    n = make_float2(fmaxf(n.x, t.x), fmaxf(n.y, t.y));
+                                }
+                                sum[c] = make_float2(sum[c].x * ex2(y[c].x - n.x), sum[c].y * ex2(y[c].y - n.y));
+                            }
+                            x = exchange(sum);
+                        }
                     }
-                    asm volatile("bar.sync %0, 128;" ::"r"(1 + part) : "memory");
-                    const float z = (xb[lane] + xb[32 + lane]) + (xb[64 + lane] + xb[96 + lane]);
+                    const float z = (x[lane] + x[32 + lane]) + (x[64 + lane] + x[96 + lane]);
                     const bool real = s * QS + half * 32 + lane < a.N;
-                    if (!safe && real && !(z >= kLowSum && z <= kHighSum)) {
+                    if ((mixed || !safe) && real && !(z >= kLowSum && z <= kHighSum)) {
                         atomicOr(s_bad + i / 32 % kBadWords, 1u << (i & 31));
                         s_again = 1;
                     }
-                    my_w[lane] = real ? __frcp_rn(z) : 0.f;
+                    my_w[lane] = real ? __frcp_rn(z) * factor : 0.f;
                     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                     __syncwarp();
                     // A key to a lane: the weighted sum of its exponentials.
@@ -492,9 +541,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
                     for (int c = 0; c < 8; ++c) w[c] = reinterpret_cast<const float4 *>(my_w)[c];
                     __syncwarp();
-#pragma unroll
-                    for (int g = kMaxTiles - 1; g >= 0; --g) {
-                        if (g > top) continue;
+#pragma unroll 1
+                    for (int g = top; g >= 0; --g) {
                         const uint32_t slot = (n_tile + (uint32_t)(top - g)) % kSlots;
                         if (g > hi) {
                             wait_tile(g);  // (so that the release before this one is over)
@@ -518,7 +566,10 @@ score_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                                 t[1] = fma2(make_float2(e[4 * c + 2], e[4 * c + 3]), make_float2(w[c].z, w[c].w), t[1]);
                             }
                         }
-                        acc[g] += (t[0].x + t[0].y) + (t[1].x + t[1].y);
+                        const float add = (t[0].x + t[0].y) + (t[1].x + t[1].y);
+#pragma unroll
+                        for (int j = 0; j < kMaxTiles; ++j)
+                            if (j == g) acc[j] += add;
                     }
                     const uint32_t used = ((2u << top) - 1) << n_tile % kSlots;
                     full_phase ^= (used | used >> kSlots) & ((1u << kSlots) - 1);
