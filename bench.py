@@ -505,7 +505,11 @@ def run_ours(args):
 def LAUNCHES_PER_STEP(w, path):
     # score: one kernel for both sums, or two passes, + head mean (the rule of score_fused_covers, and fp32 one-tile
     # prompts); search: sort/scan + bisection; compact: plan + gather; decode: one kernel per token, or stream + merge
-    one_kernel = w.N <= 128 if str(w.dtype) == "torch.float32" else w.N <= 512 or (w.N <= 640 and w.B * w.L * w.H >= 64)
+    heads, sms = w.B * w.L * w.H, 148
+    one_kernel = w.N <= 128
+    if str(w.dtype) != "torch.float32":
+        one_kernel = w.N <= 64 or (w.N <= 128 and heads <= (3 if w.D == 64 else 7) * sms) or 128 < w.N <= 384 or \
+            (384 < w.N <= 640 and heads >= 64 and not (w.N >= 600 and sms < heads < sms + sms // 8))
     return (2 if one_kernel else 3) + 2 + 2 + DECODE_KERNELS[path][3] * w.T
 
 

@@ -636,13 +636,24 @@ int selftest_wait_fused(int32_t *dev_status, cudaStream_t st)
     return check_launch("selftest_count_kernel");
 }
 
-// Prompts whose keys a CTA holds.  With five key tiles a head is 22 us of one CTA, and a few heads, spread over all SMs
-// by tiles, are faster in two passes: 8 heads of 640 tokens 23 us here, 18 there, 48 24 and 24 (heads of 64: 23 and
-// 22), 64 25 and 28 (24 and 25).  Up to four tiles this is faster throughout (8 heads of 448 tokens 16 and 17, of 64 11 and 13).
+// Prompts whose keys a CTA holds, where that is the faster way; otherwise two passes that spread heads over the SMs by tiles
+// (whole calls, us, here / there; heads of 64, then of 128):
+// - From four key tiles on a head takes one CTA 10 us or more, and few heads leave SMs idle: 512 tokens, 8 heads 16.4 / 14.5 and 16.8
+//   / 15.3, 32 16.9 / 15.6 and 17.3 / 16.8, 64 17.1 / 18.9 and 17.7 / 21.1; 448 tokens, 8 heads 15.2 / 14.4 and 15.4 / 15.2; of three
+//   tiles, 384 tokens, 12.4 / 13.4 and 12.9 / 14.1.  Of 600 tokens or more some heads above the number of SMs cost a second
+//   head's time for a few: 149 heads of 640 tokens 37.9 / 36.1 and 39.5 / 38.7, 166 38.4 / 38.6 and 39.9 / 41.5.
+// - Of 65 to 128 tokens the second strip has half of its keys masked, while there one tile takes all queries: 128 tokens, 320 heads
+//   12.9 / 14.2 and 13.2 / 16.4, 592 16.2 / 16.1 and 16.3 / 19.2, 1600 32.0 / 29.7 and 35.2 / 37.7; 65 tokens, 1024 heads 22.7 / 22.3 and
+//   22.9 / 24.3, 1184 25.0 / 22.6 and 25.3 / 25.1; 100 tokens, 4096 72 / 60 and 77.6 / 73.7.
 bool score_fused_covers(const pkv_shape *s)
 {
-    const int64_t heads = (int64_t)s->batch * s->layers * s->heads;
-    return s->prompt_len <= 4 * TT || (s->prompt_len <= kMaxTiles * TT && heads >= 64);
+    const int64_t heads = (int64_t)s->batch * s->layers * s->heads, sms = sm_count();
+    const int N = s->prompt_len;
+    if (N <= 64) return true;
+    if (N <= TT) return heads <= (s->head_dim == 64 ? 3 : 7) * sms;
+    if (N <= 3 * TT) return true;
+    if (N >= 600 && heads > sms && heads < sms + sms / 8) return false;
+    return N <= kMaxTiles * TT && heads >= 64;
 }
 
 // Returns PKV_OK, an error, or -1 when the tensor maps cannot describe the caller's layout.

@@ -1,5 +1,5 @@
-// Importance score (Sec. 3.2), tensor-core path for bf16 inputs (prompts of up to 640 tokens without the caller's
-// log-sum-exp: score_fused.cu).
+// Importance score (Sec. 3.2), tensor-core path for bf16 inputs (most prompts of up to 640 tokens without the caller's
+// log-sum-exp: score_fused.cu, whose score_fused_covers has the line).
 //
 //   pass 1: per query m, log2-sum-exp of the scaled causal logits over keys j <= m
 //   pass 2: per key n, sum over queries m >= n of exp2(logit - lse[m])

@@ -148,3 +148,15 @@ def test_heads_out_of_range_are_not_done_twice(N):
             runs.append(a.elapsed_time(b))
         times.append(sorted(runs[2:])[5])
     assert times[1] < 1.9 * times[0], times   # (1.4 measured; 2.5 with a first round that fails)
+
+
+# Both sides of every line between this kernel and the two passes.
+@pytest.mark.parametrize("heads,N,D", [(444, 100, 64), (445, 100, 64), (1036, 65, 128), (1037, 65, 128), (3, 384, 64), (3, 385, 64), (63, 450, 128), (64, 450, 128),
+                                       (148, 600, 64), (149, 600, 64), (149, 599, 64), (166, 640, 128), (165, 640, 128)])
+def test_at_the_lines_of_the_route(heads, N, D):
+    from paper_2412_03409_b200.session import Session
+    q, k = (torch.randn(1, heads, 1, N, D, device="cuda").bfloat16() for _ in range(2))
+    scale = np.full(heads, D ** -0.5, np.float32)
+    s = Session(1, heads, 1, D, N, torch.bfloat16, scale, decode_cap=0, max_budget_rows=heads)
+    ref, _ = reference(q, k, scale)
+    check_scores(s.score(q, k).cpu().numpy(), ref, 1e-5)
