@@ -579,18 +579,48 @@ static int launch_sort_items(const pkv_shape *s, const float *scores, int32_t *o
     return PKV_OK;
 }
 
+// Clusters of four of the sort kernel that run at once with an SM to each CTA (a block of 1024 threads fills one).  There
+// are fewer than SMs / 4: a cluster's SMs are of one GPC, and most of these have no multiple of four.
+static int clusters_of_four()
+{
+    static int count[64] = {};  // plus one
+    static bool attr_done[64] = {};
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if (count[dev] > 0) return count[dev] - 1;
+    const size_t smem = sort_smem_bytes(1024, 4, true);
+    if (ensure_dynamic_smem((const void *)sort_scan_kernel<4, true>, (int)smem, attr_done) != PKV_OK) return 0;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 4;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(4);
+    cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, sort_scan_kernel<4, true>, &cfg) != cudaSuccess) {
+        cudaGetLastError();  // (it only leaves segments whole)
+        n = 0;
+    }
+    count[dev] = n + 1;
+    return n;
+}
+
 // Up to 256 scores places are counted: the work grows with the square, 512 of them cost more than the passes.
 // Two items a thread beat four up to some 768 scores for one prompt (18.0 / 18.4 us with the search) and not for
 // 16 (42.8 / 37.6); beyond, four do throughout (1024: 19.8 / 19.2 and 47.9 / 40.7).  Above that as few as 1024
 // threads allow.  Long prompts whose segments leave SMs idle are split over clusters of four or two (with compaction, whole / split
 // over four: 32 segments of 4096 scores 127.9 / 125.9 us, of 4500 136.0 / 134.8, of 8192 226 / 219, of 16384 264 / 238; 64 segments, over
-// two: of 4500 230 / 235, 40 of 6000 252 / 253, 64 of 16384 431 / 421).
+// two: of 4500 230 / 235, 40 of 6000 252 / 253, 64 of 16384 431 / 421), while all clusters run at once (33 of four on a B200; the sort
+// alone, whole / split over four: 33 segments of 8193 scores 44.4 / 28.4 us, 34 43.9 / 54.2, and 36.7 over two).
 static int launch_sort(const pkv_shape *s, const float *scores, int32_t *order, uint64_t *cum,
                        int32_t *seg_flags, cudaStream_t st)
 {
     const int N = s->prompt_len, sms = sm_count();
     const int64_t segments = (int64_t)s->batch * s->layers;
-    if (N > kSplitFour && 4 * segments <= sms) return launch_sort_items<4, true>(s, scores, order, cum, seg_flags, st, 4);
+    if (N > kSplitFour && segments <= clusters_of_four()) return launch_sort_items<4, true>(s, scores, order, cum, seg_flags, st, 4);
     if (N > kSplitTwo && 2 * segments <= sms) return launch_sort_items<8, true>(s, scores, order, cum, seg_flags, st, 2);
     if (N <= 256) return launch_sort_items<1>(s, scores, order, cum, seg_flags, st);
     if (N <= 768) return launch_sort_items<2>(s, scores, order, cum, seg_flags, st);
