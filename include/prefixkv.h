@@ -326,6 +326,7 @@ int prefixkv_gini(const pkv_shape *shape, const uint64_t *cum, double *gini, voi
  * their CTAs; one block plays both parts, some flags not coming before the limit and then late,
  * and raises the same code when every flag was left as a later call needs it.
  * which = 3: the wait of the scoring kernel for short bf16 prompts for its other product warp.
+ * which = 4: the wait of the per-head decode kernel for parts of an item that other CTAs pass on, as which = 2.
  *   dev_status  [>= 1] int32, must hold PKV_DEV_OK on entry for the code to be recorded
  */
 int prefixkv_selftest_bounded_wait(int32_t which, int32_t *dev_status, void *cuda_stream);

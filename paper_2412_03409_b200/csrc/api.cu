@@ -79,6 +79,7 @@ int selftest_wait_score(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_stream(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_cluster(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_fused(int32_t *dev_status, cudaStream_t st);
+int selftest_wait_parts(int32_t *dev_status, cudaStream_t st);
 
 static size_t score_ws_bytes(const pkv_shape *s)
 {
@@ -185,5 +186,6 @@ extern "C" int prefixkv_selftest_bounded_wait(int32_t which, int32_t *dev_status
     if (which == 1) return selftest_wait_stream(dev_status, (cudaStream_t)cuda_stream);
     if (which == 2) return selftest_wait_cluster(dev_status, (cudaStream_t)cuda_stream);
     if (which == 3) return selftest_wait_fused(dev_status, (cudaStream_t)cuda_stream);
+    if (which == 4) return selftest_wait_parts(dev_status, (cudaStream_t)cuda_stream);
     return PKV_ERR_INVALID_ARG;
 }

@@ -22,9 +22,10 @@
 //
 // Long segments (SHARED): items dealt round-robin leave the CTAs with sums of tiles that differ by an item or more.  There a CTA
 // has all but the last rounds of items for its own, and the tiles of the others, the pool, are shared out as
-// consecutive ranges that make the sums alike; an item that a range cuts goes from CTA to CTA as a softmax state in
-// global memory.  A CTA takes its range from the end on and before its own items but the first, so that what the next CTA
-// waits for is there long before that is done.  Every CTA works the shares out for itself, from the lengths.
+// consecutive ranges that make the sums alike; an item that a range cuts goes on as a softmax state in global memory to
+// the CTA that has its end.  A planner warp in every CTA works the shares out from the lengths, while the first items are on their way,
+// lists what the producers issue, and at the end puts the cut item together, away from the consumers; whatever
+// happened, it puts the flags of the parts that it was owed back.  Where the lengths are short or alike already, items stay dealt.
 //
 // Measured on the 32-layer, 32-head, 128-rows-per-layer case (22.3 us per call with this design),
 // each alone: one producer thread 24.1 us, five 22.9, ten 23.1; eight stages 22.4, twelve 21.9 (with
@@ -45,6 +46,7 @@
 #include <atomic>
 #include <chrono>
 #include <mutex>
+#include <type_traits>
 
 #include "decode_plan.cuh"
 
@@ -63,9 +65,14 @@ static_assert(kHPrefetch * kHPrefetchItems <= 32, "one lane per prefetched tile"
 constexpr int kHSlots = 4;         // items whose partial results may be waiting for their last tile
 constexpr int kHMaxAct = 256;      // segments planned per call
 constexpr int kHMaxGrid = 256;
-// Mean capacity of a segment from which items are shared out by tiles (launch_decode_heads), and from which two rounds of
-// them besides the incomplete one are; one below.
-constexpr int64_t kHSharedRows = 288, kHSharedAlways = 512, kHTwoRoundsRows = 400;
+// Sharing out (the measurements stand at launch_decode_heads): mean capacity of a segment from which a call may take that form,
+// with few rounds of items and with some more, and from which two rounds of them besides the incomplete one are shared out.
+constexpr int64_t kHSharedRows = 384, kHSharedRowsMany = 512, kHTwoRoundsRows = 400;
+constexpr int kHFewRounds = 12, kHManyRounds = 40;
+// And what the lengths then decide, in tiles: a CTA's mean sum and an item's mean from which the CTAs work by list, and by how much
+// the largest sum must be above the mean for the pool to be shared out.
+constexpr int kHWorthTiles = 40, kHItemTiles = 6, kHUneven = 15;
+constexpr int kHOwnFirst = 10;  // tiles of its own (and one more to two rounds) that a CTA begins with, while the shares are worked out
 constexpr int64_t kHMaxSegRows = 1024;  // mean capacity of a segment above which calls go to the row-split kernel
 constexpr uint32_t kHTile = 8192;  // bytes of one K (or V) tile: 16 rows per row group of a warp
 constexpr int kHProducers = 2;     // issuing threads (one per warp): stage s is always filled by producer s mod kHProducers
@@ -80,7 +87,7 @@ struct TileMeta {
     int item, seg, h, nrows, flags, tiles, first_warp, slot_parity;
     long long new_row;  // cache row the new token is written to
     float sc;           // layer scale * log2(e)
-    int start;          // (a pool item) tile of the pool the item begins with
+    int pad2;
 };
 
 // Tensor maps over K and V with boxes of one head's slice by 1/kHHeights ... kHHeights/kHHeights of a
@@ -177,7 +184,7 @@ __device__ __forceinline__ void hbulk_load(void *dst, const void *src, uint32_t 
 // warp holds G = 32 / LPR rows at a time and a tile (8 KiB) is 16 such steps.
 // SHARED: the CTAs' sums of tiles are made alike, by sharing out the last items by tiles.
 template <typename T, int D, bool SHARED>
-__global__ void __launch_bounds__((kHWarps + kHProducers) * 32, 1)
+__global__ void __launch_bounds__((kHWarps + kHProducers + SHARED) * 32, 1)
 decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 {
     constexpr int VE = RowVec<T>::VE;
@@ -197,12 +204,14 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
     uint64_t *empty = full + kHStages;
     uint64_t *item_bar = empty + kHStages;     // [kHSlots] the partials of an item's other warps are in
     uint64_t *slot_empty = item_bar + kHSlots; // [kHSlots] the slot's previous item has been merged
+    __shared__ __align__(8) uint64_t own_bar[1];  // (SHARED) s_own is there
     int64_t *s_off = reinterpret_cast<int64_t *>(slot_empty + kHSlots);  // [nact] first row of the segment
     int *s_len = reinterpret_cast<int *>(s_off + a.nact);                // [nact] cached rows, or -1 (cannot take the step)
     float *s_scale = reinterpret_cast<float *>(s_len + a.nact);          // [nact]
+    int4 *s_list = reinterpret_cast<int4 *>(s_scale + a.nact);  // (SHARED) segment, head << 8 | its index, first tile, tile after the last
     __shared__ int s_abort;
     // SHARED:
-    __shared__ int s_known, s_sum[2], s_scan[kHMaxGrid / 32];
+    __shared__ int s_listed;  // entries of the list that are there
     __shared__ int s_start[SHARED ? kHMaxGrid + 1 : 1];                  // first tile of the pool of every CTA
     __shared__ __align__(16) float s_own[SHARED ? PSTRIDE : 4];          // the CTA's part of the item that another began
 
@@ -212,7 +221,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 
     if (tid == 0) {
         s_abort = 0;
-        if (SHARED) s_sum[0] = s_sum[1] = s_known = 0;
+        if (SHARED) s_listed = 0;
 #pragma unroll
         for (int i = 0; i < kHHeights; ++i) {
             prefetch_map(&maps.k[i]);
@@ -228,6 +237,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             hbar_init(item_bar + i, kHWarps - 1);
             hbar_init(slot_empty + i, 1);
         }
+        if (SHARED) hbar_init(own_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // Launched as a programmatic dependent of whatever precedes it in the stream: the set-up above
@@ -254,7 +264,8 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    if (SHARED && tid == 0) lower_flag(a.sent + blockIdx.x);  // (zero already, unless a wait ran out in an earlier launch)
+    // (it may hold anything; in a replay, whose token is the same, at most the mark of a part that was given up)
+    if (SHARED && tid == 0) lower_flag(a.sent + blockIdx.x);
     // ---- plan: what this step does to every active segment -------------------------------------
     for (int si = tid; si < a.nact; si += blockDim.x) {
         const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
@@ -274,46 +285,189 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
 
     const int nitems = a.nact * H;
     // ---- (SHARED) shares: `rounds` items of a CTA's own, and of the others' tiles as many as make all CTAs' sums alike ----
-    const int ctas = (int)gridDim.x, rounds = SHARED ? max(0, nitems / ctas - a.pool_rounds) : 0;
+    // (a call has four rounds of items or more, of which one or two complete ones are the pool's)
+    const int ctas = (int)gridDim.x, rounds = SHARED ? nitems / ctas - a.pool_rounds : 0;
     const int pool = rounds * ctas;  // items from this one on are shared out by tiles
     auto tiles_of = [&](int si) { return s_len[si] < 0 ? 0 : (s_len[si] + TILE_ROWS - 1) / TILE_ROWS; };
-    // Worked out by the consumers while the producers issue the CTA's first item.
-    auto share_out = [&]() {
-        int own = 0, both = 0;  // tiles of CTA tid's own items; of the pool
-        if (tid < ctas)
-            for (int r = 0; r < rounds; ++r) own += tiles_of((tid + r * ctas) / H);
-        for (int si = tid; si < a.nact; si += kHWarps * 32) both += tiles_of(si) * (H - min(H, max(0, pool - si * H)));
-        const int all = __reduce_add_sync(0xffffffffu, own + both);
-        both = __reduce_add_sync(0xffffffffu, both);
-        if (lane == 0) {
-            atomicAdd(&s_sum[0], all);
-            atomicAdd(&s_sum[1], both);
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(kHWarps * 32) : "memory");
-        const int pool_tiles = s_sum[1], want = tid < ctas ? max(0, (s_sum[0] + ctas - 1) / ctas - own) : 0;
-        int incl = want;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int up = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += up;
-        }
-        if (lane == 31 && warp < kHMaxGrid / 32) s_scan[warp] = incl;
-        asm volatile("bar.sync 1, %0;" ::"n"(kHWarps * 32) : "memory");
-        if (tid < ctas) {
-            int sum = incl - want;
-            for (int w = 0; w < warp; ++w) sum += s_scan[w];
-            s_start[tid] = min(pool_tiles, sum);
-        }
-        if (tid == 0) s_start[ctas] = pool_tiles;
-        asm volatile("bar.sync 1, %0;" ::"n"(kHWarps * 32) : "memory");
-        if (tid == 0) {
+    // By list, unless there is little to gain: the producers are a little slower for it, by the item.
+    bool planned = false;
+    if (SHARED && warp >= kHWarps) {
+        int all = 0;
+        for (int si = lane; si < a.nact; si += 32) all += tiles_of(si);
+        all = __reduce_add_sync(0xffffffffu, all);
+        planned = all * H >= kHWorthTiles * ctas && all >= kHItemTiles * a.nact;
+    }
+    if (SHARED && warp == kHWarps + kHProducers && !planned) {
+        // (nothing to plan)
+    } else if (SHARED && warp == kHWarps + kHProducers) {
+        // ---- planner: lists what the producers issue.  First some items of the CTA's own, and while these are on their way
+        // works out the shares (lane x has CTAs x, x + 32, ...); where those are worth it the CTA's range of the pool comes next, from
+        // the end on, so that what another CTA waits for is there early, and then its other items ----
+        const int me = (int)blockIdx.x;
+        int n = 0;  // entries
+        auto entry = [&](int si, int h, int t0, int t1) {
+            return make_int4((si / a.nl) * a.L + a.layer_begin + si % a.nl, h << 8 | si, t0, t1);
+        };
+        auto item = [&](int i) { return entry(i / H, i % H, 0, tiles_of(i / H)); };  // (a refused one has no tiles)
+        auto publish = [&](int entries) {
             __threadfence_block();
-            *(volatile int *)&s_known = 1;
+            __syncwarp();
+            if (lane == 0) *(volatile int *)&s_listed = entries;
+        };
+        {
+            const int r = 1 + lane, t = r < rounds ? tiles_of((me + r * ctas) / H) : 0;
+            int before = t;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, before, o);
+                if (lane >= o) before += up;
+            }
+            const bool now = r < rounds && before - t < kHOwnFirst + rounds / 2;
+            if (now) s_list[lane] = item(me + r * ctas);
+            n = __popc(__ballot_sync(0xffffffffu, now));
+            publish(n);
         }
-    };
-    static_assert(kHWarps * 32 >= kHMaxGrid, "a consumer thread for every CTA");
-
-    if (warp >= kHWarps) {
+        const int first = 1 + n;  // (the producers begin with the first by themselves)
+        int all = 0, pool_tiles = 0, most = 0;
+        for (int si = lane; si < a.nact; si += 32) {
+            const int t = tiles_of(si);
+            all += t * H;
+            pool_tiles += t * (H - min(H, max(0, pool - si * H)));
+        }
+        all = __reduce_add_sync(0xffffffffu, all);
+        pool_tiles = __reduce_add_sync(0xffffffffu, pool_tiles);
+        const int mean = (all + ctas - 1) / ctas;
+        // (all of a lane's CTAs at once: each round is a chain of its own)
+        constexpr int K = kHMaxGrid / 32;
+        const int steps = ctas / H, steph = ctas - steps * H;
+        int own[K], dealt[K], si[K], h[K];  // tiles of a CTA's own items, and of all that it would be dealt
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int c = k * 32 + lane;
+            own[k] = dealt[k] = 0;
+            si[k] = c / H;
+            h[k] = c - si[k] * H;
+        }
+        for (int r = 0; r * ctas < nitems; ++r)
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const int c = k * 32 + lane;
+                if (k * 32 >= ctas) break;
+                const int t = c < ctas && c + r * ctas < nitems ? tiles_of(si[k]) : 0;
+                dealt[k] += t;
+                own[k] += r < rounds ? t : 0;
+                si[k] += steps;
+                h[k] += steph;
+                if (h[k] >= H) {
+                    h[k] -= H;
+                    ++si[k];
+                }
+            }
+        int before = 0;  // tiles that the CTAs before these 32 take from the pool
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int c = k * 32 + lane;
+            if (k * 32 >= ctas) break;
+            most = max(most, dealt[k]);
+            const int want = c < ctas ? max(0, mean - own[k]) : 0;
+            int incl = want;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += up;
+            }
+            if (c < ctas) s_start[c] = min(pool_tiles, before + incl - want);
+            before += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) s_start[ctas] = pool_tiles;
+        const bool share = __reduce_max_sync(0xffffffffu, most) > mean + kHUneven;
+        __syncwarp();
+        const int x0 = share ? s_start[me] : 0, x1 = share ? s_start[me + 1] : 0;
+        if (x0 < x1) {
+            if (lane == 0) {
+                int si = pool / H, h = pool - si * H, base = 0, t = tiles_of(si);  // a segment, its first head in the pool, that one's first tile
+                while (x1 > base + (H - h) * t) {
+                    base += (H - h) * t;
+                    h = 0;
+                    t = tiles_of(++si);
+                }
+                for (int x = x1; x > x0;) {
+                    while (x <= base) {
+                        t = tiles_of(--si);
+                        h = max(0, pool - si * H);
+                        base -= (H - h) * t;
+                    }
+                    const int hh = (x - 1 - base) / t, start = base + hh * t;
+                    s_list[n++] = entry(si, h + hh, max(x0, start) - start, x - start);
+                    x = start;
+                }
+            }
+            n = __shfl_sync(0xffffffffu, n, 0);
+        }
+        const int end = share ? rounds : (nitems - me + ctas - 1) / ctas;  // items of the CTA
+        for (int r = first + lane; r < end; r += 32) s_list[n + r - first] = item(me + r * ctas);
+        n += end - first;
+        for (int i = me + end * ctas; i < nitems; i += ctas)  // those of the pool that cannot take the step are in no range
+            if (s_len[i / H] < 0) {
+                if (lane == 0) s_list[n] = item(i);
+                ++n;
+            }
+        if (lane == 0) s_list[n] = make_int4(0, 0, 0, -1);
+        publish(n + 1);
+        // Then the item that other CTAs began and this one ends, if its range starts with one: its own part from the consumers,
+        // the others' from `parts`, the nearest first.
+        if (x0 < x1) {
+            int si = pool / H, h = pool - si * H, base = 0, t = tiles_of(si);
+            while (x0 >= base + (H - h) * t) {
+                base += (H - h) * t;
+                h = 0;
+                t = tiles_of(++si);
+            }
+            h += (x0 - base) / t;
+            const int start = x0 - (x0 - base) % t;
+            if (start < x0 && start + t <= x1) {
+                bool dead = false;
+                hbar_wait(own_bar, 0u, dead, &s_abort);
+                dead = __any_sync(0xffffffffu, dead);
+                const int c = lane % (D / 4) * 4;
+                float M = s_own[D], lsum = s_own[D + 1];
+                float4 acc = *reinterpret_cast<const float4 *>(s_own + c);
+                for (int b = me - 1;; --b) {
+                    if (s_start[b] < s_start[b + 1]) {
+                        if (!await_part(a.sent + b, a.token, dead ? 0u : kHSpinLimit)) dead = true;
+                        if (!dead) {
+                            const float *p = a.parts + (size_t)b * PSTRIDE;
+                            const float4 x = __ldcg(reinterpret_cast<const float4 *>(p + c));
+                            const float M2 = __ldcg(p + D), l2 = __ldcg(p + D + 1), Mn = fmaxf(M, M2);
+                            const float f1 = exp2f(M - Mn), f2 = exp2f(M2 - Mn);
+                            lsum = lsum * f1 + l2 * f2;
+                            acc.x = acc.x * f1 + x.x * f2;
+                            acc.y = acc.y * f1 + x.y * f2;
+                            acc.z = acc.z * f1 + x.z * f2;
+                            acc.w = acc.w * f1 + x.w * f2;
+                            M = Mn;
+                        }
+                        __syncwarp();
+                        if (lane == 0) retire_part(a.sent + b, a.token, !dead);
+                    }
+                    if (s_start[b] <= start) break;
+                }
+                if (dead) {
+                    if (lane == 0) raise_status(a.dev_status, 0, PKV_DEV_TIMEOUT);
+                } else if (lane < D / 4) {
+                    const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
+                    const float inv = 1.f / lsum;
+                    T *o = reinterpret_cast<T *>(a.out) + ((size_t)seg * H + h) * D + c;
+                    if constexpr (sizeof(T) == 4) {
+                        *reinterpret_cast<float4 *>(o) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+                    } else {
+                        __nv_bfloat162 y[2] = {__floats2bfloat162_rn(acc.x * inv, acc.y * inv), __floats2bfloat162_rn(acc.z * inv, acc.w * inv)};
+                        *reinterpret_cast<uint2 *>(o) = *reinterpret_cast<const uint2 *>(y);
+                    }
+                }
+            }
+        }
+    } else if (warp >= kHWarps) {
         // ---- producers: every one walks the CTA's whole tile stream and issues the tiles that are its own ----
         const int me = warp - kHWarps;
         if (lane == 0) {
@@ -322,126 +476,100 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             int uses[kHSlots];
 #pragma unroll
             for (int i = 0; i < kHSlots; ++i) uses[i] = 0;
-            // SHARED: first an item of the CTA's own (its first tiles are on their way to L2); then its share of the pool, from
-            // the end on, so that the item that the next CTA goes on with comes early and its part is there by the
-            // time that CTA is done; then its other items.
-            int it = blockIdx.x, x0 = 0, x1 = 0;   // next item; tiles of the pool still to come
-            int ps = 0, ph = 0, base = 0, pt = 0;  // place in the pool: segment, its first head there, that one's first tile,
-            bool known = !SHARED;                  // and tiles of a head
-            for (; (SHARED || it < nitems) && !dead; it += SHARED ? 0 : gridDim.x) {
-                int si, h, t0 = 0, t1 = -1, start = 0;
-                if (SHARED && (it != (int)blockIdx.x || rounds == 0) && !known) {
-                    known = true;
-                    for (uint32_t i = 0; *(volatile int *)&s_known == 0 && i < kHSpinLimit && *(volatile int *)&s_abort == 0; ++i) {}
-                    __threadfence_block();
-                    if (*(volatile int *)&s_known == 0) {
-                        dead = true;
-                        atomicExch(&s_abort, 1);
-                        break;
+            auto walk = [&](auto by_list) {
+                constexpr bool LIST = decltype(by_list)::value;
+                int listed = 0, entries = 0;  // (LIST) entries read; known to be there
+                for (int it = blockIdx.x; (LIST || it < nitems) && !dead; it += gridDim.x) {
+                    int si, h, seg, t0 = 0, t1 = -1;
+                    if (LIST && it != (int)blockIdx.x) {
+                        if (listed >= entries) {
+                            for (uint32_t i = 0; i < kHSpinLimit && listed >= entries && *(volatile int *)&s_abort == 0; ++i)
+                                entries = *(volatile int *)&s_listed;
+                            __threadfence_block();
+                            if (listed >= entries) {
+                                dead = true;
+                                atomicExch(&s_abort, 1);
+                                break;
+                            }
+                        }
+                        const int4 e = s_list[listed++];
+                        if (e.w < 0) break;
+                        seg = e.x;
+                        si = e.y & 255;
+                        h = e.y >> 8;
+                        t0 = e.z;
+                        t1 = e.w;
+                    } else {
+                        si = it / H;
+                        h = it - si * H;
+                        seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
                     }
-                    x0 = s_start[blockIdx.x];
-                    x1 = s_start[blockIdx.x + 1];
-                    ps = pool / H;
-                    ph = pool - ps * H;
-                    if (x0 < x1) {
-                        pt = tiles_of(ps);
-                        while (x1 > base + (H - ph) * pt) {
-                            base += (H - ph) * pt;
-                            ph = 0;
-                            pt = tiles_of(++ps);
+                    const int ln = s_len[si];
+                    if (ln < 0) {
+                        // the segment cannot take the step: reported once, this head's output is zero
+                        if (me == 0) {
+                            if (h == 0) raise_status(a.dev_status, si / a.nl, PKV_DEV_CAPACITY);
+                            uint4 *o = reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.out) + ((size_t)seg * H + h) * SLICE);
+                            for (int x = 0; x < LPR; ++x) o[x] = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                        continue;
+                    }
+                    const int64_t off = s_off[si];
+                    const int item_tiles = (ln + TILE_ROWS - 1) / TILE_ROWS;
+                    if (!LIST || t1 < 0) t1 = item_tiles;
+                    const int tiles = LIST ? t1 - t0 : item_tiles;  // of the CTA's piece
+                    const int first_warp = g % kHWarps;
+                    const int slot = item_seq % kHSlots;
+                    int slot_parity = 0;
+                    if (tiles > 1) {
+                        // the slot's previous item must have been merged before its partials are overwritten
+                        // (every producer waits at every use of a slot, so that none can miss a phase)
+                        if (uses[slot] > 0) hbar_wait(slot_empty + slot, (uint32_t)(uses[slot] - 1) & 1u, dead, &s_abort);
+                        if (dead) break;
+                        slot_parity = uses[slot] & 1;  // the phase of the slot's barrier this item completes
+                        ++uses[slot];
+                    }
+                    for (int t = t0; t < t1 && !dead; ++t, ++g) {
+                        if (g % kHProducers != me) continue;
+                        const int st = g % kHStages;
+                        hbar_wait(empty + st, ((uint32_t)(g / kHStages) & 1u) ^ 1u, dead, &s_abort);
+                        if (dead) break;
+                        unsigned char *sb = stages + (size_t)st * STAGE;
+                        TileMeta *m = reinterpret_cast<TileMeta *>(sb);
+                        const bool last = t == item_tiles - 1;
+                        m->item = item_seq;
+                        m->seg = seg;
+                        m->h = h;
+                        const int nrows = min(TILE_ROWS, ln - t * TILE_ROWS);
+                        const int quarters = (nrows + TILE_ROWS / kHHeights - 1) / (TILE_ROWS / kHHeights);  // box height, in steps
+                        m->nrows = nrows;
+                        m->flags = (last && append ? kFlagNew : 0) | ((LIST ? t == t1 - 1 : last) ? kFlagItemLast : 0) |
+                                   (t + kHWarps >= t1 ? kFlagWarpLast : 0);
+                        if (LIST) m->flags |= (t0 > 0 ? kFlagBegun : 0) | (t1 < item_tiles ? kFlagGoesOn : 0);
+                        m->tiles = tiles;
+                        m->first_warp = first_warp;
+                        m->slot_parity = slot_parity;
+                        m->new_row = off + ln;
+                        m->sc = s_scale[si];
+                        const uint32_t bytes = 2 * (uint32_t)quarters * (kHTile / kHHeights) + SLICE + (last && append ? 2 * SLICE : 0u);
+                        hbar_expect_tx(full + st, bytes);
+                        const size_t hoff = ((size_t)seg * H + h) * SLICE;
+                        // rows past the segment's length (fetched up to the box's height, zero-filled past the
+                        // cache, or left in the stage by its previous tile) are masked by nrows
+                        const int row0 = (int)(off + (int64_t)t * TILE_ROWS);
+                        tma_load_2d(sb + HEAD, &maps.k[quarters - 1], full + st, h * D, row0);
+                        tma_load_2d(sb + HEAD + kHTile, &maps.v[quarters - 1], full + st, h * D, row0);
+                        hbulk_load(sb + 64, reinterpret_cast<const unsigned char *>(a.q) + hoff, SLICE, full + st);
+                        if (last && append) {
+                            hbulk_load(sb + 64 + SLICE, reinterpret_cast<const unsigned char *>(a.k_new) + hoff, SLICE, full + st);
+                            hbulk_load(sb + 64 + 2 * SLICE, reinterpret_cast<const unsigned char *>(a.v_new) + hoff, SLICE, full + st);
                         }
                     }
+                    ++item_seq;
                 }
-                if (SHARED && x0 < x1) {
-                    while (x1 <= base) {
-                        pt = tiles_of(--ps);
-                        ph = max(0, pool - ps * H);
-                        base -= (H - ph) * pt;
-                    }
-                    const int hh = (x1 - 1 - base) / pt;
-                    start = base + hh * pt;
-                    si = ps;
-                    h = ph + hh;
-                    t1 = x1 - start;
-                    x1 = max(x0, start);
-                    t0 = x1 - start;
-                } else {
-                    if (SHARED && it >= nitems) break;
-                    si = it / H;
-                    h = it - si * H;
-                    if (SHARED) {
-                        it += gridDim.x;
-                        // (items of the pool have been shared out; those that cannot take the step are in no share)
-                        if (it - (int)gridDim.x >= pool && s_len[si] >= 0) continue;
-                    }
-                }
-                const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
-                const int ln = s_len[si];
-                if (ln < 0) {
-                    // the segment cannot take the step: reported once, this head's output is zero
-                    if (me == 0) {
-                        if (h == 0) raise_status(a.dev_status, si / a.nl, PKV_DEV_CAPACITY);
-                        uint4 *o = reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.out) + ((size_t)seg * H + h) * SLICE);
-                        for (int x = 0; x < LPR; ++x) o[x] = make_uint4(0u, 0u, 0u, 0u);
-                    }
-                    continue;
-                }
-                const int64_t off = s_off[si];
-                const int item_tiles = (ln + TILE_ROWS - 1) / TILE_ROWS;
-                if (!SHARED || t1 < 0) t1 = item_tiles;
-                const int tiles = SHARED ? t1 - t0 : item_tiles;  // of the CTA's piece
-                const int first_warp = g % kHWarps;
-                const int slot = item_seq % kHSlots;
-                int slot_parity = 0;
-                if (tiles > 1) {
-                    // the slot's previous item must have been merged before its partials are overwritten
-                    // (every producer waits at every use of a slot, so that none can miss a phase)
-                    if (uses[slot] > 0) hbar_wait(slot_empty + slot, (uint32_t)(uses[slot] - 1) & 1u, dead, &s_abort);
-                    if (dead) break;
-                    slot_parity = uses[slot] & 1;  // the phase of the slot's barrier this item completes
-                    ++uses[slot];
-                }
-                for (int t = t0; t < t1 && !dead; ++t, ++g) {
-                    if (g % kHProducers != me) continue;
-                    const int st = g % kHStages;
-                    hbar_wait(empty + st, ((uint32_t)(g / kHStages) & 1u) ^ 1u, dead, &s_abort);
-                    if (dead) break;
-                    unsigned char *sb = stages + (size_t)st * STAGE;
-                    TileMeta *m = reinterpret_cast<TileMeta *>(sb);
-                    const bool last = t == item_tiles - 1;
-                    m->item = item_seq;
-                    m->seg = seg;
-                    m->h = h;
-                    const int nrows = min(TILE_ROWS, ln - t * TILE_ROWS);
-                    const int quarters = (nrows + TILE_ROWS / kHHeights - 1) / (TILE_ROWS / kHHeights);  // box height, in steps
-                    m->nrows = nrows;
-                    m->flags = (last && append ? kFlagNew : 0) | ((SHARED ? t == t1 - 1 : last) ? kFlagItemLast : 0) |
-                               (t + kHWarps >= t1 ? kFlagWarpLast : 0);
-                    if (SHARED) {
-                        m->flags |= (t0 > 0 ? kFlagBegun : 0) | (t1 < item_tiles ? kFlagGoesOn : 0);
-                        m->start = start;
-                    }
-                    m->tiles = tiles;
-                    m->first_warp = first_warp;
-                    m->slot_parity = slot_parity;
-                    m->new_row = off + ln;
-                    m->sc = s_scale[si];
-                    const uint32_t bytes = 2 * (uint32_t)quarters * (kHTile / kHHeights) + SLICE + (last && append ? 2 * SLICE : 0u);
-                    hbar_expect_tx(full + st, bytes);
-                    const size_t hoff = ((size_t)seg * H + h) * SLICE;
-                    // rows past the segment's length (fetched up to the box's height, zero-filled past the
-                    // cache, or left in the stage by its previous tile) are masked by nrows
-                    const int row0 = (int)(off + (int64_t)t * TILE_ROWS);
-                    tma_load_2d(sb + HEAD, &maps.k[quarters - 1], full + st, h * D, row0);
-                    tma_load_2d(sb + HEAD + kHTile, &maps.v[quarters - 1], full + st, h * D, row0);
-                    hbulk_load(sb + 64, reinterpret_cast<const unsigned char *>(a.q) + hoff, SLICE, full + st);
-                    if (last && append) {
-                        hbulk_load(sb + 64 + SLICE, reinterpret_cast<const unsigned char *>(a.k_new) + hoff, SLICE, full + st);
-                        hbulk_load(sb + 64 + 2 * SLICE, reinterpret_cast<const unsigned char *>(a.v_new) + hoff, SLICE, full + st);
-                    }
-                }
-                ++item_seq;
-            }
+            };
+            if (planned) walk(std::true_type());
+            else walk(std::false_type());
             // one closing tile per consumer warp
             const int g_end = g;
             for (int e = 0; e < kHWarps && !dead; ++e, ++g) {
@@ -466,79 +594,9 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
         // ---- consumers: warp w takes tiles w, w + kHWarps, ... of the CTA's stream, all through stage w ----
         const int grp = lane / LPR, c = lane % LPR;
         bool dead = false;
-        if (SHARED) share_out();
         float M = -INFINITY, lsum = 0.f, acc[VE];
 #pragma unroll
         for (int i = 0; i < VE; ++i) acc[i] = 0.f;
-        // Adds another part of the item to the state.
-        auto join = [&](float M2, float l2, const float4 *x) {
-            const float Mn2 = fmaxf(M, M2);
-            const float f1 = exp2f(M - Mn2), f2 = exp2f(M2 - Mn2);
-            lsum = lsum * f1 + l2 * f2;
-#pragma unroll
-            for (int i = 0; i < VE; i += 4) {
-                const float4 y = x[i / 4];
-                acc[i] = acc[i] * f1 + y.x * f2;
-                acc[i + 1] = acc[i + 1] * f1 + y.y * f2;
-                acc[i + 2] = acc[i + 2] * f1 + y.z * f2;
-                acc[i + 3] = acc[i + 3] * f1 + y.w * f2;
-            }
-            M = Mn2;
-        };
-        auto write_out = [&](int seg, int h) {
-            if (grp == 0) {
-                const float inv = 1.f / lsum;
-                float x[VE];
-#pragma unroll
-                for (int i = 0; i < VE; ++i) x[i] = acc[i] * inv;
-                *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.out) + ((size_t)seg * H + h) * SLICE + c * 16) =
-                    RowVec<T>::pack(x);
-            }
-        };
-        auto leave = [&](float *p) {  // the state, for another warp to join
-            if (grp == 0) {
-#pragma unroll
-                for (int i = 0; i < VE; i += 4)
-                    *reinterpret_cast<float4 *>(p + c * VE + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
-                if (c == 0) {
-                    p[D] = M;
-                    p[D + 1] = lsum;
-                }
-            }
-            __syncwarp();
-        };
-        // The parts of an item that begins at tile `start` of the pool, from the CTAs before this one, the nearest first: when
-        // all are there (`last`: all that come within the limit).  False when one is still to come.
-        auto collect = [&](int start, bool last) {
-            for (int b = (int)blockIdx.x - 1;; --b) {
-                if (s_start[b] < s_start[b + 1]) {
-                    unsigned long long v = load_flag(a.sent + b);
-                    for (uint32_t i = 0; last && v != a.token && i < kHSpinLimit; ++i) v = load_flag(a.sent + b);
-                    if (!__all_sync(0xffffffffu, v == a.token)) {
-                        if (!last) return false;
-                        dead = true;
-                    }
-                }
-                if (s_start[b] <= start) break;
-            }
-            asm volatile("fence.acq_rel.gpu;" ::: "memory");
-            for (int b = (int)blockIdx.x - 1;; --b) {
-                if (s_start[b] < s_start[b + 1]) {
-                    if (!dead) {
-                        const float *p = a.parts + (size_t)b * PSTRIDE;
-                        float4 x[VE / 4];
-#pragma unroll
-                        for (int i = 0; i < VE / 4; ++i) x[i] = __ldcg(reinterpret_cast<const float4 *>(p + c * VE) + i);
-                        join(__ldcg(p + D), __ldcg(p + D + 1), x);
-                    }
-                    // back to zero; one that has not come gets it from its own CTA
-                    if (lane == 0 && (!dead || atomicExch(a.sent + b, a.token ^ kGone) == a.token)) lower_flag(a.sent + b);
-                }
-                if (s_start[b] <= start) break;
-            }
-            return true;
-        };
-        int late_seg = -1, late_h = 0, late_start = 0;  // an item of this warp whose other parts are still to come
         unsigned long long sent_held = 0;
         for (int g = warp;; g += kHWarps) {
             const int st = g % kHStages;
@@ -687,30 +745,36 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
                     __syncwarp();
                     if (lane == 0) hbar_arrive(slot_empty + slot);
                 }
-                if (SHARED && (m.flags & kFlagGoesOn)) {
-                    leave(a.parts + (size_t)blockIdx.x * PSTRIDE);
-                    if (lane == 0) sent_held = raise_flag(a.sent + blockIdx.x, a.token);
-                } else if (SHARED && (m.flags & kFlagBegun) && !collect(m.start, false)) {
-                    leave(s_own);
-                    late_seg = m.seg;
-                    late_h = m.h;
-                    late_start = m.start;
-                } else {
-                    write_out(m.seg, m.h);
+                if (SHARED && (m.flags & (kFlagGoesOn | kFlagBegun))) {
+                    // (an item cut by the CTA's range: the part goes to the next CTA, or waits for those of the CTAs before)
+                    float *p = m.flags & kFlagGoesOn ? a.parts + (size_t)blockIdx.x * PSTRIDE : s_own;
+                    if (grp == 0) {
+#pragma unroll
+                        for (int i = 0; i < VE; i += 4)
+                            *reinterpret_cast<float4 *>(p + c * VE + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
+                        if (c == 0) {
+                            p[D] = M;
+                            p[D + 1] = lsum;
+                        }
+                    }
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (m.flags & kFlagGoesOn) sent_held = raise_flag(a.sent + blockIdx.x, a.token);
+                        else hbar_arrive(own_bar);
+                    }
+                } else if (grp == 0) {
+                    const float inv = 1.f / lsum;
+                    float x[VE];
+#pragma unroll
+                    for (int i = 0; i < VE; ++i) x[i] = acc[i] * inv;
+                    *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(a.out) + ((size_t)m.seg * H + m.h) * SLICE + c * 16) =
+                        RowVec<T>::pack(x);
                 }
             }
             M = -INFINITY;
             lsum = 0.f;
 #pragma unroll
             for (int i = 0; i < VE; ++i) acc[i] = 0.f;
-        }
-        if (SHARED && late_seg >= 0 && !dead) {
-            float4 x[VE / 4];
-#pragma unroll
-            for (int i = 0; i < VE / 4; ++i) x[i] = reinterpret_cast<const float4 *>(s_own + c * VE)[i];
-            join(s_own[D], s_own[D + 1], x);
-            collect(late_start, true);
-            write_out(late_seg, late_h);
         }
         if (SHARED && lane == 0) unraise_flag(a.sent + blockIdx.x, a.token, sent_held);
         if (dead && lane == 0) raise_status(a.dev_status, 0, PKV_DEV_TIMEOUT);
@@ -769,6 +833,46 @@ bool make_cache_map(CUtensorMap *map, void *ptr, const pkv_shape *s, int64_t row
 
 constexpr int kHMaxSmem = 224 * 1024;  // dynamic; there are up to 1.7 KiB of static variables beside it
 
+// The wait for parts that CTAs pass on, in isolation: some are there, one does not come in time, others are given up after it; flags
+// of parts that were there are zero then, late ones get zero from their own CTAs, and a second run with the same token is whole.
+__global__ void selftest_parts_kernel(int32_t *dev_status, uint32_t limit)
+{
+    constexpr int n = 8;
+    __shared__ unsigned long long flags[n];
+    const unsigned long long token = 0x9e3779b97f4a7c15ull;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool late = lane == 5 || lane == 6;
+    if (threadIdx.x < n) flags[threadIdx.x] = threadIdx.x % 3 ? 0ull : ~(unsigned long long)threadIdx.x;
+    __syncthreads();
+    bool ok = true;
+    for (int run = 0; run < 2; ++run) {
+        unsigned long long held = 0;
+        if (warp == 1 && lane < n && !(run == 0 && late)) held = raise_flag(flags + lane, token);
+        __syncthreads();
+        if (warp == 0) {
+            bool dead = false;
+            for (int b = 0; b < n; ++b) {
+                if (!await_part(flags + b, token, dead ? 0u : limit)) dead = true;
+                __syncwarp();
+                if (lane == 0) retire_part(flags + b, token, !dead);
+            }
+            ok = ok && dead == (run == 0);
+        }
+        __syncthreads();
+        if (warp == 1 && lane < n) {
+            ok = ok && flags[lane] == (run == 0 && late ? token ^ kGone : 0ull);
+            if (run == 0 && late) held = raise_flag(flags + lane, token);
+            ok = unraise_flag(flags + lane, token, held) == (run == 0 && late) && ok;
+            ok = ok && *(volatile unsigned long long *)(flags + lane) == 0ull;
+        }
+        __syncthreads();
+    }
+    if (__syncthreads_and(ok) && threadIdx.x == 0) raise_status(dev_status, 0, PKV_DEV_TIMEOUT);
+}
+
+// Entries that a CTA's list may need: its own items, all of the pool, and the end.
+int list_entries(const HeadArgs &a, int grid) { return a.nact * a.H / grid + (a.pool_rounds + 1) * grid + 2; }
+
 template <typename T, int D, bool SHARED>
 int launch_heads(const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t st)
 {
@@ -776,11 +880,12 @@ int launch_heads(const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t
     constexpr uint32_t SLICE = D * sizeof(T);
     constexpr uint32_t HEAD = (64 + 3 * SLICE + 127) / 128 * 128;
     const size_t smem = (size_t)kHStages * (HEAD + 2 * kHTile) + (size_t)kHSlots * kHWarps * (D + 4) * sizeof(float) +
-                        (2 * kHStages + 2 * kHSlots) * sizeof(uint64_t) + (size_t)a.nact * (sizeof(int64_t) + 2 * sizeof(int));
+                        (2 * kHStages + 2 * kHSlots) * sizeof(uint64_t) + (size_t)a.nact * (sizeof(int64_t) + 2 * sizeof(int)) +
+                        (SHARED ? (size_t)list_entries(a, grid) * sizeof(int4) : 0);
     int rc = ensure_dynamic_smem((const void *)decode_heads_kernel<T, D, SHARED>, kHMaxSmem, done);
     if (rc != PKV_OK) return rc;
     if (smem > kHMaxSmem) return -1;
-    cudaError_t e = launch_dependent(decode_heads_kernel<T, D, SHARED>, dim3(grid), dim3((kHWarps + kHProducers) * 32), smem, st, maps, a);
+    cudaError_t e = launch_dependent(decode_heads_kernel<T, D, SHARED>, dim3(grid), dim3((kHWarps + kHProducers + SHARED) * 32), smem, st, maps, a);
     if (e != cudaSuccess) {
         set_cuda_error(e, "decode_heads_kernel");
         return PKV_ERR_CUDA;
@@ -790,11 +895,20 @@ int launch_heads(const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t
 
 template <typename T> int launch_heads(int D, bool shared, const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t st)
 {
-    if (D == 128) return shared ? launch_heads<T, 128, true>(maps, a, grid, st) : launch_heads<T, 128, false>(maps, a, grid, st);
-    return shared ? launch_heads<T, 64, true>(maps, a, grid, st) : launch_heads<T, 64, false>(maps, a, grid, st);
+    if (shared) {  // (-1: its list does not fit)
+        const int rc = D == 128 ? launch_heads<T, 128, true>(maps, a, grid, st) : launch_heads<T, 64, true>(maps, a, grid, st);
+        if (rc != -1) return rc;
+    }
+    return D == 128 ? launch_heads<T, 128, false>(maps, a, grid, st) : launch_heads<T, 64, false>(maps, a, grid, st);
 }
 
 }  // namespace
+
+int selftest_wait_parts(int32_t *dev_status, cudaStream_t st)
+{
+    selftest_parts_kernel<<<1, 64, 0, st>>>(dev_status, 4096u);
+    return check_launch("selftest_parts_kernel");
+}
 
 // Flags of either kind, and a part of an item for every CTA.
 size_t decode_heads_ws_bytes() { return round_up((size_t)kHMaxGrid * (2 * sizeof(unsigned long long) + (128 + 4) * sizeof(float)), kWsAlign); }
@@ -876,14 +990,14 @@ int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const v
     a.total_cap_rows = c->total_cap_rows;
     const int items = nact * H;
     const int grid = items < sms ? items : sms;
-    // Segments of some hundred rows differ in length and an item is a good part of a CTA's work: CTAs' sums of tiles
-    // made alike.  It costs 2 us a call, the shares' arithmetic and the parts that pass through global memory:
-    // 32 x 32 heads, 128 rows 19.3 us a call without / 23.0 with; 256 31.5 / 31.5 (and caches are mostly below their
-    // capacity); 300 37.5 / 36.0 (two rounds shared
-    // out 38.8); 40 x 40 heads, 500 rows 77 / 77 (74); 800 rows of 32 x 32 heads 87 / 82 (77); 4 x 32 x 32 heads of 819 rows 296
-    // / 284 (279); fp32, 16 x 40 heads of 600 rows 81 / 67 (66).
-    // With many rounds of items the sums are alike without it: 80 x 40 heads (21 rounds) of 361 rows 105 / 108, of 604 171 / 162.
-    const bool shared = seg_rows >= kHSharedAlways || (seg_rows >= kHSharedRows && items <= 12 * sms);
+    // Segments of some hundred rows differ in length, and an item is a good part of a CTA's work: CTAs' sums of tiles made alike.
+    // What that gives is up to the lengths, which the kernel sees; for a call that may gain, this form costs up to 0.5 us (two calls
+    // and a copy, us, dealt / here; lengths lognormal with sigma 0.5, then all alike, then a tenth of the capacity):
+    // 32 x 32 heads, 400 rows of capacity 57.4 / 55.3, 71.3 / 73.4; 512 rows 60.3 / 57.2, 52.0 / 53.6, 22.6 / 23.4; 800 rows 100.6 / 90.2,
+    // 127.2 / 128.7; 1000 rows 121.3 / 107.9, 155.7 / 157.4; fp32, 16 x 40 heads, 600 rows 90.6 / 85.3, 124.9 / 124.2.  More rounds
+    // of items are more alike by themselves: 4 x 32 x 32 heads (28 rounds) of 520 rows 346 / 325, 318 / 327, 6 x 40 x 40
+    // (65) 755 / 767, 742 / 765, 250 x 30 heads of 64 (51) 205 / 203, 304 / 315: dealt there.
+    const bool shared = seg_rows >= kHSharedRowsMany ? items <= kHManyRounds * sms : seg_rows >= kHSharedRows && items <= kHFewRounds * sms;
     a.pool_rounds = seg_rows >= kHTwoRoundsRows ? 2 : 1;
     return s->dtype == PKV_BF16 ? launch_heads<__nv_bfloat16>(D, shared, maps, a, grid, st) : launch_heads<float>(D, shared, maps, a, grid, st);
 }

@@ -180,4 +180,20 @@ __device__ __forceinline__ bool settle_flags(unsigned long long *flags, int n, u
     return all_in;
 }
 
+// ---- parts of an item that CTAs pass on: a flag of the same kind for each, which the CTA that takes the parts puts back ----
+// A whole warp: waits for a part; false when the limit ran out.
+__device__ __forceinline__ bool await_part(const unsigned long long *flag, unsigned long long token, uint32_t limit)
+{
+    unsigned long long v = load_flag(flag);
+    for (uint32_t i = 0; v != token && i < limit; ++i) v = load_flag(flag);
+    const bool came = __all_sync(0xffffffffu, v == token);
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    return came;
+}
+// One thread, after the part has been read or given up: the flag is zero again, or will be when a late part comes.
+__device__ __forceinline__ void retire_part(unsigned long long *flag, unsigned long long token, bool came)
+{
+    if (came || atomicExch(flag, token ^ kGone) == token) lower_flag(flag);
+}
+
 }  // namespace pkv

@@ -1,5 +1,6 @@
-"""Decode calls of long segments, whose tiles the per-head kernel shares out evenly over the CTAs (needs a B200): an item
-may be begun by one CTA, gone on with by others and ended by another."""
+"""Decode calls of long segments, whose tiles the per-head kernel shares out evenly over the CTAs where they are uneven (needs
+a B200): an item may be begun by one CTA, gone on with by others and ended by another.  Calls of 300 rows of capacity
+(test_shared_tiles) have the same lengths and edges in the form that deals items out."""
 import numpy as np
 import pytest
 import torch
@@ -15,7 +16,6 @@ def ready(L, H, D, lens, dtype, T, seed=5):
     from paper_2412_03409_b200.session import Session
     N = max(lens)
     g = torch.Generator(device="cuda").manual_seed(seed)
-    # (the mean capacity, 300 rows and more, is what sends the call to the shared form)
     s = Session(1, L, H, D, N, dtype, np.full(L, D ** -0.5, np.float32), decode_cap=T, max_budget_rows=max(sum(lens), 300 * L), poison=True)
     s.apply_lengths(torch.tensor(lens, dtype=torch.int32), scores=torch.rand(1, L, N, device="cuda", generator=g))
     k, v = (torch.randn(1, L, H, N, D, device="cuda", generator=g).to(dtype) for _ in range(2))
@@ -84,3 +84,130 @@ def test_shared_tiles(L, H, kind, D, dtype):
     got = a.decode(tok[0][0], None, None)
     assert torch.equal(a.cache.len, want)
     assert float((got.double() - reference(a, tok[0][0], D)).abs().max()) <= TOL[dtype]
+
+
+def test_a_wait_for_parts_that_runs_out():
+    """Parts that come late, or were given up, leave nothing that a replay with the same token could mistake for its own."""
+    from paper_2412_03409_b200 import api
+    status = torch.zeros(2, dtype=torch.int32, device="cuda")
+    api.prefixkv_selftest_bounded_wait(4, status)
+    torch.cuda.synchronize()
+    assert status.cpu().tolist() == [api.DEV_TIMEOUT, 0]
+
+
+SMS = 148
+
+
+def uneven(B, L, H, lens, tile, rows):
+    """Whether the kernel shares the tiles out, as its rule has it: enough tiles for a CTA and in an item, CTAs' sums unlike."""
+    items = np.repeat([(n + tile - 1) // tile for n in lens], H)
+    rounds = len(items) / SMS
+    if rounds < 4 or not (rounds <= 40 if rows >= 512 else rows >= 384 and rounds <= 12):
+        return False
+    sums = np.zeros(SMS, int)
+    for i, t in enumerate(items):
+        sums[i % SMS] += t
+    mean = -(-items.sum() // SMS)
+    return items.sum() >= 40 * SMS and items.sum() >= 6 * len(items) and sums.max() > mean + 15
+
+
+def unlike(kind, n, rows, tile):
+    rng = np.random.default_rng(n * rows)
+    if kind == "unlike":
+        x = rng.lognormal(0, 0.7, n)
+        return [int(v) for v in np.maximum(1, x / x.mean() * 0.8 * rows)]
+    if kind == "edges":      # whole tiles, a row more, a row less; a few rows
+        m = max(1, rows // tile)
+        return [int(v) for v in rng.choice([1, tile, m * tile, m * tile - 1, m // 2 * tile + 1], n)]
+    if kind == "even":
+        return [int(0.9 * rows)] * n
+    if kind == "short":
+        return [int(v) for v in rng.integers(1, 3 * tile, n)]
+    long = rows * n // 3     # (one in a hundred holds a third of all rows)
+    at = n - 1 if kind == "long last" else 0
+    return [long if i == at else rows // 2 for i in range(n)]
+
+
+@pytest.mark.parametrize("B,L,H,lb,le,rows,kind", [
+    (1, 37, 16, 0, 37, 400, "unlike"), (1, 19, 32, 0, 19, 384, "edges"), (1, 19, 32, 0, 19, 399, "unlike"), (1, 19, 32, 0, 19, 401, "unlike"),
+    (1, 75, 8, 0, 75, 511, "unlike"), (1, 75, 8, 0, 75, 512, "edges"), (1, 20, 40, 0, 20, 1024, "unlike"), (2, 20, 16, 0, 20, 600, "edges"),
+    (1, 60, 16, 10, 50, 450, "unlike"), (2, 40, 16, 20, 40, 800, "unlike"), (4, 32, 20, 0, 32, 520, "unlike"), (1, 250, 20, 0, 250, 512, "unlike"),
+    (1, 40, 16, 0, 40, 420, "long last"), (1, 40, 16, 0, 40, 800, "long first"), (1, 20, 40, 0, 20, 800, "even"), (1, 40, 16, 0, 40, 700, "short")])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_uneven_segments(B, L, H, lb, le, rows, kind, D, dtype):
+    """One round of items in the pool and two, batches, ranges of layers; refused segments, appended rows, and a captured call
+    replayed over a stale workspace."""
+    from paper_2412_03409_b200 import api
+    from paper_2412_03409_b200.session import Session
+    T, tile, n = 3, TILE[dtype, D], B * (le - lb)
+    lens = unlike(kind, n, rows, tile)
+    if tile < 64 and kind in ("unlike", "long last", "long first"):   # (of 64 rows there are too few for a CTA in the shorter ones)
+        assert uneven(B, L, H, lens, tile, rows)
+    elif kind == "short":
+        assert not uneven(B, L, H, lens, tile, rows)
+    full = np.ones((B, L), np.int64)
+    full[:, lb:le] = np.reshape(lens, (B, le - lb))
+    full = full.reshape(-1)
+    N = max(max(lens), rows)
+    assert int(full.sum()) <= B * L * (rows - T)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    both = []
+    for _ in range(2):
+        s = Session(B, L, H, D, N, dtype, np.full(L, D ** -0.5, np.float32), decode_cap=T, max_budget_rows=L * (rows - T))
+        both.append(s)
+        assert s.cache.total_cap_rows // (B * L) == rows
+        off = np.concatenate([[0], np.cumsum(full + T)])
+        s.cache.row_offset.copy_(torch.from_numpy(off))
+        s.cache.cap.copy_(torch.from_numpy((full + T).astype(np.int32)))
+        s.cache.len.copy_(torch.from_numpy(full.astype(np.int32)))
+    a, b = both
+    a.cache.k.normal_(generator=g)
+    a.cache.v.normal_(generator=g)
+    b.cache.k.copy_(a.cache.k)
+    b.cache.v.copy_(a.cache.v)
+    act = [x * L + l for x in range(B) for l in range(lb, le)]
+    refused = [act[n // 3], act[n - 2]]
+    before = a.cache.len.clone()
+    for s in both:
+        s.cache.len[refused] = 0
+        s.out.zero_()
+    tok = [[torch.randn(B, L, H, D, device="cuda", generator=g).to(dtype) for _ in range(3)] for _ in range(T)]
+    buf = [x.clone() for x in tok[0]]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        b.decode(*buf, layer_begin=lb, layer_end=le)
+    b.ws_decode.fill_(0xff)
+    steps = torch.zeros_like(before)
+    steps[act] = 1
+    steps[refused] = 0
+
+    def check(s, q, what):
+        m, o = s.cache.len.tolist(), s.cache.row_offset.tolist()
+        for i in act:
+            got = s.out[i // L, i % L].double()
+            if m[i] < 1:
+                assert (got == 0).all()
+                continue
+            k, v = (x[o[i]:o[i] + m[i]].double() for x in (s.cache.k, s.cache.v))
+            p = torch.softmax(torch.einsum("hd,rhd->hr", q[i // L, i % L].double(), k) * float(np.float32(D ** -0.5)), -1)
+            assert float((got - torch.einsum("hr,rhd->hd", p, v)).abs().max()) <= TOL[dtype], (what, i)
+
+    for t in range(T):
+        for x, y in zip(buf, tok[t]):
+            x.copy_(y)
+        a.decode(*tok[t], layer_begin=lb, layer_end=le)
+        graph.replay()
+        torch.cuda.synchronize()
+        want = torch.where(before > 0, before + (t + 1) * steps, before)
+        want[refused] = 0
+        assert torch.equal(a.cache.len, want) and torch.equal(b.cache.len, want)
+        for i in (act[0], act[-1]):
+            row = int(a.cache.row_offset[i]) + int(before[i]) + t
+            assert torch.equal(a.cache.k[row], tok[t][1][i // L, i % L]) and torch.equal(a.cache.v[row], tok[t][2][i // L, i % L])
+        check(a, tok[t][0], t)
+        assert torch.equal(a.out, b.out), t
+    assert a.status.max().item() == api.DEV_CAPACITY == b.status.max().item()
+    a.decode(tok[0][0], None, None, layer_begin=lb, layer_end=le)   # nothing appended
+    assert torch.equal(a.cache.len, want)
+    check(a, tok[0][0], "nothing appended")
