@@ -79,6 +79,7 @@ constexpr int kHProducers = 2;     // issuing threads (one per warp): stage s is
 static_assert(kHStages % kHProducers == 0, "a stage must keep its producer, which then sees each of its phases in turn");
 constexpr uint32_t kHSpinLimit = 1u << 22;
 constexpr float kLog2eH = 1.4426950408889634f;
+constexpr float kHNoMax = -0x1.fffffep127f;  // maximum of no rows: finite, so that its differences are numbers
 
 // (kFlagItemLast: the last tile of an item, or of the CTA's piece of one)
 enum { kFlagNew = 1, kFlagItemLast = 2, kFlagWarpLast = 4, kFlagEnd = 8, kFlagBegun = 16, kFlagGoesOn = 32 };
@@ -594,7 +595,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
         // ---- consumers: warp w takes tiles w, w + kHWarps, ... of the CTA's stream, all through stage w ----
         const int grp = lane / LPR, c = lane % LPR;
         bool dead = false;
-        float M = -INFINITY, lsum = 0.f, acc[VE];
+        float M = kHNoMax, lsum = 0.f, acc[VE];
 #pragma unroll
         for (int i = 0; i < VE; ++i) acc[i] = 0.f;
         unsigned long long sent_held = 0;
@@ -652,9 +653,9 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
             mx = fmaxf(mx, s[16]);
 #pragma unroll
             for (int o = LPR; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            // one rescale per tile (mx is finite: a tile has at least one row)
+            // one rescale per tile (mx is -infinity when infinite elements mask all of its rows: exponentials of 0)
             const float Mn = fmaxf(M, mx);
-            const float corr = exp2f(M - Mn);  // 0 for the first tile of an item (M = -inf)
+            const float corr = exp2f(M - Mn);  // 0 for the first tile of an item
             M = Mn;
             lsum *= corr;
 #pragma unroll
@@ -771,7 +772,7 @@ decode_heads_kernel(const __grid_constant__ HeadMaps maps, const HeadArgs a)
                         RowVec<T>::pack(x);
                 }
             }
-            M = -INFINITY;
+            M = kHNoMax;
             lsum = 0.f;
 #pragma unroll
             for (int i = 0; i < VE; ++i) acc[i] = 0.f;

@@ -211,3 +211,29 @@ def test_uneven_segments(B, L, H, lb, le, rows, kind, D, dtype):
     a.decode(tok[0][0], None, None, layer_begin=lb, layer_end=le)   # nothing appended
     assert torch.equal(a.cache.len, want)
     check(a, tok[0][0], "nothing appended")
+
+
+@pytest.mark.parametrize("rows,lo,hi", [(140, 0, 64), (140, 70, 139), (700, 0, 100), (700, 320, 480), (700, 600, 699), (900, 64, 800)])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_rows_masked_by_an_infinite_element(rows, lo, hi, D, dtype):
+    """Rows with logits of -infinity have no part in the output, wherever a CTA's tiles begin, whole tiles of them included."""
+    from paper_2412_03409_b200.session import Session
+    L, H, T = 20, 32, 1
+    rng = np.random.default_rng(rows + lo)
+    lens = [int(v) for v in np.minimum(rng.lognormal(0, 0.6, L) * rows, 1500)]
+    lens[3:6] = [rows] * 3
+    s = Session(1, L, H, D, max(lens), dtype, np.full(L, D ** -0.5, np.float32), decode_cap=T, max_budget_rows=sum(lens))
+    off = np.concatenate([[0], np.cumsum(np.array(lens) + T)])
+    s.cache.row_offset.copy_(torch.from_numpy(off))
+    s.cache.cap.copy_(torch.tensor([n + T for n in lens], dtype=torch.int32))
+    s.cache.len.copy_(torch.tensor(lens, dtype=torch.int32))
+    s.cache.k.normal_()
+    s.cache.v.normal_()
+    for l in range(L):
+        a, b = min(lo, lens[l] - 1), min(hi, lens[l] - 1)   # (a row is left)
+        s.cache.k[off[l] + a:off[l] + b, :, 0] = -float("inf")
+    q, kn, vn = (torch.randn(1, L, H, D, device="cuda").to(dtype) for _ in range(3))
+    q[..., 0] = q[..., 0].abs() + 1
+    got = s.decode(q, kn, vn)
+    assert float((got.double() - reference(s, q, D)).abs().max()) <= TOL[dtype]
