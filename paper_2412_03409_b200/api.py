@@ -119,11 +119,18 @@ def _stream():
     return _raw_stream(_raw_device())
 
 
+def _call_by_ctypes(shape, cache, q, k_new, v_new, layer_scale, layer_begin, layer_end, out, dev_status, ws):
+    return _lib.prefixkv_decode_attn(ctypes.byref(shape), ctypes.byref(cache), _ptr(q), _ptr(k_new), _ptr(v_new),
+                                     _ptr(layer_scale), int(layer_begin), int(layer_end), _ptr(out), _ptr(dev_status),
+                                     *_ws(ws), _stream())
+
+
 def _load_call():
     """The decode call's own binding: of all calls it alone is made per layer and token."""
     if not os.path.exists(_build.CALL_PATH):
-        raise ImportError("_decode_call.so is not built; run `python -m paper_2412_03409_b200.build`. "
-                          "There is no fallback path.")
+        if not _build.python_headers():    # (it cannot be built here)
+            return _call_by_ctypes
+        raise ImportError("%s is not built; run `python -m paper_2412_03409_b200.build`." % os.path.basename(_build.CALL_PATH))
     loader = importlib.machinery.ExtensionFileLoader("_decode_call", _build.CALL_PATH)
     mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_decode_call", loader))
     loader.exec_module(mod)

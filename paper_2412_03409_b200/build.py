@@ -11,7 +11,8 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 LIB_PATH = os.path.join(_HERE, "libprefixkv.so")
 CALL_SRC = os.path.join(_HERE, "csrc", "decode_call.c")
-CALL_PATH = os.path.join(_HERE, "_decode_call.so")
+# (for this interpreter: another one builds, and loads, its own)
+CALL_PATH = os.path.join(_HERE, "_decode_call" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 
 def _sources():
@@ -35,14 +36,26 @@ def is_stale() -> bool:
     return any(os.path.getmtime(f) > t for f in _sources() + _headers())
 
 
-def build_call(force: bool = False) -> str:
-    newest = max(os.path.getmtime(f) for f in (CALL_SRC, os.path.join(_ROOT, "include", "prefixkv.h")))
-    if force or not os.path.exists(CALL_PATH) or os.path.getmtime(CALL_PATH) < newest:
-        tmp = CALL_PATH + ".%d.tmp" % os.getpid()
-        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", os.path.join(_ROOT, "include"),
-                               "-I", sysconfig.get_paths()["include"], "-o", tmp, CALL_SRC])
-        os.replace(tmp, CALL_PATH)
-    return CALL_PATH
+def python_headers() -> bool:
+    return os.path.exists(os.path.join(sysconfig.get_paths()["include"], "Python.h"))
+
+
+def call_is_stale() -> bool:
+    if not os.path.exists(CALL_PATH):
+        return True
+    t = os.path.getmtime(CALL_PATH)
+    return any(os.path.getmtime(f) > t for f in (CALL_SRC, os.path.join(_ROOT, "include", "prefixkv.h"), os.path.abspath(__file__)))
+
+
+def build_call(force: bool = False) -> None:
+    if not force and not call_is_stale():
+        return
+    if not python_headers():
+        return    # (the decode call goes through ctypes then: the same library, some 2 us a call slower)
+    tmp = CALL_PATH + ".%d.tmp" % os.getpid()
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", os.path.join(_ROOT, "include"),
+                           "-I", sysconfig.get_paths()["include"], "-o", tmp, CALL_SRC])
+    os.replace(tmp, CALL_PATH)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:

@@ -75,3 +75,36 @@ def test_null_and_range_arguments_rejected_on_host(api):
     assert lib.prefixkv_score(sh, 16, odd, 16, odd, 16, None, 16, 256, 1 << 30, None) == \
         api.PKV_ERR_INVALID_ARG
     assert lib.prefixkv_gini(sh, None, None, None) == api.PKV_ERR_INVALID_ARG
+
+
+def test_the_decode_binding_is_this_interpreters(api, monkeypatch, tmp_path):
+    """It carries the interpreter's suffix, is built again when what it is built from or with changes, and where there is no
+    Python.h to build it with the call goes through ctypes."""
+    import sysconfig
+
+    import torch
+
+    from paper_2412_03409_b200 import build
+    assert build.CALL_PATH.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and not build.call_is_stale()
+    copy = tmp_path / os.path.basename(build.CALL_PATH)
+    copy.write_bytes(open(build.CALL_PATH, "rb").read())
+    monkeypatch.setattr(build, "CALL_PATH", str(copy))
+    for src in (build.CALL_SRC, build.__file__):
+        t = os.path.getmtime(src)
+        os.utime(copy, (t + 1e6, t + 1e6))
+        assert not build.call_is_stale()
+        os.utime(copy, (t - 1, t - 1))
+        assert build.call_is_stale()
+    os.unlink(copy)
+    with pytest.raises(ImportError):
+        api._load_call()
+    monkeypatch.setattr(build, "python_headers", lambda: False)
+    build.build_call()
+    by_ctypes = api._load_call()
+    assert not copy.exists()
+    sh = api.make_shape(1, 2, 4, 64, 32, torch.float32)
+    cache = api.CacheStruct(None, None, None, None, None, 10, 1, 0, None, None, None)
+    monkeypatch.setattr(api, "_stream", lambda: None)
+    for call in (api._decode_attn, by_ctypes):
+        if call is by_ctypes or torch.cuda.is_available():
+            assert call(sh, cache, None, None, None, None, 0, 2, None, None, None) == api.PKV_ERR_INVALID_ARG
