@@ -68,7 +68,7 @@ constexpr int kHMaxGrid = 256;
 // Sharing out (the measurements stand at launch_decode_heads): mean capacity of a segment from which a call may take that form,
 // with few rounds of items and with some more, and from which two rounds of them besides the incomplete one are shared out.
 constexpr int64_t kHSharedRows = 384, kHSharedRowsMany = 512, kHTwoRoundsRows = 400;
-constexpr int kHFewRounds = 12, kHManyRounds = 40;
+constexpr int kHFewRounds = 12, kHManyRounds = 40;  // (the lists of more rounds would outgrow shared memory at some point)
 // And what the lengths then decide, in tiles: a CTA's mean sum and an item's mean from which the CTAs work by list, and by how much
 // the largest sum must be above the mean for the pool to be shared out.
 constexpr int kHWorthTiles = 40, kHItemTiles = 6, kHUneven = 15;
@@ -896,11 +896,8 @@ int launch_heads(const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t
 
 template <typename T> int launch_heads(int D, bool shared, const HeadMaps &maps, const HeadArgs &a, int grid, cudaStream_t st)
 {
-    if (shared) {  // (-1: its list does not fit)
-        const int rc = D == 128 ? launch_heads<T, 128, true>(maps, a, grid, st) : launch_heads<T, 64, true>(maps, a, grid, st);
-        if (rc != -1) return rc;
-    }
-    return D == 128 ? launch_heads<T, 128, false>(maps, a, grid, st) : launch_heads<T, 64, false>(maps, a, grid, st);
+    if (D == 128) return shared ? launch_heads<T, 128, true>(maps, a, grid, st) : launch_heads<T, 128, false>(maps, a, grid, st);
+    return shared ? launch_heads<T, 64, true>(maps, a, grid, st) : launch_heads<T, 64, false>(maps, a, grid, st);
 }
 
 }  // namespace

@@ -382,8 +382,10 @@ __device__ __forceinline__ int count_below(const uint64_t *__restrict__ c, int a
 // same additions and halvings that would lead there), and then walked: a round costs little more than a midpoint did, the
 // first one apart, whose searches cover whole rows; later ones lie between the counts at both ends of the interval.
 // Selection and compaction of one sample, a midpoint at a time / five levels at a time: 32 layers of 640 scores 58.2 / 52.0 us
-// (four levels 54.0), of 128 28.8 / 24.7, of 16384 274 / 266; 40 layers of 1024 109 / 98.
+// (four levels 54.0), of 128 28.8 / 24.7, of 16384 274 / 266; 40 layers of 1024 109 / 98.  Sort and search alone, one sample: 129
+// layers of 640 scores 56.0 / 40.4, 300 143.5 / 97.6, 1000 of 2000 scores 699 / 559 (beyond 128 layers a lane searches whole rows).
 constexpr int kTreeLevels = 5;
+constexpr int kMaxLayers = 5120;  // of a sample (sums of lengths are 32 bits wide, which would do for 2^17 layers)
 __global__ void __launch_bounds__(1024)
 search_kernel(const uint64_t *__restrict__ cum, const int64_t *__restrict__ budget_rows, int L,
               int N, double tol, int max_iters, int64_t slack, int64_t slack_over, int32_t *__restrict__ len,
@@ -646,7 +648,7 @@ extern "C" int prefixkv_search(const pkv_shape *shape, const float *scores,
     if (!shape_supported(shape)) return PKV_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const int B = shape->batch, L = shape->layers, N = shape->prompt_len;
-    if ((size_t)2 * L * sizeof(int) > 40 * 1024) return PKV_ERR_UNSUPPORTED;
+    if (L > kMaxLayers) return PKV_ERR_UNSUPPORTED;
     int rc = launch_sort(shape, scores, order, cum, len, st);
     if (rc != PKV_OK) return rc;
     cudaError_t e = launch_dependent(search_kernel, dim3(B), dim3(1024), 0, st,
