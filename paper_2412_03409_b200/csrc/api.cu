@@ -77,7 +77,7 @@ int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const
                        const float *scale, const float *lse, float *scores, void *ws, cudaStream_t st);
 int selftest_wait_score(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_stream(int32_t *dev_status, cudaStream_t st);
-int selftest_wait_cluster(int32_t *dev_status, cudaStream_t st);
+int selftest_wait_flags(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_fused(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_parts(int32_t *dev_status, cudaStream_t st);
 
@@ -184,7 +184,7 @@ extern "C" int prefixkv_selftest_bounded_wait(int32_t which, int32_t *dev_status
     if (!dev_status) return PKV_ERR_INVALID_ARG;
     if (which == 0) return selftest_wait_score(dev_status, (cudaStream_t)cuda_stream);
     if (which == 1) return selftest_wait_stream(dev_status, (cudaStream_t)cuda_stream);
-    if (which == 2) return selftest_wait_cluster(dev_status, (cudaStream_t)cuda_stream);
+    if (which == 2) return selftest_wait_flags(dev_status, (cudaStream_t)cuda_stream);
     if (which == 3) return selftest_wait_fused(dev_status, (cudaStream_t)cuda_stream);
     if (which == 4) return selftest_wait_parts(dev_status, (cudaStream_t)cuda_stream);
     return PKV_ERR_INVALID_ARG;

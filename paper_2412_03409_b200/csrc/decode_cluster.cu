@@ -8,23 +8,25 @@
 // CTAs' partial softmax states go to the first CTA of the cluster through distributed shared memory,
 // which merges them in rank order and writes the head's output: one launch, nothing in global memory
 // in between.  The last CTA of a cluster also attends to the new row and appends it.
-// Lengths: every CTA reads its segment's length at the start and raises its flag (a per-call token
-// in the workspace); one extra cluster at the end of the grid, which has no rows, waits (bounded) for
-// all flags while the others work, and then writes the lengths of the next step.  However the wait
-// ends, all flags are zero once the launch is over: a call replayed from a CUDA graph comes with the
-// same token and must not find flags of its previous run.
+// Lengths: a CTA reads its segment's length by adding one to the upper bits of its word, which so counts
+// the CTAs that have been there; the last of them writes the length of the next step over it.  A call
+// that appends nothing leaves the word alone.  (Before, every CTA raised a flag in the workspace and an
+// extra cluster waited for them: its chain of round trips ended after the rows', 4.43 us a call below for 3.96 without.)
+// Where the rows are is also read ahead, while the kernel in front still runs: the rows of that guess are
+// asked for as soon as it has completed, and the guess is held against the plan made afterwards.  The
+// values are not looked at before then, so that a CTA that starts late has both loads on their way at once
+// (looked at before: 19.3 us for 17.7 in the case of 8 x 40 x 410 rows; one thread's loads, passed on through
+// shared memory: 20.1, and 4.15 for 3.77 in the smallest).
 //
-// Measured, device time of calls replayed from a graph, against the row-split kernel and its merge
-// kernel (one layer, bf16, D = 128): 1 segment x 32 heads x 128 rows 4.5 us (10.0), 1024 rows 8.0
-// (26.4); 4 x 32 x 128 rows 6.1 (12.1); 8 x 40 x 410 rows 17.4 (25.7; 10.3 us of bytes: SMs hold four
-// or five of the 642 CTAs); 8 x 64 x 900 rows 50 (51).  A second wave of CTAs costs as much as the
+// Measured, device time of calls replayed from a graph, one layer, bf16, D = 128, every call on another layer: 1 segment
+// x 32 heads x 128 rows 3.77 us (4.43 with flags and without the guess), 4 x 32 x 128 rows 5.46 (6.00), 16 x 32 x 128 10.98 (11.55),
+// 1 x 40 x 410 5.05 (5.63), 8 x 40 x 410 17.7 (18.8; 10.3 us of bytes); against the row-split kernel and its merge
+// kernel, before that: 1 x 32 x 128 rows 4.5 (10.0), 1024 rows 8.0 (26.4); 4 x 32 x 128 rows 6.1 (12.1);
+// 8 x 40 x 410 rows 17.4 (25.7); 8 x 64 x 900 rows 50 (51).  A second wave of CTAs costs as much as the
 // first's latency, 4-5 us (C = 8 for 4 x 32 x 128 rows: 8.9 us), hence the choice of C below.  Loads to
 // registers instead of the rings, eight steps of K and V in flight: the same for one round of rows,
 // 20.5 us for 8 x 40 x 410.  Ring shapes (steps, rounds, CTAs per SM): 4, 2, 5 as here; 8, 2, 3 and
 // 4, 3, 4 18.9-19.4 us there; 2, 4, 5 18.7.  Clusters of 12 or 16: slower throughout.
-#include <atomic>
-#include <chrono>
-
 #include "decode_plan.cuh"
 
 namespace pkv {
@@ -39,8 +41,6 @@ constexpr int kCStages = 2;            // rounds in flight per warp
 constexpr int kCPerSm = 5;             // CTAs an SM holds at a time (their rings fill its shared memory)
 constexpr uint32_t kCRound = kCU * 512;  // bytes of a round's K (or V) rows: a warp reads 512 bytes per step
 constexpr int kCMaxCluster = 8;        // portable cluster size
-constexpr int kCMaxCtas = 8192;        // CTAs of a call (flags in the workspace)
-constexpr uint32_t kCSpinLimit = 1u << 22;
 constexpr float kLog2eC = 1.4426950408889634f;
 constexpr float kNoLogit = -3.402823466e38f;  // the lowest finite number
 
@@ -49,10 +49,8 @@ struct ClusterArgs {
     const void *q, *k_new, *v_new;
     void *ck, *cv, *out;
     const float *layer_scale;
-    unsigned long long *flags;  // [CTAs with rows] per-call tokens: "this CTA has read the lengths"
-    unsigned long long token;
     int32_t *dev_status;
-    int H;
+    int H, visit_shift;  // a length's word counts its readers from this bit on
     uint32_t row_bytes;
 };
 
@@ -80,32 +78,6 @@ __device__ __forceinline__ void copy16(void *dst, const unsigned char *src)
     asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 
-// The give-up path in isolation: some CTAs' flags are raised, the wait for all of them runs out, the other flags
-// come late; all are zero after that, and a second run with the same token finds every flag it waits for.
-__global__ void selftest_flags_kernel(int32_t *dev_status, uint32_t limit)
-{
-    constexpr int n = 80, came = 50;
-    __shared__ unsigned long long flags[n];
-    const unsigned long long token = 0x9e3779b97f4a7c15ull;
-    const int i = threadIdx.x;
-    if (i < n) flags[i] = i % 3 ? 0ull : ~(unsigned long long)i;  // (left from anything)
-    __syncthreads();
-    bool ok = true;
-    if (i < came) ok = !unraise_flag(flags + i, token, raise_flag(flags + i, token));
-    __syncthreads();
-    ok = !settle_flags(flags, n, token, limit) && ok;
-    __syncthreads();
-    if (i >= came && i < n) ok = unraise_flag(flags + i, token, raise_flag(flags + i, token)) && ok;
-    __syncthreads();
-    if (i < n) ok = ok && flags[i] == 0ull;
-    if (i < n) ok = !unraise_flag(flags + i, token, raise_flag(flags + i, token)) && ok;
-    __syncthreads();
-    ok = settle_flags(flags, n, token, limit) && ok;
-    __syncthreads();
-    if (i < n) ok = ok && flags[i] == 0ull;
-    if (__syncthreads_and(ok) && i == 0) raise_status(dev_status, 0, PKV_DEV_TIMEOUT);
-}
-
 // A head's slice of a row is D * sizeof(T) bytes: LPR lanes share a row, a warp reads G = 32 / LPR
 // rows per step.
 template <typename T, int D>
@@ -120,36 +92,81 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
     __shared__ float s_acc[kCWarps][D], s_ml[kCWarps][2];
     __shared__ float c_acc[kCMaxCluster][D], c_ml[kCMaxCluster][2];  // (first CTA) the cluster's partials
 
+    __shared__ SegPlan s_plan[2];
+
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int C = (int)cluster_size(), rank = (int)cluster_rank();
     const int item = blockIdx.x / C;
-    const int nitems = a.p.nact * a.H;
     // (the first CTA must be running before anyone writes to its shared memory)
     if (C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-    if (item == nitems) {
-        // ---- the extra cluster: lengths of the next step, once every CTA has read this step's ----------
-        if (C > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-        if (rank != 0) return;
-        if (!settle_flags(a.flags, nitems * C, a.token, kCSpinLimit)) {
-            if (tid == 0) raise_status(a.dev_status, 0, PKV_DEV_TIMEOUT);
-            return;
-        }
-        for (int si = tid; si < a.p.nact; si += kCWarps * 32) {
-            const SegPlan sp = segment_plan(a.p, si);
-            if (sp.rows < 0) raise_status(a.dev_status, si / a.p.nl, PKV_DEV_CAPACITY);
-            else if (a.p.append) segment_advance(a.p, si, sp);
-        }
-        return;
-    }
 
     const int si = item / a.H, h = item - si * a.H;
     const int seg = (si / a.p.nl) * a.p.L + a.p.layer_begin + si % a.p.nl;
     const size_t hoff = ((size_t)seg * a.H + h) * SLICE;
     const int grp = lane / LPR, c = lane % LPR;
     const bool takes_new = a.p.append && rank == C - 1 && warp == 0;
+    // What this CTA reads of a segment: the cached rows less the slot that the new row reuses, a C-th of them.
+    struct Rows {
+        const unsigned char *kb, *vb;
+        int r0, r1, skip;
+    };
+    auto rows_of = [&](const SegPlan &sp) {
+        const int cached = sp.rows < 0 ? 0 : (a.p.append ? (sp.evict ? sp.rows : sp.rows - 1) : sp.rows);
+        const int per = (cached + C - 1) / C;
+        Rows r;
+        r.r0 = min(cached, rank * per);
+        r.r1 = min(cached, r.r0 + per);
+        r.skip = sp.evict ? sp.dst : -1;
+        r.kb = static_cast<const unsigned char *>(a.ck) + (size_t)sp.off * a.row_bytes + (size_t)h * SLICE + c * 16;
+        r.vb = static_cast<const unsigned char *>(a.cv) + (size_t)sp.off * a.row_bytes + (size_t)h * SLICE + c * 16;
+        return r;
+    };
+    // Every warp runs its own ring: a lane copies, and later reads, the same 16 bytes of a step's rows, so
+    // that waiting for its own copies is all that it needs.
+    unsigned char *ring = s_ring + (size_t)warp * kCStages * 2 * kCRound + lane * 16;
+    auto request = [&](const Rows &rw, int base, int stage) {
+        unsigned char *d = ring + stage * 2 * kCRound;
+#pragma unroll
+        for (int j = 0; j < kCU; ++j) {
+            const int r = base + j * G + grp;
+            if (r < rw.r1 && r != rw.skip) {
+                copy16(d + j * 512, rw.kb + (size_t)r * a.row_bytes);
+                copy16(d + kCRound + j * 512, rw.vb + (size_t)r * a.row_bytes);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // Where the rows are is read before the kernel in front has completed, and the first rounds are asked for as soon
+    // as it has, together with the plan that counts.  Should that one be another, they are asked for again.
+    const bool guesses = a.p.evict_distance == 0;
+    int guess_ln = 0, guess_cp = 0;
+    int64_t guess_off = 0;
+    if (guesses) {  // (not looked at yet: a CTA that starts late must not wait for these before it asks for the others)
+        guess_ln = load_l2(a.p.len + seg);
+        guess_cp = load_l2(a.p.cap + seg);
+        guess_off = load_l2(a.p.row_offset + seg);
+    }
+    dependent_entry();
+    // The length is read by adding to its word's upper bits: whoever finds that all CTAs of the segment but itself have
+    // been there writes what the step leaves.  (With pruning what else the plan is made of has been read before that.)
+    uint32_t word = 0;
+    int cp = 0;
+    int64_t off = 0;
+    PruneState ps;
+    if (tid == 0) {
+        ps = prune_state(a.p, seg);
+        if (!a.p.append) word = (uint32_t)load_l2(a.p.len + seg);
+        else if (a.p.evict_distance == 0) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], %2;" : "=r"(word) : "l"(a.p.len + seg), "r"(1u << a.visit_shift) : "memory");
+        else asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(word) : "l"(a.p.len + seg), "r"(1u << a.visit_shift) : "memory");
+        cp = load_l2(a.p.cap + seg);
+        off = load_l2(a.p.row_offset + seg);
+    }
+    Rows rw{nullptr, nullptr, 0, 0, -1};
+    if (guesses) {
+        rw = rows_of(plan_of(a.p, guess_ln, guess_cp, guess_off, PruneState{0, 0, -1}));
+#pragma unroll
+        for (int i = 0; i < kCStages; ++i) request(rw, rw.r0 + (warp + i * kCWarps) * STEP, i);
+    }
     uint4 qraw = *reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(a.q) + hoff + c * 16);
     uint4 knew = make_uint4(0u, 0u, 0u, 0u), vnew = knew;
     if (takes_new) {
@@ -157,16 +174,30 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         vnew = *reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(a.v_new) + hoff + c * 16);
     }
     const float sc = a.layer_scale[a.p.layer_begin + si % a.p.nl] * kLog2eC;
-    const SegPlan sp = segment_plan(a.p, si);
-    __syncthreads();  // all of this CTA's reads of the lengths are done
-    unsigned long long held = 0;
-    if (tid == 0) held = raise_flag(a.flags + blockIdx.x, a.token);
+    if (tid == 0) {
+        const uint32_t before = a.p.append ? word >> a.visit_shift : 0u, all = (uint32_t)(a.H * C);
+        const int ln = a.p.append ? (int)(word & ((1u << a.visit_shift) - 1u)) : (int)word;
+        SegPlan sp = plan_of(a.p, ln, cp, off, ps);
+        if (before >= all) sp.rows = -1;  // (the word was no length)
+        if (sp.rows < 0) {  // (every CTA finds the same, and takes back what it added)
+            raise_status(a.dev_status, si / a.p.nl, PKV_DEV_CAPACITY);
+            if (a.p.append) atomicSub(reinterpret_cast<unsigned int *>(a.p.len + seg), 1u << a.visit_shift);
+        } else if (a.p.append && before == all - 1) {
+            segment_advance(a.p, si, sp);
+        }
+        s_plan[1] = sp;
+    }
+    __syncthreads();
+    const SegPlan sp = s_plan[1];
+    const Rows now = rows_of(sp);
+    if (now.r0 != rw.r0 || now.r1 != rw.r1 || now.skip != rw.skip || now.kb != rw.kb) {
+        // (a row more or less at the end: the same bytes come to the same places again)
+        if (now.r0 != rw.r0 || now.skip != rw.skip || now.kb != rw.kb) asm volatile("cp.async.wait_all;" ::: "memory");
+        rw = now;
+#pragma unroll
+        for (int i = 0; i < kCStages; ++i) request(rw, rw.r0 + (warp + i * kCWarps) * STEP, i);
+    }
 
-    // cached rows of the segment that are attended to: all of them, less the slot that the new row reuses
-    const int cached = sp.rows < 0 ? 0 : (a.p.append ? (sp.evict ? sp.rows : sp.rows - 1) : sp.rows);
-    const int skip = sp.evict ? sp.dst : -1;
-    const int per = (cached + C - 1) / C;
-    const int r0 = min(cached, rank * per), r1 = min(cached, r0 + per);
     // M: the running maximum of the logits, from the lowest finite number on, so that exp2f(s - M) is 0 for a logit
     // of -infinity and NaN for NaN whatever came before it.
     float qf[VE], acc[VE], M = kNoLogit, lsum = 0.f;
@@ -176,8 +207,6 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         qf[i] *= sc;
         acc[i] = 0.f;
     }
-    const unsigned char *kb = static_cast<const unsigned char *>(a.ck) + (size_t)sp.off * a.row_bytes + (size_t)h * SLICE + c * 16;
-    const unsigned char *vb = static_cast<const unsigned char *>(a.cv) + (size_t)sp.off * a.row_bytes + (size_t)h * SLICE + c * 16;
     // One round: logits of the warp's rows, one rescale, accumulation (every lane group keeps the
     // warp-wide running maximum, so that the groups' sums simply add at the end).
     auto dot = [&](const uint4 &raw) {
@@ -207,26 +236,8 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
 #pragma unroll
         for (int i = 0; i < VE; ++i) acc[i] *= corr;
     };
-    // Every warp runs its own ring: a lane copies, and later reads, the same 16 bytes of a step's rows, so
-    // that waiting for its own copies is all that it needs.
-    unsigned char *ring = s_ring + (size_t)warp * kCStages * 2 * kCRound + lane * 16;
-    auto request = [&](int base, int stage) {
-        unsigned char *d = ring + stage * 2 * kCRound;
-#pragma unroll
-        for (int j = 0; j < kCU; ++j) {
-            const int r = base + j * G + grp;
-            if (r < r1 && r != skip) {
-                copy16(d + j * 512, kb + (size_t)r * a.row_bytes);
-                copy16(d + kCRound + j * 512, vb + (size_t)r * a.row_bytes);
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    const int first = r0 + warp * STEP;
-#pragma unroll
-    for (int i = 0; i < kCStages; ++i) request(first + i * kCWarps * STEP, i);
     int stage = 0;
-    for (int base = first; base < r1; base += kCWarps * STEP) {
+    for (int base = rw.r0 + warp * STEP; base < rw.r1; base += kCWarps * STEP) {
         asm volatile("cp.async.wait_group %0;" ::"n"(kCStages - 1) : "memory");
         const unsigned char *kt = ring + stage * 2 * kCRound;
         float s[kCU], mx = -INFINITY;
@@ -239,17 +250,17 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
 #pragma unroll
         for (int j = 0; j < kCU; ++j) {
             const int r = base + j * G + grp;  // (what was not copied may be anything, NaN included)
-            if (r >= r1 || r == skip) s[j] = -INFINITY;
+            if (r >= rw.r1 || r == rw.skip) s[j] = -INFINITY;
             mx = fmaxf(mx, s[j]);
         }
         rescale(mx);
 #pragma unroll
         for (int j = 0; j < kCU; ++j) {
             const int r = base + j * G + grp;
-            if (r < r1 && r != skip)
+            if (r < rw.r1 && r != rw.skip)
                 add(exp2f(s[j] - M), *reinterpret_cast<const uint4 *>(kt + kCRound + j * 512));
         }
-        request(base + kCStages * kCWarps * STEP, stage);
+        request(rw, base + kCStages * kCWarps * STEP, stage);
         if (++stage == kCStages) stage = 0;
     }
     if (takes_new && sp.rows >= 0) {
@@ -300,10 +311,7 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
             store_first_cta(&c_ml[rank][1], z);
         }
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        if (rank != 0) {  // (only the first CTA's memory is written, and it waits for everyone)
-            unraise_flag(a.flags + blockIdx.x, a.token, held);
-            return;
-        }
+        if (rank != 0) return;  // (only the first CTA's memory is written, and it waits for everyone)
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         m = kNoLogit;
         for (int r = 0; r < C; ++r) m = fmaxf(m, c_ml[r][0]);
@@ -315,9 +323,8 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
             if (tid < D) o = fmaf(f, c_acc[r][tid], o);
         }
     }
-    if (tid < D)  // (a segment that cannot take the step is reported by the extra cluster; its output is zero)
+    if (tid < D)  // (the output of a segment that cannot take the step is zero)
         reinterpret_cast<T *>(static_cast<unsigned char *>(a.out) + hoff)[tid] = from_float<T>(sp.rows < 0 ? 0.f : o * (1.f / z));
-    unraise_flag(a.flags + blockIdx.x, a.token, held);
 }
 
 template <typename T, int D> int launch_cluster(const ClusterArgs &a, int C, cudaStream_t st)
@@ -333,7 +340,7 @@ template <typename T, int D> int launch_cluster(const ClusterArgs &a, int C, cud
     attr[1].val.clusterDim.x = (unsigned)C;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((a.p.nact * a.H + 1) * C));
+    cfg.gridDim = dim3((unsigned)(a.p.nact * a.H * C));
     cfg.blockDim = dim3(kCWarps * 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -349,17 +356,9 @@ template <typename T, int D> int launch_cluster(const ClusterArgs &a, int C, cud
 
 }  // namespace
 
-int selftest_wait_cluster(int32_t *dev_status, cudaStream_t st)
-{
-    selftest_flags_kernel<<<1, 96, 0, st>>>(dev_status, 4096u);
-    return check_launch("selftest_flags_kernel");
-}
-
-size_t decode_cluster_ws_bytes() { return (size_t)kCMaxCtas * sizeof(unsigned long long); }
-
 // Returns PKV_OK, an error, or -1 when this call is outside what the kernel covers.
 int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn, const void *vn,
-                          const float *scale, int lb, int le, void *out, int32_t *dev_status, void *ws, cudaStream_t st)
+                          const float *scale, int lb, int le, void *out, int32_t *dev_status, cudaStream_t st)
 {
     const int H = s->heads, D = s->head_dim, nl = le - lb, nact = s->batch * nl;
     const int sms = sm_count();
@@ -387,21 +386,21 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     int C = 1;
     while (C < kCMaxCluster) {
         const int n = C + 1;
-        const bool one_wave = (int64_t)(items + 1) * n <= (int64_t)kCPerSm * sms &&
+        const bool one_wave = (int64_t)items * n <= (int64_t)kCPerSm * sms &&
                               (seg_rows >= 32 * n || (int64_t)items * n <= 2 * (int64_t)sms);
         if (!one_wave && seg_rows < 256 * (int64_t)n) break;
         C = n;
     }
-    if ((int64_t)(items + 1) * C > kCMaxCtas) return -1;
+    // (the bits of a length's word that its readers are counted in leave room for any length)
+    int visit_bits = 1;
+    while ((H * C) >> visit_bits) ++visit_bits;
+    if (c->total_cap_rows >> (32 - visit_bits)) return -1;
 
-    static std::atomic<unsigned long long> g_token{
-        0x9e3779b97f4a7c15ull ^ (unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count()};
     ClusterArgs a;
     a.p = decode_plan_args(s, c, kn != nullptr, lb, nl);
     a.q = q; a.k_new = kn; a.v_new = vn; a.ck = c->k; a.cv = c->v; a.out = out;
     a.layer_scale = scale;
-    a.flags = (unsigned long long *)ws;
-    a.token = g_token.fetch_add(0x9e3779b97f4a7c15ull) | 1ull;
+    a.visit_shift = 32 - visit_bits;
     a.dev_status = dev_status;
     a.H = H;
     a.row_bytes = (uint32_t)((size_t)H * D * esize(s));

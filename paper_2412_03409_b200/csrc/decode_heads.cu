@@ -834,6 +834,32 @@ bool make_cache_map(CUtensorMap *map, void *ptr, const pkv_shape *s, int64_t row
 
 constexpr int kHMaxSmem = 224 * 1024;  // dynamic; there are up to 1.7 KiB of static variables beside it
 
+// The give-up path in isolation: some CTAs' flags are raised, the wait for all of them runs out, the other flags
+// come late; all are zero after that, and a second run with the same token finds every flag it waits for.
+__global__ void selftest_flags_kernel(int32_t *dev_status, uint32_t limit)
+{
+    constexpr int n = 80, came = 50;
+    __shared__ unsigned long long flags[n];
+    const unsigned long long token = 0x9e3779b97f4a7c15ull;
+    const int i = threadIdx.x;
+    if (i < n) flags[i] = i % 3 ? 0ull : ~(unsigned long long)i;  // (left from anything)
+    __syncthreads();
+    bool ok = true;
+    if (i < came) ok = !unraise_flag(flags + i, token, raise_flag(flags + i, token));
+    __syncthreads();
+    ok = !settle_flags(flags, n, token, limit) && ok;
+    __syncthreads();
+    if (i >= came && i < n) ok = unraise_flag(flags + i, token, raise_flag(flags + i, token)) && ok;
+    __syncthreads();
+    if (i < n) ok = ok && flags[i] == 0ull;
+    if (i < n) ok = !unraise_flag(flags + i, token, raise_flag(flags + i, token)) && ok;
+    __syncthreads();
+    ok = settle_flags(flags, n, token, limit) && ok;
+    __syncthreads();
+    if (i < n) ok = ok && flags[i] == 0ull;
+    if (__syncthreads_and(ok) && i == 0) raise_status(dev_status, 0, PKV_DEV_TIMEOUT);
+}
+
 // The wait for parts that CTAs pass on, in isolation: some are there, one does not come in time, others are given up after it; flags
 // of parts that were there are zero then, late ones get zero from their own CTAs, and a second run with the same token is whole.
 __global__ void selftest_parts_kernel(int32_t *dev_status, uint32_t limit)
@@ -901,6 +927,12 @@ template <typename T> int launch_heads(int D, bool shared, const HeadMaps &maps,
 }
 
 }  // namespace
+
+int selftest_wait_flags(int32_t *dev_status, cudaStream_t st)
+{
+    selftest_flags_kernel<<<1, 96, 0, st>>>(dev_status, 4096u);
+    return check_launch("selftest_flags_kernel");
+}
 
 int selftest_wait_parts(int32_t *dev_status, cudaStream_t st)
 {

@@ -74,15 +74,41 @@ struct SegPlan {
     bool evict;
     int64_t off;
 };
-__device__ __forceinline__ SegPlan segment_plan(const DecodePlanArgs &a, int si)
+// (Read past the L1 cache: a kernel may ask once while the kernel in front still runs, as a guess, and again after it.)
+__device__ __forceinline__ int32_t load_l2(const int32_t *p)
 {
-    const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
-    const int ln = a.len[seg], cp = a.cap[seg];
+    int32_t v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int64_t load_l2(const int64_t *p)
+{
+    int64_t v;
+    asm volatile("ld.relaxed.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+// What decode-time pruning goes by: tokens so far, rows kept by compaction, the place of the token `distance` back.
+struct PruneState {
+    int g, len0, slot;
+};
+__device__ __forceinline__ PruneState prune_state(const DecodePlanArgs &a, int seg)
+{
+    PruneState s{0, 0, -1};
+    const int d = a.append ? a.evict_distance : 0;
+    if (d > 0) {
+        s.g = load_l2(a.gen + seg);
+        s.len0 = load_l2(a.len0 + seg);
+        if (s.g >= d) s.slot = load_l2(a.slot_ring + (size_t)seg * (d + 1) + (s.g - d) % (d + 1));
+    }
+    return s;
+}
+__device__ __forceinline__ SegPlan plan_of(const DecodePlanArgs &a, int ln, int cp, int64_t off, const PruneState &ps)
+{
     SegPlan p;
-    p.off = a.row_offset[seg];
+    p.off = off;
     p.evict = false;
     p.dst = ln;
-    bool ok = ln >= 1 && p.off >= 0 && p.off + cp <= a.total_cap_rows && ln <= cp;
+    bool ok = ln >= 1 && p.off >= 0 && p.off <= a.total_cap_rows - cp && ln <= cp;
     if (!a.append) {  // nothing to append: attend over the rows that are there
         p.dst = 0x3fffffff;
         p.rows = ok ? ln : -1;
@@ -91,20 +117,23 @@ __device__ __forceinline__ SegPlan segment_plan(const DecodePlanArgs &a, int si)
     }
     const int d = a.evict_distance;
     if (ok && d > 0) {
-        const int g = a.gen[seg];
-        const int64_t target = ((int64_t)a.len0[seg] * ((int64_t)a.N + g + 1)) / a.N;
-        if ((int64_t)ln + 1 > target && g >= d) {
-            const int r = a.slot_ring[(size_t)seg * (d + 1) + (g - d) % (d + 1)];
-            if (r >= 0 && r < ln) {
-                p.evict = true;
-                p.dst = r;
-            }
+        const int64_t target = ((int64_t)ps.len0 * ((int64_t)a.N + ps.g + 1)) / a.N;
+        if ((int64_t)ln + 1 > target && ps.g >= d && ps.slot >= 0 && ps.slot < ln) {
+            p.evict = true;
+            p.dst = ps.slot;
         }
     }
     if (!p.evict && ln >= cp) ok = false;  // appending needs head-room
     p.rows = ok ? (p.evict ? ln : ln + 1) : -1;
     p.len_after = p.rows;
     return p;
+}
+__device__ __forceinline__ SegPlan segment_plan(const DecodePlanArgs &a, int si)
+{
+    const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
+    const int ln = load_l2(a.len + seg), cp = load_l2(a.cap + seg);
+    const int64_t off = load_l2(a.row_offset + seg);
+    return plan_of(a, ln, cp, off, prune_state(a, seg));
 }
 // Writes what the step leaves for the next one: the length and, with pruning, the token's place.
 // (Only one thread of the call touches a segment's token count and slot ring.)

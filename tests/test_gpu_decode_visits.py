@@ -1,0 +1,99 @@
+"""Layer-by-layer decode calls: the length's word counts its readers, and rows are asked for by a length read ahead
+(needs a B200).  Outputs against attention in 64 bits over the rows as they stand."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2412_03409_b200 import api
+from paper_2412_03409_b200.session import Session
+
+pytestmark = pytest.mark.gpu
+
+TOL = {torch.float32: 2e-5, torch.bfloat16: 8e-3}  # one rounding to bf16 of |out| < 4
+
+
+def _session(B, L, H, D, lens, dtype, T):
+    s = Session(B, L, H, D, max(lens), dtype, np.full(L, 1.0 / np.sqrt(D), np.float32), decode_cap=T,
+                max_budget_rows=int(np.ceil(sum(lens) / B)))
+    cap = torch.tensor(lens, dtype=torch.int32, device="cuda") + T
+    s.cache.cap.copy_(cap)
+    s.cache.len.copy_(cap - T)
+    s.cache.row_offset.copy_(torch.cat([cap.new_zeros(1), cap.cumsum(0)])[:s.cache.row_offset.numel()])
+    g = torch.Generator(device="cuda").manual_seed(H * 131 + sum(lens))
+    s.cache.k.copy_(torch.randn(s.cache.k.shape, device="cuda", generator=g).to(dtype))
+    s.cache.v.copy_(torch.randn(s.cache.v.shape, device="cuda", generator=g).to(dtype))
+    tok = [[torch.randn(B, L, H, D, device="cuda", generator=g).to(dtype) for _ in range(3)] for _ in range(T)]
+    return s, tok
+
+
+def _attend(s, q, i, n):
+    """Segment i's output over its first n rows, 64 bits."""
+    o, L = int(s.cache.row_offset[i]), q.shape[1]
+    k, v = (x[o:o + n].double().reshape(n, q.shape[2], q.shape[3]) for x in (s.cache.k, s.cache.v))
+    w = torch.einsum("hd,nhd->hn", q[i // L, i % L].double(), k) / np.sqrt(q.shape[3])
+    return torch.einsum("hn,nhd->hd", torch.softmax(w, -1), v)
+
+
+# readers of a word (heads x CTAs of a cluster) at and around powers of two; lengths around a CTA's and a round's rows
+@pytest.mark.parametrize("B,L,H,D,lens,dtype", [
+    (1, 1, 1, 64, [1], torch.bfloat16), (1, 1, 1, 128, [700], torch.float32), (1, 1, 2, 128, [255], torch.bfloat16),
+    (1, 2, 31, 64, [32, 129], torch.bfloat16), (1, 1, 32, 128, [127], torch.bfloat16), (2, 1, 33, 64, [64, 33], torch.float32),
+    (3, 1, 63, 64, [31, 257, 8], torch.bfloat16), (2, 2, 64, 128, [16, 17, 90, 5], torch.bfloat16), (1, 1, 80, 64, [300], torch.bfloat16),
+    (8, 1, 40, 128, [410, 380, 409, 3, 411, 64, 128, 256], torch.bfloat16), (1, 1, 512, 64, [40], torch.bfloat16),
+])
+@pytest.mark.parametrize("layerwise", [False, True])
+def test_tokens_back_to_back(B, L, H, D, lens, dtype, layerwise):
+    """Every call but the first starts while the one in front may still be writing the lengths."""
+    T = 5
+    s, tok = _session(B, L, H, D, lens, dtype, T)
+    outs = [torch.empty_like(tok[0][0]) for _ in range(T)]
+    torch.cuda.synchronize()
+    for t in range(T):
+        if layerwise:
+            for l in range(L):
+                s.decode(*tok[t], out=outs[t], layer_begin=l, layer_end=l + 1)
+        else:
+            s.decode(*tok[t], out=outs[t])
+    torch.cuda.synchronize()
+    assert s.cache.len.tolist() == [n + T for n in lens] and s.status.tolist() == [0] * B
+    for i, n in enumerate(lens):
+        o = int(s.cache.row_offset[i])
+        for t in range(T):
+            for mine, new in ((s.cache.k, tok[t][1]), (s.cache.v, tok[t][2])):
+                assert torch.equal(mine[o + n + t].reshape(H, D), new[i // L, i % L])
+            ref = _attend(s, tok[t][0], i, n + t + 1)
+            assert (outs[t][i // L, i % L].double() - ref).abs().max().item() <= TOL[dtype], (i, t)
+
+
+@pytest.mark.parametrize("word", [0, -1, 2**31 - 1, -2**31, 0x7f7f7f7f, "full", "above"])
+@pytest.mark.parametrize("H", [1, 5, 64])
+def test_a_segment_that_cannot_take_the_row_keeps_its_word(word, H):
+    s, tok = _session(2, 1, H, 64, [40, 30], torch.bfloat16, 2)
+    word = {"full": 32, "above": 33}.get(word, word)  # (of the second segment: 30 rows and two to come)
+    s.cache.len[1] = word
+    before = s.cache.k.clone()
+    out = s.decode(*tok[0])
+    torch.cuda.synchronize()
+    assert s.status.tolist() == [0, api.DEV_CAPACITY]
+    assert s.cache.len.tolist() == [41, word]
+    assert (out[1] == 0).all()
+    assert (out[0, 0].double() - _attend(s, tok[0][0], 0, 41)).abs().max().item() <= TOL[torch.bfloat16]
+    o = int(s.cache.row_offset[1])
+    assert torch.equal(s.cache.k[o:], before[o:])
+
+
+@pytest.mark.parametrize("place", ["len", "row_offset"])
+def test_a_plan_changed_just_before_the_call(place):
+    """The rows that count are those of the plan after the kernel in front, whatever was there while it ran."""
+    s, tok = _session(1, 2, 8, 64, [200, 90], torch.bfloat16, 4)
+    for n in (200, 17, 131, 64):
+        s.cache.len.copy_(torch.tensor([n, 90], dtype=torch.int32))
+        if place == "row_offset":
+            s.cache.row_offset[:2].copy_(torch.tensor([n % 3, 204 + n % 4]))
+            s.cache.cap.copy_(torch.tensor([n + 1, 91], dtype=torch.int32))
+        s.decode(*tok[0])      # changes the lengths while the next call is being set up
+        out = s.decode(tok[1][0], None, None)
+        torch.cuda.synchronize()
+        for i, rows in enumerate((n + 1, 91)):
+            ref = _attend(s, tok[1][0], i, rows)
+            assert (out[0, i].double() - ref).abs().max().item() <= TOL[torch.bfloat16], (n, i)
