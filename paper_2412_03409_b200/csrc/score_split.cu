@@ -19,12 +19,17 @@
 // per SM, 13 warps.  A prompt of at most 128 tokens is one tile: both passes then run on it in one
 // launch (MODE 0), the second on the transposed product of the operands already in shared memory.
 //
-// Measured, 8 layers x 16 heads of 128, 777 tokens: 190 us for the whole call (1263 us with 64 x 64
-// tiles on FMA units), 94 and 98 us a pass.  A tile needs 48 MMAs of 64 clocks = 3072; it takes 6200: the
-// issuing warp waits 1800 of them for chunks, because a chunk costs a loader warp about 2300 clocks
-// (the latency of its loads, of which one chunk is in flight, and its share of the issue slots).
-// Sixteen loader warps leave 80 registers a thread and spill (211 us).  4 layers x 4 heads of 64,
-// 128 tokens (one tile each): 12.3 us for the call, 30.7 with three FMA kernels.
+// Prompts of a few tiles keep their logits (MODE 3): one pass, one launch and the mean.
+//
+// Measured, 8 layers x 16 heads of 128, 777 tokens: 161 us for the whole call (1263 us with 64 x 64 tiles on FMA units; 167
+// in two passes, 175 before a loader's lane took 32 bytes of a row at a time, with 16-byte stores and half the address
+// arithmetic), 92 us with the caller's log-sum-exp.  A tile needs 48 MMAs of 64 clocks = 3072, during which their operands
+// take all of shared memory's bandwidth; storing the split ones takes 768 more.  It takes 5250: the issuing warp
+// waits 1250 of them for chunks.  Pairs of CTAs (cta_group::2, a streamed row split once for two tiles): 198 us.
+// Sixteen loader warps leave 80 registers a thread and spill (211 us).  4 layers x 4 heads of 64, 300 tokens:
+// 17.4 us (26.9 in two passes before), 128 tokens (one tile each): 10.9 us for the call (30.7 with three FMA kernels).
+// Reading the logits back: eight rows at a time 168 us, sixteen 161; by three warps of their own 177-187; kept in blocks that
+// pass through shared memory 177-206 (memory's latency, not the stores, is what the warps wait for).
 #include "score_tiles.cuh"
 
 namespace pkv {
@@ -33,13 +38,17 @@ namespace {
 
 constexpr int kReaders = 4;                  // accumulator reader warps (warps 0-3: one TMEM lane quarter each)
 constexpr int kLoaders = 8;                  // loader warps (warps 5-12; warp 4 issues the MMAs)
-constexpr int kVecs = TT / kLoaders / 2;     // float4 of a chunk per loader lane
+constexpr int kRows = TT / kLoaders / 4;     // rows of a chunk per loader lane, eight elements of each
+constexpr int kVecs = 2 * kRows;
 constexpr int kSplitThreads = (kReaders + 1 + kLoaders) * 32;
 constexpr int kRing = 2;                     // streamed chunks in shared memory
 static_assert(kRing == 2, "with two chunks a tile, chunk c of every tile goes through ring slot c");
 constexpr uint32_t kPart = TT * 128;         // bytes of one bf16 part of a chunk: 128 rows x 64 elements
 constexpr uint32_t kChunk = 3 * kPart;
 constexpr uint32_t kBuf = 256;               // tensor-memory columns of one of the two accumulator buffers
+constexpr int kKeepTiles = 16;               // tiles of the longest prompt whose logits are kept (1 MiB a CTA), heads of 64
+constexpr size_t kKeepCtas = 148;            // CTAs of such a call at most
+constexpr int kBack = 16;                    // rows of them a warp reads back at a time
 constexpr int kQueue = 4;                    // item numbers in flight between the loaders and the other roles
 
 struct SplitArgs {
@@ -49,7 +58,8 @@ struct SplitArgs {
     const float *lse_in;  // pass 2: [B*L*H][N] log-sum-exp; times lse_mul it is in the log2 domain
     float lse_mul;
     float *lse2;          // pass 1 out, same layout, log2 domain
-    float *partial;       // [B*L*H][N] per-head column sums
+    float *partial;       // [B*L*H][N] per-head column sums; mode 3: [B*L*H][pairs of a query and a key tile][quarter of the queries][128]
+    float *logits;        // mode 3: [CTA][tiles][128 queries][128 keys], of the item at hand
     int32_t *abort_word;  // set when a bounded wait runs out: the head mean then writes NaN scores
     int *next_item;       // work counter of this pass, zeroed before it; NULL: a CTA takes item blockIdx.x alone
     int clear_abort;      // this launch is the call's first and nothing has zeroed the abort word
@@ -61,10 +71,11 @@ struct SplitArgs {
 __device__ __forceinline__ void split2(float x, float y, uint32_t &p0, uint32_t &p1, uint32_t &p2)
 {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p0) : "f"(y), "f"(x));
-    const float rx = x - __uint_as_float(p0 << 16), ry = y - __uint_as_float(p0 & 0xffff0000u);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p1) : "f"(ry), "f"(rx));
-    const float sx = rx - __uint_as_float(p1 << 16), sy = ry - __uint_as_float(p1 & 0xffff0000u);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p2) : "f"(sy), "f"(sx));
+    const float2 neg = make_float2(-1.f, -1.f);  // (the remainders are exact, whichever way they are formed)
+    const float2 r = fma2(make_float2(__uint_as_float(p0 << 16), __uint_as_float(p0 & 0xffff0000u)), neg, make_float2(x, y));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p1) : "f"(r.y), "f"(r.x));
+    const float2 u = fma2(make_float2(__uint_as_float(p1 << 16), __uint_as_float(p1 & 0xffff0000u)), neg, r);
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p2) : "f"(u.y), "f"(u.x));
 }
 
 // An accumulator buffer holds one unit of a tile: UN columns, in NACC partial accumulators.
@@ -79,14 +90,12 @@ template <int D> struct Unit {
 template <int D> __device__ __forceinline__ void load_logits(uint32_t taddr, float (&v)[32])
 {
     float w[32];
-    tmem_ld32(taddr, v);
-    tmem_ld32(taddr + Unit<D>::UN, w);
+    tmem_ld32x2(taddr, taddr + Unit<D>::UN, v, w);
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] += w[i];
     if (Unit<D>::NACC == 4) {
         float x[32];
-        tmem_ld32(taddr + 2 * Unit<D>::UN, w);
-        tmem_ld32(taddr + 3 * Unit<D>::UN, x);
+        tmem_ld32x2(taddr + 2 * Unit<D>::UN, taddr + 3 * Unit<D>::UN, w, x);
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] += w[i] + x[i];
     }
@@ -111,13 +120,21 @@ __device__ __forceinline__ const float *head_rows(const float *p, const pkv_stri
     const int seg = sh / a.H, h = sh - seg * a.H, b = seg / a.L, l = seg - b * a.L;
     return p + b * st.b + l * st.l + h * st.h;
 }
-// Running maximum and sum of a query over the keys of the tile from key0 on.
+__device__ __forceinline__ void store8(float *p, const float *v)
+{
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]),
+                 "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+
+// Running maximum and sum of a query over the keys of the tile from key0 on; `keep` (or NULL) gets the logits.
 template <int D>
-__device__ __noinline__ float2 redo_lse(const SplitArgs &a, int sh, int query, int key0, float sc, float run_max, float run_sum)
+__device__ __noinline__ float2 redo_lse(const SplitArgs &a, int sh, int query, int key0, float sc, float run_max, float run_sum, float *keep)
 {
     const float *q = head_rows(a.q, a.qs, a, sh) + query * a.qs.n, *k = head_rows(a.k, a.ks, a, sh);
     for (int key = key0; key <= min(query, key0 + TT - 1); ++key) {
-        const float x = fma_logit<D>(q, k + key * a.ks.n) * sc;
+        const float v = fma_logit<D>(q, k + key * a.ks.n), x = v * sc;
+        if (keep) keep[key - key0] = v;
         const float nm = fmaxf(run_max, x), base = nm == -INFINITY ? 0.f : nm;
         run_sum = fmaf(run_sum, ex2(run_max - base), ex2(x - base));
         run_max = nm;
@@ -135,6 +152,9 @@ __device__ __noinline__ float redo_colsum(const SplitArgs &a, int sh, int key, i
     return sum;
 }
 
+// MODE 3: as MODE 1, and the item's logits are kept (64 KiB a tile, which mostly stay in the L2); once a query's
+// normaliser is known, the reader warp that has its row reads them back and adds up what the warp's queries give to every
+// key: the second pass without its products and splits.
 // MODE 1: stationary = Q tile t, streamed = K tiles 0..t (log-sum-exp).  MODE 2: stationary = K tile
 // t, streamed = Q tiles t..tiles-1 (column sums).  MODE 0: one tile, Q stationary, both results.
 template <int MODE, int D>
@@ -195,14 +215,17 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
     if (warp > kReaders) {
         // ---- loaders: fp32 rows -> three bf16 parts in shared memory --------------------------------
         const int lw = warp - kReaders - 1;
-        const int r0 = lw * 2 * kVecs + (lane >> 4), c4 = lane & 15;  // rows r0, r0 + 2, ...; float4 c4 of the row
+        // Lane: eight neighbouring elements of the rows r0, r0 + 4, ... of a chunk.
+        const int r0 = lw * 4 * kRows + (lane >> 3), c8 = lane & 7;
+        const uint32_t off0 = r0 * 128 + ((c8 ^ (r0 & 7)) << 4), off1 = (off0 ^ 64u) + 512u;  // rows r0 + 8 i and r0 + 8 i + 4
         bool dead = false;
         Ring2 rb{0, 0u}, rq{0, 0u}, rp{0, 0u};
         uint32_t a_phase = 0;
-        // the chunk whose global loads come next
-        int w = -1, step = 0, nsteps = 0, t = 0;
-        const float *stat = nullptr, *strm = nullptr;
-        int64_t stat_n = 0, strm_n = 0;
+        // the chunk whose global loads come next: steps of the item done and in all; of either operand the place of this
+        // lane's first row in the tile at hand, a row's length, and how many rows from there the prompt still has
+        int step = 0, nsteps = 0, a_left = 0, b_left = 0;
+        const float *pa = nullptr, *pb = nullptr;
+        int64_t an = 0, bn = 0;
         // (only the announcing thread) the next item number, asked for one item ahead
         int ahead = blockIdx.x;
         if (a.next_item && lw == 0 && lane == 0) ahead = atomicAdd(a.next_item, 1);
@@ -218,42 +241,52 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
         auto next_item = [&]() {
             if (lw == 0 && lane == 0) announce();
             warp_wait(q_full + rq.idx, rq.phase, dead, &s_abort);
-            w = dead ? -1 : *(volatile int *)(q_item + rq.idx);
+            const int w = dead ? -1 : *(volatile int *)(q_item + rq.idx);
             __syncwarp();
             if (lane == 0) bar_arrive(q_empty + rq.idx);
             rq.next(kQueue);
-            if (w < 0) return;
-            int sh;
+            if (w < 0) {
+                nsteps = -1;  // (nothing comes after the end)
+                return;
+            }
+            int sh, t;
             decode_item<PASS>(w, a.nsh, a.tiles, a.group, sh, t);
             const int seg = sh / a.H, h = sh - seg * a.H, b = seg / a.L, l = seg - b * a.L;
-            const float *qb = a.q + b * a.qs.b + l * a.qs.l + h * a.qs.h;
-            const float *kb = a.k + b * a.ks.b + l * a.ks.l + h * a.ks.h;
-            stat = PASS == 1 ? qb : kb;
-            strm = PASS == 1 ? kb : qb;
-            stat_n = PASS == 1 ? a.qs.n : a.ks.n;
-            strm_n = PASS == 1 ? a.ks.n : a.qs.n;
+            const float *qb = a.q + b * a.qs.b + l * a.qs.l + h * a.qs.h + c8 * 8;
+            const float *kb = a.k + b * a.ks.b + l * a.ks.l + h * a.ks.h + c8 * 8;
+            const int arow = t * TT + r0, brow = (PASS == 1 ? 0 : t) * TT + r0;
+            an = PASS == 1 ? a.qs.n : a.ks.n;
+            bn = PASS == 1 ? a.ks.n : a.qs.n;
+            pa = (PASS == 1 ? qb : kb) + arow * an;
+            pb = (PASS == 1 ? kb : qb) + brow * bn;
+            a_left = a.N - arow;
+            b_left = a.N - brow;
             step = 0;
             nsteps = KH + KH * (PASS == 1 ? t + 1 : a.tiles - t);
         };
-        // Step s of an item: the stationary chunk c and the first streamed tile's chunk c in turn, then
+        // Steps of an item: the stationary chunk c and the first streamed tile's chunk c in turn, then
         // the chunks of the other streamed tiles.
         auto fetch = [&](float4 (&x)[kVecs], int &where) {
             if (step == nsteps) next_item();
-            if (w < 0) {
+            if (nsteps < 0) {
                 where = -1;
                 return;
             }
-            const bool head = step < 2 * KH;
-            const bool is_a = head && (step & 1) == 0;
-            const int u = head ? step >> 1 : step - KH;  // streamed chunk number (the stationary one: its own)
-            const int c = u % KH;
-            const int tile = is_a ? t : (PASS == 1 ? 0 : t) + u / KH;
-            const float *p = (is_a ? stat : strm) + c * 64 + c4 * 4;
-            const int64_t rn = is_a ? stat_n : strm_n;
+            const bool head = step < 2 * KH, is_a = head && (step & 1) == 0;
+            const int c = KH == 1 ? 0 : head ? step >> 1 : step & 1;
+            const int64_t rn = is_a ? an : bn;
+            const float *p = (is_a ? pa : pb) + c * 64;
+            const int left = is_a ? a_left : b_left;
+            if (!is_a && c == KH - 1) {  // the streamed tile's last chunk
+                pb += TT * bn;
+                b_left -= TT;
+            }
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int i = 0; i < kVecs; ++i) {
-                const int row = tile * TT + r0 + 2 * i;
-                x[i] = row < a.N ? __ldg(reinterpret_cast<const float4 *>(p + row * rn)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int i = 0; i < kRows; ++i) {
+                const float4 *v = reinterpret_cast<const float4 *>(p + 4 * i * rn);
+                x[2 * i] = 4 * i < left ? __ldg(v) : zero;
+                x[2 * i + 1] = 4 * i < left ? __ldg(v + 1) : zero;
             }
             where = is_a ? c : KH;  // which stationary chunk, or KH: the ring
             ++step;
@@ -274,15 +307,16 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
             }
             if (dead) return;
 #pragma unroll
-            for (int i = 0; i < kVecs; ++i) {
-                const int r = r0 + 2 * i;
-                uint2 p0, p1, p2;
-                split2(x[i].x, x[i].y, p0.x, p1.x, p2.x);
-                split2(x[i].z, x[i].w, p0.y, p1.y, p2.y);
-                unsigned char *d = dst + r * 128 + (((c4 >> 1) ^ (r & 7)) << 4) + (c4 & 1) * 8;
-                *reinterpret_cast<uint2 *>(d) = p0;
-                *reinterpret_cast<uint2 *>(d + kPart) = p1;
-                *reinterpret_cast<uint2 *>(d + 2 * kPart) = p2;
+            for (int i = 0; i < kRows; ++i) {
+                uint4 p0, p1, p2;
+                split2(x[2 * i].x, x[2 * i].y, p0.x, p1.x, p2.x);
+                split2(x[2 * i].z, x[2 * i].w, p0.y, p1.y, p2.y);
+                split2(x[2 * i + 1].x, x[2 * i + 1].y, p0.z, p1.z, p2.z);
+                split2(x[2 * i + 1].z, x[2 * i + 1].w, p0.w, p1.w, p2.w);
+                unsigned char *d = dst + (i % 2 == 0 ? off0 : off1) + i / 2 * 1024;
+                *reinterpret_cast<uint4 *>(d) = p0;
+                *reinterpret_cast<uint4 *>(d + kPart) = p1;
+                *reinterpret_cast<uint4 *>(d + 2 * kPart) = p2;
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
@@ -448,6 +482,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
             decode_item<PASS>(w, a.nsh, a.tiles, a.group, sh, t);
             const float sc = a.layer_scale[(sh / a.H) % a.L] * kLog2eT;
             const int grow = t * TT + row;  // query (pass 1) or key (pass 2) of this thread
+            float *kept = MODE == 3 ? a.logits + ((size_t)blockIdx.x * a.tiles * TT + row) * TT : nullptr;
             float run_max = -INFINITY, run_sum = 0.f, col_sum = 0.f;
             if (PASS == 1) {
                 for (int j = 0; j <= t; ++j) {
@@ -461,6 +496,10 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
                         for (int cb = u * U::BLOCKS; cb < (u + 1) * U::BLOCKS && cb <= c_hi; ++cb) {
                             float v[32];
                             load_logits<D>(lane_addr + rs.idx * kBuf + (cb - u * U::BLOCKS) * 32, v);
+                            if (MODE == 3) {
+#pragma unroll
+                                for (int i = 0; i < 32; i += 8) store8(kept + j * TT * TT + cb * 32 + i, v + i);
+                            }
                             if (j == t && cb == warp) {  // the block the causal boundary crosses
 #pragma unroll
                                 for (int i = 0; i < 32; ++i) v[i] = i <= lane ? v[i] : -INFINITY;
@@ -472,7 +511,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
                     const bool redo = run_sum != run_sum && old_sum == old_sum && grow < a.N;
                     if (__any_sync(0xffffffffu, redo)) {
                         if (redo) {
-                            const float2 r = redo_lse<D>(a, sh, grow, j * TT, sc, old_max, old_sum);
+                            const float2 r = redo_lse<D>(a, sh, grow, j * TT, sc, old_max, old_sum, MODE == 3 ? kept + j * TT * TT : nullptr);
                             run_max = r.x;
                             run_sum = r.y;
                         }
@@ -480,7 +519,35 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
                     }
                 }
                 const float lse = run_max + log2f(run_sum);
-                if (MODE == 1) {
+                if (MODE == 3) {
+                    // What the warp's 32 queries give to every key of a tile, four keys to a lane.
+                    __syncwarp();  // (the rows are the warp's own: its lanes' stores are seen from here on)
+                    const int rows = min(32, a.N - t * TT - warp * 32);
+                    const float *back = kept - lane * TT + lane * 4;
+                    float *out = a.partial + ((size_t)sh * (a.tiles * (a.tiles + 1) / 2) + t * (t + 1) / 2) * (4 * TT) + warp * TT + lane * 4;
+                    for (int j = 0; j <= t; ++j) {
+                        float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
+                        const int edge = j == t ? warp * 32 - lane * 4 : TT;  // key e of query i counts when e <= edge + i
+#pragma unroll 1
+                        for (int i0 = 0; i0 < rows; i0 += kBack) {
+                            float4 x[kBack];
+#pragma unroll
+                            for (int i = 0; i < kBack; ++i)  // (rows past the prompt's end have a place too, and are left out below)
+                                x[i] = __ldcg(reinterpret_cast<const float4 *>(back + j * TT * TT + (i0 + i) * TT));
+#pragma unroll
+                            for (int i = 0; i < kBack; ++i) {
+                                const float nl = -__shfl_sync(0xffffffffu, lse, i0 + i);
+                                const int last = i0 + i < rows ? edge + i0 + i : -1;
+                                s0.x += last >= 0 ? ex2(fmaf(x[i].x, sc, nl)) : 0.f;
+                                s0.y += last >= 1 ? ex2(fmaf(x[i].y, sc, nl)) : 0.f;
+                                s1.x += last >= 2 ? ex2(fmaf(x[i].z, sc, nl)) : 0.f;
+                                s1.y += last >= 3 ? ex2(fmaf(x[i].w, sc, nl)) : 0.f;
+                            }
+                        }
+                        *reinterpret_cast<float4 *>(out + j * (4 * TT)) = make_float4(s0.x, s0.y, s1.x, s1.y);
+                    }
+                    __syncwarp();  // the next item's logits go to the same place
+                } else if (MODE == 1) {
                     if (grow < a.N) a.lse2[(size_t)sh * a.N + grow] = lse;
                 } else {
                     // every reader warp needs all 128 normalisers (two buffers in turn, so that
@@ -529,6 +596,34 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
     }
 }
 
+// Mode 3's part sums: 32 keys of a segment to a block, a warp to the heads w, w + 8, ...; the sums of the warps in order.
+__global__ void __launch_bounds__(256) split_mean_kernel(const float *__restrict__ partial, int H, int N, int tiles, float *__restrict__ scores,
+                                                         const int32_t *__restrict__ abort_word)
+{
+    __shared__ float s_sum[8][32];
+    const int blocks = (N + 31) / 32, seg = blockIdx.x / blocks, n = (blockIdx.x - seg * blocks) * 32 + (threadIdx.x & 31), w = threadIdx.x >> 5;
+    const int j = n / TT, all = tiles * (tiles + 1) / 2;
+    dependent_entry();
+    float sum = 0.f;
+    for (int h = w; h < H; h += 8) {
+        const float *p = partial + (size_t)(seg * H + h) * all * (4 * TT) + n % TT;
+        for (int t = j; t < tiles; ++t) {
+            const float *q = p + (size_t)(t * (t + 1) / 2 + j) * (4 * TT);
+            sum += (__ldcg(q) + __ldcg(q + TT)) + (__ldcg(q + 2 * TT) + __ldcg(q + 3 * TT));
+        }
+    }
+    s_sum[w][threadIdx.x & 31] = sum;
+    __syncthreads();
+    if (w != 0 || n >= N) return;
+    for (int i = 1; i < 8; ++i) sum += s_sum[i][threadIdx.x];
+    scores[(size_t)seg * N + n] = *abort_word != 0 ? __int_as_float(0x7fc00000) : sum / (float)H;
+}
+
+// Whether mode 3 takes a prompt, without the caller's log-sum-exp.  Two passes / kept logits, us a call, tokens x heads: heads
+// of 128, 130 x 192 50.2 / 36.2, 300 x 16 27.5 / 19.1, 512 x 128 79.9 / 69.7, 777 x 128 167.5 / 161.2, 900 x 6 48.6 / 44.5, but
+// 1500 x 4 66.2 / 69.8 and x 16 109.8 / 111.9; heads of 64, 256 x 192 45.1 / 35.3, 777 x 128 145.7 / 126.2, 1500 x 4 68.1 / 58.1.
+bool keeps_logits(int tiles, int D) { return tiles >= 2 && tiles <= (D == 128 ? kKeepTiles / 2 : kKeepTiles); }
+
 template <int MODE, int D> int launch_split(const SplitArgs &a, int sms, cudaStream_t st)
 {
     static bool done[64] = {};
@@ -549,24 +644,43 @@ template <int MODE, int D> int launch_split(const SplitArgs &a, int sms, cudaStr
 int launch_head_mean(const float *partial, int H, int N, size_t total, float *scores, const int32_t *abort_word,
                      cudaStream_t st);
 
-// Workspace: partial [rows][N], lse2 [rows][N], then two work counters and the abort word.
-size_t score_split_ws_bytes(const pkv_shape *s)
+// Workspace: partial [rows][N], lse2 [rows][N], then two work counters and the abort word.  Short prompts: part sums of every
+// pair of tiles in the place of these, and the logits of a CTA's item.
+struct SplitSpace {
+    size_t partial, lse2, logits, words, bytes;
+};
+static SplitSpace split_space(const pkv_shape *s)
 {
-    const size_t per = (size_t)s->batch * s->layers * s->heads * s->prompt_len * sizeof(float);
-    return round_up(2 * per, kWsAlign) + kWsAlign;
+    const size_t heads = (size_t)s->batch * s->layers * s->heads, tiles = ((size_t)s->prompt_len + TT - 1) / TT;
+    const size_t per = heads * s->prompt_len * sizeof(float);
+    SplitSpace w = {0, per, 0, 0, 0};
+    size_t end = 2 * per;
+    if (keeps_logits((int)tiles, s->head_dim)) {
+        const size_t parts = heads * (tiles * (tiles + 1) / 2) * (4 * TT) * sizeof(float);
+        const size_t ctas = heads * tiles < kKeepCtas ? heads * tiles : kKeepCtas;
+        w.logits = round_up(parts, kWsAlign);
+        const size_t kept = w.logits + ctas * tiles * TT * TT * sizeof(float);
+        if (kept > end) end = kept;
+    }
+    w.words = round_up(end, kWsAlign);
+    w.bytes = w.words + kWsAlign;
+    return w;
 }
+size_t score_split_ws_bytes(const pkv_shape *s) { return split_space(s).bytes; }
 
 int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const float *k, pkv_strides ks,
                        const float *scale, const float *lse, float *scores, void *ws, cudaStream_t st)
 {
     const int B = s->batch, L = s->layers, H = s->heads, N = s->prompt_len;
-    const size_t per = (size_t)B * L * H * N;
+    const SplitSpace space = split_space(s);
+    unsigned char *mem = (unsigned char *)ws;
     SplitArgs a = {};
     a.q = q; a.k = k; a.qs = qs; a.ks = ks;
     a.layer_scale = scale;
-    a.partial = (float *)ws;
-    a.lse2 = a.partial + per;
-    int *words = (int *)((unsigned char *)ws + round_up(2 * per * sizeof(float), kWsAlign));
+    a.partial = (float *)(mem + space.partial);
+    a.lse2 = (float *)(mem + space.lse2);
+    a.logits = (float *)(mem + space.logits);
+    int *words = (int *)(mem + space.words);
     a.abort_word = words + 2;
     a.L = L; a.H = H; a.N = N;
     a.tiles = (N + TT - 1) / TT;
@@ -575,7 +689,7 @@ int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const
     const int sms = sm_count();
     if (sms <= 0) return PKV_ERR_CUDA;
     // With an item for every CTA there is nothing to hand out: no counter, and so nothing to zero first.
-    const bool counted = a.nsh * a.tiles > sms;
+    const bool counted = a.nsh * a.tiles > (sms < (int)kKeepCtas ? sms : (int)kKeepCtas);
     if (counted) {
         cudaError_t e = cudaMemsetAsync(words, 0, 4 * sizeof(int), st);
         if (e != cudaSuccess) {
@@ -589,6 +703,18 @@ int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const
     if (!lse && a.tiles == 1) {
         a.next_item = counted ? words : nullptr;
         rc = wide ? launch_split<0, 128>(a, sms, st) : launch_split<0, 64>(a, sms, st);
+    } else if (!lse && keeps_logits(a.tiles, s->head_dim)) {
+        a.next_item = counted ? words : nullptr;
+        const int ctas = sms < (int)kKeepCtas ? sms : (int)kKeepCtas;
+        rc = wide ? launch_split<3, 128>(a, ctas, st) : launch_split<3, 64>(a, ctas, st);
+        if (rc != PKV_OK) return rc;
+        cudaError_t e = launch_dependent(split_mean_kernel, dim3((unsigned)((size_t)B * L * ((N + 31) / 32))), dim3(256), 0, st, a.partial, H, N, a.tiles, scores,
+                                         a.abort_word);
+        if (e != cudaSuccess) {
+            set_cuda_error(e, "split_mean_kernel");
+            return PKV_ERR_CUDA;
+        }
+        return PKV_OK;
     } else {
         if (!lse) {
             a.next_item = counted ? words : nullptr;

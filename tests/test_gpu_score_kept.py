@@ -1,0 +1,59 @@
+"""fp32 prompts whose logits are kept for the column sums (2 to 8 tiles of 128 tokens, 16 with heads of 64) and the lengths
+around them (needs a B200).  Against 64 bits."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2412_03409_b200.session import Session
+
+pytestmark = pytest.mark.gpu
+
+# An fp32 logit is off by up to 2^-22 of the sum of its terms' magnitudes (here below 30): 7e-6; a probability as much of itself,
+# and a score is a mean of sums of them.
+TOL = 2e-5
+
+
+def _exact(q, k, scale):
+    x = torch.matmul(q.double(), k.double().transpose(-1, -2)) * torch.from_numpy(scale).double().cuda()[None, :, None, None, None]
+    later = torch.ones(x.shape[-2:], dtype=torch.bool, device="cuda").triu(1)
+    return torch.softmax(x.masked_fill_(later, -float("inf")), -1).masked_fill_(later, 0).sum(-2).mean(2)
+
+
+@pytest.mark.parametrize("B,L,H,D,N", [
+    (1, 1, 1, 64, 129), (1, 2, 3, 128, 129), (1, 1, 9, 64, 255), (2, 1, 8, 128, 256), (1, 3, 5, 64, 257), (1, 1, 2, 128, 1000),
+    (1, 1, 2, 128, 1024), (1, 1, 2, 128, 1025), (1, 1, 1, 64, 1921), (1, 1, 1, 64, 2048), (1, 1, 1, 64, 2049),
+    (1, 12, 16, 64, 150),      # more items than CTAs
+    (3, 9, 17, 128, 130),
+])
+@pytest.mark.parametrize("sign", [1, -1])
+def test_scores(B, L, H, D, N, sign):
+    g = torch.Generator(device="cuda").manual_seed(N * 3 + H)
+    # heads and tokens in another order than the shape's
+    q = torch.randn(B, L, N, H, D, device="cuda", generator=g).transpose(2, 3)
+    k = (torch.randn(B, L, H, N, D + 4, device="cuda", generator=g) * 2)[..., :D]
+    scale = sign * np.linspace(0.5, 1.5, L).astype(np.float32) / np.float32(np.sqrt(D))
+    s = Session(B, L, H, D, N, torch.float32, scale, decode_cap=0, max_budget_rows=L)
+    s.scores.fill_(float("nan"))
+    got = s.score(q, k).clone()
+    ref = _exact(q, k, scale)
+    assert ((got.double() - ref).abs() / ref.clamp(min=1e-3)).max().item() <= TOL
+    s.ws_score.fill_(255)      # over a workspace of NaN words
+    assert torch.equal(got, s.score(q, k))
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf"), 3.4e38])
+def test_elements_that_have_no_split(D, bad):
+    """What a NaN query or an infinite key does to the other keys is what the definition has, and no more."""
+    N = 400
+    g = torch.Generator(device="cuda").manual_seed(D)
+    q, k = (torch.randn(1, 1, 2, N, D, device="cuda", generator=g) for _ in range(2))
+    scale = np.full(1, D ** -0.5, np.float32)
+    q[..., 0] = 2.0 ** -122 if bad == 3.4e38 else q[..., 0].abs() + 1
+    (q if np.isnan(bad) else k)[0, 0, 1, 200, 0] = bad
+    s = Session(1, 1, 2, D, N, torch.float32, scale, decode_cap=0, max_budget_rows=1)
+    got, ref = s.score(q, k)[0, 0].double(), _exact(q, k, scale)[0, 0]
+    assert torch.equal(torch.isnan(got), torch.isnan(ref))
+    ok = ~torch.isnan(ref)
+    assert bool(ok.any()) or bad == float("inf")
+    assert bool((((got - ref).abs() / ref.clamp(min=1e-3))[ok] <= TOL).all())
