@@ -27,7 +27,8 @@
 // take all of shared memory's bandwidth; storing the split ones takes 768 more.  It takes 5250: the issuing warp
 // waits 1250 of them for chunks.  Pairs of CTAs (cta_group::2, a streamed row split once for two tiles): 198 us.
 // Sixteen loader warps leave 80 registers a thread and spill (211 us).  4 layers x 4 heads of 64, 300 tokens:
-// 17.4 us (26.9 in two passes before), 128 tokens (one tile each): 10.9 us for the call (30.7 with three FMA kernels).
+// 17.4 us (26.9 in two passes before), 128 tokens (one tile each): 10.2 us for the call (11.3 with the mean in a launch of its
+// own, 30.7 with three FMA kernels).
 // Reading the logits back: eight rows at a time 168 us, sixteen 161; by three warps of their own 177-187; kept in blocks that
 // pass through shared memory 177-206 (memory's latency, not the stores, is what the warps wait for).
 #include "score_tiles.cuh"
@@ -46,6 +47,7 @@ static_assert(kRing == 2, "with two chunks a tile, chunk c of every tile goes th
 constexpr uint32_t kPart = TT * 128;         // bytes of one bf16 part of a chunk: 128 rows x 64 elements
 constexpr uint32_t kChunk = 3 * kPart;
 constexpr uint32_t kBuf = 256;               // tensor-memory columns of one of the two accumulator buffers
+constexpr int kMeanHeads = 8;                // CTAs of a portable cluster
 constexpr int kKeepTiles = 16;               // tiles of the longest prompt whose logits are kept (1 MiB a CTA), heads of 64
 constexpr size_t kKeepCtas = 148;            // CTAs of such a call at most
 constexpr int kBack = 16;                    // rows of them a warp reads back at a time
@@ -60,6 +62,7 @@ struct SplitArgs {
     float *lse2;          // pass 1 out, same layout, log2 domain
     float *partial;       // [B*L*H][N] per-head column sums; mode 3: [B*L*H][pairs of a query and a key tile][quarter of the queries][128]
     float *logits;        // mode 3: [CTA][tiles][128 queries][128 keys], of the item at hand
+    float *scores;        // mode 0 by clusters (below): [B*L][N], or NULL
     int32_t *abort_word;  // set when a bounded wait runs out: the head mean then writes NaN scores
     int *next_item;       // work counter of this pass, zeroed before it; NULL: a CTA takes item blockIdx.x alone
     int clear_abort;      // this launch is the call's first and nothing has zeroed the abort word
@@ -152,11 +155,20 @@ __device__ __noinline__ float redo_colsum(const SplitArgs &a, int sh, int key, i
     return sum;
 }
 
+// Store into the first CTA of the cluster, at the place that `p` has in this CTA's shared memory.
+__device__ __forceinline__ void store_in_first(float *p, float v)
+{
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(saddr(p)));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
+}
+
 // MODE 3: as MODE 1, and the item's logits are kept (64 KiB a tile, which mostly stay in the L2); once a query's
 // normaliser is known, the reader warp that has its row reads them back and adds up what the warp's queries give to every
 // key: the second pass without its products and splits.
 // MODE 1: stationary = Q tile t, streamed = K tiles 0..t (log-sum-exp).  MODE 2: stationary = K tile
-// t, streamed = Q tiles t..tiles-1 (column sums).  MODE 0: one tile, Q stationary, both results.
+// t, streamed = Q tiles t..tiles-1 (column sums).  MODE 0: one tile, Q stationary, both results.  With a CTA for every
+// head and at most eight heads a segment's CTAs are a cluster, whose first one takes the mean: no second launch.
 template <int MODE, int D>
 __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __grid_constant__ SplitArgs a)
 {
@@ -173,6 +185,8 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
     __shared__ int s_abort;
     __shared__ int q_item[kQueue];
     __shared__ __align__(16) float s_lse[2][kReaders][TT];
+    __shared__ float s_col[MODE == 0 ? TT : 1], s_cols[MODE == 0 ? kMeanHeads : 1][TT];  // column sums; (first CTA) those of all heads
+    __shared__ int s_gave_up[kMeanHeads];
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int nitems = a.nsh * a.tiles;
@@ -205,6 +219,9 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    const bool by_cluster = MODE == 0 && a.scores != nullptr;
+    // (the first CTA must be running before anyone writes to its shared memory)
+    if (by_cluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     fence_before();
     __syncthreads();
     fence_after();
@@ -559,7 +576,8 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
                     sum_tile(s_lse[flip][0], sh, grow, t, true, sc, col_sum);
                     flip ^= 1;
                     if (flip == 0) lse_phase ^= 1u;
-                    if (grow < a.N) a.partial[(size_t)sh * a.N + grow] = col_sum;
+                    if (by_cluster) s_col[row] = col_sum;
+                    else if (grow < a.N) a.partial[(size_t)sh * a.N + grow] = col_sum;
                 }
             } else {
                 const float *lrow = a.lse_in + (size_t)sh * a.N;
@@ -589,10 +607,28 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
     fence_before();
     __syncthreads();
     fence_after();
-    if (tid == 0 && s_abort) atomicExch(a.abort_word, (int)PKV_DEV_TIMEOUT);
+    if (tid == 0 && s_abort && !by_cluster) atomicExch(a.abort_word, (int)PKV_DEV_TIMEOUT);
     if (warp == kReaders) {
         __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * kBuf) : "memory");
+    }
+    if (MODE == 0 && by_cluster) {
+        const int seg = blockIdx.x / a.H, h = blockIdx.x - seg * a.H;
+        asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+        if (tid < TT) store_in_first(&s_cols[h][tid], s_col[tid]);
+        if (tid == 0) store_in_first(reinterpret_cast<float *>(s_gave_up + h), __int_as_float(s_abort));
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        if (h != 0) return;  // (only the first CTA's memory is written, and it waits for everyone)
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (tid < a.N) {  // (at most a tile)
+            float sum = 0.f;
+            int gave_up = 0;
+            for (int i = 0; i < a.H; ++i) {
+                sum += s_cols[i][tid];
+                gave_up |= s_gave_up[i];
+            }
+            a.scores[(size_t)seg * a.N + tid] = gave_up ? __int_as_float(0x7fc00000) : sum / (float)a.H;
+        }
     }
 }
 
@@ -631,7 +667,20 @@ template <int MODE, int D> int launch_split(const SplitArgs &a, int sms, cudaStr
     int rc = ensure_dynamic_smem((const void *)score_split_kernel<MODE, D>, (int)smem, done);
     if (rc != PKV_OK) return rc;
     const int items = a.nsh * a.tiles;
-    cudaError_t e = launch_dependent(score_split_kernel<MODE, D>, dim3(items < sms ? items : sms), dim3(kSplitThreads), smem, st, a);
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)a.H;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(items < sms ? items : sms);
+    cfg.blockDim = dim3(kSplitThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.scores ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, score_split_kernel<MODE, D>, a);
     if (e != cudaSuccess) {
         set_cuda_error(e, "score_split_kernel");
         return PKV_ERR_CUDA;
@@ -702,6 +751,12 @@ int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const
     int rc = PKV_OK;
     if (!lse && a.tiles == 1) {
         a.next_item = counted ? words : nullptr;
+        // (clusters that run at once: 12 segments of 8 heads 13.7 -> 10.5 us, 6 of 3 12.3 -> 10.7, but 16 of 8, 128 CTAs
+        // of 148 SMs, take two waves, 13.9 -> 19.5)
+        if (3 * a.nsh <= 2 * sms && H <= kMeanHeads) {
+            a.scores = scores;
+            return wide ? launch_split<0, 128>(a, sms, st) : launch_split<0, 64>(a, sms, st);
+        }
         rc = wide ? launch_split<0, 128>(a, sms, st) : launch_split<0, 64>(a, sms, st);
     } else if (!lse && keeps_logits(a.tiles, s->head_dim)) {
         a.next_item = counted ? words : nullptr;

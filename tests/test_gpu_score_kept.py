@@ -41,6 +41,21 @@ def test_scores(B, L, H, D, N, sign):
     assert torch.equal(got, s.score(q, k))
 
 
+# one tile: a cluster of a segment's heads takes the mean up to eight heads and 98 in all
+@pytest.mark.parametrize("B,L,H,D,N", [(1, 1, 1, 128, 128), (1, 4, 4, 64, 128), (1, 3, 7, 64, 65), (2, 6, 8, 128, 127), (1, 7, 7, 128, 90),
+                                       (1, 14, 7, 64, 100), (1, 33, 3, 64, 100), (1, 2, 9, 128, 100), (2, 8, 8, 64, 66)])
+def test_one_tile(B, L, H, D, N):
+    g = torch.Generator(device="cuda").manual_seed(N + L)
+    q, k = (torch.randn(B, L, H, N, D, device="cuda", generator=g) for _ in range(2))
+    q[0, L - 1, H - 1, N // 2, 3] = float("nan")
+    scale = np.linspace(0.5, 1.5, L).astype(np.float32) / np.float32(np.sqrt(D))
+    s = Session(B, L, H, D, N, torch.float32, scale, decode_cap=0, max_budget_rows=L)
+    got = [s.score(q, k).clone() for _ in range(3)]
+    ref = _exact(q, k, scale)
+    assert torch.equal(torch.isnan(got[0]), torch.isnan(ref)) and torch.equal(got[0].nan_to_num(7.0), got[2].nan_to_num(7.0))
+    assert ((got[0].double() - ref).abs() / ref.clamp(min=1e-3)).nan_to_num(0.0).max().item() <= TOL
+
+
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf"), 3.4e38])
 def test_elements_that_have_no_split(D, bad):
