@@ -71,7 +71,7 @@ def measured_peaks():
 
 
 # Which kernel a decode call takes: the library's rules (launch_decode_cluster and launch_decode_heads)
-# restated for the workloads below (the cluster kernel's line for long segments is far from them), for the
+# restated for the workloads below (the cluster kernel's line for long segments of few pairs is far from them), for the
 # kernel's name, the launch count and the traffic figure.
 DECODE_KERNELS = {
     "cluster": ("decode_cluster_kernel", "decode_cluster.cu", "decode_cluster_kernel(const ClusterArgs a)", 1),
@@ -82,9 +82,23 @@ DECODE_KERNELS = {
 
 def decode_path(w, sms):
     nact = w.B * w.L
-    if nact * w.H < 4 * sms:
-        return "cluster"
+    pairs = nact * w.H
     cap_rows = w.B * (min(w.budget_rows(), w.L * w.N) + w.L * w.T)       # as Session sizes the cache
+    kb = (cap_rows // nact - w.T // 2) * w.D * 2 * w.esize >> 10
+    if pairs < 4 * sms:
+        return "cluster"
+    if pairs <= 5 * sms:
+        cluster = kb <= 256
+    elif pairs <= 6 * sms:
+        cluster = kb <= 176
+    elif pairs <= 7 * sms:
+        cluster = kb <= 96
+    elif pairs < 10 * sms:
+        cluster = 96 <= kb <= 256
+    else:
+        cluster = kb >= (96 if nact > 256 else 64) and (pairs >= 20 * sms or kb <= 320)
+    if cluster:
+        return "cluster"
     heads = w.D in (64, 128) and nact <= 256 and cap_rows // nact <= 1024
     return "heads" if heads else "stream"
 

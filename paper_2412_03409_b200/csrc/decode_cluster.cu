@@ -1,7 +1,8 @@
-// Decode attention over the ragged cache (Sec. 3.1, Fig. 2a) for calls with few (segment, head)
-// pairs: a layer at a time, or a few layers, of a small batch.
+// Decode attention over the ragged cache (Sec. 3.1, Fig. 2a), (segment, head) pair by pair: calls with few pairs (a layer at
+// a time, or a few layers, of a small batch) by a cluster of CTAs to a pair, most others by a CTA to a pair
+// (launch_decode_cluster has the lines).
 //
-// Such a call moves a few megabytes, so what counts is the chain of latencies of one launch and that
+// A call of few pairs moves a few megabytes, so what counts is the chain of latencies of one launch and that
 // every SM has a share.  A cluster of C CTAs takes one (segment, head); each CTA takes a C-th of its
 // rows.  Every warp copies its rows' slices of the head into a ring of its own with 16-byte cp.async
 // and reads back what the same lane copied, so that no warp waits for another until the merge.  The
@@ -26,7 +27,9 @@
 // first's latency, 4-5 us (C = 8 for 4 x 32 x 128 rows: 8.9 us), hence the choice of C below.  Loads to
 // registers instead of the rings, eight steps of K and V in flight: the same for one round of rows,
 // 20.5 us for 8 x 40 x 410.  Ring shapes (steps, rounds, CTAs per SM): 4, 2, 5 as here; 8, 2, 3 and
-// 4, 3, 4 18.9-19.4 us there; 2, 4, 5 18.7.  Clusters of 12 or 16: slower throughout.
+// 4, 3, 4 18.9-19.4 us there; 2, 4, 5 18.7.  With a CTA to a pair (1024 of 136 rows / 4096 of 820; 17.4 / 259 us as here): one warp
+// with four to eight rounds in flight 23.1-29.2 / 336-396, two 19.5-21 / 300, eight 19.8 / 262; a loop over several pairs with the next
+// one's rows under way, 10-18 % slower throughout.  Clusters of 12 or 16: slower throughout.
 #include "decode_plan.cuh"
 
 namespace pkv {
@@ -36,11 +39,10 @@ bool decode_stream_covers(const pkv_shape *s, int nact);
 namespace {
 
 constexpr int kCWarps = 4;             // warps per CTA
-constexpr int kCU = 4;                 // row steps of a round
 constexpr int kCStages = 2;            // rounds in flight per warp
-constexpr int kCPerSm = 5;             // CTAs an SM holds at a time (their rings fill its shared memory)
-constexpr uint32_t kCRound = kCU * 512;  // bytes of a round's K (or V) rows: a warp reads 512 bytes per step
+constexpr int kCPerSm = 5;             // CTAs an SM holds at a time, rounds of four steps (their rings fill its shared memory)
 constexpr int kCMaxCluster = 8;        // portable cluster size
+constexpr int kCSmShared = 228 * 1024; // an SM's shared memory; a CTA takes 1 KiB more than it asks for
 constexpr float kLog2eC = 1.4426950408889634f;
 constexpr float kNoLogit = -3.402823466e38f;  // the lowest finite number
 
@@ -51,6 +53,7 @@ struct ClusterArgs {
     const float *layer_scale;
     int32_t *dev_status;
     int H, visit_shift;  // a length's word counts its readers from this bit on
+    uint32_t guess_mask;  // what a length read ahead is taken from: the word without that count, where CTAs come in waves
     uint32_t row_bytes;
 };
 
@@ -80,9 +83,12 @@ __device__ __forceinline__ void copy16(void *dst, const unsigned char *src)
 
 // A head's slice of a row is D * sizeof(T) bytes: LPR lanes share a row, a warp reads G = 32 / LPR
 // rows per step.
-template <typename T, int D>
-__global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(const ClusterArgs a)
+// A round is U steps; an SM holds P CTAs (their rings and registers are cut for that).
+template <typename T, int D, int U, int P>
+__global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const ClusterArgs a)
 {
+    constexpr int kCU = U;
+    constexpr uint32_t kCRound = U * 512;  // bytes of a round's K (or V) rows: a warp reads 512 bytes per step
     constexpr int VE = RowVec<T>::VE;
     constexpr uint32_t SLICE = D * sizeof(T);
     constexpr int LPR = SLICE / 16, G = 32 / LPR;
@@ -90,7 +96,7 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
     static_assert(kCWarps * 32 >= D, "a thread per element of the output");
     extern __shared__ __align__(16) unsigned char s_ring[];  // [kCWarps][kCStages][K, V][kCRound]
     __shared__ float s_acc[kCWarps][D], s_ml[kCWarps][2];
-    __shared__ float c_acc[kCMaxCluster][D], c_ml[kCMaxCluster][2];  // (first CTA) the cluster's partials
+    __shared__ float c_acc[P == kCPerSm ? kCMaxCluster : 1][D], c_ml[kCMaxCluster][2];  // (first CTA of a cluster) the cluster's partials
 
     __shared__ SegPlan s_plan[2];
 
@@ -136,6 +142,8 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    // A length's word: the length, and above it how many of the segment's CTAs have been there.
+    const uint32_t ln_mask = a.p.append ? (1u << a.visit_shift) - 1u : 0xffffffffu;
     // Where the rows are is read before the kernel in front has completed, and the first rounds are asked for as soon
     // as it has, together with the plan that counts.  Should that one be another, they are asked for again.
     const bool guesses = a.p.evict_distance == 0;
@@ -163,7 +171,7 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
     }
     Rows rw{nullptr, nullptr, 0, 0, -1};
     if (guesses) {
-        rw = rows_of(plan_of(a.p, guess_ln, guess_cp, guess_off, PruneState{0, 0, -1}));
+        rw = rows_of(plan_of(a.p, (int)((uint32_t)guess_ln & a.guess_mask), guess_cp, guess_off, PruneState{0, 0, -1}));
 #pragma unroll
         for (int i = 0; i < kCStages; ++i) request(rw, rw.r0 + (warp + i * kCWarps) * STEP, i);
     }
@@ -176,8 +184,7 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
     const float sc = a.layer_scale[a.p.layer_begin + si % a.p.nl] * kLog2eC;
     if (tid == 0) {
         const uint32_t before = a.p.append ? word >> a.visit_shift : 0u, all = (uint32_t)(a.H * C);
-        const int ln = a.p.append ? (int)(word & ((1u << a.visit_shift) - 1u)) : (int)word;
-        SegPlan sp = plan_of(a.p, ln, cp, off, ps);
+        SegPlan sp = plan_of(a.p, (int)(word & ln_mask), cp, off, ps);
         if (before >= all) sp.rows = -1;  // (the word was no length)
         if (sp.rows < 0) {  // (every CTA finds the same, and takes back what it added)
             raise_status(a.dev_status, si / a.p.nl, PKV_DEV_CAPACITY);
@@ -327,11 +334,17 @@ __global__ void __launch_bounds__(kCWarps * 32, kCPerSm) decode_cluster_kernel(c
         reinterpret_cast<T *>(static_cast<unsigned char *>(a.out) + hoff)[tid] = from_float<T>(sp.rows < 0 ? 0.f : o * (1.f / z));
 }
 
-template <typename T, int D> int launch_cluster(const ClusterArgs &a, int C, cudaStream_t st)
+template <typename T, int D, int U, int P> int launch_cluster(const ClusterArgs &a, int C, cudaStream_t st)
 {
-    constexpr int smem = kCWarps * kCStages * 2 * (int)kCRound;
+    // Room for P CTAs and not for one more.  (Clusters have the first shape; the others need no place for partials.)
+    constexpr int rings = kCWarps * kCStages * 2 * U * 512;
+    // (its static part, rounded up, and what every CTA takes)
+    constexpr int fixed = kCWarps * (D + 2) * (int)sizeof(float) + (P == kCPerSm ? kCMaxCluster : 1) * D * (int)sizeof(float) + 1344;
+    constexpr int one_more = kCSmShared / (P + 1) - fixed + 512;
+    constexpr int smem = rings > one_more ? rings : one_more;
+    static_assert(P * (smem + fixed) <= kCSmShared, "P CTAs fit");
     static bool smem_done[64] = {};
-    int rc = ensure_dynamic_smem((const void *)decode_cluster_kernel<T, D>, smem, smem_done);
+    int rc = ensure_dynamic_smem((const void *)decode_cluster_kernel<T, D, U, P>, smem, smem_done);
     if (rc != PKV_OK) return rc;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -346,12 +359,18 @@ template <typename T, int D> int launch_cluster(const ClusterArgs &a, int C, cud
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, decode_cluster_kernel<T, D>, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, decode_cluster_kernel<T, D, U, P>, a);
     if (e != cudaSuccess) {
         set_cuda_error(e, "decode_cluster_kernel");
         return PKV_ERR_CUDA;
     }
     return PKV_OK;
+}
+template <int U, int P> int launch_shape(const pkv_shape *s, const ClusterArgs &a, int C, cudaStream_t st)
+{
+    if (s->dtype == PKV_BF16)
+        return s->head_dim == 128 ? launch_cluster<__nv_bfloat16, 128, U, P>(a, C, st) : launch_cluster<__nv_bfloat16, 64, U, P>(a, C, st);
+    return s->head_dim == 128 ? launch_cluster<float, 128, U, P>(a, C, st) : launch_cluster<float, 64, U, P>(a, C, st);
 }
 
 }  // namespace
@@ -363,9 +382,30 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     const int H = s->heads, D = s->head_dim, nl = le - lb, nact = s->batch * nl;
     const int sms = sm_count();
     if (sms <= 0) return PKV_ERR_CUDA;
-    if ((int64_t)nact * H >= 4 * (int64_t)sms) return -1;  // (the per-head kernel's and the row-split kernel's calls)
-    const int items = nact * H;
-    const int64_t seg_rows = c->total_cap_rows / ((int64_t)s->batch * s->layers);
+    const int64_t items = (int64_t)nact * H, seg_rows = c->total_cap_rows / ((int64_t)s->batch * s->layers);
+    const int64_t pair_bytes = seg_rows * D * 2 * (int64_t)esize(s);
+    const int wave = kCPerSm * sms;
+    if (items >= 4 * (int64_t)sms) {
+        // A CTA for every pair.  Measured, the per-head (or row-split) kernel / this one, us a call, bf16, heads of 128, lengths alike and
+        // from 0.3 to 1.7 of the mean.  One wave: 640 pairs of 30 rows 7.5 / 4.9, 8.4 / 5.4, of 128 12.7 / 10.4, 13.4 / 11.6, of 400
+        // 28.3 / 25.6, 28.7 / 28.6, but of 820 48.9 / 48.6, 46.9 / 50.2: the longest pairs end alone.  740 pairs of 128 14.0 / 12.0.
+        // Up to seven CTAs an SM, in one wave too: 800 x 64 11.2 / 9.1, x 256 22.7 / 22.3, 26.7 / 24.4, x 400 33.1 / 31.8, 33.8 / 35.2, 1024 x 30 8.9 / 7.1, 10.2 / 7.4, x 128 16.6 / 15.5, 18.0 / 16.5,
+        // but x 256 26.1 / 27.1, 31.8 / 30.1, x 400 38.8 / 39.6, 39.8 / 43.5.  More waves: CTAs that begin cost the first rows' latency,
+        // which is little against long rows, and is hidden where lengths differ, as they do after a search: 1280 x 256 31.9 / 33.1,
+        // 38.4 / 31.9, 1536 x 384 54.5 / 54.2, 55.3 / 52.7, 2048 x 64 20.0 / 21.4, 19.9 / 20.6, x 128 27.6 / 29.5, 28.8 / 28.1, x 256 46.5 / 48.3,
+        // 52.1 / 48.1, 1600 x 820 104.4 / 107.4, 107.1 / 110.2, 4096 x 128 50.7 / 51.9, 52.3 / 50.9, x 400 130.7 / 128.1, 143.9 / 129.8, 8192 x 400
+        // 257 / 248, 284 / 247; against the row-split kernel 12800 x 410 395 / 377, 16384 x 128 174 / 177, x 256 343 / 313;
+        // with pruning 640 x 64 17.0 / 10.3, 4096 x 64 33.9 / 36.7, x 200 75.3 / 74.1.
+        // By a pair's bytes halfway through the tokens that the cache has room for.
+        const int64_t kb = (seg_rows - c->decode_cap / 2) * D * 2 * (int64_t)esize(s) >> 10;
+        bool here;
+        if (items <= wave) here = kb <= 256;
+        else if (items <= 6 * (int64_t)sms) here = kb <= 176;
+        else if (items <= 7 * (int64_t)sms) here = kb <= 96;
+        else if (items < 10 * (int64_t)sms) here = kb >= 96 && kb <= 256;
+        else here = kb >= (nact > 256 || c->evict_distance > 0 ? 96 : 64) && (items >= 20 * (int64_t)sms || kb <= 320) && items <= INT32_MAX / 2;
+        if (!here) return -1;
+    }
     // Long segments are the row-split kernel's, where it covers the shape: eight CTAs of a pair keep 256 KiB in
     // flight however long it is, and CTAs that come in waves read the slices of a row at different times.
     // Measured, one layer, this kernel / row-split.  Few pairs, by a pair's bytes: 1 head of 128, bf16, 12000 rows
@@ -375,8 +415,8 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     // rows: 128 x 6000 rows 73 / 73, x 12000 137 / 130; 320 x 1800 58 / 59, x 3200 86 / 92; 512 x 1100 55 / 59, x
     // 1800 89 / 83 (heads of 64: 34 / 36, 55 / 49); 576 x 1100 60 / 60, x 1800 96 / 90; and by bytes: 64 pairs of 8000 rows of fp32
     // (524 MB) 90 / 90, 12000 134 / 126.
-    const int64_t pair_bytes = seg_rows * D * 2 * (int64_t)esize(s);
-    if ((pair_bytes > ((int64_t)(items < 24 ? 6 : 12) << 20) || items * seg_rows > (items <= 320 ? 1 << 20 : 704 << 10) ||
+    if (items < 4 * (int64_t)sms &&
+        (pair_bytes > ((int64_t)(items < 24 ? 6 : 12) << 20) || items * seg_rows > (items <= 320 ? 1 << 20 : 704 << 10) ||
          items * pair_bytes > ((int64_t)512 << 20)) &&
         decode_stream_covers(s, nact))
         return -1;
@@ -384,10 +424,10 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     // the call is so small that SMs would be idle; further waves only for CTAs of 256 rows and more,
     // whose bytes outweigh a wave's latency (16 x 32 x 2048 rows: C = 1 111 us, 6 89 us in one run, 99 in another).
     int C = 1;
-    while (C < kCMaxCluster) {
+    while (C < kCMaxCluster && items < 4 * (int64_t)sms) {
         const int n = C + 1;
-        const bool one_wave = (int64_t)items * n <= (int64_t)kCPerSm * sms &&
-                              (seg_rows >= 32 * n || (int64_t)items * n <= 2 * (int64_t)sms);
+        const bool one_wave = items * n <= wave &&
+                              (seg_rows >= 32 * n || items * n <= 2 * (int64_t)sms);
         if (!one_wave && seg_rows < 256 * (int64_t)n) break;
         C = n;
     }
@@ -401,11 +441,13 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     a.q = q; a.k_new = kn; a.v_new = vn; a.ck = c->k; a.cv = c->v; a.out = out;
     a.layer_scale = scale;
     a.visit_shift = 32 - visit_bits;
+    a.guess_mask = kn != nullptr && items * C > wave ? (1u << a.visit_shift) - 1u : 0xffffffffu;
     a.dev_status = dev_status;
     a.H = H;
     a.row_bytes = (uint32_t)((size_t)H * D * esize(s));
-    if (s->dtype == PKV_BF16) return D == 128 ? launch_cluster<__nv_bfloat16, 128>(a, C, st) : launch_cluster<__nv_bfloat16, 64>(a, C, st);
-    return D == 128 ? launch_cluster<float, 128>(a, C, st) : launch_cluster<float, 64>(a, C, st);
+    if (C == 1 && items > wave && items <= 6 * (int64_t)sms) return launch_shape<4, 6>(s, a, C, st);
+    if (C == 1 && items > wave && items <= 7 * (int64_t)sms) return launch_shape<3, 7>(s, a, C, st);
+    return launch_shape<4, kCPerSm>(s, a, C, st);
 }
 
 }  // namespace pkv

@@ -96,9 +96,9 @@ __device__ __forceinline__ PruneState prune_state(const DecodePlanArgs &a, int s
     PruneState s{0, 0, -1};
     const int d = a.append ? a.evict_distance : 0;
     if (d > 0) {
-        s.g = load_l2(a.gen + seg);
-        s.len0 = load_l2(a.len0 + seg);
-        if (s.g >= d) s.slot = load_l2(a.slot_ring + (size_t)seg * (d + 1) + (s.g - d) % (d + 1));
+        s.g = a.gen[seg];
+        s.len0 = a.len0[seg];
+        if (s.g >= d) s.slot = a.slot_ring[(size_t)seg * (d + 1) + (s.g - d) % (d + 1)];
     }
     return s;
 }
@@ -131,9 +131,7 @@ __device__ __forceinline__ SegPlan plan_of(const DecodePlanArgs &a, int ln, int 
 __device__ __forceinline__ SegPlan segment_plan(const DecodePlanArgs &a, int si)
 {
     const int seg = (si / a.nl) * a.L + a.layer_begin + si % a.nl;
-    const int ln = load_l2(a.len + seg), cp = load_l2(a.cap + seg);
-    const int64_t off = load_l2(a.row_offset + seg);
-    return plan_of(a, ln, cp, off, prune_state(a, seg));
+    return plan_of(a, a.len[seg], a.cap[seg], a.row_offset[seg], prune_state(a, seg));
 }
 // Writes what the step leaves for the next one: the length and, with pruning, the token's place.
 // (Only one thread of the call touches a segment's token count and slot ring.)

@@ -65,6 +65,35 @@ def test_tokens_back_to_back(B, L, H, D, lens, dtype, layerwise):
             assert (outs[t][i // L, i % L].double() - ref).abs().max().item() <= TOL[dtype], (i, t)
 
 
+# a CTA to a pair: one wave of five, six and seven CTAs an SM (740, 888, 1036 pairs on a B200) and the next pair after
+# each, and several waves (pairs of 64 KiB and more, 96 with more than 256 segments); the wrong side of each line goes elsewhere
+@pytest.mark.parametrize("B,L,H,D,rows,dtype", [
+    (1, 37, 20, 128, 60, torch.bfloat16), (1, 13, 57, 64, 33, torch.bfloat16), (1, 24, 37, 64, 20, torch.float32), (1, 127, 7, 64, 50, torch.bfloat16),
+    (2, 14, 37, 128, 30, torch.bfloat16), (1, 17, 61, 128, 230, torch.bfloat16), (1, 20, 74, 64, 300, torch.bfloat16), (2, 25, 32, 128, 140, torch.bfloat16),
+    (1, 20, 80, 128, 70, torch.float32), (8, 33, 6, 128, 210, torch.bfloat16), (8, 33, 8, 64, 500, torch.bfloat16),
+])
+def test_a_cta_to_a_pair(B, L, H, D, rows, dtype):
+    rng = np.random.default_rng(rows)
+    lens = [int(x) for x in rng.integers(1, 2 * rows, B * L)]
+    T = 3
+    s, tok = _session(B, L, H, D, lens, dtype, T)
+    outs = [torch.empty_like(tok[0][0]) for _ in range(T)]
+    torch.cuda.synchronize()
+    for t in range(T):
+        s.decode(*tok[t], out=outs[t])
+    again = s.decode(tok[0][0], None, None) if H <= 64 else None
+    torch.cuda.synchronize()
+    assert s.cache.len.tolist() == [n + T for n in lens] and s.status.tolist() == [0] * B
+    for i in sorted({0, 1, B * L // 2, B * L - 1}):
+        n, o = lens[i], int(s.cache.row_offset[i])
+        for t in range(T):
+            assert torch.equal(s.cache.v[o + n + t].reshape(H, D), tok[t][2][i // L, i % L])
+            ref = _attend(s, tok[t][0], i, n + t + 1)
+            assert (outs[t][i // L, i % L].double() - ref).abs().max().item() <= TOL[dtype], (i, t)
+        if again is not None:
+            assert (again[i // L, i % L].double() - _attend(s, tok[0][0], i, n + T)).abs().max().item() <= TOL[dtype]
+
+
 @pytest.mark.parametrize("word", [0, -1, 2**31 - 1, -2**31, 0x7f7f7f7f, "full", "above"])
 @pytest.mark.parametrize("H", [1, 5, 64])
 def test_a_segment_that_cannot_take_the_row_keeps_its_word(word, H):
