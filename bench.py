@@ -84,19 +84,16 @@ def decode_path(w, sms):
     nact = w.B * w.L
     pairs = nact * w.H
     cap_rows = w.B * (min(w.budget_rows(), w.L * w.N) + w.L * w.T)       # as Session sizes the cache
-    kb = (cap_rows // nact - w.T // 2) * w.D * 2 * w.esize >> 10
+    rows = cap_rows // nact - w.T // 2
+    kb = rows * w.D * 2 * w.esize >> 10
     if pairs < 4 * sms:
         return "cluster"
-    if pairs <= 5 * sms:
-        cluster = kb <= 256
-    elif pairs <= 6 * sms:
-        cluster = kb <= 176
-    elif pairs <= 7 * sms:
-        cluster = kb <= 96
-    elif pairs < 10 * sms:
-        cluster = 96 <= kb <= 256
+    if pairs < 10 * sms:
+        cluster = kb <= (448 if pairs <= 5 * sms else 256 if pairs <= 6 * sms else 320 if pairs <= 7 * sms else 448)
+    elif nact > 256:
+        cluster = rows >= (0 if w.H * w.D * w.esize <= 1024 else 112)
     else:
-        cluster = kb >= (96 if nact > 256 else 64) and (pairs >= 20 * sms or kb <= 320)
+        cluster = rows >= (96 if pairs < 20 * sms else 80)
     if cluster:
         return "cluster"
     heads = w.D in (64, 128) and nact <= 256 and cap_rows // nact <= 1024

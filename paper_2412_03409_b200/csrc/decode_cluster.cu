@@ -19,9 +19,13 @@
 // (looked at before: 19.3 us for 17.7 in the case of 8 x 40 x 410 rows; one thread's loads, passed on through
 // shared memory: 20.1, and 4.15 for 3.77 in the smallest).
 //
+// A round's arithmetic is half of what a warp does: dot products and sums two elements to an instruction, whole rounds without a look at
+// their ends, rescaling where the maximum moves, pointers instead of products of row numbers: 8 x 40 x 410 17.7 -> 15.9 us, 1024 pairs of
+// 136 rows 16.7 -> 15.0.  (Partial sums of four rows reduced together, 12 shuffles for 17: no gain.)
+//
 // Measured, device time of calls replayed from a graph, one layer, bf16, D = 128, every call on another layer: 1 segment
-// x 32 heads x 128 rows 3.77 us (4.43 with flags and without the guess), 4 x 32 x 128 rows 5.46 (6.00), 16 x 32 x 128 10.98 (11.55),
-// 1 x 40 x 410 5.05 (5.63), 8 x 40 x 410 17.7 (18.8; 10.3 us of bytes); against the row-split kernel and its merge
+// x 32 heads x 128 rows 3.77 us (4.44 before all of this), 4 x 32 x 128 rows 5.23 (6.01), 16 x 32 x 128 9.84 (11.55),
+// 1 x 40 x 410 4.96 (5.65), 8 x 40 x 410 15.9 (18.8; 10.3 us of bytes); against the row-split kernel and its merge
 // kernel, before that: 1 x 32 x 128 rows 4.5 (10.0), 1024 rows 8.0 (26.4); 4 x 32 x 128 rows 6.1 (12.1);
 // 8 x 40 x 410 rows 17.4 (25.7); 8 x 64 x 900 rows 50 (51).  A second wave of CTAs costs as much as the
 // first's latency, 4-5 us (C = 8 for 4 x 32 x 128 rows: 8.9 us), hence the choice of C below.  Loads to
@@ -76,6 +80,27 @@ __device__ __forceinline__ void store_first_cta(float *p, float v)
     asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"((uint32_t)__cvta_generic_to_shared(p)));
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
 }
+// Two fp32 operations in one instruction (same rounding as the scalar ones): half the issue slots.
+__device__ __forceinline__ float2 fma_pair(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, z, w;\n\t"
+        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
+        "fma.rn.f32x2 w, x, y, z;\n\tmov.b64 {%0, %1}, w;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 mul_pair(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, w;\n\t"
+        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+        "mul.rn.f32x2 w, x, y;\n\tmov.b64 {%0, %1}, w;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
 __device__ __forceinline__ void copy16(void *dst, const unsigned char *src)
 {
     asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
@@ -95,7 +120,8 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
     constexpr int STEP = kCU * G;  // rows of one round of a warp
     static_assert(kCWarps * 32 >= D, "a thread per element of the output");
     extern __shared__ __align__(16) unsigned char s_ring[];  // [kCWarps][kCStages][K, V][kCRound]
-    __shared__ float s_acc[kCWarps][D], s_ml[kCWarps][2];
+    __shared__ __align__(8) float s_acc[kCWarps][D];
+    __shared__ float s_ml[kCWarps][2];
     __shared__ float c_acc[P == kCPerSm ? kCMaxCluster : 1][D], c_ml[kCMaxCluster][2];  // (first CTA of a cluster) the cluster's partials
 
     __shared__ SegPlan s_plan[2];
@@ -132,13 +158,18 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
     unsigned char *ring = s_ring + (size_t)warp * kCStages * 2 * kCRound + lane * 16;
     auto request = [&](const Rows &rw, int base, int stage) {
         unsigned char *d = ring + stage * 2 * kCRound;
+        const size_t first = (size_t)(base + grp) * a.row_bytes;
+        const unsigned char *kp = rw.kb + first, *vp = rw.vb + first;
+        const uint32_t step = G * a.row_bytes;
 #pragma unroll
         for (int j = 0; j < kCU; ++j) {
             const int r = base + j * G + grp;
             if (r < rw.r1 && r != rw.skip) {
-                copy16(d + j * 512, rw.kb + (size_t)r * a.row_bytes);
-                copy16(d + kCRound + j * 512, rw.vb + (size_t)r * a.row_bytes);
+                copy16(d + j * 512, kp);
+                copy16(d + kCRound + j * 512, vp);
             }
+            kp += step;
+            vp += step;
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -207,41 +238,40 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
 
     // M: the running maximum of the logits, from the lowest finite number on, so that exp2f(s - M) is 0 for a logit
     // of -infinity and NaN for NaN whatever came before it.
-    float qf[VE], acc[VE], M = kNoLogit, lsum = 0.f;
+    float qf[VE], M = kNoLogit, lsum = 0.f;
+    float2 acc[VE / 2];
     RowVec<T>::unpack(qraw, qf);
 #pragma unroll
     for (int i = 0; i < VE; ++i) {
         qf[i] *= sc;
-        acc[i] = 0.f;
+        acc[i / 2] = make_float2(0.f, 0.f);
     }
     // One round: logits of the warp's rows, one rescale, accumulation (every lane group keeps the
     // warp-wide running maximum, so that the groups' sums simply add at the end).
     auto dot = [&](const uint4 &raw) {
-        float x[VE], d0 = 0.f, d1 = 0.f;
+        float x[VE];
+        float2 d = make_float2(0.f, 0.f);
         RowVec<T>::unpack(raw, x);
 #pragma unroll
-        for (int i = 0; i < VE; i += 2) {
-            d0 = fmaf(qf[i], x[i], d0);
-            d1 = fmaf(qf[i + 1], x[i + 1], d1);
-        }
-        return d0 + d1;
+        for (int i = 0; i < VE; i += 2) d = fma_pair(make_float2(qf[i], qf[i + 1]), make_float2(x[i], x[i + 1]), d);
+        return d.x + d.y;
     };
     auto add = [&](float p, const uint4 &raw) {
         float x[VE];
         RowVec<T>::unpack(raw, x);
         lsum += p;
 #pragma unroll
-        for (int i = 0; i < VE; ++i) acc[i] = fmaf(p, x[i], acc[i]);
+        for (int i = 0; i < VE; i += 2) acc[i / 2] = fma_pair(make_float2(p, p), make_float2(x[i], x[i + 1]), acc[i / 2]);
     };
     auto rescale = [&](float mx) {
 #pragma unroll
         for (int o = LPR; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        const float Mn = fmaxf(M, mx);
-        const float corr = exp2f(M - Mn);
-        M = Mn;
+        if (!(mx > M)) return;  // (the same in all lanes)
+        const float corr = exp2f(M - mx);
+        M = mx;
         lsum *= corr;
 #pragma unroll
-        for (int i = 0; i < VE; ++i) acc[i] *= corr;
+        for (int i = 0; i < VE / 2; ++i) acc[i] = mul_pair(acc[i], make_float2(corr, corr));
     };
     int stage = 0;
     for (int base = rw.r0 + warp * STEP; base < rw.r1; base += kCWarps * STEP) {
@@ -254,18 +284,25 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
         for (int o = LPR / 2; o > 0; o >>= 1)
 #pragma unroll
             for (int j = 0; j < kCU; ++j) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o);
+        if (base + STEP <= rw.r1 && rw.skip < 0) {
 #pragma unroll
-        for (int j = 0; j < kCU; ++j) {
-            const int r = base + j * G + grp;  // (what was not copied may be anything, NaN included)
-            if (r >= rw.r1 || r == rw.skip) s[j] = -INFINITY;
-            mx = fmaxf(mx, s[j]);
-        }
-        rescale(mx);
+            for (int j = 0; j < kCU; ++j) mx = fmaxf(mx, s[j]);
+            rescale(mx);
 #pragma unroll
-        for (int j = 0; j < kCU; ++j) {
-            const int r = base + j * G + grp;
-            if (r < rw.r1 && r != rw.skip)
-                add(exp2f(s[j] - M), *reinterpret_cast<const uint4 *>(kt + kCRound + j * 512));
+            for (int j = 0; j < kCU; ++j) add(exp2f(s[j] - M), *reinterpret_cast<const uint4 *>(kt + kCRound + j * 512));
+        } else {
+#pragma unroll
+            for (int j = 0; j < kCU; ++j) {
+                const int r = base + j * G + grp;  // (what was not copied may be anything, NaN included)
+                if (r >= rw.r1 || r == rw.skip) s[j] = -INFINITY;
+                mx = fmaxf(mx, s[j]);
+            }
+            rescale(mx);
+#pragma unroll
+            for (int j = 0; j < kCU; ++j) {
+                const int r = base + j * G + grp;
+                if (r < rw.r1 && r != rw.skip) add(exp2f(s[j] - M), *reinterpret_cast<const uint4 *>(kt + kCRound + j * 512));
+            }
         }
         request(rw, base + kCStages * kCWarps * STEP, stage);
         if (++stage == kCStages) stage = 0;
@@ -289,11 +326,14 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
     for (int o = LPR; o < 32; o <<= 1) {
         lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
 #pragma unroll
-        for (int i = 0; i < VE; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+        for (int i = 0; i < VE / 2; ++i) {
+            acc[i].x += __shfl_xor_sync(0xffffffffu, acc[i].x, o);
+            acc[i].y += __shfl_xor_sync(0xffffffffu, acc[i].y, o);
+        }
     }
     if (grp == 0) {
 #pragma unroll
-        for (int i = 0; i < VE; ++i) s_acc[warp][c * VE + i] = acc[i];
+        for (int i = 0; i < VE; i += 2) *reinterpret_cast<float2 *>(&s_acc[warp][c * VE + i]) = acc[i / 2];
     }
     if (lane == 0) {
         s_ml[warp][0] = M;
@@ -387,37 +427,38 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     const int wave = kCPerSm * sms;
     if (items >= 4 * (int64_t)sms) {
         // A CTA for every pair.  Measured, the per-head (or row-split) kernel / this one, us a call, bf16, heads of 128, lengths alike and
-        // from 0.3 to 1.7 of the mean.  One wave: 640 pairs of 30 rows 7.5 / 4.9, 8.4 / 5.4, of 128 12.7 / 10.4, 13.4 / 11.6, of 400
-        // 28.3 / 25.6, 28.7 / 28.6, but of 820 48.9 / 48.6, 46.9 / 50.2: the longest pairs end alone.  740 pairs of 128 14.0 / 12.0.
-        // Up to seven CTAs an SM, in one wave too: 800 x 64 11.2 / 9.1, x 256 22.7 / 22.3, 26.7 / 24.4, x 400 33.1 / 31.8, 33.8 / 35.2, 1024 x 30 8.9 / 7.1, 10.2 / 7.4, x 128 16.6 / 15.5, 18.0 / 16.5,
-        // but x 256 26.1 / 27.1, 31.8 / 30.1, x 400 38.8 / 39.6, 39.8 / 43.5.  More waves: CTAs that begin cost the first rows' latency,
-        // which is little against long rows, and is hidden where lengths differ, as they do after a search: 1280 x 256 31.9 / 33.1,
-        // 38.4 / 31.9, 1536 x 384 54.5 / 54.2, 55.3 / 52.7, 2048 x 64 20.0 / 21.4, 19.9 / 20.6, x 128 27.6 / 29.5, 28.8 / 28.1, x 256 46.5 / 48.3,
-        // 52.1 / 48.1, 1600 x 820 104.4 / 107.4, 107.1 / 110.2, 4096 x 128 50.7 / 51.9, 52.3 / 50.9, x 400 130.7 / 128.1, 143.9 / 129.8, 8192 x 400
-        // 257 / 248, 284 / 247; against the row-split kernel 12800 x 410 395 / 377, 16384 x 128 174 / 177, x 256 343 / 313;
-        // with pruning 640 x 64 17.0 / 10.3, 4096 x 64 33.9 / 36.7, x 200 75.3 / 74.1.
-        // By a pair's bytes halfway through the tokens that the cache has room for.
-        const int64_t kb = (seg_rows - c->decode_cap / 2) * D * 2 * (int64_t)esize(s) >> 10;
-        bool here;
-        if (items <= wave) here = kb <= 256;
-        else if (items <= 6 * (int64_t)sms) here = kb <= 176;
-        else if (items <= 7 * (int64_t)sms) here = kb <= 96;
-        else if (items < 10 * (int64_t)sms) here = kb >= 96 && kb <= 256;
-        else here = kb >= (nact > 256 || c->evict_distance > 0 ? 96 : 64) && (items >= 20 * (int64_t)sms || kb <= 320) && items <= INT32_MAX / 2;
-        if (!here) return -1;
+        // from 0.3 to 1.7 of the mean.  One wave: 640 pairs of 30 rows 7.5 / 4.9, 8.4 / 5.4, of 128 12.7 / 9.9, 13.4 / 10.7, of 820 48.8 / 45.8,
+        // 46.7 / 46.0.  Up to seven CTAs an SM, in one wave too: 888 x 64 12.2 / 9.1, 11.8 / 9.2, x 400 34.9 / 33.6, 36.7 / 35.6, x 600 47.3 / 46.7,
+        // 47.4 / 49.7; 1024 x 32 10.5 / 7.1, 10.3 / 7.2, x 128 16.6 / 14.8, 18.1 / 15.2, x 256 25.9 / 25.7, 31.9 / 27.3, x 400 38.8 / 38.1, 39.8 / 39.3,
+        // x 600 53.0 / 53.5, 54.7 / 55.8, x 820 69.3 / 71.2, 71.2 / 73.8.  More waves: CTAs that begin cost the first rows' latency,
+        // which is little against long rows, and is hidden where lengths differ, as they do after a search: 1280 x 32 11.9 / 10.8, 11.7 / 10.7,
+        // x 128 19.5 / 20.1, 21.5 / 18.4, x 256 31.9 / 32.3, 38.4 / 31.5; 1600 x 128 23.0 / 24.4, 24.3 / 23.3, x 820 104.5 / 106.4, 106.6 / 104.5;
+        // 2048 x 32 15.8 / 16.5, 15.5 / 16.3, x 128 27.8 / 28.8, 29.2 / 27.2, x 400 68.6 / 67.4, 77.0 / 69.3; 4096 x 32 27.0 / 29.0, 26.2 / 28.6, x 64 35.5 / 35.3,
+        // 35.9 / 34.4, x 256 87.3 / 84.3, 95.7 / 83.4; 8192 x 128 97.2 / 90.0, 99.0 / 88.5; against the row-split kernel 16384 x 64 97.8 / 118.2,
+        // 96.5 / 114.9, x 128 180 / 169, 174 / 168; with pruning 640 x 64 17.0 / 9.7, 2048 x 64 22.7 / 21.3, 4096 x 64 34.1 / 37.4, x 128 51.8 / 51.2,
+        // 8192 x 128 94.1 / 94.5, x 200 138.6 / 130.3.
+        // More than 256 segments, always the row-split kernel's otherwise: 288 x 16 heads of 64, 64 rows 28.9 / 29.5, 128 42.3 / 36.0, 256 69.8 / 53.5;
+        // 960 x 32, 32 rows 99 / 179, 128 318 / 313, 256 601 / 573, but rows of 1 KiB, which it splits badly, 288 x 8 of 64, 32 rows 18.6 / 14.3, 960 x 8,
+        // 64 rows 65.6 / 43.9.
+        // By a pair's rows, and their bytes, halfway through the tokens that the cache has room for.
+        const int64_t rows = seg_rows - c->decode_cap / 2, kb = rows * D * 2 * (int64_t)esize(s) >> 10;
+        int64_t least = 0, most_kb = INT64_MAX;
+        if (items <= wave) most_kb = 448;
+        else if (items <= 6 * (int64_t)sms) most_kb = 256;
+        else if (items <= 7 * (int64_t)sms) most_kb = 320;
+        else if (items < 10 * (int64_t)sms) most_kb = 448;
+        else if (c->evict_distance > 0) least = items < 20 * (int64_t)sms ? 80 : 200;
+        else if (nact > 256) least = (size_t)H * D * esize(s) <= 1024 ? 0 : 112;
+        else least = items < 20 * (int64_t)sms ? 96 : 80;
+        if (rows < least || kb > most_kb || items > INT32_MAX / 2) return -1;
     }
-    // Long segments are the row-split kernel's, where it covers the shape: eight CTAs of a pair keep 256 KiB in
-    // flight however long it is, and CTAs that come in waves read the slices of a row at different times.
-    // Measured, one layer, this kernel / row-split.  Few pairs, by a pair's bytes: 1 head of 128, bf16, 12000 rows
-    // (6.1 MB) 29 / 33 us, 16000 (8.2) 38 / 35, fp32 6000 rows 29 / 30, 8000 38 / 31, 16000 70 / 35; 8 heads
-    // fp32 8000 38 / 40, 12000 56 / 45.  From 24 pairs on the row-split kernel's merge costs more: 24 heads fp32
-    // 12000 rows (12.3 MB) 64 / 81, 32 pairs of 4 segments 72 / 73, 16000 rows 94 / 92.  Many pairs, by pairs x
-    // rows: 128 x 6000 rows 73 / 73, x 12000 137 / 130; 320 x 1800 58 / 59, x 3200 86 / 92; 512 x 1100 55 / 59, x
-    // 1800 89 / 83 (heads of 64: 34 / 36, 55 / 49); 576 x 1100 60 / 60, x 1800 96 / 90; and by bytes: 64 pairs of 8000 rows of fp32
-    // (524 MB) 90 / 90, 12000 134 / 126.
+    // Few pairs, but the longest, for which the row-split kernel is as fast where it covers the shape, row-split / this one, one layer: 1 head
+    // of 128, bf16, 8000 rows 18.1 / 13.4, 15000 31.1 / 21.8, fp32 8000 26.8 / 20.9; 8 heads fp32 8000 40.1 / 31.9, 12000 (12.3 MB a pair) 45.0 / 45.6;
+    // 32 pairs of 12000 67.9 / 63.3; 128 pairs of bf16, 6000 72.5 / 65.1, 12000 129 / 121; 320 x 1800 57.6 / 53.4, x 4500 120 / 110; 512 x 1800 79.9 / 77.9,
+    // x 2400 103 / 98, heads of 64 47.5 / 48.3; 576 x 1800 88.3 / 85.2.  (Nothing longer measured.)
     if (items < 4 * (int64_t)sms &&
-        (pair_bytes > ((int64_t)(items < 24 ? 6 : 12) << 20) || items * seg_rows > (items <= 320 ? 1 << 20 : 704 << 10) ||
-         items * pair_bytes > ((int64_t)512 << 20)) &&
+        (pair_bytes > ((int64_t)(items < 24 ? 11 : 13) << 20) ||
+         items * seg_rows > (D == 64 ? (items <= 320 ? 1 << 20 : 704 << 10) : 1536 << 10) || items * pair_bytes > ((int64_t)800 << 20)) &&
         decode_stream_covers(s, nact))
         return -1;
     // As many CTAs as the SMs hold at a time, none of them with less than one round of rows (32) unless

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+import test_gpu_decode_paths as paths
 from paper_2412_03409_b200 import api
 from paper_2412_03409_b200.session import Session
 
@@ -126,3 +127,18 @@ def test_a_plan_changed_just_before_the_call(place):
         for i, rows in enumerate((n + 1, 91)):
             ref = _attend(s, tok[1][0], i, rows)
             assert (out[0, i].double() - ref).abs().max().item() <= TOL[torch.bfloat16], (n, i)
+
+
+# What the pair kernel leaves: more than 256 segments of few rows (row-split kernel, whose lanes, heads a warp, rows a unit and warps
+# go by the row's bytes), pairs just too long for one wave (per-head kernel, tiles shared out where lengths differ), short ones of several waves.
+@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d", [
+    (9, 32, 16, 128, 40, 15, torch.bfloat16, 3), (9, 32, 40, 128, 40, 15, torch.bfloat16, 3), (9, 30, 64, 128, 24, 15, torch.bfloat16, 3),
+    (9, 32, 16, 64, 60, 30, torch.bfloat16, 3), (9, 32, 32, 64, 60, 20, torch.bfloat16, 0), (9, 32, 40, 64, 40, 15, torch.bfloat16, 3),
+    (9, 30, 64, 64, 40, 15, torch.bfloat16, 0), (9, 32, 16, 128, 40, 12, torch.float32, 3), (9, 32, 32, 128, 40, 12, torch.float32, 3),
+    (9, 30, 40, 128, 24, 8, torch.float32, 0), (9, 32, 16, 64, 40, 12, torch.float32, 3),
+    (9, 32, 32, 64, 40, 12, torch.float32, 3), (9, 30, 40, 64, 24, 9, torch.float32, 0), (9, 30, 64, 64, 24, 9, torch.float32, 3),
+    (1, 32, 32, 128, 1500, 700, torch.bfloat16, 0), (2, 18, 25, 128, 900, 640, torch.bfloat16, 0), (3, 32, 32, 64, 90, 40, torch.bfloat16, 0),
+    (2, 32, 32, 128, 90, 30, torch.float32, 0),
+])
+def test_what_goes_elsewhere(B, L, H, D, N, rows, dtype, d):
+    paths.test_decode_steps_match_the_oracle(B, L, H, D, N, rows, dtype, d)
