@@ -373,33 +373,83 @@ __device__ __forceinline__ int count_below(const uint64_t *__restrict__ c, int a
     }
     return a;
 }
+// The same for two rows side by side: the numbers end up in a.
+template <int M>
+__device__ __forceinline__ void count_below(const uint64_t *__restrict__ c0, const uint64_t *__restrict__ c1, int (&a)[M],
+                                            int (&b)[M], const uint64_t (&theta)[M])
+{
+    while (a[0] < b[0] || a[M - 1] < b[M - 1]) {
+        uint64_t x[M][3];
+        int i[M][3];
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            const int from = a[m] < b[m] ? a[m] : 0, width = max(b[m] - a[m], 0);  // (a row done: its first value)
+            const uint64_t *c = m ? c1 : c0;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                i[m][j] = from + ((j + 1) * width >> 2);
+                x[m][j] = c[i[m][j]];
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            if (a[m] >= b[m]) continue;
+            if (x[m][1] < theta[m]) {
+                a[m] = x[m][2] < theta[m] ? i[m][2] + 1 : i[m][1] + 1;
+                b[m] = x[m][2] < theta[m] ? b[m] : i[m][2];
+            } else {
+                b[m] = x[m][0] < theta[m] ? i[m][1] : i[m][0];
+                a[m] = x[m][0] < theta[m] ? i[m][0] + 1 : a[m];
+            }
+        }
+    }
+}
 
 // Length rule of Sec. 3.3 (a layer keeps one row more than there are cumulative values below p * total, at most N) and the
 // bisection on p that makes the lengths meet the budget.  One CTA per sample, warp per layer.
 //
 // A midpoint by itself is a chain of latencies -- a load or two, the sum over the layers, a barrier -- of some 1000
-// clocks.  So the tree of the next five bisections is evaluated at once, a lane to each of its 31 midpoints (formed by the
-// same additions and halvings that would lead there), and then walked: a round costs little more than a midpoint did, the
-// first one apart, whose searches cover whole rows; later ones lie between the counts at both ends of the interval.
-// Selection and compaction of one sample, a midpoint at a time / five levels at a time: 32 layers of 640 scores 58.2 / 52.0 us
-// (four levels 54.0), of 128 28.8 / 24.7, of 16384 274 / 266; 40 layers of 1024 109 / 98.  Sort and search alone, one sample: 129
-// layers of 640 scores 56.0 / 40.4, 300 143.5 / 97.6, 1000 of 2000 scores 699 / 559 (beyond 128 layers a lane searches whole rows).
+// clocks.  So the tree of the next five bisections is evaluated at once, a lane to each of its 31 midpoints (the values that the
+// same additions and halvings would lead to), and the way through it is found by all lanes at once from bit masks of what each
+// midpoint came to: a round costs little more than a midpoint did, the first one apart, whose searches cover whole rows; later
+// ones lie between the counts at both ends of the interval.  What a warp's layers need is kept in registers for kHoist of them,
+// and they are searched two at a time, so that their loads are in flight together.  kHoist is the least that covers the layers of
+// a sample: code for layers that are not there costs as much as a layer's (32 layers of 640 scores with four hoisted: 16.2 us).
+// Sort and search of one sample, in us, sorting alone in brackets; five levels walked one by one in fp64, four layers hoisted and
+// searched one after the other / as here: 32 layers of 640 scores 19.3 / 13.1 (7.9), of 128 12.2 / 7.0 (3.5), of 4096 39.1 / 32.3
+// (23.8); 40 of 640 21.8 / 14.8, eight samples 29.5 / 21.4 (13.6); 64 of 640 24.1 / 17.1; 96 27.5 / 22.8; 128 37.4 / 28.1; 200 of
+// 300 46.0 / 32.0 (with four hoisted 42.8); 1000 of 2000 478 / 389 (beyond 256 layers a lane searches whole rows).  A midpoint at
+// a time cost some 6 us more than the former at 32 layers of 640.
 constexpr int kTreeLevels = 5;
+// After so many rounds the ends are multiples of 2^-50: every midpoint until then is a sum without rounding, found at once.
+constexpr int kExactRounds = 50 / kTreeLevels;
 constexpr int kMaxLayers = 5120;  // of a sample (sums of lengths are 32 bits wide, which would do for 2^17 layers)
+template <int kHoist>
 __global__ void __launch_bounds__(1024)
 search_kernel(const uint64_t *__restrict__ cum, const int64_t *__restrict__ budget_rows, int L,
               int N, double tol, int max_iters, int64_t slack, int64_t slack_over, int32_t *__restrict__ len,
               double *__restrict__ p_out, int32_t *__restrict__ iters_out, int32_t *dev_status)
 {
+    __shared__ int s_flags;
     __shared__ int s_sum[3][32];  // total length at every midpoint of the tree; buffers in turn
     const int b = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const uint64_t *cb = cum + (size_t)b * L * N;
     if (threadIdx.x < 96) s_sum[threadIdx.x / 32][lane] = 0;
+    if (threadIdx.x == 0) s_flags = 0;
+    const int depth = 31 - __clz(lane | 1);  // of the lane's node, whose interval is `part` of the tree's,
+    const double part = ldexp(1.0, -depth);  // and its midpoint at `place` of it (lane 0: as lane 1)
+    const double place = (2 * (lane & ((1 << depth) - 1)) + 1) * part * 0.5;
+    uint32_t above = 0, upper = 0;  // the nodes above the lane's, and those of them in whose upper half it is
+    for (int i = 0; i < depth; ++i) {
+        above |= 1u << (lane >> (i + 1));
+        upper |= (uint32_t)(lane >> i & 1) << (lane >> (i + 1));
+    }
+    __syncthreads();
     dependent_entry();  // the sort kernel's sums and flags are complete
-    // What a layer's searches need, kept in registers for the first kHoist layers of the warp: its total, the counts at both
-    // ends of the interval, and a pivot per lane, c[(lane + 1) * chunk - 1] (or ~0 past the end).
-    constexpr int kHoist = 4;
+    // What a layer's searches need, for the first kHoist layers of the warp: its total, the counts at both ends of the interval,
+    // and a pivot per lane, c[(lane + 1) * chunk - 1] (or ~0 past the end).
+    constexpr int M = kHoist > 1 ? 2 : 1;  // rows searched side by side
     const int chunk = (N + 31) >> 5;
     double tot[kHoist];
     uint64_t pivot[kHoist];
@@ -422,9 +472,7 @@ search_kernel(const uint64_t *__restrict__ cum, const int64_t *__restrict__ budg
     {
         int flags = 0;
         for (int l = threadIdx.x; l < L; l += blockDim.x) flags |= len[(size_t)b * L + l];
-        // (the block-wide "or" is of predicates, so one per bit)
-        flags = (__syncthreads_or(flags & 1) ? 1 : 0) | (__syncthreads_or(flags & 2) ? 2 : 0);
-        if (threadIdx.x == 0) dev_status[b] = status_from_flags(flags);  // overwrites: this call's status starts here
+        if (flags) atomicOr(&s_flags, flags);  // (looked at after a round's barrier, as the slots are written after one)
     }
 
     auto threshold = [](double p, double total) { return __double2ull_ru(__dmul_rn(p, total)); };
@@ -432,73 +480,102 @@ search_kernel(const uint64_t *__restrict__ cum, const int64_t *__restrict__ budg
 
     double p_final = 0.0;
     int iters = 0, taken = -1;  // taken: the midpoint, of the last tree, that is p_final
-    if (budget < (int64_t)L) {
-        if (threadIdx.x == 0) raise_status(dev_status, b, PKV_DEV_BUDGET_TOO_SMALL);
-    } else if ((int64_t)L * (int64_t)N <= budget) {
-        p_final = 1.0;
+    if (budget < (int64_t)L || (int64_t)L * (int64_t)N <= budget) {
+        if (budget >= (int64_t)L) p_final = 1.0;
+        __syncthreads();
     } else {
         double p1 = 0.0, p2 = 1.0;
         bool done = false;
         for (int round = 0; !done; ++round) {
             // the lane's midpoint: node `lane` of the tree (root 1; the upper half of a node's interval is its odd child)
-            double a1 = p1, a2 = p2, p = (p1 + p2) * 0.5;
-            for (int bit = 30 - __clz(lane | 1); bit >= 0; --bit) {
-                if (lane >> bit & 1) a1 = p;
-                else a2 = p;
-                p = (a1 + a2) * 0.5;
+            double p;
+            bool stop;  // no bisection of the node's interval: its ends are neighbours or within the tolerance
+            if (round < kExactRounds) {
+                const double width = p2 - p1;
+                p = fma(width, place, p1);
+                stop = width * part <= tol;
+            } else {
+                double a1 = p1, a2 = p2;
+                p = (p1 + p2) * 0.5;
+                for (int bit = depth - 1; bit >= 0; --bit) {
+                    if (lane >> bit & 1) a1 = p;
+                    else a2 = p;
+                    p = (a1 + a2) * 0.5;
+                }
+                stop = p == a1 || p == a2 || a2 - a1 <= tol;
             }
+            const uint32_t stops = __ballot_sync(0xffffffffu, stop || depth >= max_iters - iters);
             int total = 0;
 #pragma unroll
-            for (int k = 0; k < kHoist; ++k) {
+            for (int k = 0; k < kHoist; k += M) {
                 const int l = warp + k * nwarp;
                 if (l >= L) continue;
-                const uint64_t theta = threshold(p, tot[k]);
-                int x = lo[k], y = hi[k];
-                if (y - x > chunk) {  // (the first round: which 32nd of the row)
-                    int n = 0;
+                uint64_t theta[M];
+                int x[M], y[M];
 #pragma unroll
-                    for (int step = 16; step > 0; step >>= 1)
-                        n += __shfl_sync(0xffffffffu, pivot[k], n + step - 1) < theta ? step : 0;
-                    n += __shfl_sync(0xffffffffu, pivot[k], 31) < theta ? n == 31 : 0;
-                    x = max(x, n * chunk);
-                    y = min(y, (n + 1) * chunk - 1);
+                for (int m = 0; m < M; ++m) {
+                    theta[m] = threshold(p, tot[k + m]);
+                    x[m] = lo[k + m];
+                    y[m] = hi[k + m];
+                    if (m == 1 && l + nwarp >= L) {
+                        x[m] = y[m] = 0;
+                    } else if (y[m] - x[m] > chunk) {  // (the first round: which 32nd of the row)
+                        int n = 0;
+#pragma unroll
+                        for (int step = 16; step > 0; step >>= 1)
+                            n += __shfl_sync(0xffffffffu, pivot[k + m], n + step - 1) < theta[m] ? step : 0;
+                        n += __shfl_sync(0xffffffffu, pivot[k + m], 31) < theta[m] ? n == 31 : 0;
+                        x[m] = max(x[m], n * chunk);
+                        y[m] = min(y[m], (n + 1) * chunk - 1);
+                    }
                 }
-                at[k] = p < 1.0 ? count_below(cb + (size_t)l * N, x, y, theta) : N;
-                total += length_of(at[k]);
+                const uint64_t *row = cb + (size_t)l * N;
+                if (M == 1 || l + nwarp >= L) {
+                    at[k] = p < 1.0 ? count_below(row, x[0], y[0], theta[0]) : N;
+                    total += length_of(at[k]);
+                } else {
+                    count_below(row, row + (size_t)nwarp * N, x, y, theta);
+#pragma unroll
+                    for (int m = 0; m < M; ++m) {
+                        at[k + m] = p < 1.0 ? x[m] : N;
+                        total += length_of(at[k + m]);
+                    }
+                }
             }
-            for (int l = warp + kHoist * nwarp; l < L; l += nwarp) {
-                const uint64_t *c = cb + (size_t)l * N;
-                total += length_of(p < 1.0 ? count_below(c, 0, N, threshold(p, (double)c[N - 1])) : N);
+            for (int l = warp + kHoist * nwarp; M > 1 && l < L; l += M * nwarp) {
+                const uint64_t *row[2] = {cb + (size_t)l * N, cb + (size_t)(l + nwarp < L ? l + nwarp : l) * N};
+                int x[M], y[M];
+                uint64_t theta[M];
+#pragma unroll
+                for (int m = 0; m < M; ++m) {
+                    x[m] = 0;
+                    y[m] = l + m * nwarp < L ? N : 0;
+                    theta[m] = threshold(p, (double)row[m][N - 1]);
+                }
+                count_below(row[0], row[1], x, y, theta);
+#pragma unroll
+                for (int m = 0; m < M; ++m)
+                    if (l + m * nwarp < L) total += length_of(p < 1.0 ? x[m] : N);
             }
             int *sums = s_sum[round % 3];
             atomicAdd(sums + lane, total);
             if (warp == 0) s_sum[(round + 1) % 3][lane] = 0;  // (read two rounds ago, before the last barrier)
             __syncthreads();
-            int node = 1, at1 = -1, at2 = -1;  // nodes that became the ends of the interval
-            for (int level = 0; level < kTreeLevels; ++level) {
-                const double mid = (p1 + p2) * 0.5;
-                if (mid == p1 || mid == p2 || iters == max_iters || p2 - p1 <= tol) {
-                    p_final = p1;
-                    done = true;
-                    break;
-                }
-                ++iters;
-                const int64_t delta = (int64_t)sums[node] - budget;
-                if (delta >= -slack && delta <= slack_over) {  // within the threshold on delta (Sec. 3.3)
-                    p_final = mid;
-                    taken = node;
-                    done = true;
-                    break;
-                }
-                if (delta < 0) {
-                    p1 = mid;
-                    at1 = node;
-                } else {
-                    p2 = mid;
-                    at2 = node;
-                }
-                node = 2 * node + (delta < 0 ? 1 : 0);
-            }
+            const int64_t delta = (int64_t)sums[lane] - budget;
+            const uint32_t low = __ballot_sync(0xffffffffu, delta < 0);
+            const uint32_t met = __ballot_sync(0xffffffffu, delta >= -slack && delta <= slack_over);  // (Sec. 3.3)
+            // the nodes that the bisection goes through, the interval's new ends among them, and the one where it ends
+            const uint32_t path =
+                __ballot_sync(0xffffffffu, lane > 0 && ((low ^ upper) & above) == 0 && ((stops | met) & above) == 0);
+            const uint32_t met_at = path & met & ~stops, went = path & ~stops & ~met;
+            const int at1 = 31 - __clz(went & low), at2 = 31 - __clz(went & ~low);  // (-1: none)
+            iters += __popc(path & ~stops);
+            taken = 31 - __clz(met_at);
+            done = (path & (stops | met)) != 0;
+            const double q1 = __shfl_sync(0xffffffffu, p, at1 & 31), q2 = __shfl_sync(0xffffffffu, p, at2 & 31);
+            if (at1 >= 0) p1 = q1;
+            if (at2 >= 0) p2 = q2;
+            if (done) p_final = taken >= 0 ? __shfl_sync(0xffffffffu, p, taken) : p1;
 #pragma unroll
             for (int k = 0; k < kHoist; ++k) {
                 const int n1 = __shfl_sync(0xffffffffu, at[k], at1 & 31), n2 = __shfl_sync(0xffffffffu, at[k], at2 & 31);
@@ -519,6 +596,8 @@ search_kernel(const uint64_t *__restrict__ cum, const int64_t *__restrict__ budg
         if (lane == 0) len[(size_t)b * L + l] = length_of(count);
     }
     if (threadIdx.x == 0) {
+        dev_status[b] = status_from_flags(s_flags);  // overwrites: this call's status starts here
+        if (budget < (int64_t)L) raise_status(dev_status, b, PKV_DEV_BUDGET_TOO_SMALL);
         p_out[b] = p_final;
         iters_out[b] = iters;
     }
@@ -651,7 +730,7 @@ extern "C" int prefixkv_search(const pkv_shape *shape, const float *scores,
     if (L > kMaxLayers) return PKV_ERR_UNSUPPORTED;
     int rc = launch_sort(shape, scores, order, cum, len, st);
     if (rc != PKV_OK) return rc;
-    cudaError_t e = launch_dependent(search_kernel, dim3(B), dim3(1024), 0, st,
+    cudaError_t e = launch_dependent(L <= 32 ? search_kernel<1> : L <= 64 ? search_kernel<2> : L <= 128 ? search_kernel<4> : search_kernel<8>, dim3(B), dim3(1024), 0, st,
                                      (const uint64_t *)cum, budget_rows, L, N, tol, (int)max_iters, slack_rows, slack_over_rows, len,
                                      p_out, iters_out, dev_status);
     if (e != cudaSuccess) {
