@@ -20,14 +20,13 @@ namespace pkv {
 // shared memory), turns the table of the warps' counts into offsets with one scan in the order (digit,
 // warp), and moves keys and positions to their places in shared memory.
 //
-// Up to 256 scores, one a thread, there are no passes: an item's place is the number of items before it, counted.
+// One item a thread (IPT 1) takes no passes but merges: a warp's 32 by counting, four warps' runs into one, those into the whole.
+// An item's place in a merge is its own among its run and the number of each other run's items before it, a binary search.
 //
-// Bounded by the issue slots of the ranking (some 60 instructions an item and pass) and, after it, by the
+// The passes are bounded by the issue slots of the ranking (some 60 instructions an item and pass) and, after it, by the
 // scattered stores; with few items by the barriers of the passes and, as each warp brings a table of 256 counts
-// to be scanned, by the number of warps.  64 segments of 16384: 204 us with a bitonic network of 64-bit keys,
-// 75 now.  Sort and search together, 32 segments, bitonic / one item a thread / as here: 64 scores 18.3 / 19.2 /
-// 17.3 us, 256 16.2 / 16.4 / 15.1, 640 28.6 / 25.9 / 24.2, 1024 34.9 / 37.1 / 31.5, 2048 44.5 / 38.2 (two items)
-// / 33.8; 512 segments of 1024 62.8 / 67.0 / 40.7.
+// to be scanned, by the number of warps, which is why merging beats them there (the figures are at launch_sort).
+// 64 segments of 16384: 204 us with a bitonic network of 64-bit keys, 75 now.
 // ---------------------------------------------------------------------------
 // Fixed-point weight of a sort key (inverted score bits): round-half-even(score * 2^32).  In integers:
 // fp64 instructions are few per clock here, and two conversions and a product per key took a good part of
@@ -49,7 +48,8 @@ __device__ __forceinline__ uint64_t weight_of_key(uint32_t key, bool &range_bad)
 }
 
 constexpr int kDigits = 256;
-constexpr int kSplitFour = 4096, kSplitTwo = 8192;  // scores above which a segment may be split over a cluster of so many
+constexpr int kSplit = 1024;        // scores of a segment above which a cluster of four may share it; one thread each to there,
+constexpr int kMergeCrowded = 768;  // or to here where segments outnumber the SMs
 
 // Shared memory: keys [items], counts [warps][kDigits] (a warp's lanes then meet in a bank by chance only; with
 // the warps of a digit side by side they always did), positions [items].
@@ -90,6 +90,18 @@ __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// How many of a sorted run of WIDTH keys come before an item of another run: of equal keys those of an earlier run do.
+template <int WIDTH>
+__device__ __forceinline__ uint32_t not_after(const uint32_t *run, uint32_t key, bool earlier)
+{
+    const uint32_t last = earlier ? key : key - 1;
+    const uint32_t *at = run;
+#pragma unroll
+    for (int step = WIDTH / 2; step > 0; step >>= 1) at += at[step - 1] <= last ? step : 0;
+    at += *at <= last ? 1 : 0;
+    return earlier || key != 0 ? (uint32_t)(at - run) : 0u;
 }
 
 // SPLIT: a cluster takes a segment.  Each of its CTAs sorts and sums a run of consecutive positions; an item's place is then its
@@ -137,27 +149,46 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
         }
     }
     if constexpr (IPT == 1) {
-        skey[tid] = key[0];
-        __syncthreads();
         uint32_t place = 0;
-        const uint4 *four = reinterpret_cast<const uint4 *>(skey);
-        for (int i = 0; i < warp * 8; ++i) {  // equal keys of earlier places come first
-            const uint4 x = four[i];
-            place += (x.x <= key[0]) + (x.y <= key[0]) + (x.z <= key[0]) + (x.w <= key[0]);
-        }
-        for (int i = (warp + 1) * 8; i < nthr / 4; ++i) {
-            const uint4 x = four[i];
-            place += (x.x < key[0]) + (x.y < key[0]) + (x.z < key[0]) + (x.w < key[0]);
-        }
 #pragma unroll 8
         for (int i = 0; i < 32; ++i) {
             const uint32_t x = __shfl_sync(0xffffffffu, key[0], i);
             place += x < key[0] || (x == key[0] && i < lane);
         }
+        skey[warp * 32 + place] = key[0];
+        spos[warp * 32 + place] = pos[0];
         __syncthreads();
-        skey[place] = key[0];
-        spos[place] = pos[0];
-        __syncthreads();
+        if (nwarp > 1) {
+            // runs of a warp's items into runs of four warps', these into the whole
+            key[0] = skey[tid];
+            pos[0] = spos[tid];
+            place = lane;
+            const int mine = warp & 3, from = warp - mine;
+#pragma unroll
+            for (int g = 1; g < 4; ++g) {
+                const int other = (mine + g) & 3;
+                if (from + other < nwarp) place += not_after<32>(skey + (from + other) * 32, key[0], other < mine);
+            }
+            __syncthreads();
+            skey[from * 32 + place] = key[0];
+            spos[from * 32 + place] = pos[0];
+            __syncthreads();
+        }
+        if (nwarp > 4) {
+            key[0] = skey[tid];
+            pos[0] = spos[tid];
+            place = tid & 127;
+            const int mine = tid >> 7, runs = nwarp >> 2;
+#pragma unroll 1
+            for (int g = 1; g < runs; ++g) {
+                const int other = mine + g < runs ? mine + g : mine + g - runs;
+                place += not_after<128>(skey + other * 128, key[0], other < mine);
+            }
+            __syncthreads();
+            skey[place] = key[0];
+            spos[place] = pos[0];
+            __syncthreads();
+        }
         key[0] = skey[tid];
         pos[0] = spos[tid];
     } else
@@ -633,7 +664,8 @@ static int launch_sort_items(const pkv_shape *s, const float *scores, int32_t *o
                              int32_t *seg_flags, cudaStream_t st, int split = 1)
 {
     const int N = s->prompt_len, share = (N + split - 1) / split;
-    const int threads = ((share + IPT - 1) / IPT + 31) / 32 * 32;
+    int threads = ((share + IPT - 1) / IPT + 31) / 32 * 32;
+    if (IPT == 1 && threads > 128) threads = (threads + 127) / 128 * 128;  // (whole runs)
     const size_t smem = sort_smem_bytes(threads, IPT, SPLIT);
     // (for every size: the default limit of 48 KiB is for the kernel's static variables and these together)
     static bool attr_done[64] = {};
@@ -689,22 +721,30 @@ static int clusters_of_four()
     return n;
 }
 
-// Up to 256 scores places are counted: the work grows with the square, 512 of them cost more than the passes.
-// Two items a thread beat four up to some 768 scores for one prompt (18.0 / 18.4 us with the search) and not for
-// 16 (42.8 / 37.6); beyond, four do throughout (1024: 19.8 / 19.2 and 47.9 / 40.7).  Above that as few as 1024
-// threads allow.  Long prompts whose segments leave SMs idle are split over clusters of four or two (with compaction, whole / split
-// over four: 32 segments of 4096 scores 127.9 / 125.9 us, of 4500 136.0 / 134.8, of 8192 226 / 219, of 16384 264 / 238; 64 segments, over
-// two: of 4500 230 / 235, 40 of 6000 252 / 253, 64 of 16384 431 / 421), while all clusters run at once (33 of four on a B200; the sort
-// alone, whole / split over four: 33 segments of 8193 scores 44.4 / 28.4 us, 34 43.9 / 54.2, and 36.7 over two).
+// One item a thread, merged, or radix passes; whole segments, or clusters of two or four to a segment.  Sort alone and a short
+// kernel behind it, in us, one item a thread / radix passes over whole segments, split as taken here in brackets:
+//   32 segments of 256 scores 4.2 / 4.7 (places counted against all), 300 4.6 / 6.9, 640 5.6 / 7.9 (one a thread over clusters of
+//   two 6.5), 768 6.4 / 8.3, 1024 8.2 / 9.0 (7.6); 512 of 256 6.7 / 9.5, 640 14.6 / 17.8, 768 18.1 / 21.2, 1024 24.9 / 18.7;
+//   of 1024 148 8.5 / 9.3, 160 13.7 / 11.9.
+// Merging takes the square of the runs, so the line falls to 768 where a block of 1024 threads is more than an SM's first.
+//   Clusters of two, one item a thread: 64 of 1024 12.1 at 2048 (13.0); two and four items: 32 of 3000 15.6 (18.0), 4096 18.2 (24.0).
+//   Clusters of four: 32 of 1536 9.3 (two: 9.5), 2048 10.6 (11.7), 3000 13.1 (15.6), 4096 16.4 (18.2), while all run at once (33 of
+//   four on a B200): 40 of 2048 13.9 (11.9), of 4096 26.9 (18.1).  Beyond 4096 radix passes in clusters of four or two: with
+//   compaction, whole / four, 32 of 4500 136.0 / 134.8, of 16384 264 / 238; whole / two, 64 of 16384 431 / 421; the sort alone,
+//   33 of 8193 44.4 / 28.4, 34 43.9 / 54.2, and 36.7 over two.
 static int launch_sort(const pkv_shape *s, const float *scores, int32_t *order, uint64_t *cum,
                        int32_t *seg_flags, cudaStream_t st)
 {
     const int N = s->prompt_len, sms = sm_count();
     const int64_t segments = (int64_t)s->batch * s->layers;
-    if (N > kSplitFour && segments <= clusters_of_four()) return launch_sort_items<4, true>(s, scores, order, cum, seg_flags, st, 4);
-    if (N > kSplitTwo && 2 * segments <= sms) return launch_sort_items<8, true>(s, scores, order, cum, seg_flags, st, 2);
-    if (N <= 256) return launch_sort_items<1>(s, scores, order, cum, seg_flags, st);
-    if (N <= 768) return launch_sort_items<2>(s, scores, order, cum, seg_flags, st);
+    if (N > kSplit && segments <= clusters_of_four())
+        return N <= 4096 ? launch_sort_items<1, true>(s, scores, order, cum, seg_flags, st, 4)
+                         : launch_sort_items<4, true>(s, scores, order, cum, seg_flags, st, 4);
+    if (N > kMergeCrowded && N <= 4096 && 2 * segments <= sms)
+        return N <= 2048 ? launch_sort_items<1, true>(s, scores, order, cum, seg_flags, st, 2)
+                         : launch_sort_items<4, true>(s, scores, order, cum, seg_flags, st, 2);
+    if (N > 8192 && 2 * segments <= sms) return launch_sort_items<8, true>(s, scores, order, cum, seg_flags, st, 2);
+    if (N <= (segments <= sms ? kSplit : kMergeCrowded)) return launch_sort_items<1>(s, scores, order, cum, seg_flags, st);
     if (N <= 4096) return launch_sort_items<4>(s, scores, order, cum, seg_flags, st);
     if (N <= 8192) return launch_sort_items<8>(s, scores, order, cum, seg_flags, st);
     return launch_sort_items<16>(s, scores, order, cum, seg_flags, st);
