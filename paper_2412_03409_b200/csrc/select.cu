@@ -26,7 +26,9 @@ namespace pkv {
 // The passes are bounded by the issue slots of the ranking (some 60 instructions an item and pass) and, after it, by the
 // scattered stores; with few items by the barriers of the passes and, as each warp brings a table of 256 counts
 // to be scanned, by the number of warps, which is why merging beats them there (the figures are at launch_sort).
-// 64 segments of 16384: 204 us with a bitonic network of 64-bit keys, 75 now.
+// 64 segments of 16384: 204 us with a bitonic network of 64-bit keys, 75 by passes; over clusters of two 57, and 45 with a
+// warp's items placed among few keys of the other CTA and the counts in separate banks (128 of 16384 77 / 74, 256 of 8192
+// 73 / 65, of 4096 46 / 39, 160 of 3000 34 / 31, 320 of 800 14.7 / 14.2).
 // ---------------------------------------------------------------------------
 // Fixed-point weight of a sort key (inverted score bits): round-half-even(score * 2^32).  In integers:
 // fp64 instructions are few per clock here, and two conversions and a product per key took a good part of
@@ -102,6 +104,31 @@ __device__ __forceinline__ uint32_t not_after(const uint32_t *run, uint32_t key,
     for (int step = WIDTH / 2; step > 0; step >>= 1) at += at[step - 1] <= last ? step : 0;
     at += *at <= last ? 1 : 0;
     return earlier || key != 0 ? (uint32_t)(at - run) : 0u;
+}
+
+// For a warp's sorted items, item i of the lanes after item i - 1: the number of the sorted `keys` that come before each (of equal
+// ones EARLIER says).  They are neighbours: a search for the first and the last of them leaves the others few keys to look among
+// (searching all 8192 keys for each of eight items a thread: 23400 clocks; so: 6600).
+template <int IPT, bool EARLIER>
+__device__ __forceinline__ void places_among(const uint32_t *keys, int items, const uint32_t (&key)[IPT], int lane, int (&n)[IPT])
+{
+    auto before = [](uint32_t x, uint32_t k) { return EARLIER ? x <= k : x < k; };
+    const uint32_t first = __shfl_sync(0xffffffffu, key[0], 0), last = __shfl_sync(0xffffffffu, key[IPT - 1], 31);
+    const uint32_t end = lane < 16 ? first : last;
+    int low = 0;
+    for (int width = items; width > 0; width >>= 1) {
+        const int half = (width + 1) >> 1;
+        low += before(keys[low + half - 1], end) ? half : 0;
+    }
+    const int high = __shfl_sync(0xffffffffu, low, 31);
+    low = __shfl_sync(0xffffffffu, low, 0);
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) n[i] = low;
+    for (int width = high - low; width > 0; width >>= 1) {
+        const int half = (width + 1) >> 1;
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) n[i] += before(keys[n[i] + half - 1], key[i]) ? half : 0;
+    }
 }
 
 // SPLIT: a cluster takes a segment.  Each of its CTAs sorts and sums a run of consecutive positions; an item's place is then its
@@ -191,14 +218,19 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
         }
         key[0] = skey[tid];
         pos[0] = spos[tid];
-    } else
+    } else {
+    // A warp counts a digit at the digit with `turned` turned over.  A thread of the scan goes through four warps' counts of a digit
+    // and the next four's; where warps come in eights, all of one digit, the threads of a warp do so in 32 banks (32 warps: four
+    // ways into eight without, 2950 clocks a scan, 1800 so).
+    const int turn = nwarp & 4 ? 0 : nwarp > 16 ? 8 : 16;
+    const uint32_t turned = (warp >> 3) * turn;
     for (int shift = 0; shift < 32; shift += 8) {
         for (int i = tid; i < kDigits * nwarp; i += nthr) count[i] = 0;
         __syncthreads();  // (and every item of the pass before is in registers)
         uint32_t rank[IPT];
 #pragma unroll
         for (int i = 0; i < IPT; ++i) {
-            const uint32_t digit = (key[i] >> shift) & (kDigits - 1);
+            const uint32_t digit = ((key[i] >> shift) & (kDigits - 1)) ^ turned;
             // lanes with this digit: bit by bit, or by match.any where digits are few (sign and exponent); it
             // takes a step per distinct value (16 items a warp: 31000 clocks a pass, 6500 on the last digit;
             // bit by bit 16000 throughout)
@@ -221,16 +253,14 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
         }
         __syncthreads();
         {  // exclusive scan in the order (digit, warp): eight entries a thread (kDigits * nwarp = 8 * nthr)
-            const int d0 = tid * 8 / nwarp, w0 = tid * 8 - d0 * nwarp;
+            const int d0 = tid * 8 / nwarp, w0 = tid * 8 - d0 * nwarp, w1 = w0 + 4 < nwarp ? w0 + 4 : 0;
+            uint32_t *four[2] = {count + w0 * kDigits + (d0 ^ (w0 >> 3) * turn),
+                                 count + w1 * kDigits + ((w1 ? d0 : d0 + 1) ^ (w1 >> 3) * turn)};
             uint32_t x[8], total = 0;
 #pragma unroll
-            for (int e = 0, d = d0, w = w0; e < 8; ++e) {
-                x[e] = count[w * kDigits + d];
+            for (int e = 0; e < 8; ++e) {
+                x[e] = four[e >> 2][(e & 3) * kDigits];
                 total += x[e];
-                if (++w == nwarp) {
-                    w = 0;
-                    ++d;
-                }
             }
             uint32_t incl = total;
 #pragma unroll
@@ -242,19 +272,15 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
             __syncthreads();
             uint32_t run = __reduce_add_sync(0xffffffffu, lane < warp ? warp_sum[lane] : 0u) + incl - total;
 #pragma unroll
-            for (int e = 0, d = d0, w = w0; e < 8; ++e) {
-                count[w * kDigits + d] = run;
+            for (int e = 0; e < 8; ++e) {
+                four[e >> 2][(e & 3) * kDigits] = run;
                 run += x[e];
-                if (++w == nwarp) {
-                    w = 0;
-                    ++d;
-                }
             }
         }
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < IPT; ++i) {
-            const uint32_t at = count[warp * kDigits + ((key[i] >> shift) & (kDigits - 1))] + rank[i];
+            const uint32_t at = count[warp * kDigits + (((key[i] >> shift) & (kDigits - 1)) ^ turned)] + rank[i];
             skey[at] = key[i];
             spos[at] = pos[i];
         }
@@ -264,6 +290,7 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
             key[i] = skey[base + i * 32];
             pos[i] = spos[base + i * 32];
         }
+    }
     }
 
     // Inclusive scan of the fixed-point weights.  Each is below 2^53; sums of their high parts cannot wrap
@@ -333,17 +360,8 @@ sort_scan_kernel(const float *__restrict__ scores, int N, int32_t *__restrict__ 
             __syncthreads();
             // (of equal keys those of earlier positions, another CTA's as a whole, come first)
             int n[IPT];
-#pragma unroll
-            for (int i = 0; i < IPT; ++i) n[i] = 0;
-            for (int half = 1 << (31 - __clz(items)); half > 0; half >>= 1)
-#pragma unroll
-                for (int i = 0; i < IPT; ++i) {
-                    const int at = n[i] + half - 1;
-                    if (at < items) {
-                        const uint32_t x = count[at];
-                        if (other < rank ? x <= key[i] : x < key[i]) n[i] += half;
-                    }
-                }
+            if (other < rank) places_among<IPT, true>(count, items, key, lane, n);
+            else places_among<IPT, false>(count, items, key, lane, n);
             const uint32_t sums = in_cta(ssum, other);
 #pragma unroll
             for (int i = 0; i < IPT; ++i) {
@@ -665,7 +683,7 @@ static int launch_sort_items(const pkv_shape *s, const float *scores, int32_t *o
 {
     const int N = s->prompt_len, share = (N + split - 1) / split;
     int threads = ((share + IPT - 1) / IPT + 31) / 32 * 32;
-    if (IPT == 1 && threads > 128) threads = (threads + 127) / 128 * 128;  // (whole runs)
+    if (threads > 128) threads = (threads + 127) / 128 * 128;  // (whole runs; the passes' scan goes by four warps)
     const size_t smem = sort_smem_bytes(threads, IPT, SPLIT);
     // (for every size: the default limit of 48 KiB is for the kernel's static variables and these together)
     static bool attr_done[64] = {};

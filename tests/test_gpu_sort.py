@@ -1,6 +1,6 @@
-"""The sort by merging runs, and clusters of two and four to shorter segments: numbers of scores at and around the runs' ends, the
-lines between the variants and shares that leave a cluster's last blocks without items, with many equal scores and zeros.
-Order and sums are compared exactly."""
+"""The sort: runs merged, radix passes with any number of quads of warps, clusters of two and four.  Numbers of scores at and around
+the runs' ends, the lines between the variants and shares that leave a cluster's last blocks without items, with many equal
+scores and zeros.  Order and sums are compared exactly."""
 import numpy as np
 import pytest
 import torch
@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
                                                          767, 768, 769, 1000, 1023, 1024, 1025, 1026, 1400, 2047, 2048, 2049, 3001,
                                                          4095, 4096, 4097)]
                          + [(33, 1030), (34, 1030), (34, 2049), (74, 1024), (75, 1024), (74, 2048), (74, 4096), (75, 2100), (148, 1000),
-                            (149, 1000), (149, 768)])
+                            (149, 1000), (149, 768), (149, 769), (149, 1500), (149, 2817),
+                            (75, 4500), (75, 6001), (40, 9000), (75, 8193), (3, 16384), (40, 16384), (75, 16001)])
 def test_order_and_sums(segments, N, kind):
     rng = np.random.default_rng(segments * 10000 + N)
     shape = (segments, N)
