@@ -745,11 +745,10 @@ static int clusters_of_four()
 //   two 6.5), 768 6.4 / 8.3, 1024 8.2 / 9.0 (7.6); 512 of 256 6.7 / 9.5, 640 14.6 / 17.8, 768 18.1 / 21.2, 1024 24.9 / 18.7;
 //   of 1024 148 8.5 / 9.3, 160 13.7 / 11.9.
 // Merging takes the square of the runs, so the line falls to 768 where a block of 1024 threads is more than an SM's first.
-//   Clusters of two, one item a thread: 64 of 1024 12.1 at 2048 (13.0); two and four items: 32 of 3000 15.6 (18.0), 4096 18.2 (24.0).
-//   Clusters of four: 32 of 1536 9.3 (two: 9.5), 2048 10.6 (11.7), 3000 13.1 (15.6), 4096 16.4 (18.2), while all run at once (33 of
-//   four on a B200): 40 of 2048 13.9 (11.9), of 4096 26.9 (18.1).  Beyond 4096 radix passes in clusters of four or two: with
-//   compaction, whole / four, 32 of 4500 136.0 / 134.8, of 16384 264 / 238; whole / two, 64 of 16384 431 / 421; the sort alone,
-//   33 of 8193 44.4 / 28.4, 34 43.9 / 54.2, and 36.7 over two.
+//   Clusters of two: 64 of 2048 12.1 with one item a thread (whole 13.0), of 3000 15.6 with four (18.0), 4096 18.2 (24.0), 5000 19.1
+//   (24.1), 8192 25.7 (33.5); with eight 25.2 there, 44.5 for 64 of 16384.
+//   Clusters of four, while all run at once (33 of them on a B200): 32 of 1536 9.3 (two: 9.5), 2048 10.6 (11.7), 3000 13.1 (15.6),
+//   4096 16.4 (18.2), 4500 16.2 (18.8), 8192 20.2 (25.2), 16384 34.7 (44.7); beyond that 40 of 2048 13.9 (11.9), of 16384 65.7 (44.6).
 static int launch_sort(const pkv_shape *s, const float *scores, int32_t *order, uint64_t *cum,
                        int32_t *seg_flags, cudaStream_t st)
 {
@@ -758,10 +757,10 @@ static int launch_sort(const pkv_shape *s, const float *scores, int32_t *order, 
     if (N > kSplit && segments <= clusters_of_four())
         return N <= 4096 ? launch_sort_items<1, true>(s, scores, order, cum, seg_flags, st, 4)
                          : launch_sort_items<4, true>(s, scores, order, cum, seg_flags, st, 4);
-    if (N > kMergeCrowded && N <= 4096 && 2 * segments <= sms)
-        return N <= 2048 ? launch_sort_items<1, true>(s, scores, order, cum, seg_flags, st, 2)
-                         : launch_sort_items<4, true>(s, scores, order, cum, seg_flags, st, 2);
-    if (N > 8192 && 2 * segments <= sms) return launch_sort_items<8, true>(s, scores, order, cum, seg_flags, st, 2);
+    if (N > kMergeCrowded && 2 * segments <= sms)
+        return N <= 2048   ? launch_sort_items<1, true>(s, scores, order, cum, seg_flags, st, 2)
+               : N <= 8192 ? launch_sort_items<4, true>(s, scores, order, cum, seg_flags, st, 2)
+                           : launch_sort_items<8, true>(s, scores, order, cum, seg_flags, st, 2);
     if (N <= (segments <= sms ? kSplit : kMergeCrowded)) return launch_sort_items<1>(s, scores, order, cum, seg_flags, st);
     if (N <= 4096) return launch_sort_items<4>(s, scores, order, cum, seg_flags, st);
     if (N <= 8192) return launch_sort_items<8>(s, scores, order, cum, seg_flags, st);

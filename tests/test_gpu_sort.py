@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
                                                          4095, 4096, 4097)]
                          + [(33, 1030), (34, 1030), (34, 2049), (74, 1024), (75, 1024), (74, 2048), (74, 4096), (75, 2100), (148, 1000),
                             (149, 1000), (149, 768), (149, 769), (149, 1500), (149, 2817),
-                            (75, 4500), (75, 6001), (40, 9000), (75, 8193), (3, 16384), (40, 16384), (75, 16001)])
+                            (75, 4500), (75, 6001), (34, 4097), (34, 6001), (74, 8192), (40, 9000), (75, 8193), (3, 16384), (40, 16384), (75, 16001)])
 def test_order_and_sums(segments, N, kind):
     rng = np.random.default_rng(segments * 10000 + N)
     shape = (segments, N)
