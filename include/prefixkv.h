@@ -101,7 +101,8 @@ const char *prefixkv_last_cuda_error(void);
  * tensor map can describe, e.g. a zero stride, use FMA, and so do fp32 prompts of up to 64 tokens
  * with heads of 64 and the caller's lse.
  * The workspace holds per-head partial sums and work counters: calls that share one must
- * not overlap on the GPU.  The call has no status argument: if a bounded wait inside the
+ * not overlap on the GPU.  An fp32 prompt of a few hundred tokens keeps its logits there, too; a
+ * workspace that was sized for a longer prompt serves without.  The call has no status argument: if a bounded wait inside the
  * tensor-core kernel runs out, every score of the call is written as NaN, which
  * prefixkv_search / prefixkv_apply_lengths report as PKV_DEV_BAD_SCORE.
  */

@@ -72,21 +72,22 @@ int launch_score_tc(const pkv_shape *s, const void *q, pkv_strides qs, const voi
 bool score_tc_usable(const pkv_shape *s, const void *q, pkv_strides qs, const void *k, pkv_strides ks);
 
 size_t score_tc_ws_bytes(const pkv_shape *s);
-size_t score_split_ws_bytes(const pkv_shape *s);
+size_t score_split_ws_bytes(const pkv_shape *s, bool least);
 int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const float *k, pkv_strides ks,
-                       const float *scale, const float *lse, float *scores, void *ws, cudaStream_t st);
+                       const float *scale, const float *lse, float *scores, void *ws, size_t ws_bytes, cudaStream_t st);
 int selftest_wait_score(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_stream(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_flags(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_fused(int32_t *dev_status, cudaStream_t st);
 int selftest_wait_parts(int32_t *dev_status, cudaStream_t st);
 
-static size_t score_ws_bytes(const pkv_shape *s)
+// (least: what a call cannot do without; with all of it fp32 prompts of a few tiles take one pass instead of two)
+static size_t score_ws_bytes(const pkv_shape *s, bool least)
 {
     // per-head column sums + per-query log-sum-exp, both [B, L, H, N] fp32; the tensor-core
     // path pads the second to whole 128-query tiles
     size_t per = (size_t)s->batch * s->layers * s->heads * s->prompt_len * sizeof(float);
-    size_t simt = round_up(2 * per, kWsAlign), tc = score_tc_ws_bytes(s), split = score_split_ws_bytes(s);
+    size_t simt = round_up(2 * per, kWsAlign), tc = score_tc_ws_bytes(s), split = score_split_ws_bytes(s, least);
     size_t need = simt > tc ? simt : tc;
     return need > split ? need : split;
 }
@@ -126,7 +127,7 @@ extern "C" size_t prefixkv_workspace_bytes(const pkv_shape *shape, int which)
 {
     if (!shape_ok(shape) || !shape_supported(shape)) return 0;
     switch (which) {
-    case PKV_WS_SCORE: return score_ws_bytes(shape);
+    case PKV_WS_SCORE: return score_ws_bytes(shape, false);
     case PKV_WS_SEARCH: return kWsAlign;
     case PKV_WS_COMPACT:
         return round_up((size_t)shape->batch * shape->layers * shape->prompt_len * sizeof(int32_t),
@@ -149,7 +150,7 @@ extern "C" int prefixkv_score(const pkv_shape *shape, const void *q, pkv_strides
     if (!aligned(q, 16) || !aligned(k, 16)) return PKV_ERR_INVALID_ARG;
     if ((size_t)shape->batch * shape->layers > 65535 || shape->heads > 65535)
         return PKV_ERR_UNSUPPORTED;
-    if (!ws || !aligned(ws, kWsAlign) || ws_bytes < score_ws_bytes(shape)) return PKV_ERR_WORKSPACE;
+    if (!ws || !aligned(ws, kWsAlign) || ws_bytes < score_ws_bytes(shape, true)) return PKV_ERR_WORKSPACE;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     if (shape->dtype == PKV_BF16) {
         if (score_tc_usable(shape, q, qs, k, ks)) {
@@ -167,7 +168,8 @@ extern "C" int prefixkv_score(const pkv_shape *shape, const void *q, pkv_strides
     // 16.7 / 58.9 and 12.4 / 57.6; heads of 128 14.1 / 52.3 and 9.8 / 47.2; 100 tokens 14.6 / 84.0 and 10.3 / 43.5.
     if (lse && shape->head_dim == 64 && shape->prompt_len <= 64)
         return launch_score_simt<float, 64>(shape, q, qs, k, ks, layer_scale, lse, scores, ws, stream);
-    return launch_score_split(shape, (const float *)q, qs, (const float *)k, ks, layer_scale, lse, scores, ws, stream);
+    return launch_score_split(shape, (const float *)q, qs, (const float *)k, ks, layer_scale, lse, scores, ws, ws_bytes,
+                              stream);
 }
 
 extern "C" int prefixkv_gini(const pkv_shape *shape, const uint64_t *cum, double *gini,

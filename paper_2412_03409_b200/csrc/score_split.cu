@@ -694,17 +694,18 @@ int launch_head_mean(const float *partial, int H, int N, size_t total, float *sc
                      cudaStream_t st);
 
 // Workspace: partial [rows][N], lse2 [rows][N], then two work counters and the abort word.  Short prompts: part sums of every
-// pair of tiles in the place of these, and the logits of a CTA's item.
+// pair of tiles in the place of these, and the logits of a CTA's item, where the workspace has room for them: one that was sized
+// for a longer prompt need not, and then serves two passes.
 struct SplitSpace {
     size_t partial, lse2, logits, words, bytes;
 };
-static SplitSpace split_space(const pkv_shape *s)
+static SplitSpace split_space(const pkv_shape *s, bool keep)
 {
     const size_t heads = (size_t)s->batch * s->layers * s->heads, tiles = ((size_t)s->prompt_len + TT - 1) / TT;
     const size_t per = heads * s->prompt_len * sizeof(float);
     SplitSpace w = {0, per, 0, 0, 0};
     size_t end = 2 * per;
-    if (keeps_logits((int)tiles, s->head_dim)) {
+    if (keep) {
         const size_t parts = heads * (tiles * (tiles + 1) / 2) * (4 * TT) * sizeof(float);
         const size_t ctas = heads * tiles < kKeepCtas ? heads * tiles : kKeepCtas;
         w.logits = round_up(parts, kWsAlign);
@@ -715,13 +716,18 @@ static SplitSpace split_space(const pkv_shape *s)
     w.bytes = w.words + kWsAlign;
     return w;
 }
-size_t score_split_ws_bytes(const pkv_shape *s) { return split_space(s).bytes; }
+static bool split_keeps(const pkv_shape *s)
+{
+    return s->dtype == PKV_F32 && keeps_logits((s->prompt_len + TT - 1) / TT, s->head_dim);
+}
+size_t score_split_ws_bytes(const pkv_shape *s, bool least) { return split_space(s, !least && split_keeps(s)).bytes; }
 
 int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const float *k, pkv_strides ks,
-                       const float *scale, const float *lse, float *scores, void *ws, cudaStream_t st)
+                       const float *scale, const float *lse, float *scores, void *ws, size_t ws_bytes, cudaStream_t st)
 {
     const int B = s->batch, L = s->layers, H = s->heads, N = s->prompt_len;
-    const SplitSpace space = split_space(s);
+    const bool keep = !lse && split_keeps(s) && ws_bytes >= split_space(s, true).bytes;
+    const SplitSpace space = split_space(s, keep);
     unsigned char *mem = (unsigned char *)ws;
     SplitArgs a = {};
     a.q = q; a.k = k; a.qs = qs; a.ks = ks;
@@ -758,7 +764,7 @@ int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const
             return wide ? launch_split<0, 128>(a, sms, st) : launch_split<0, 64>(a, sms, st);
         }
         rc = wide ? launch_split<0, 128>(a, sms, st) : launch_split<0, 64>(a, sms, st);
-    } else if (!lse && keeps_logits(a.tiles, s->head_dim)) {
+    } else if (keep) {
         a.next_item = counted ? words : nullptr;
         const int ctas = sms < (int)kKeepCtas ? sms : (int)kKeepCtas;
         rc = wide ? launch_split<3, 128>(a, ctas, st) : launch_split<3, 64>(a, ctas, st);

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2412_03409_b200 import api
 from paper_2412_03409_b200.session import Session
 
 pytestmark = pytest.mark.gpu
@@ -72,3 +73,16 @@ def test_elements_that_have_no_split(D, bad):
     ok = ~torch.isnan(ref)
     assert bool(ok.any()) or bad == float("inf")
     assert bool((((got - ref).abs() / ref.clamp(min=1e-3))[ok] <= TOL).all())
+
+
+@pytest.mark.parametrize("D,N,longer", [(128, 512, 4096), (64, 1500, 2100), (128, 129, 1025)])
+def test_workspace_of_a_longer_prompt(D, N, longer):
+    """It holds less than keeping the logits takes, and serves all the same."""
+    g = torch.Generator(device="cuda").manual_seed(N)
+    q, k = (torch.randn(1, 1, 2, N, D, device="cuda", generator=g) for _ in range(2))
+    scale = np.full(1, 1 / np.sqrt(D), np.float32)
+    s = Session(1, 1, 2, D, N, torch.float32, scale, decode_cap=0, max_budget_rows=1)
+    s.ws_score = api.alloc_workspace(api.make_shape(1, 1, 2, D, longer, torch.float32), api.WS_SCORE, "cuda")
+    assert s.ws_score.numel() < api.alloc_workspace(s.shape, api.WS_SCORE, "cuda").numel()
+    ref = _exact(q, k, scale)
+    assert ((s.score(q, k).double() - ref).abs() / ref.clamp(min=1e-3)).max().item() <= TOL
