@@ -263,7 +263,7 @@ int prefixkv_compact_merge(const pkv_shape *shape, const void *k, pkv_strides ks
  * generated token g would push a layer past floor(len0 * (N + g + 1) / N) rows and token
  * g - d is still cached, the new row takes that token's slot and len stays; otherwise it is
  * appended.  Prompt rows are never dropped.  Calls on one cache, or sharing one workspace, must not overlap on
- * the GPU; while a call runs that appends, the words of len may hold other values than lengths.
+ * the GPU.
  * The call only enqueues kernels on cuda_stream, so it may be captured into a CUDA graph and
  * replayed once per token (same pointers, new contents); make one call on the device outside
  * any capture first, which sets the kernels up.

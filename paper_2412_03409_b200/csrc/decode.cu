@@ -164,7 +164,7 @@ size_t decode_stream_ws_bytes(const pkv_shape *s);
 size_t decode_heads_ws_bytes();
 bool decode_stream_covers(const pkv_shape *s, int nact);
 int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn, const void *vn,
-                          const float *scale, int lb, int le, void *out, int32_t *dev_status, cudaStream_t st);
+                          const float *scale, int lb, int le, void *out, int32_t *dev_status, void *ws, cudaStream_t st);
 int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn, const void *vn,
                         const float *scale, int lb, int le, void *out, int32_t *dev_status, void *ws, cudaStream_t st);
 int launch_decode_stream(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn,
@@ -233,7 +233,7 @@ extern "C" int prefixkv_decode_attn(const pkv_shape *shape, pkv_cache *cache, co
     if (covered) {
         // Few (segment, head) pairs, a layer at a time: a cluster for each, one launch.
         int rc = launch_decode_cluster(shape, cache, q, k_new, v_new, layer_scale, layer_begin, layer_end, out, dev_status,
-                                       st);
+                                       ws, st);
         if (rc >= 0) return rc;  // -1: not a case for that kernel
     }
     {

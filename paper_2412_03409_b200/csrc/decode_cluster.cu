@@ -9,10 +9,13 @@
 // CTAs' partial softmax states go to the first CTA of the cluster through distributed shared memory,
 // which merges them in rank order and writes the head's output: one launch, nothing in global memory
 // in between.  The last CTA of a cluster also attends to the new row and appends it.
-// Lengths: a CTA reads its segment's length by adding one to the upper bits of its word, which so counts
-// the CTAs that have been there; the last of them writes the length of the next step over it.  A call
-// that appends nothing leaves the word alone.  (Before, every CTA raised a flag in the workspace and an
-// extra cluster waited for them: its chain of round trips ended after the rows', 4.43 us a call below for 3.96 without.)
+// Lengths: every CTA reads its segment's length and then counts itself in a word of the workspace; the one that
+// completes the count writes the length of the next step.  A call that appends nothing counts nothing.  (Every CTA
+// raising a flag in the workspace, and an extra cluster waiting for them: its chain of round trips ended after the rows',
+// 4.43 us a call below for 3.96 without.  A count in the upper bits of the length's own word: a word that was no length
+// before the call could pass for one that some CTAs had been at.  Plan and count by a thread of the first warp, which
+// may have the new row to take: 3.65 us a call for 3.51; the count only after the barrier: 3.82; its answer looked at
+// before the rows: 3.80; by the clusters' first CTAs alone, after their merge's first barrier: 3.90.)
 // Where the rows are is also read ahead, while the kernel in front still runs: the rows of that guess are
 // asked for as soon as it has completed, and the guess is held against the plan made afterwards.  The
 // values are not looked at before then, so that a CTA that starts late has both loads on their way at once
@@ -43,6 +46,7 @@ bool decode_stream_covers(const pkv_shape *s, int nact);
 namespace {
 
 constexpr int kCWarps = 4;             // warps per CTA
+constexpr int kPlanner = kCWarps * 32 - 32;  // the thread that reads a CTA's plan and counts: not of the warp that takes the new row
 constexpr int kCStages = 2;            // rounds in flight per warp
 constexpr int kCPerSm = 5;             // CTAs an SM holds at a time, rounds of four steps (their rings fill its shared memory)
 constexpr int kCMaxCluster = 8;        // portable cluster size
@@ -55,9 +59,10 @@ struct ClusterArgs {
     const void *q, *k_new, *v_new;
     void *ck, *cv, *out;
     const float *layer_scale;
+    unsigned long long *visits;  // [active segments][kVisitStride] how many CTAs have read the segment's length
+    unsigned long long visit_tag;
     int32_t *dev_status;
-    int H, visit_shift;  // a length's word counts its readers from this bit on
-    uint32_t guess_mask;  // what a length read ahead is taken from: the word without that count, where CTAs come in waves
+    int H;
     uint32_t row_bytes;
 };
 
@@ -124,12 +129,11 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
     __shared__ float s_ml[kCWarps][2];
     __shared__ float c_acc[P == kCPerSm ? kCMaxCluster : 1][D], c_ml[kCMaxCluster][2];  // (first CTA of a cluster) the cluster's partials
 
-    __shared__ SegPlan s_plan[2];
+    __shared__ SegPlan s_plan;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int C = (int)cluster_size(), rank = (int)cluster_rank();
-    const int item = blockIdx.x / C;
-    // (the first CTA must be running before anyone writes to its shared memory)
+    const int item = blockIdx.x / C;    // (the first CTA must be running before anyone writes to its shared memory)
     if (C > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
     const int si = item / a.H, h = item - si * a.H;
@@ -173,8 +177,6 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    // A length's word: the length, and above it how many of the segment's CTAs have been there.
-    const uint32_t ln_mask = a.p.append ? (1u << a.visit_shift) - 1u : 0xffffffffu;
     // Where the rows are is read before the kernel in front has completed, and the first rounds are asked for as soon
     // as it has, together with the plan that counts.  Should that one be another, they are asked for again.
     const bool guesses = a.p.evict_distance == 0;
@@ -186,23 +188,28 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
         guess_off = load_l2(a.p.row_offset + seg);
     }
     dependent_entry();
-    // The length is read by adding to its word's upper bits: whoever finds that all CTAs of the segment but itself have
-    // been there writes what the step leaves.  (With pruning what else the plan is made of has been read before that.)
-    uint32_t word = 0;
-    int cp = 0;
+    int ln = 0, cp = 0;
     int64_t off = 0;
+    unsigned long long seen = 0, before = 0, *const visits = a.visits + (size_t)si * kVisitStride;
     PruneState ps;
-    if (tid == 0) {
+    if (tid == kPlanner) {
         ps = prune_state(a.p, seg);
-        if (!a.p.append) word = (uint32_t)load_l2(a.p.len + seg);
-        else if (a.p.evict_distance == 0) asm volatile("atom.relaxed.gpu.global.add.u32 %0, [%1], %2;" : "=r"(word) : "l"(a.p.len + seg), "r"(1u << a.visit_shift) : "memory");
-        else asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(word) : "l"(a.p.len + seg), "r"(1u << a.visit_shift) : "memory");
+        ln = load_l2(a.p.len + seg);
         cp = load_l2(a.p.cap + seg);
         off = load_l2(a.p.row_offset + seg);
+        if (a.p.append) seen = load_flag(visits);
     }
+    // When all of the segment's CTAs have read its length.  The answer comes while the rows are looked at; it is not kept waiting where six
+    // and seven CTAs of an SM leave a thread few registers (1024 pairs of 140 rows 15.6 us so, 15.9 after the rows; 2048 pairs, five CTAs
+    // an SM: 27.2 and 26.2).
+    auto last_one = [&]() {
+        if (tid != kPlanner || before != a.visit_tag + (uint32_t)(a.H * C - 1)) return;
+        settle_visits(visits, a.visit_tag, a.p.evict_distance > 0);
+        segment_advance(a.p, si, s_plan);
+    };
     Rows rw{nullptr, nullptr, 0, 0, -1};
     if (guesses) {
-        rw = rows_of(plan_of(a.p, (int)((uint32_t)guess_ln & a.guess_mask), guess_cp, guess_off, PruneState{0, 0, -1}));
+        rw = rows_of(plan_of(a.p, guess_ln, guess_cp, guess_off, PruneState{0, 0, -1}));
 #pragma unroll
         for (int i = 0; i < kCStages; ++i) request(rw, rw.r0 + (warp + i * kCWarps) * STEP, i);
     }
@@ -213,20 +220,16 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
         vnew = *reinterpret_cast<const uint4 *>(static_cast<const unsigned char *>(a.v_new) + hoff + c * 16);
     }
     const float sc = a.layer_scale[a.p.layer_begin + si % a.p.nl] * kLog2eC;
-    if (tid == 0) {
-        const uint32_t before = a.p.append ? word >> a.visit_shift : 0u, all = (uint32_t)(a.H * C);
-        SegPlan sp = plan_of(a.p, (int)(word & ln_mask), cp, off, ps);
-        if (before >= all) sp.rows = -1;  // (the word was no length)
-        if (sp.rows < 0) {  // (every CTA finds the same, and takes back what it added)
-            raise_status(a.dev_status, si / a.p.nl, PKV_DEV_CAPACITY);
-            if (a.p.append) atomicSub(reinterpret_cast<unsigned int *>(a.p.len + seg), 1u << a.visit_shift);
-        } else if (a.p.append && before == all - 1) {
-            segment_advance(a.p, si, sp);
-        }
-        s_plan[1] = sp;
+    if (tid == kPlanner) {
+        const SegPlan sp = plan_of(a.p, ln, cp, off, ps);
+        s_plan = sp;
+        // (a segment that cannot take the step is counted by nobody; the count's answer is looked at later)
+        if (sp.rows < 0) raise_status(a.dev_status, si / a.p.nl, PKV_DEV_CAPACITY);
+        else if (a.p.append) before = count_visit(visits, a.visit_tag, seen, a.p.evict_distance > 0);
     }
     __syncthreads();
-    const SegPlan sp = s_plan[1];
+    const SegPlan sp = s_plan;
+    if (P != kCPerSm) last_one();
     const Rows now = rows_of(sp);
     if (now.r0 != rw.r0 || now.r1 != rw.r1 || now.skip != rw.skip || now.kb != rw.kb) {
         // (a row more or less at the end: the same bytes come to the same places again)
@@ -320,6 +323,8 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
             *reinterpret_cast<uint4 *>(static_cast<unsigned char *>(a.cv) + at) = vnew;
         }
     }
+
+    if (P == kCPerSm) last_one();
 
     // ---- merge: lane groups, warps, then the CTAs of the cluster ---------------------------------------
 #pragma unroll
@@ -417,7 +422,7 @@ template <int U, int P> int launch_shape(const pkv_shape *s, const ClusterArgs &
 
 // Returns PKV_OK, an error, or -1 when this call is outside what the kernel covers.
 int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn, const void *vn,
-                          const float *scale, int lb, int le, void *out, int32_t *dev_status, cudaStream_t st)
+                          const float *scale, int lb, int le, void *out, int32_t *dev_status, void *ws, cudaStream_t st)
 {
     const int H = s->heads, D = s->head_dim, nl = le - lb, nact = s->batch * nl;
     const int sms = sm_count();
@@ -472,17 +477,14 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
         if (!one_wave && seg_rows < 256 * (int64_t)n) break;
         C = n;
     }
-    // (the bits of a length's word that its readers are counted in leave room for any length)
-    int visit_bits = 1;
-    while ((H * C) >> visit_bits) ++visit_bits;
-    if (c->total_cap_rows >> (32 - visit_bits)) return -1;
+    if ((int64_t)H * C >= (int64_t)1 << kVisitBits) return -1;
 
     ClusterArgs a;
     a.p = decode_plan_args(s, c, kn != nullptr, lb, nl);
     a.q = q; a.k_new = kn; a.v_new = vn; a.ck = c->k; a.cv = c->v; a.out = out;
     a.layer_scale = scale;
-    a.visit_shift = 32 - visit_bits;
-    a.guess_mask = kn != nullptr && items * C > wave ? (1u << a.visit_shift) - 1u : 0xffffffffu;
+    a.visits = (unsigned long long *)ws;
+    a.visit_tag = visit_tag();
     a.dev_status = dev_status;
     a.H = H;
     a.row_bytes = (uint32_t)((size_t)H * D * esize(s));

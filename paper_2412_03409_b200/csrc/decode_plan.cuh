@@ -1,6 +1,8 @@
-// What one decode step does to a segment, 16-byte row vectors, and the flags that order the reads of the
-// lengths before their writes: shared by the decode kernels.
+// What one decode step does to a segment, 16-byte row vectors, and the flags and counts that order the reads of
+// the lengths before their writes: shared by the decode kernels.
 #pragma once
+#include <chrono>
+
 #include "common.cuh"
 
 namespace pkv {
@@ -205,6 +207,39 @@ __device__ __forceinline__ bool settle_flags(unsigned long long *flags, int n, u
     for (int i = threadIdx.x; i < n; i += blockDim.x)
         if (all_in || atomicExch(flags + i, token ^ kGone) == token) lower_flag(flags + i);
     return all_in;
+}
+
+// ---- counts: how many of a segment's CTAs have read its length ----------------------------------------
+// One word per segment in the workspace, which may hold anything before: a tag of this process in the upper bits says that the
+// lower ones are a count.  Calls leave it at none.
+constexpr int kVisitBits = 20;
+constexpr int kVisitStride = 16;  // words from one segment's to the next (in one line, 32 segments' counts are made one by one: +0.1 us)
+
+inline unsigned long long visit_tag()
+{
+    static const unsigned long long tag =
+        (0x9e3779b97f4a7c15ull ^ (unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count()) << kVisitBits;
+    return tag;
+}
+// One thread of a CTA, after its reads; `seen` is what the word held a moment ago.  Tag and count, itself not included: the first
+// to come makes the word a count.  (Whether to count at all hangs on the length, so the count cannot come before its read;
+// `others` asks for the same of what else was read.)
+__device__ __forceinline__ unsigned long long count_visit(unsigned long long *word, unsigned long long tag, unsigned long long seen, bool others)
+{
+    unsigned long long before;
+    if (others) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    if (seen >> kVisitBits != tag >> kVisitBits) {
+        before = atomicCAS(word, seen, tag + 1);
+        if (before == seen) return tag;
+    }
+    asm volatile("atom.relaxed.gpu.global.add.u64 %0, [%1], 1;" : "=l"(before) : "l"(word) : "memory");
+    return before;
+}
+// The thread that found itself to be the last, before it writes what all have read.
+__device__ __forceinline__ void settle_visits(unsigned long long *word, unsigned long long tag, bool others)
+{
+    if (others) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    *(volatile unsigned long long *)word = tag;
 }
 
 // ---- parts of an item that CTAs pass on: a flag of the same kind for each, which the CTA that takes the parts puts back ----

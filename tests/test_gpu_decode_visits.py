@@ -95,7 +95,9 @@ def test_a_cta_to_a_pair(B, L, H, D, rows, dtype):
             assert (again[i // L, i % L].double() - _attend(s, tok[0][0], i, n + T)).abs().max().item() <= TOL[dtype]
 
 
-@pytest.mark.parametrize("word", [0, -1, 2**31 - 1, -2**31, 0x7f7f7f7f, "full", "above"])
+# (words whose lower bits would be a length, with bits set above them: anything but a length is refused)
+@pytest.mark.parametrize("word", [0, -1, 2**31 - 1, -2**31, 0x7f7f7f7f, "full", "above", 30 + (1 << 20), 30 + (1 << 28), 5 + (3 << 28),
+                                  5 + (3 << 26), 31 + (7 << 24), 31 + (100 << 24), 5 - 2**31, 30 - 2**31 + (1 << 26)])
 @pytest.mark.parametrize("H", [1, 5, 64])
 def test_a_segment_that_cannot_take_the_row_keeps_its_word(word, H):
     s, tok = _session(2, 1, H, 64, [40, 30], torch.bfloat16, 2)
