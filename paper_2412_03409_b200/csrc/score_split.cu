@@ -48,7 +48,7 @@ constexpr uint32_t kPart = TT * 128;         // bytes of one bf16 part of a chun
 constexpr uint32_t kChunk = 3 * kPart;
 constexpr uint32_t kBuf = 256;               // tensor-memory columns of one of the two accumulator buffers
 constexpr int kMeanHeads = 8;                // CTAs of a portable cluster
-constexpr int kKeepTiles = 16;               // tiles of the longest prompt whose logits are kept (1 MiB a CTA), heads of 64
+constexpr int kKeepTiles = 8, kKeepTilesFew = 16;  // tiles of the longest prompt whose logits are kept (1 MiB a CTA)
 constexpr size_t kKeepCtas = 148;            // CTAs of such a call at most
 constexpr int kBack = 16;                    // rows of them a warp reads back at a time
 constexpr int kQueue = 4;                    // item numbers in flight between the loaders and the other roles
@@ -655,10 +655,22 @@ __global__ void __launch_bounds__(256) split_mean_kernel(const float *__restrict
     scores[(size_t)seg * N + n] = *abort_word != 0 ? __int_as_float(0x7fc00000) : sum / (float)H;
 }
 
-// Whether mode 3 takes a prompt, without the caller's log-sum-exp.  Two passes / kept logits, us a call, tokens x heads: heads
-// of 128, 130 x 192 50.2 / 36.2, 300 x 16 27.5 / 19.1, 512 x 128 79.9 / 69.7, 777 x 128 167.5 / 161.2, 900 x 6 48.6 / 44.5, but
-// 1500 x 4 66.2 / 69.8 and x 16 109.8 / 111.9; heads of 64, 256 x 192 45.1 / 35.3, 777 x 128 145.7 / 126.2, 1500 x 4 68.1 / 58.1.
-bool keeps_logits(int tiles, int D) { return tiles >= 2 && tiles <= (D == 128 ? kKeepTiles / 2 : kKeepTiles); }
+// Whether mode 3 takes a prompt, without the caller's log-sum-exp.  Us a call, tokens x heads:
+//   heads of 128    two passes  kept      heads of 64     two passes  kept
+//   130 x 192          53.0     37.4      256 x 192          49.3     36.9
+//   300 x 1024          333      237      256 x 1536          227      160
+//   777 x 128           168      163      777 x 128           146      128
+//   1024 x 1024        1575     1540      1024 x 1536        1959     1872
+//   1500 x 4           84.1     71.9      1152 x 128          224      231
+//   1500 x 16           107      125      2048 x 1536        7086     8370
+// With more than eight tiles to an item the logits in use leave the L2, unless a CTA has one item: with heads of 64, 1152 x 16
+// 56.6 / 50.6, 1500 x 12 73.2 / 65.1, x 16 (192 items) 92.0 / 98.3, 2048 x 7 89.9 / 79.6, x 9 91.9 / 92.5.
+bool keeps_logits(size_t heads, int tiles, int D)
+{
+    if (tiles < 2) return false;
+    if (tiles <= kKeepTiles) return true;
+    return D == 64 && tiles <= kKeepTilesFew && heads * tiles <= kKeepCtas;
+}
 
 template <int MODE, int D> int launch_split(const SplitArgs &a, int sms, cudaStream_t st)
 {
@@ -718,7 +730,7 @@ static SplitSpace split_space(const pkv_shape *s, bool keep)
 }
 static bool split_keeps(const pkv_shape *s)
 {
-    return s->dtype == PKV_F32 && keeps_logits((s->prompt_len + TT - 1) / TT, s->head_dim);
+    return s->dtype == PKV_F32 && keeps_logits((size_t)s->batch * s->layers * s->heads, (s->prompt_len + TT - 1) / TT, s->head_dim);
 }
 size_t score_split_ws_bytes(const pkv_shape *s, bool least) { return split_space(s, !least && split_keeps(s)).bytes; }
 

@@ -108,3 +108,15 @@ def test_the_decode_binding_is_this_interpreters(api, monkeypatch, tmp_path):
     for call in (api._decode_attn, by_ctypes):
         if call is by_ctypes or torch.cuda.is_available():
             assert call(sh, cache, None, None, None, None, 0, 2, None, None, None) == api.PKV_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("heads,D,N,kept", [(1, 64, 128, False), (9999, 64, 129, True), (9999, 64, 1024, True), (16, 64, 1025, True), (17, 64, 1025, False),
+                                            (9, 64, 2048, True), (10, 64, 2048, False), (8, 64, 2049, False), (9999, 128, 1024, True),
+                                            (1, 128, 1025, False)])
+def test_which_fp32_prompts_keep_their_logits(api, heads, D, N, kept):
+    """By the workspace they ask for: logits that leave the L2 cost more than a second pass."""
+    import torch
+    two = 2 * heads * N * 4
+    need = api.prefixkv_workspace_bytes(api.make_shape(1, 1, heads, D, N, torch.float32), api.WS_SCORE)
+    least = api.prefixkv_workspace_bytes(api.make_shape(1, 1, heads, D, N, torch.bfloat16), api.WS_SCORE)
+    assert (need > max(two, least) + 1024) == kept, (need, two, least)

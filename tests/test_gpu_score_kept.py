@@ -1,5 +1,5 @@
-"""fp32 prompts whose logits are kept for the column sums (2 to 8 tiles of 128 tokens, 16 with heads of 64) and the lengths
-around them (needs a B200).  Against 64 bits."""
+"""fp32 prompts whose logits are kept for the column sums (2 to 8 tiles of 128 tokens; with heads of 64 16, with a CTA for
+each) and the lengths around them (needs a B200).  Against 64 bits."""
 import numpy as np
 import pytest
 import torch
@@ -25,6 +25,7 @@ def _exact(q, k, scale):
     (1, 1, 2, 128, 1024), (1, 1, 2, 128, 1025), (1, 1, 1, 64, 1921), (1, 1, 1, 64, 2048), (1, 1, 1, 64, 2049),
     (1, 12, 16, 64, 150),      # more items than CTAs
     (3, 9, 17, 128, 130),
+    (1, 3, 7, 64, 1024), (1, 1, 17, 64, 1025), (1, 1, 14, 64, 1280), (1, 1, 15, 64, 1280),   # ten tiles: 140 items, and 150 in two passes
 ])
 @pytest.mark.parametrize("sign", [1, -1])
 def test_scores(B, L, H, D, N, sign):
