@@ -71,10 +71,11 @@ typedef struct {
     int64_t b, l, h, n;
 } pkv_strides;
 
-enum { PKV_WS_SCORE = 0, PKV_WS_SEARCH = 1, PKV_WS_COMPACT = 2, PKV_WS_DECODE = 3 };
+enum { PKV_WS_SCORE = 0, PKV_WS_SEARCH = 1, PKV_WS_COMPACT = 2, PKV_WS_DECODE = 3, PKV_WS_SCORE_LEAST = 4 };
 
 /* Bytes of 256-byte-aligned workspace the named call needs for this shape.
- * Returns 0 for an unknown `which` or an unsupported shape. */
+ * Returns 0 for an unknown `which` or an unsupported shape.  PKV_WS_SCORE_LEAST: what prefixkv_score cannot do
+ * without, and all that it uses with the caller's log-sum-exp; PKV_WS_SCORE: what it can use besides. */
 size_t prefixkv_workspace_bytes(const pkv_shape *shape, int which);
 
 /* Text of the last CUDA error seen by this library on the calling thread (host). */
@@ -101,8 +102,10 @@ const char *prefixkv_last_cuda_error(void);
  * tensor map can describe, e.g. a zero stride, use FMA, and so do fp32 prompts of up to 64 tokens
  * with heads of 64 and the caller's lse.
  * The workspace holds per-head partial sums and work counters: calls that share one must
- * not overlap on the GPU.  An fp32 prompt of a few hundred tokens keeps its logits there, too; a
- * workspace that was sized for a longer prompt serves without.  The call has no status argument: if a bounded wait inside the
+ * not overlap on the GPU.  The logits of fp32 prompts of 129 to 1024 tokens (2048 with heads of 64 while
+ * heads x tiles of 128 tokens are no more than 148) are kept there, too, a thread block's at a time: PKV_WS_SCORE asks for up to
+ * 74 (148) MiB for them and 128 MiB of part sums, of which longer prompts need none.  A workspace of
+ * PKV_WS_SCORE_LEAST serves without, in a second pass over Q and K.  The call has no status argument: if a bounded wait inside the
  * tensor-core kernel runs out, every score of the call is written as NaN, which
  * prefixkv_search / prefixkv_apply_lengths report as PKV_DEV_BAD_SCORE.
  */

@@ -20,7 +20,7 @@ from . import build as _build
  PKV_ERR_STATIC_LIMIT) = range(6)
 (DEV_OK, DEV_BAD_SCORE, DEV_RANGE, DEV_BUDGET_TOO_SMALL, DEV_BAD_LENGTH, DEV_CAPACITY,
  DEV_TIMEOUT) = range(7)
-WS_SCORE, WS_SEARCH, WS_COMPACT, WS_DECODE = range(4)
+WS_SCORE, WS_SEARCH, WS_COMPACT, WS_DECODE, WS_SCORE_LEAST = range(5)
 MERGE_POSITION, MERGE_FEATURE = 1, 2
 F32, BF16 = 0, 1
 

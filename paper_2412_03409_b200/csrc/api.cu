@@ -128,6 +128,7 @@ extern "C" size_t prefixkv_workspace_bytes(const pkv_shape *shape, int which)
     if (!shape_ok(shape) || !shape_supported(shape)) return 0;
     switch (which) {
     case PKV_WS_SCORE: return score_ws_bytes(shape, false);
+    case PKV_WS_SCORE_LEAST: return score_ws_bytes(shape, true);
     case PKV_WS_SEARCH: return kWsAlign;
     case PKV_WS_COMPACT:
         return round_up((size_t)shape->batch * shape->layers * shape->prompt_len * sizeof(int32_t),

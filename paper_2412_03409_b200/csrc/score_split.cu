@@ -50,6 +50,7 @@ constexpr uint32_t kBuf = 256;               // tensor-memory columns of one of 
 constexpr int kMeanHeads = 8;                // CTAs of a portable cluster
 constexpr int kKeepTiles = 8, kKeepTilesFew = 16;  // tiles of the longest prompt whose logits are kept (1 MiB a CTA)
 constexpr size_t kKeepCtas = 148;            // CTAs of such a call at most
+constexpr size_t kPartBytes = 128u << 20;    // and its part sums: more segments than these hold take turns
 constexpr int kBack = 16;                    // rows of them a warp reads back at a time
 constexpr int kQueue = 4;                    // item numbers in flight between the loaders and the other roles
 
@@ -67,6 +68,7 @@ struct SplitArgs {
     int *next_item;       // work counter of this pass, zeroed before it; NULL: a CTA takes item blockIdx.x alone
     int clear_abort;      // this launch is the call's first and nothing has zeroed the abort word
     int L, H, N, tiles, nsh, group;
+    int seg0;             // the segment of the launch's first heads (mode 3)
 };
 
 // One float into its three bf16 parts, two elements at a time (packed low, high).  (Above the largest bf16,
@@ -120,7 +122,7 @@ template <int D> __device__ __forceinline__ float fma_logit(const float *x, cons
 }
 __device__ __forceinline__ const float *head_rows(const float *p, const pkv_strides &st, const SplitArgs &a, int sh)
 {
-    const int seg = sh / a.H, h = sh - seg * a.H, b = seg / a.L, l = seg - b * a.L;
+    const int turn = sh / a.H, h = sh - turn * a.H, seg = a.seg0 + turn, b = seg / a.L, l = seg - b * a.L;
     return p + b * st.b + l * st.l + h * st.h;
 }
 __device__ __forceinline__ void store8(float *p, const float *v)
@@ -268,7 +270,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
             }
             int sh, t;
             decode_item<PASS>(w, a.nsh, a.tiles, a.group, sh, t);
-            const int seg = sh / a.H, h = sh - seg * a.H, b = seg / a.L, l = seg - b * a.L;
+            const int turn = sh / a.H, h = sh - turn * a.H, seg = a.seg0 + turn, b = seg / a.L, l = seg - b * a.L;
             const float *qb = a.q + b * a.qs.b + l * a.qs.l + h * a.qs.h + c8 * 8;
             const float *kb = a.k + b * a.ks.b + l * a.ks.l + h * a.ks.h + c8 * 8;
             const int arow = t * TT + r0, brow = (PASS == 1 ? 0 : t) * TT + r0;
@@ -497,7 +499,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
             if (w < 0) break;
             int sh, t;
             decode_item<PASS>(w, a.nsh, a.tiles, a.group, sh, t);
-            const float sc = a.layer_scale[(sh / a.H) % a.L] * kLog2eT;
+            const float sc = a.layer_scale[(a.seg0 + sh / a.H) % a.L] * kLog2eT;
             const int grow = t * TT + row;  // query (pass 1) or key (pass 2) of this thread
             float *kept = MODE == 3 ? a.logits + ((size_t)blockIdx.x * a.tiles * TT + row) * TT : nullptr;
             float run_max = -INFINITY, run_sum = 0.f, col_sum = 0.f;
@@ -655,6 +657,14 @@ __global__ void __launch_bounds__(256) split_mean_kernel(const float *__restrict
     scores[(size_t)seg * N + n] = *abort_word != 0 ? __int_as_float(0x7fc00000) : sum / (float)H;
 }
 
+// (Calls of several turns) every score of a call is NaN when a wait in any of them ran out.
+__global__ void __launch_bounds__(256) split_abort_kernel(float *__restrict__ scores, size_t total, const int32_t *__restrict__ abort_word)
+{
+    dependent_entry();
+    if (*abort_word == 0) return;
+    for (size_t i = blockIdx.x * 256ull + threadIdx.x; i < total; i += gridDim.x * 256ull) scores[i] = __int_as_float(0x7fc00000);
+}
+
 // Whether mode 3 takes a prompt, without the caller's log-sum-exp.  Us a call, tokens x heads:
 //   heads of 128    two passes  kept      heads of 64     two passes  kept
 //   130 x 192          53.0     37.4      256 x 192          49.3     36.9
@@ -665,11 +675,12 @@ __global__ void __launch_bounds__(256) split_mean_kernel(const float *__restrict
 //   1500 x 16           107      125      2048 x 1536        7086     8370
 // With more than eight tiles to an item the logits in use leave the L2, unless a CTA has one item: with heads of 64, 1152 x 16
 // 56.6 / 50.6, 1500 x 12 73.2 / 65.1, x 16 (192 items) 92.0 / 98.3, 2048 x 7 89.9 / 79.6, x 9 91.9 / 92.5.
-bool keeps_logits(size_t heads, int tiles, int D)
+size_t part_bytes(size_t heads, size_t tiles) { return heads * (tiles * (tiles + 1) / 2) * (4 * TT) * sizeof(float); }
+bool keeps_logits(const pkv_shape *s)
 {
-    if (tiles < 2) return false;
-    if (tiles <= kKeepTiles) return true;
-    return D == 64 && tiles <= kKeepTilesFew && heads * tiles <= kKeepCtas;
+    const size_t heads = (size_t)s->batch * s->layers * s->heads, tiles = ((size_t)s->prompt_len + TT - 1) / TT;
+    if (s->dtype != PKV_F32 || tiles < 2 || part_bytes(s->heads, tiles) > kPartBytes) return false;
+    return tiles <= kKeepTiles || (s->head_dim == 64 && tiles <= kKeepTilesFew && heads * tiles <= kKeepCtas);
 }
 
 template <int MODE, int D> int launch_split(const SplitArgs &a, int sms, cudaStream_t st)
@@ -706,21 +717,26 @@ int launch_head_mean(const float *partial, int H, int N, size_t total, float *sc
                      cudaStream_t st);
 
 // Workspace: partial [rows][N], lse2 [rows][N], then two work counters and the abort word.  Short prompts: part sums of every
-// pair of tiles in the place of these, and the logits of a CTA's item, where the workspace has room for them: one that was sized
-// for a longer prompt need not, and then serves two passes.
+// pair of tiles in the place of these, of as many segments at a time as kPartBytes hold, and the logits of a CTA's item, where the
+// workspace has room for them: one that was sized for a longer prompt, or for the caller's log-sum-exp, need not, and then
+// serves two passes.  (1024 tokens, us at once, in turns of 128 MiB, 64, 16: 6144 heads of 64, 432 MiB, 7626, 7742, 7796, 8424; 1024 heads
+// of 128, 72 MiB, 1525, 1526, 1589, 1770.)
 struct SplitSpace {
     size_t partial, lse2, logits, words, bytes;
+    int turn;  // segments of a turn
 };
 static SplitSpace split_space(const pkv_shape *s, bool keep)
 {
-    const size_t heads = (size_t)s->batch * s->layers * s->heads, tiles = ((size_t)s->prompt_len + TT - 1) / TT;
+    const size_t segs = (size_t)s->batch * s->layers, heads = segs * s->heads, tiles = ((size_t)s->prompt_len + TT - 1) / TT;
     const size_t per = heads * s->prompt_len * sizeof(float);
-    SplitSpace w = {0, per, 0, 0, 0};
+    SplitSpace w = {0, per, 0, 0, 0, 0};
     size_t end = 2 * per;
     if (keep) {
-        const size_t parts = heads * (tiles * (tiles + 1) / 2) * (4 * TT) * sizeof(float);
-        const size_t ctas = heads * tiles < kKeepCtas ? heads * tiles : kKeepCtas;
-        w.logits = round_up(parts, kWsAlign);
+        const size_t one = part_bytes(s->heads, tiles), most = kPartBytes / one, turns = (segs + most - 1) / most;
+        const size_t turn = (segs + turns - 1) / turns;
+        const size_t ctas = turn * s->heads * tiles < kKeepCtas ? turn * s->heads * tiles : kKeepCtas;
+        w.turn = (int)turn;
+        w.logits = round_up(turn * one, kWsAlign);
         const size_t kept = w.logits + ctas * tiles * TT * TT * sizeof(float);
         if (kept > end) end = kept;
     }
@@ -728,17 +744,13 @@ static SplitSpace split_space(const pkv_shape *s, bool keep)
     w.bytes = w.words + kWsAlign;
     return w;
 }
-static bool split_keeps(const pkv_shape *s)
-{
-    return s->dtype == PKV_F32 && keeps_logits((size_t)s->batch * s->layers * s->heads, (s->prompt_len + TT - 1) / TT, s->head_dim);
-}
-size_t score_split_ws_bytes(const pkv_shape *s, bool least) { return split_space(s, !least && split_keeps(s)).bytes; }
+size_t score_split_ws_bytes(const pkv_shape *s, bool least) { return split_space(s, !least && keeps_logits(s)).bytes; }
 
 int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const float *k, pkv_strides ks,
                        const float *scale, const float *lse, float *scores, void *ws, size_t ws_bytes, cudaStream_t st)
 {
     const int B = s->batch, L = s->layers, H = s->heads, N = s->prompt_len;
-    const bool keep = !lse && split_keeps(s) && ws_bytes >= split_space(s, true).bytes;
+    const bool keep = !lse && keeps_logits(s) && ws_bytes >= split_space(s, true).bytes;
     const SplitSpace space = split_space(s, keep);
     unsigned char *mem = (unsigned char *)ws;
     SplitArgs a = {};
@@ -777,15 +789,27 @@ int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const
         }
         rc = wide ? launch_split<0, 128>(a, sms, st) : launch_split<0, 64>(a, sms, st);
     } else if (keep) {
+        const int ctas = sms < (int)kKeepCtas ? sms : (int)kKeepCtas, segs = B * L;
         a.next_item = counted ? words : nullptr;
-        const int ctas = sms < (int)kKeepCtas ? sms : (int)kKeepCtas;
-        rc = wide ? launch_split<3, 128>(a, ctas, st) : launch_split<3, 64>(a, ctas, st);
-        if (rc != PKV_OK) return rc;
-        cudaError_t e = launch_dependent(split_mean_kernel, dim3((unsigned)((size_t)B * L * ((N + 31) / 32))), dim3(256), 0, st, a.partial, H, N, a.tiles, scores,
-                                         a.abort_word);
-        if (e != cudaSuccess) {
-            set_cuda_error(e, "split_mean_kernel");
-            return PKV_ERR_CUDA;
+        for (a.seg0 = 0; a.seg0 < segs; a.seg0 += space.turn) {
+            const int now = segs - a.seg0 < space.turn ? segs - a.seg0 : space.turn;
+            a.nsh = now * H;
+            a.group = head_group(a.nsh, N, s->head_dim, 4);
+            cudaError_t e = a.seg0 > 0 ? cudaMemsetAsync(words, 0, sizeof(int), st) : cudaSuccess;
+            if (e != cudaSuccess) {
+                set_cuda_error(e, "cudaMemsetAsync(score work counter)");
+                return PKV_ERR_CUDA;
+            }
+            rc = wide ? launch_split<3, 128>(a, ctas, st) : launch_split<3, 64>(a, ctas, st);
+            if (rc != PKV_OK) return rc;
+            e = launch_dependent(split_mean_kernel, dim3((unsigned)((size_t)now * ((N + 31) / 32))), dim3(256), 0, st, a.partial, H, N, a.tiles,
+                                 scores + (size_t)a.seg0 * N, a.abort_word);
+            if (e == cudaSuccess && now < segs && a.seg0 + now == segs)
+                e = launch_dependent(split_abort_kernel, dim3((unsigned)sms), dim3(256), 0, st, scores, (size_t)segs * N, a.abort_word);
+            if (e != cudaSuccess) {
+                set_cuda_error(e, "split_mean_kernel");
+                return PKV_ERR_CUDA;
+            }
         }
         return PKV_OK;
     } else {

@@ -28,7 +28,7 @@ class Session:
         self.iters = torch.empty(B, dtype=torch.int32, device=dev)
         self.status = torch.zeros(B, dtype=torch.int32, device=dev)
         self.budget = torch.empty(B, dtype=torch.int64, device=dev)
-        self.ws_score = None
+        self.ws_score = self.ws_score_lse = None
         self.ws_compact = api.alloc_workspace(self.shape, api.WS_COMPACT, dev)
         self.ws_decode = api.alloc_workspace(self.shape, api.WS_DECODE, dev)
         rows = L * N if max_budget_rows is None else min(int(max_budget_rows), L * N)
@@ -39,9 +39,16 @@ class Session:
 
     # -- compress ---------------------------------------------------------
     def score(self, q, k, lse=None):
-        if self.ws_score is None:
-            self.ws_score = api.alloc_workspace(self.shape, api.WS_SCORE, self.device)
-        api.prefixkv_score(self.shape, q, k, self.layer_scale, self.scores, self.ws_score, lse=lse)
+        # (a buffer for each kind of call: a captured one keeps using its own)
+        if lse is None:
+            if self.ws_score is None:
+                self.ws_score = api.alloc_workspace(self.shape, api.WS_SCORE, self.device)
+            ws = self.ws_score
+        else:
+            if self.ws_score_lse is None:
+                self.ws_score_lse = api.alloc_workspace(self.shape, api.WS_SCORE_LEAST, self.device)
+            ws = self.ws_score_lse
+        api.prefixkv_score(self.shape, q, k, self.layer_scale, self.scores, ws, lse=lse)
         return self.scores
 
     def search(self, budget_rows, tol=1e-6, max_iters=64, slack_rows=0, scores=None, slack_over_rows=0):

@@ -110,13 +110,23 @@ def test_the_decode_binding_is_this_interpreters(api, monkeypatch, tmp_path):
             assert call(sh, cache, None, None, None, None, 0, 2, None, None, None) == api.PKV_ERR_INVALID_ARG
 
 
-@pytest.mark.parametrize("heads,D,N,kept", [(1, 64, 128, False), (9999, 64, 129, True), (9999, 64, 1024, True), (16, 64, 1025, True), (17, 64, 1025, False),
-                                            (9, 64, 2048, True), (10, 64, 2048, False), (8, 64, 2049, False), (9999, 128, 1024, True),
+@pytest.mark.parametrize("heads,D,N,kept", [(1, 64, 128, False), (9999, 64, 129, True), (1820, 64, 1024, True), (1821, 64, 1024, False), (16, 64, 1025, True), (17, 64, 1025, False),
+                                            (9, 64, 2048, True), (10, 64, 2048, False), (8, 64, 2049, False), (800, 128, 1024, True),
                                             (1, 128, 1025, False)])
 def test_which_fp32_prompts_keep_their_logits(api, heads, D, N, kept):
-    """By the workspace they ask for: logits that leave the L2 cost more than a second pass."""
+    """By the workspace they ask for beyond the least: logits that leave the L2 cost more than a second pass."""
     import torch
-    two = 2 * heads * N * 4
-    need = api.prefixkv_workspace_bytes(api.make_shape(1, 1, heads, D, N, torch.float32), api.WS_SCORE)
-    least = api.prefixkv_workspace_bytes(api.make_shape(1, 1, heads, D, N, torch.bfloat16), api.WS_SCORE)
-    assert (need > max(two, least) + 1024) == kept, (need, two, least)
+    sh = api.make_shape(1, 1, heads, D, N, torch.float32)
+    assert (api.prefixkv_workspace_bytes(sh, api.WS_SCORE) > api.prefixkv_workspace_bytes(sh, api.WS_SCORE_LEAST)) == kept
+
+
+@pytest.mark.parametrize("B,L,H,D,N", [(1, 8, 16, 128, 777), (1, 32, 32, 128, 1024), (16, 24, 16, 64, 1024), (1, 1, 9, 64, 2048), (64, 40, 40, 128, 1000),
+                                       (1, 2, 5000, 64, 1024), (16, 24, 16, 64, 2048)])
+def test_kept_logits_take_bounded_memory(api, B, L, H, D, N):
+    """Logits of 148 blocks and 128 MiB of part sums, however many heads there are; with the caller's log-sum-exp nothing but
+    sums and normalisers of every query."""
+    import torch
+    sh, tiles = api.make_shape(B, L, H, D, N, torch.float32), (N + 127) // 128
+    two = 2 * B * L * H * N * 4
+    assert api.prefixkv_workspace_bytes(sh, api.WS_SCORE) <= max(two * 1.2, 148 * tiles * 65536 + (128 << 20)) + 1024
+    assert two <= api.prefixkv_workspace_bytes(sh, api.WS_SCORE_LEAST) <= two * 1.2 + 1024

@@ -87,3 +87,42 @@ def test_workspace_of_a_longer_prompt(D, N, longer):
     assert s.ws_score.numel() < api.alloc_workspace(s.shape, api.WS_SCORE, "cuda").numel()
     ref = _exact(q, k, scale)
     assert ((s.score(q, k).double() - ref).abs() / ref.clamp(min=1e-3)).max().item() <= TOL
+
+
+@pytest.mark.parametrize("B,L,H,D,N", [(3, 71, 9, 64, 1000), (2, 40, 33, 128, 1024), (1, 3, 1800, 128, 1020), (1, 13, 900, 64, 300)])
+def test_segments_in_turns(B, L, H, D, N):
+    """More part sums than the workspace holds: as many segments at a time, no longer than the two passes' bound."""
+    g = torch.Generator(device="cuda").manual_seed(N + H)
+    q, k = (torch.randn(B, L, H, N, D, device="cuda", generator=g) for _ in range(2))
+    scale = np.linspace(0.5, 1.5, L).astype(np.float32) / np.float32(np.sqrt(D))
+    s = Session(B, L, H, D, N, torch.float32, scale, decode_cap=0, max_budget_rows=L)
+    tiles = (N + 127) // 128
+    assert s.B * s.L * H * (tiles * (tiles + 1) // 2) * 2048 > 128 << 20      # (more than one turn)
+    got = s.score(q, k).clone()
+    for b, l in {(0, 0), (B // 2, L // 2), (B - 1, L - 1), (B - 1, 0)}:
+        ref = torch.zeros(N, dtype=torch.float64, device="cuda")
+        for h in range(H):
+            ref += _exact(q[b:b + 1, l:l + 1, h:h + 1], k[b:b + 1, l:l + 1, h:h + 1], scale[l:l + 1])[0, 0]
+        ref /= H
+        assert ((got[b, l].double() - ref).abs() / ref.clamp(min=1e-3)).max().item() <= TOL
+    # each segment by itself, in one turn: the same sums
+    for b, l in {(0, L // 3), (B - 1, L - 1)}:
+        one = Session(1, 1, H, D, N, torch.float32, scale[l:l + 1], decode_cap=0, max_budget_rows=1)
+        assert torch.equal(one.score(q[b:b + 1, l:l + 1], k[b:b + 1, l:l + 1])[0, 0], got[b, l])
+
+
+def test_with_a_log_sum_exp_the_least_will_do():
+    """A call with the caller's log-sum-exp has no logits to keep, and a session none to make room for."""
+    N = 600
+    g = torch.Generator(device="cuda").manual_seed(N)
+    q, k = (torch.randn(1, 2, 3, N, 128, device="cuda", generator=g) for _ in range(2))
+    scale = np.full(2, 128 ** -0.5, np.float32)
+    s = Session(1, 2, 3, 128, N, torch.float32, scale, decode_cap=0, max_budget_rows=2)
+    x = torch.matmul(q.double(), k.double().transpose(-1, -2)) * float(scale[0])
+    later = torch.ones(N, N, dtype=torch.bool, device="cuda").triu(1)
+    lse = torch.logsumexp(x.masked_fill_(later, -float("inf")), -1).float()
+    a = s.score(q, k, lse=lse).clone()
+    assert s.ws_score is None and s.ws_score_lse.numel() == api.prefixkv_workspace_bytes(s.shape, api.WS_SCORE_LEAST)
+    b = s.score(q, k)
+    assert s.ws_score.numel() > s.ws_score_lse.numel()
+    assert ((a - b).abs() / b.clamp(min=1e-3)).max().item() <= TOL
