@@ -106,13 +106,13 @@ compact_plan_kernel(const int32_t *__restrict__ order, const int32_t *__restrict
 constexpr int kGatherThreads = 128;
 constexpr int kGatherHeads = 8;
 
-// grid (segments, row slices, groups of kGatherHeads heads).
+// grid (segments, row slices, groups of kGatherHeads heads from `group0` on).
 template <int VEC_PER_HEAD>
 __global__ void __launch_bounds__(kGatherThreads)
 gather_rows_kernel(const uint4 *__restrict__ k, const uint4 *__restrict__ v, pkv_strides ks16,
                    pkv_strides vs16, const int32_t *__restrict__ kept,
                    const int32_t *__restrict__ len, const int64_t *__restrict__ row_offset, int L,
-                   int N, int H, uint4 *__restrict__ ck, uint4 *__restrict__ cv)
+                   int N, int H, uint4 *__restrict__ ck, uint4 *__restrict__ cv, int group0)
 {
     constexpr int ROWS = kGatherThreads / VEC_PER_HEAD;
     const int seg = blockIdx.x;
@@ -122,7 +122,7 @@ gather_rows_kernel(const uint4 *__restrict__ k, const uint4 *__restrict__ v, pkv
     const int64_t off = row_offset[seg];
     const int row_vecs = H * VEC_PER_HEAD;
     const int i = threadIdx.x / VEC_PER_HEAD, c = threadIdx.x % VEC_PER_HEAD;
-    const int h0 = blockIdx.z * kGatherHeads, nh = min(H - h0, kGatherHeads);
+    const int h0 = (group0 + blockIdx.z) * kGatherHeads, nh = min(H - h0, kGatherHeads);
     const uint4 *kb = k + b * ks16.b + l * ks16.l + h0 * ks16.h + c;
     const uint4 *vb = v + b * vs16.b + l * vs16.l + h0 * vs16.h + c;
     const int32_t *kp = kept + (size_t)seg * N;
@@ -212,18 +212,21 @@ extern "C" int prefixkv_compact(const pkv_shape *shape, const void *k, pkv_strid
     const int groups = (H + kGatherHeads - 1) / kGatherHeads, rows_at_once = kGatherThreads / vph;
     const int slices = std::max(1, std::min((148 * 128 + nseg * groups - 1) / (nseg * groups),
                                             (N + rows_at_once - 1) / rows_at_once));
-    dim3 grid(nseg, slices, groups);
+    constexpr int kMostGroups = 65535;  // of a launch
+    for (int group0 = 0; group0 < groups && e == cudaSuccess; group0 += kMostGroups) {
+        dim3 grid(nseg, slices, std::min(groups - group0, kMostGroups));
 #define PKV_GATHER(V)                                                                                  \
     e = launch_dependent(gather_rows_kernel<V>, grid, dim3(kGatherThreads), 0, stream, (const uint4 *)k, \
                          (const uint4 *)v, k16, v16, (const int32_t *)kept, (const int32_t *)cache->len, \
-                         (const int64_t *)cache->row_offset, L, N, H, (uint4 *)cache->k, (uint4 *)cache->v)
-    switch (vph) {
-    case 8: PKV_GATHER(8); break;
-    case 16: PKV_GATHER(16); break;
-    case 32: PKV_GATHER(32); break;
-    default: return PKV_ERR_UNSUPPORTED;
-    }
+                         (const int64_t *)cache->row_offset, L, N, H, (uint4 *)cache->k, (uint4 *)cache->v, group0)
+        switch (vph) {
+        case 8: PKV_GATHER(8); break;
+        case 16: PKV_GATHER(16); break;
+        case 32: PKV_GATHER(32); break;
+        default: return PKV_ERR_UNSUPPORTED;
+        }
 #undef PKV_GATHER
+    }
     if (e != cudaSuccess) {
         set_cuda_error(e, "gather_rows_kernel");
         return PKV_ERR_CUDA;

@@ -1,9 +1,11 @@
 """The compaction copy where its tiles of rows and groups of heads end: single heads, heads one below,
 at and one above a group, a whole tile of rows and one more, several rounds of a CTA, and sources laid
 out by head, by token and with a gap between rows.  Rows are moved, so every comparison is exact."""
+import numpy as np
 import pytest
 import torch
 
+from paper_2412_03409_b200 import api
 from paper_2412_03409_b200.session import Session
 
 pytestmark = pytest.mark.gpu
@@ -49,3 +51,20 @@ def test_rows_are_copied_exactly(B, L, H, N, keep, dtype, D, layout):
             got = dst[offs[seg]:offs[seg + 1]]
             assert torch.equal(got[:lens[seg]].contiguous().view(raw), want), (seg, lens[seg])
             assert torch.isnan(got[lens[seg]:]).all()
+
+
+def test_more_groups_of_heads_than_a_grid_holds():
+    H, N, D = 8 * 65535 + 9, 3, 64
+    shape = api.make_shape(1, 1, H, D, N, torch.bfloat16)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    k, v = (torch.randn((1, 1, H, N, D), generator=gen, device="cuda").bfloat16() for _ in range(2))
+    cache = api.alloc_cache(shape, 2, 0, "cuda")
+    order = torch.tensor([[[2, 0, 1]]], dtype=torch.int32, device="cuda")
+    length = torch.tensor([[2]], dtype=torch.int32, device="cuda")
+    kept = torch.empty((1, 1, N), dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    api.prefixkv_compact(shape, k, v, order, length, cache, status, None, kept=kept)
+    torch.cuda.synchronize()
+    assert status.tolist() == [0]
+    for src, dst in ((k, cache.k), (v, cache.v)):
+        assert torch.equal(dst[:2].view(2, H, D), src[0, 0][:, [0, 2]].transpose(0, 1))
