@@ -277,6 +277,23 @@ int prefixkv_decode_attn(const pkv_shape *shape, pkv_cache *cache, const void *q
                          int32_t *dev_status, void *ws, size_t ws_bytes, void *cuda_stream);
 
 /*
+ * Which kernel prefixkv_decode_attn takes for a call (a diagnostic for tests and benchmarks; the paper has no counterpart).
+ * Host only: of the cache it reads total_cap_rows, decode_cap and evict_distance, and no pointer; the device is asked for
+ * its number of SMs.  appends: whether k_new and v_new are given.  PKV_KERNEL_NONE: the call is refused, or the device cannot
+ * be asked.
+ */
+enum {
+    PKV_KERNEL_NONE = 0,
+    PKV_KERNEL_CLUSTER = 1,      /* a cluster of thread blocks to a (segment, head) pair                */
+    PKV_KERNEL_PAIR = 2,         /* a thread block to a pair                                           */
+    PKV_KERNEL_HEADS = 3,        /* pairs dealt to a thread block per SM                               */
+    PKV_KERNEL_HEADS_SHARED = 4, /* the same, tiles shared out where lengths are uneven                */
+    PKV_KERNEL_ROWS = 5,         /* rows of all segments split over the SMs, and a merge               */
+    PKV_KERNEL_TWO = 6           /* the same without that kernel's limits                              */
+};
+int prefixkv_decode_kernel(const pkv_shape *shape, const pkv_cache *cache, int32_t appends, int32_t layer_begin, int32_t layer_end);
+
+/*
  * The same decode step for callers that have no workspace to give.  (The paper
  * has no counterpart to this call; it exists for deployment.)
  *

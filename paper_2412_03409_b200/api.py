@@ -22,13 +22,15 @@ from . import build as _build
  DEV_TIMEOUT) = range(7)
 WS_SCORE, WS_SEARCH, WS_COMPACT, WS_DECODE, WS_SCORE_LEAST = range(5)
 MERGE_POSITION, MERGE_FEATURE = 1, 2
+KERNEL_NONE, KERNEL_CLUSTER, KERNEL_PAIR, KERNEL_HEADS, KERNEL_HEADS_SHARED, KERNEL_ROWS, KERNEL_TWO = range(7)
 F32, BF16 = 0, 1
 
 EXPORTS = ["prefixkv_workspace_bytes", "prefixkv_last_cuda_error", "prefixkv_score",
            "prefixkv_search", "prefixkv_apply_lengths", "prefixkv_compact",
            "prefixkv_decode_attn", "prefixkv_gini", "prefixkv_rescale",
            "prefixkv_estimate_config", "prefixkv_decode_attn_static",
-           "prefixkv_selftest_bounded_wait", "prefixkv_compact_merge", "prefixkv_decode_static_limit_bytes"]
+           "prefixkv_selftest_bounded_wait", "prefixkv_compact_merge", "prefixkv_decode_kernel",
+           "prefixkv_decode_static_limit_bytes"]
 
 
 class Shape(ctypes.Structure):
@@ -82,6 +84,7 @@ def _load():
     lib.prefixkv_selftest_bounded_wait.argtypes = [i32, vp, vp]
     lib.prefixkv_compact_merge.argtypes = [sp, vp, Strides, vp, Strides, vp, vp, ctypes.POINTER(CacheStruct), i32,
                                            vp, vp, vp, vp, sz, vp]
+    lib.prefixkv_decode_kernel.argtypes = [sp, ctypes.POINTER(CacheStruct), i32, i32, i32]
     for name in EXPORTS[2:-1]:
         getattr(lib, name).restype = ctypes.c_int
     lib.prefixkv_decode_static_limit_bytes.restype = ctypes.c_size_t
@@ -243,6 +246,12 @@ def prefixkv_compact(shape, k, v, order, length, cache: Cache, dev_status, ws, k
     _check(_lib.prefixkv_compact(ctypes.byref(shape), _ptr(k), strides_of(k), _ptr(v), strides_of(v),
                                  _ptr(order), _ptr(length), ctypes.byref(cache.c), _ptr(kept),
                                  _ptr(dev_status), p, n, _stream()), "prefixkv_compact")
+
+
+def prefixkv_decode_kernel(shape, cache, appends=True, layer_begin=0, layer_end=None) -> int:
+    """KERNEL_*: what a decode call of this shape over `cache` (a Cache, or a CacheStruct without pointers) runs."""
+    return _lib.prefixkv_decode_kernel(ctypes.byref(shape), ctypes.byref(getattr(cache, "c", cache)), int(appends), layer_begin,
+                                       shape.layers if layer_end is None else layer_end)
 
 
 def prefixkv_decode_attn(shape, cache: Cache, q, k_new, v_new, layer_scale, out, dev_status, ws,

@@ -163,6 +163,8 @@ static int pick_splits(int nseg_active)
 size_t decode_stream_ws_bytes(const pkv_shape *s);
 size_t decode_heads_ws_bytes();
 bool decode_stream_covers(const pkv_shape *s, int nact);
+int decode_cluster_ctas(const pkv_shape *s, const pkv_cache *c, int nact, int sms);
+int decode_heads_form(const pkv_shape *s, const pkv_cache *c, int nact, int sms);
 int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn, const void *vn,
                           const float *scale, int lb, int le, void *out, int32_t *dev_status, void *ws, cudaStream_t st);
 int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn, const void *vn,
@@ -180,6 +182,18 @@ size_t decode_ws_bytes(const pkv_shape *s)
     size_t two = round_up(slots * per, kWsAlign), one = decode_stream_ws_bytes(s), heads = decode_heads_ws_bytes();
     size_t need = two > one ? two : one;
     return heads > need ? heads : need;
+}
+
+// Pruning and attending without appending are for shapes within the streaming kernel's limits.
+static bool decode_pairs_allowed(const pkv_shape *s, const pkv_cache *c, bool appends, int nact)
+{
+    return (c->evict_distance == 0 && appends) || decode_stream_covers(s, nact);
+}
+// Layers of a launch of that kernel.
+static int decode_stream_layers(int batch, int layers)
+{
+    const int max_active = 1024;
+    return (size_t)batch * layers > (size_t)max_active && batch <= max_active ? max_active / batch : layers;
 }
 
 template <typename T, int D>
@@ -227,17 +241,15 @@ extern "C" int prefixkv_decode_attn(const pkv_shape *shape, pkv_cache *cache, co
     if ((size_t)shape->batch * (layer_end - layer_begin) > 65535) return PKV_ERR_UNSUPPORTED;
     if (!ws || !aligned(ws, kWsAlign) || ws_bytes < decode_ws_bytes(shape)) return PKV_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // Pruning and attending without appending are for shapes within the streaming kernel's limits.
-    const bool covered = (cache->evict_distance == 0 && k_new) ||
-                         decode_stream_covers(shape, shape->batch * (layer_end - layer_begin));
+    const bool covered = decode_pairs_allowed(shape, cache, k_new != nullptr, shape->batch * (layer_end - layer_begin));
     if (covered) {
-        // Few (segment, head) pairs, a layer at a time: a cluster for each, one launch.
+        // A cluster of CTAs, or a CTA, to each (segment, head) pair: most calls, one launch.
         int rc = launch_decode_cluster(shape, cache, q, k_new, v_new, layer_scale, layer_begin, layer_end, out, dev_status,
                                        ws, st);
         if (rc >= 0) return rc;  // -1: not a case for that kernel
     }
     {
-        // Few segments: whole (segment, head) items per CTA, no partials and no second kernel.
+        // Up to 256 segments: (segment, head) pairs dealt to the SMs, no second kernel.
         int rc = launch_decode_heads(shape, cache, q, k_new, v_new, layer_scale, layer_begin, layer_end, out, dev_status,
                                      ws, st);
         if (rc >= 0) return rc;  // -1: not a case for that kernel
@@ -245,10 +257,7 @@ extern "C" int prefixkv_decode_attn(const pkv_shape *shape, pkv_cache *cache, co
     {
         // The streaming kernel plans at most 1024 segments at a time: a larger batch x layer range
         // goes through it in layer chunks, one launch after the other on the stream.
-        const int max_active = 1024;
-        int step = layer_end - layer_begin;
-        if ((size_t)shape->batch * step > (size_t)max_active && shape->batch <= max_active)
-            step = max_active / shape->batch;
+        const int step = decode_stream_layers(shape->batch, layer_end - layer_begin);
         int rc = -1;
         for (int lb = layer_begin; lb < layer_end; lb += step) {
             const int le = lb + step < layer_end ? lb + step : layer_end;
@@ -270,6 +279,20 @@ extern "C" int prefixkv_decode_attn(const pkv_shape *shape, pkv_cache *cache, co
         PKV_DEC(__nv_bfloat16, 128);
     }
 #undef PKV_DEC
+}
+
+extern "C" int prefixkv_decode_kernel(const pkv_shape *shape, const pkv_cache *cache, int32_t appends, int32_t layer_begin, int32_t layer_end)
+{
+    if (!shape_ok(shape) || !cache || layer_begin < 0 || layer_end > shape->layers || layer_begin >= layer_end || cache->evict_distance < 0 ||
+        !shape_supported(shape) || (size_t)shape->batch * (layer_end - layer_begin) > 65535)
+        return PKV_KERNEL_NONE;
+    const int nact = shape->batch * (layer_end - layer_begin), sms = sm_count();
+    if (sms <= 0) return PKV_KERNEL_NONE;
+    if (decode_pairs_allowed(shape, cache, appends != 0, nact) && decode_cluster_ctas(shape, cache, nact, sms) > 0)
+        return (int64_t)nact * shape->heads < 4 * (int64_t)sms ? PKV_KERNEL_CLUSTER : PKV_KERNEL_PAIR;
+    if (const int form = decode_heads_form(shape, cache, nact, sms)) return form == 2 ? PKV_KERNEL_HEADS_SHARED : PKV_KERNEL_HEADS;
+    if (decode_stream_covers(shape, shape->batch * decode_stream_layers(shape->batch, layer_end - layer_begin))) return PKV_KERNEL_ROWS;
+    return cache->evict_distance == 0 && appends ? PKV_KERNEL_TWO : PKV_KERNEL_NONE;
 }
 
 // ---------------------------------------------------------------------------

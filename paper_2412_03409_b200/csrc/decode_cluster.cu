@@ -420,13 +420,10 @@ template <int U, int P> int launch_shape(const pkv_shape *s, const ClusterArgs &
 
 }  // namespace
 
-// Returns PKV_OK, an error, or -1 when this call is outside what the kernel covers.
-int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn, const void *vn,
-                          const float *scale, int lb, int le, void *out, int32_t *dev_status, void *ws, cudaStream_t st)
+// CTAs to a pair for a call of nact segments; 0 when another kernel is to take it.
+int decode_cluster_ctas(const pkv_shape *s, const pkv_cache *c, int nact, int sms)
 {
-    const int H = s->heads, D = s->head_dim, nl = le - lb, nact = s->batch * nl;
-    const int sms = sm_count();
-    if (sms <= 0) return PKV_ERR_CUDA;
+    const int H = s->heads, D = s->head_dim;
     const int64_t items = (int64_t)nact * H, seg_rows = c->total_cap_rows / ((int64_t)s->batch * s->layers);
     const int64_t pair_bytes = seg_rows * D * 2 * (int64_t)esize(s);
     const int wave = kCPerSm * sms;
@@ -455,7 +452,7 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
         else if (c->evict_distance > 0) least = items < 20 * (int64_t)sms ? 80 : 200;
         else if (nact > 256) least = (size_t)H * D * esize(s) <= 1024 ? 0 : 112;
         else least = items < 20 * (int64_t)sms ? 96 : 80;
-        if (rows < least || kb > most_kb || items > INT32_MAX / 2) return -1;
+        if (rows < least || kb > most_kb || items > INT32_MAX / 2) return 0;
     }
     // Few pairs, but the longest, for which the row-split kernel is as fast where it covers the shape, row-split / this one, one layer: 1 head
     // of 128, bf16, 8000 rows 18.1 / 13.4, 15000 31.1 / 21.8, fp32 8000 26.8 / 20.9; 8 heads fp32 8000 40.1 / 31.9, 12000 (12.3 MB a pair) 45.0 / 45.6;
@@ -465,7 +462,7 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
         (pair_bytes > ((int64_t)(items < 24 ? 11 : 13) << 20) ||
          items * seg_rows > (D == 64 ? (items <= 320 ? 1 << 20 : 704 << 10) : 1536 << 10) || items * pair_bytes > ((int64_t)800 << 20)) &&
         decode_stream_covers(s, nact))
-        return -1;
+        return 0;
     // As many CTAs as the SMs hold at a time, none of them with less than one round of rows (32) unless
     // the call is so small that SMs would be idle; further waves only for CTAs of 256 rows and more,
     // whose bytes outweigh a wave's latency (16 x 32 x 2048 rows: C = 1 111 us, 6 89 us in one run, 99 in another).
@@ -477,8 +474,19 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
         if (!one_wave && seg_rows < 256 * (int64_t)n) break;
         C = n;
     }
-    if ((int64_t)H * C >= (int64_t)1 << kVisitBits) return -1;
+    return (int64_t)H * C >= (int64_t)1 << kVisitBits ? 0 : C;
+}
 
+// Returns PKV_OK, an error, or -1 when this call is outside what the kernel covers.
+int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn, const void *vn,
+                          const float *scale, int lb, int le, void *out, int32_t *dev_status, void *ws, cudaStream_t st)
+{
+    const int H = s->heads, D = s->head_dim, nl = le - lb, nact = s->batch * nl;
+    const int sms = sm_count();
+    if (sms <= 0) return PKV_ERR_CUDA;
+    const int C = decode_cluster_ctas(s, c, nact, sms);
+    if (C == 0) return -1;
+    const int64_t items = (int64_t)nact * H;
     ClusterArgs a;
     a.p = decode_plan_args(s, c, kn != nullptr, lb, nl);
     a.q = q; a.k_new = kn; a.v_new = vn; a.ck = c->k; a.cv = c->v; a.out = out;
@@ -488,8 +496,8 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     a.dev_status = dev_status;
     a.H = H;
     a.row_bytes = (uint32_t)((size_t)H * D * esize(s));
-    if (C == 1 && items > wave && items <= 6 * (int64_t)sms) return launch_shape<4, 6>(s, a, C, st);
-    if (C == 1 && items > wave && items <= 7 * (int64_t)sms) return launch_shape<3, 7>(s, a, C, st);
+    if (C == 1 && items > kCPerSm * (int64_t)sms && items <= 6 * (int64_t)sms) return launch_shape<4, 6>(s, a, C, st);
+    if (C == 1 && items > kCPerSm * (int64_t)sms && items <= 7 * (int64_t)sms) return launch_shape<3, 7>(s, a, C, st);
     return launch_shape<4, kCPerSm>(s, a, C, st);
 }
 

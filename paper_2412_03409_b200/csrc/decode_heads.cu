@@ -943,27 +943,43 @@ int selftest_wait_parts(int32_t *dev_status, cudaStream_t st)
 // Flags of either kind, and a part of an item for every CTA.
 size_t decode_heads_ws_bytes() { return round_up((size_t)kHMaxGrid * (2 * sizeof(unsigned long long) + (128 + 4) * sizeof(float)), kWsAlign); }
 
+// How the per-head kernel takes a call of nact segments: 0 not at all, 1 its items dealt, 2 with the tiles of the last rounds shared out.
+int decode_heads_form(const pkv_shape *s, const pkv_cache *c, int nact, int sms)
+{
+    if (c->evict_distance != 0 || nact > kHMaxAct || (s->head_dim != 64 && s->head_dim != 128)) return 0;
+    if (sms > kHMaxGrid) sms = kHMaxGrid;
+    // What the kernel with a CTA to a pair leaves (decode_cluster_ctas): pairs that are too short for it, or too long for one wave, and
+    // queries that append nothing with more than 64 heads.  Worth it while complete (segment, head) items balance over the SMs (at
+    // least four per SM) and the segments are short.  Measured on 128 segments of 32 heads of 128, against the row-split kernel, it wins
+    // while they hold under about 1000 rows (341 / 352 us) and loses beyond (561 / 502 us at 1800
+    // rows): the CTAs that work on neighbouring heads of a segment drift apart over a long item,
+    // and the 256-byte slices of a row are then fetched from DRAM one by one, while the row-split
+    // kernel always reads whole 8 KiB rows.  Lengths live on the device; the capacity bounds them.
+    const int64_t seg_rows = c->total_cap_rows / ((int64_t)s->batch * s->layers), items = (int64_t)nact * s->heads;
+    if (items < 4 * (int64_t)sms || seg_rows > kHMaxSegRows) return 0;
+    // Segments of some hundred rows differ in length, and an item is a good part of a CTA's work: CTAs' sums of tiles made alike.
+    // What that gives is up to the lengths, which the kernel sees; for a call that may gain, this form costs up to 0.5 us (two calls
+    // and a copy, us, dealt / here; lengths lognormal with sigma 0.5, then all alike, then a tenth of the capacity):
+    // 32 x 32 heads, 800 rows 100.6 / 90.2, 127.2 / 128.7; 1000 rows 121.3 / 107.9, 155.7 / 157.4; fp32, 16 x 40 heads, 600 rows
+    // 90.6 / 85.3, 124.9 / 124.2.  More rounds of items, which come here only with queries that append nothing, are more alike by
+    // themselves: 4 x 32 x 32 heads (28 rounds) of 520 rows 346 / 325, 318 / 327, 6 x 40 x 40 (65) 755 / 767, 742 / 765, 250 x 30 heads of
+    // 64 (51) 205 / 203, 304 / 315: dealt there.
+    const bool shared = seg_rows >= kHSharedRowsMany ? items <= kHManyRounds * (int64_t)sms : seg_rows >= kHSharedRows && items <= kHFewRounds * (int64_t)sms;
+    return shared ? 2 : 1;
+}
+
 // Returns PKV_OK, an error, or -1 when this call is outside what the per-head kernel covers (the
 // caller then takes the row-split streaming kernel).
 int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const void *kn, const void *vn,
                         const float *scale, int lb, int le, void *out, int32_t *dev_status, void *ws, cudaStream_t st)
 {
     const int H = s->heads, D = s->head_dim, nl = le - lb, nact = s->batch * nl;
-    if (c->evict_distance != 0 || nact > kHMaxAct) return -1;
-    if (D != 64 && D != 128) return -1;
     int sms = sm_count();
     if (sms <= 0) return PKV_ERR_CUDA;
+    const int form = decode_heads_form(s, c, nact, sms);
+    if (form == 0) return -1;
     if (sms > kHMaxGrid) sms = kHMaxGrid;
-    // Worth it while complete (segment, head) items balance over the SMs (at least four per SM)
-    // and the segments are short.  Measured on 32 layers x 32 heads of 128, 128-256 rows per
-    // segment, against the row-split kernel: 21.1 / 26.0 us per call at batch 1, 67.4 / 71.4 at
-    // batch 4, 129.3 / 134.0 at batch 8 (256 segments).  On 128 segments of a long prompt it wins
-    // while they hold under about 1000 rows (341 / 352 us) and loses beyond (561 / 502 us at 1800
-    // rows): the CTAs that work on neighbouring heads of a segment drift apart over a long item,
-    // and the 256-byte slices of a row are then fetched from DRAM one by one, while the row-split
-    // kernel always reads whole 8 KiB rows.  Lengths live on the device; the capacity bounds them.
     const int64_t seg_rows = c->total_cap_rows / ((int64_t)s->batch * s->layers);
-    if ((int64_t)nact * H < 4 * (int64_t)sms || seg_rows > kHMaxSegRows) return -1;
     const size_t es = esize(s);
     const int tile_rows = (int)(kHTile / ((size_t)D * es));
     // The maps depend on the cache's buffers and shape alone: the last few sets are kept, so that a
@@ -1020,14 +1036,7 @@ int launch_decode_heads(const pkv_shape *s, pkv_cache *c, const void *q, const v
     a.total_cap_rows = c->total_cap_rows;
     const int items = nact * H;
     const int grid = items < sms ? items : sms;
-    // Segments of some hundred rows differ in length, and an item is a good part of a CTA's work: CTAs' sums of tiles made alike.
-    // What that gives is up to the lengths, which the kernel sees; for a call that may gain, this form costs up to 0.5 us (two calls
-    // and a copy, us, dealt / here; lengths lognormal with sigma 0.5, then all alike, then a tenth of the capacity):
-    // 32 x 32 heads, 400 rows of capacity 57.4 / 55.3, 71.3 / 73.4; 512 rows 60.3 / 57.2, 52.0 / 53.6, 22.6 / 23.4; 800 rows 100.6 / 90.2,
-    // 127.2 / 128.7; 1000 rows 121.3 / 107.9, 155.7 / 157.4; fp32, 16 x 40 heads, 600 rows 90.6 / 85.3, 124.9 / 124.2.  More rounds
-    // of items are more alike by themselves: 4 x 32 x 32 heads (28 rounds) of 520 rows 346 / 325, 318 / 327, 6 x 40 x 40
-    // (65) 755 / 767, 742 / 765, 250 x 30 heads of 64 (51) 205 / 203, 304 / 315: dealt there.
-    const bool shared = seg_rows >= kHSharedRowsMany ? items <= kHManyRounds * sms : seg_rows >= kHSharedRows && items <= kHFewRounds * sms;
+    const bool shared = form == 2;
     a.pool_rounds = seg_rows >= kHTwoRoundsRows ? 2 : 1;
     return s->dtype == PKV_BF16 ? launch_heads<__nv_bfloat16>(D, shared, maps, a, grid, st) : launch_heads<float>(D, shared, maps, a, grid, st);
 }
