@@ -52,3 +52,14 @@ def check_scores(got: np.ndarray, ref: np.ndarray, tol: float):
     worst = float((err / bound).max())
     assert worst <= 1.0, "score error %.3g x bound (max abs err %.3g)" % (worst, err.max())
     return worst
+
+
+# What prefixkv_decode_kernel calls the kernels (148 SMs; the lines between them move with the number).
+NONE, CLUSTER, PAIR, HEADS, SHARED, ROWS, TWO = range(7)
+
+
+def check_kernel(s, kernel, appends=True, layer_begin=0, layer_end=None):
+    """The case runs the kernel that it is there for."""
+    from paper_2412_03409_b200 import api
+    got = api.prefixkv_decode_kernel(s.shape, s.cache, appends, layer_begin, layer_end)
+    assert got == kernel, "kernel %d, meant for %d" % (got, kernel)

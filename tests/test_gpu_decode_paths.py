@@ -1,13 +1,13 @@
 """Decode calls that take each of the library's kernels, against the oracle on the cache as it stands
-(needs a B200).  Few (segment, head) pairs: the cluster kernel; from four pairs per SM (592) the
-per-head kernel, the row-split kernel (long segments, more than 256 of them, pruning) or, above 64 heads, the
-two-kernel path."""
+(needs a B200), and says which it is.  Few (segment, head) pairs: a cluster to each; from four pairs per SM (592) a CTA to each
+or, where pairs are short or too long for one wave, the per-head kernel, the row-split kernel (more than 256 segments, more than 1024
+rows, pruning) or, above 64 heads, the two-kernel path."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
-from helpers import to_np32
+from helpers import CLUSTER, HEADS, PAIR, ROWS, SHARED, TWO, check_kernel, to_np32
 from paper_2412_03409_b200 import workloads as wl
 
 pytestmark = pytest.mark.gpu
@@ -16,52 +16,65 @@ pytestmark = pytest.mark.gpu
 # rounding to bf16 is at most 2^-9 * 4 = 8e-3
 TOL = {torch.float32: 2e-5, torch.bfloat16: 8e-3}
 
-CASES = [  # B, L, H, D, N, rows per layer, dtype, evict_distance
-    (1, 2, 1, 64, 40, 1, torch.bfloat16, 0),          # single cached row per layer
-    (1, 1, 32, 128, 300, 33, torch.bfloat16, 0),      # a row more than one round of a cluster's CTA
-    (2, 3, 5, 64, 300, 131, torch.float32, 0),
-    (1, 1, 3, 128, 3000, 2900, torch.float32, 0),     # eight CTAs of many rounds each
-    (3, 1, 7, 64, 2500, 1111, torch.bfloat16, 0),
-    (1, 4, 80, 64, 200, 50, torch.bfloat16, 0),       # above the row-split kernel's 64 heads
-    (2, 2, 4, 128, 64, 16, torch.bfloat16, 3),        # pruning: reused slots are skipped
-    (1, 3, 9, 64, 90, 30, torch.float32, 2),
-    (1, 20, 32, 128, 200, 60, torch.bfloat16, 3),     # 640 pairs with pruning: row-split kernel
-    (1, 20, 32, 64, 1100, 1050, torch.bfloat16, 0),   # 640 pairs, long segments: row-split kernel
-    (1, 9, 72, 64, 100, 20, torch.bfloat16, 0),       # 648 pairs, 72 heads: two-kernel path when segments are long
-    (1, 9, 72, 64, 1300, 1200, torch.bfloat16, 0),
-    # the row-split kernel: the (lanes per row, heads per warp, rows per unit, block size) that fewer than 900 segments
-    # choose, and one that more do.
-    # Rows of up to 8.9 KB go in units of eight, up to 16.5 KB of four, up to 28.9 KB of two; many segments leave
-    # less room for the ring.
-    (1, 38, 16, 128, 40, 12, torch.bfloat16, 3),      # 8, 1, 8
-    (1, 15, 40, 128, 40, 12, torch.bfloat16, 3),      # 16, 4, 4, 12 warps
-    (1, 10, 64, 128, 40, 12, torch.bfloat16, 3),      # 16, 4, 4, 17 warps
-    (4, 32, 64, 128, 24, 6, torch.bfloat16, 3),       # 16, 4, 2, 17 warps
-    (2, 19, 16, 64, 40, 12, torch.bfloat16, 3),       # 8, 1, 8
-    (2, 10, 32, 64, 40, 12, torch.bfloat16, 3),       # 8, 2, 8
-    (1, 15, 40, 64, 40, 12, torch.bfloat16, 3),       # 8, 4, 8, 12 warps
-    (1, 10, 64, 64, 40, 12, torch.bfloat16, 3),       # 8, 4, 8, 17 warps
-    (1, 38, 16, 128, 40, 12, torch.float32, 3),       # 8, 1, 8
-    (30, 32, 16, 128, 20, 4, torch.float32, 3),       # 8, 1, 4
-    (1, 20, 32, 128, 40, 12, torch.float32, 3),       # 16, 2, 4
-    (4, 32, 32, 128, 24, 6, torch.float32, 3),        # 16, 2, 2
-    (1, 15, 40, 128, 40, 12, torch.float32, 3),       # 16, 4, 2, 12 warps
-    (1, 11, 56, 128, 40, 12, torch.float32, 3),       # 16, 4, 2, 17 warps
-    (1, 38, 16, 64, 40, 12, torch.float32, 3),        # 8, 1, 8
-    (1, 20, 32, 64, 40, 12, torch.float32, 3),        # 16, 2, 8
-    (1, 15, 40, 64, 40, 12, torch.float32, 3),        # 16, 4, 4, 12 warps
-    (1, 10, 64, 64, 40, 12, torch.float32, 3),        # 16, 4, 4, 17 warps
-    (10, 32, 2, 128, 40, 9, torch.bfloat16, 0),       # 320 segments
-    (1, 1, 2, 128, 6600, 6500, torch.float32, 0),     # two pairs of 6.7 MB each: split over all SMs
-    (2, 12, 32, 128, 1100, 1040, torch.bfloat16, 0),  # segments split over a few CTAs each
+CASES = [  # B, L, H, D, N, rows per layer, dtype, evict_distance, kernel
+    (1, 2, 1, 64, 40, 1, torch.bfloat16, 0, CLUSTER),        # single cached row per layer
+    (1, 1, 32, 128, 300, 33, torch.bfloat16, 0, CLUSTER),    # a row more than one round of a cluster's CTA
+    (2, 3, 5, 64, 300, 131, torch.float32, 0, CLUSTER),
+    (1, 1, 3, 128, 3000, 2900, torch.float32, 0, CLUSTER),   # eight CTAs of many rounds each
+    (3, 1, 7, 64, 2500, 1111, torch.bfloat16, 0, CLUSTER),
+    (1, 4, 80, 64, 200, 50, torch.bfloat16, 0, CLUSTER),     # above the row-split kernel's 64 heads
+    (2, 2, 4, 128, 64, 16, torch.bfloat16, 3, CLUSTER),      # pruning: reused slots are skipped
+    (1, 3, 9, 64, 90, 30, torch.float32, 2, CLUSTER),
+    (1, 20, 32, 128, 200, 60, torch.bfloat16, 3, PAIR),      # 640 pairs with pruning
+    (1, 20, 32, 64, 1100, 1050, torch.bfloat16, 0, PAIR),    # 640 pairs, long segments
+    (1, 9, 72, 64, 100, 20, torch.bfloat16, 0, PAIR),        # 648 pairs, 72 heads
+    (1, 9, 72, 64, 1300, 1200, torch.bfloat16, 0, PAIR),
+    # short segments with pruning, heads of either size.  (Behind those of the row-split kernel: lanes per row, heads per warp, rows per
+    # unit and block size.  Rows of up to 8.9 KB go in units of eight, up to 16.5 KB of four, up to 28.9 KB of two; many segments
+    # leave less room for the ring.  test_what_goes_elsewhere has the other combinations.)
+    (1, 38, 16, 128, 40, 12, torch.bfloat16, 3, PAIR),
+    (1, 15, 40, 128, 40, 12, torch.bfloat16, 3, PAIR),
+    (1, 10, 64, 128, 40, 12, torch.bfloat16, 3, PAIR),
+    (4, 32, 64, 128, 24, 6, torch.bfloat16, 3, ROWS),        # 16, 4, 2, 17 warps
+    (2, 19, 16, 64, 40, 12, torch.bfloat16, 3, PAIR),
+    (2, 10, 32, 64, 40, 12, torch.bfloat16, 3, PAIR),
+    (1, 15, 40, 64, 40, 12, torch.bfloat16, 3, PAIR),
+    (1, 10, 64, 64, 40, 12, torch.bfloat16, 3, PAIR),
+    (1, 38, 16, 128, 40, 12, torch.float32, 3, PAIR),
+    (30, 32, 16, 128, 20, 4, torch.float32, 3, ROWS),        # 8, 1, 4
+    (1, 20, 32, 128, 40, 12, torch.float32, 3, PAIR),
+    (4, 32, 32, 128, 24, 6, torch.float32, 3, ROWS),         # 16, 2, 2
+    (1, 15, 40, 128, 40, 12, torch.float32, 3, PAIR),
+    (1, 11, 56, 128, 40, 12, torch.float32, 3, PAIR),
+    (1, 38, 16, 64, 40, 12, torch.float32, 3, PAIR),
+    (1, 20, 32, 64, 40, 12, torch.float32, 3, PAIR),
+    (1, 15, 40, 64, 40, 12, torch.float32, 3, PAIR),
+    (1, 10, 64, 64, 40, 12, torch.float32, 3, PAIR),
+    (10, 32, 2, 128, 40, 9, torch.bfloat16, 0, PAIR),        # 320 segments
+    (1, 1, 2, 128, 6600, 6500, torch.float32, 0, CLUSTER),   # two pairs of 6.7 MB each: split over all SMs
+    (2, 12, 32, 128, 1100, 1040, torch.bfloat16, 0, ROWS),   # segments split over a few CTAs each
+    (1, 24, 64, 128, 40, 12, torch.bfloat16, 3, ROWS),       # 1536 short pairs with pruning
+    (9, 32, 16, 128, 40, 15, torch.bfloat16, 3, ROWS),       # 288 segments
+    (40, 32, 16, 64, 24, 5, torch.bfloat16, 0, ROWS),        # 1280 segments: two launches, of 25 layers and of seven
+    (1, 32, 48, 128, 100, 20, torch.bfloat16, 0, HEADS),     # 1536 short pairs
+    (2, 16, 48, 64, 90, 40, torch.bfloat16, 0, HEADS),
+    (1, 32, 48, 64, 100, 40, torch.float32, 0, HEADS),
+    (1, 20, 40, 128, 500, 300, torch.float32, 0, HEADS),     # 800 pairs too long for one wave
+    (1, 27, 32, 128, 600, 560, torch.bfloat16, 0, SHARED),
+    (1, 27, 32, 64, 600, 560, torch.float32, 0, SHARED),
+    (1, 9, 72, 128, 1300, 1200, torch.bfloat16, 0, TWO),     # 648 long pairs of 72 heads
+    (9, 30, 72, 64, 24, 8, torch.bfloat16, 0, TWO),          # 270 segments of 72 heads
 ]
+REPLAYED = [c for i, c in enumerate(CASES) if i in (4, 6, 8, 9) or (i >= 31 and c[0] < 40)]
 
 
-def _ready(B, L, H, D, N, rows, dtype, d, T, seed=3):
+def _ready(B, L, H, D, N, rows, dtype, d, T, seed=3, kernel=None):
     from paper_2412_03409_b200.session import Session
     g = torch.Generator(device="cuda").manual_seed(seed + N)
     scale = np.full(L, 1.0 / np.sqrt(D), np.float32)
     s = Session(B, L, H, D, N, dtype, scale, decode_cap=T, max_budget_rows=L * rows, evict_distance=d, poison=True)
+    if kernel is not None:
+        check_kernel(s, kernel)
     scores = np.stack([wl.synthetic_scores(L, N, seed + b) for b in range(B)])
     s.search(L * rows, scores=torch.from_numpy(scores).cuda())
     k, v = (torch.randn(B, L, H, N, D, device="cuda", generator=g).to(dtype) for _ in range(2))
@@ -70,10 +83,10 @@ def _ready(B, L, H, D, N, rows, dtype, d, T, seed=3):
     return s, scale, tok
 
 
-@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d", CASES)
-def test_decode_steps_match_the_oracle(B, L, H, D, N, rows, dtype, d):
+@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d,kernel", CASES)
+def test_decode_steps_match_the_oracle(B, L, H, D, N, rows, dtype, d, kernel):
     T = 8 if d else 2
-    s, scale, tok = _ready(B, L, H, D, N, rows, dtype, d, T)
+    s, scale, tok = _ready(B, L, H, D, N, rows, dtype, d, T, kernel=kernel)
     ring = {i: np.full(d + 1, -1, np.int32) for i in range(B * L)}
     len0 = s.cache.len.cpu().numpy()
     off = s.cache.row_offset.cpu().numpy()
@@ -110,13 +123,13 @@ def test_decode_steps_match_the_oracle(B, L, H, D, N, rows, dtype, d):
             assert np.abs(got[b, l] - ref).max() <= TOL[dtype]
 
 
-@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d", [CASES[4], CASES[6], CASES[8], CASES[9], CASES[-2], CASES[-1]])
+@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d,kernel", REPLAYED)
 @pytest.mark.parametrize("byte", [0x7f, 0xff])
-def test_replay_and_stale_workspace(B, L, H, D, N, rows, dtype, d, byte):
+def test_replay_and_stale_workspace(B, L, H, D, N, rows, dtype, d, kernel, byte):
     """A captured call replayed token after token, over a workspace that holds anything, gives bit for
     bit what separate calls give; a segment without rows is reported and zero."""
     T = 6
-    a, _, tok = _ready(B, L, H, D, N, rows, dtype, d, T)
+    a, _, tok = _ready(B, L, H, D, N, rows, dtype, d, T, kernel=kernel)
     b, _, _ = _ready(B, L, H, D, N, rows, dtype, d, T)
     warm, _, _ = _ready(B, L, H, D, N, rows, dtype, d, T)
     buf = [x.clone() for x in tok[0]]

@@ -1,10 +1,11 @@
-"""Layer-by-layer decode calls: the length's word counts its readers, and rows are asked for by a length read ahead
+"""Decode calls pair by pair: the readers of a length are counted, and rows are asked for by a length read ahead
 (needs a B200).  Outputs against attention in 64 bits over the rows as they stand."""
 import numpy as np
 import pytest
 import torch
 
 import test_gpu_decode_paths as paths
+from helpers import CLUSTER, HEADS, PAIR, ROWS, SHARED, check_kernel
 from paper_2412_03409_b200 import api
 from paper_2412_03409_b200.session import Session
 
@@ -35,7 +36,7 @@ def _attend(s, q, i, n):
     return torch.einsum("hn,nhd->hd", torch.softmax(w, -1), v)
 
 
-# readers of a word (heads x CTAs of a cluster) at and around powers of two; lengths around a CTA's and a round's rows
+# readers of a length (heads x CTAs of a cluster) at and around powers of two; lengths around a CTA's and a round's rows
 @pytest.mark.parametrize("B,L,H,D,lens,dtype", [
     (1, 1, 1, 64, [1], torch.bfloat16), (1, 1, 1, 128, [700], torch.float32), (1, 1, 2, 128, [255], torch.bfloat16),
     (1, 2, 31, 64, [32, 129], torch.bfloat16), (1, 1, 32, 128, [127], torch.bfloat16), (2, 1, 33, 64, [64, 33], torch.float32),
@@ -47,6 +48,7 @@ def test_tokens_back_to_back(B, L, H, D, lens, dtype, layerwise):
     """Every call but the first starts while the one in front may still be writing the lengths."""
     T = 5
     s, tok = _session(B, L, H, D, lens, dtype, T)
+    check_kernel(s, CLUSTER)
     outs = [torch.empty_like(tok[0][0]) for _ in range(T)]
     torch.cuda.synchronize()
     for t in range(T):
@@ -67,17 +69,18 @@ def test_tokens_back_to_back(B, L, H, D, lens, dtype, layerwise):
 
 
 # a CTA to a pair: one wave of five, six and seven CTAs an SM (740, 888, 1036 pairs on a B200) and the next pair after
-# each, and several waves (pairs of 64 KiB and more, 96 with more than 256 segments); the wrong side of each line goes elsewhere
+# each, and several waves (pairs of 96 rows and more, 112 with more than 256 segments); test_what_goes_elsewhere has the others
 @pytest.mark.parametrize("B,L,H,D,rows,dtype", [
     (1, 37, 20, 128, 60, torch.bfloat16), (1, 13, 57, 64, 33, torch.bfloat16), (1, 24, 37, 64, 20, torch.float32), (1, 127, 7, 64, 50, torch.bfloat16),
     (2, 14, 37, 128, 30, torch.bfloat16), (1, 17, 61, 128, 230, torch.bfloat16), (1, 20, 74, 64, 300, torch.bfloat16), (2, 25, 32, 128, 140, torch.bfloat16),
-    (1, 20, 80, 128, 70, torch.float32), (8, 33, 6, 128, 210, torch.bfloat16), (8, 33, 8, 64, 500, torch.bfloat16),
+    (1, 20, 80, 128, 100, torch.float32), (8, 33, 6, 128, 210, torch.bfloat16), (8, 33, 8, 64, 500, torch.bfloat16),
 ])
 def test_a_cta_to_a_pair(B, L, H, D, rows, dtype):
     rng = np.random.default_rng(rows)
     lens = [int(x) for x in rng.integers(1, 2 * rows, B * L)]
     T = 3
     s, tok = _session(B, L, H, D, lens, dtype, T)
+    check_kernel(s, PAIR)
     outs = [torch.empty_like(tok[0][0]) for _ in range(T)]
     torch.cuda.synchronize()
     for t in range(T):
@@ -133,14 +136,36 @@ def test_a_plan_changed_just_before_the_call(place):
 
 # What the pair kernel leaves: more than 256 segments of few rows (row-split kernel, whose lanes, heads a warp, rows a unit and warps
 # go by the row's bytes), pairs just too long for one wave (per-head kernel, tiles shared out where lengths differ), short ones of several waves.
-@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d", [
-    (9, 32, 16, 128, 40, 15, torch.bfloat16, 3), (9, 32, 40, 128, 40, 15, torch.bfloat16, 3), (9, 30, 64, 128, 24, 15, torch.bfloat16, 3),
-    (9, 32, 16, 64, 60, 30, torch.bfloat16, 3), (9, 32, 32, 64, 60, 20, torch.bfloat16, 0), (9, 32, 40, 64, 40, 15, torch.bfloat16, 3),
-    (9, 30, 64, 64, 40, 15, torch.bfloat16, 0), (9, 32, 16, 128, 40, 12, torch.float32, 3), (9, 32, 32, 128, 40, 12, torch.float32, 3),
-    (9, 30, 40, 128, 24, 8, torch.float32, 0), (9, 32, 16, 64, 40, 12, torch.float32, 3),
-    (9, 32, 32, 64, 40, 12, torch.float32, 3), (9, 30, 40, 64, 24, 9, torch.float32, 0), (9, 30, 64, 64, 24, 9, torch.float32, 3),
-    (1, 32, 32, 128, 1500, 700, torch.bfloat16, 0), (2, 18, 25, 128, 900, 640, torch.bfloat16, 0), (3, 32, 32, 64, 90, 40, torch.bfloat16, 0),
-    (2, 32, 32, 128, 90, 30, torch.float32, 0),
+@pytest.mark.parametrize("B,L,H,D,N,rows,dtype,d,kernel", [
+    (9, 32, 16, 128, 40, 15, torch.bfloat16, 3, ROWS), (9, 32, 40, 128, 40, 15, torch.bfloat16, 3, ROWS), (9, 30, 64, 128, 24, 15, torch.bfloat16, 3, ROWS),
+    (9, 32, 16, 64, 60, 30, torch.bfloat16, 3, ROWS), (9, 32, 32, 64, 60, 20, torch.bfloat16, 0, ROWS), (9, 32, 40, 64, 40, 15, torch.bfloat16, 3, ROWS),
+    (9, 30, 64, 64, 40, 15, torch.bfloat16, 0, ROWS), (9, 32, 16, 128, 40, 12, torch.float32, 3, ROWS), (9, 32, 32, 128, 40, 12, torch.float32, 3, ROWS),
+    (9, 30, 40, 128, 24, 8, torch.float32, 0, ROWS), (9, 32, 16, 64, 40, 12, torch.float32, 3, ROWS),
+    (9, 32, 32, 64, 40, 12, torch.float32, 3, ROWS), (9, 30, 40, 64, 24, 9, torch.float32, 0, ROWS), (9, 30, 64, 64, 24, 9, torch.float32, 3, ROWS),
+    (1, 32, 32, 128, 1500, 700, torch.bfloat16, 0, SHARED), (2, 18, 25, 128, 900, 660, torch.bfloat16, 0, SHARED), (3, 32, 32, 64, 90, 40, torch.bfloat16, 0, HEADS),
+    (2, 32, 32, 128, 90, 30, torch.float32, 0, HEADS),
 ])
-def test_what_goes_elsewhere(B, L, H, D, N, rows, dtype, d):
-    paths.test_decode_steps_match_the_oracle(B, L, H, D, N, rows, dtype, d)
+def test_what_goes_elsewhere(B, L, H, D, N, rows, dtype, d, kernel):
+    paths.test_decode_steps_match_the_oracle(B, L, H, D, N, rows, dtype, d, kernel)
+
+
+@pytest.mark.parametrize("B,L,H,D,rows,dtype", [(1, 37, 16, 128, 60, torch.bfloat16), (1, 9, 8, 64, 500, torch.float32), (1, 16, 96, 128, 120, torch.bfloat16)])
+def test_a_workspace_that_holds_anything(B, L, H, D, rows, dtype):
+    """Counts are made anew over any words: over what another call's layout left, over all ones, and over the call's own."""
+    T = 4
+    lens = [rows + i % 5 for i in range(B * L)]
+    a, tok = _session(B, L, H, D, lens, dtype, T)
+    b, _ = _session(B, L, H, D, lens, dtype, T)
+    for t in range(T):
+        ref = a.decode(*tok[t]).clone()
+        if t == 1:
+            b.ws_decode.fill_(255)
+        elif t == 2:        # a layer at a time: other places for the same segments
+            b.cache.len.copy_(a.cache.len - 1)
+            for l in range(L):
+                b.decode(*tok[t], layer_begin=l, layer_end=l + 1)
+            b.cache.len.copy_(a.cache.len - 1)
+        got = b.decode(*tok[t])
+        torch.cuda.synchronize()
+        assert torch.equal(got, ref) and torch.equal(a.cache.len, b.cache.len), t
+    assert a.cache.len.tolist() == [n + T for n in lens] and b.status.tolist() == [0] * B

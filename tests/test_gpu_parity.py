@@ -4,7 +4,7 @@ import pytest
 import torch
 
 import oracle
-from helpers import check_scores, oracle_scores, oracle_select, to_np32
+from helpers import CLUSTER, HEADS, PAIR, ROWS, TWO, check_kernel, check_scores, oracle_scores, oracle_select, to_np32
 from paper_2412_03409_b200 import workloads as wl
 
 pytestmark = pytest.mark.gpu
@@ -264,34 +264,44 @@ def _decode_reference(w, s, k, v, ref_sel, steps, layer_scale):
     return worst
 
 
-@pytest.mark.parametrize("name,kw", [
-    ("tiny", {}),
-    ("llava7b_b1", dict(L=3, H=8, N=200, T=5)),
-    ("llava7b_b16", dict(B=3, L=2, H=4, N=97, T=4)),
-    ("tiny", dict(D=128, H=2, T=3)),
-    ("llava7b_b1", dict(L=2, H=5, D=64, N=130, T=3)),
-    ("tiny", dict(D=128, H=32, L=2, N=100, T=3)),           # fp32 rows of 16 KiB
-    ("llava7b_b1", dict(L=2, H=64, N=90, T=2)),              # 64 heads
-    ("llava7b_b1", dict(L=2, H=72, D=64, N=90, T=2)),        # more heads than the row-split kernel takes
-    ("llava7b_b16", dict(B=40, L=32, H=2, D=64, N=24, T=2)),  # 1280 segments: two layer chunks through the row-split kernel
-    # few segments, many (segment, head) items: the per-head kernel (whole softmax rows per CTA)
-    ("llava7b_b1", dict(L=20, H=32, N=100, T=3)),            # bf16, 256-byte head slices
-    ("tiny", dict(L=16, H=40, N=70, T=3)),                   # fp32, D = 64
-    ("tiny", dict(B=2, L=10, H=32, D=128, N=50, T=2)),       # fp32, D = 128: 512-byte slices, one row per warp step
-    ("llava7b_b1", dict(L=10, H=64, D=64, N=150, T=2)),      # bf16, D = 64: 128-byte slices, four rows per warp step
-    ("llava7b_b1", dict(L=20, H=32, N=700, T=2, budget_ratios=(1.0,))),   # 22 tiles per item: more than consumer warps
-    ("llava7b_b1", dict(L=24, H=27, N=100, T=2)),            # odd head count
-    ("llava7b_b1", dict(L=24, H=40, D=64, N=100, T=2)),      # bf16, D = 64, 40 heads
-    ("llava7b_b1", dict(L=37, H=18, N=100, T=2)),            # 666 items over 148 CTAs: four or five each
-    ("llava7b_b1", dict(B=4, L=32, H=8, N=60, T=2)),         # 128 segments (several samples) on the per-head kernel
+@pytest.mark.parametrize("name,kw,kernel", [
+    ("tiny", {}, CLUSTER),
+    ("llava7b_b1", dict(L=3, H=8, N=200, T=5), CLUSTER),
+    ("llava7b_b16", dict(B=3, L=2, H=4, N=97, T=4), CLUSTER),
+    ("tiny", dict(D=128, H=2, T=3), CLUSTER),
+    ("llava7b_b1", dict(L=2, H=5, D=64, N=130, T=3), CLUSTER),
+    ("tiny", dict(D=128, H=32, L=2, N=100, T=3), CLUSTER),           # fp32 rows of 16 KiB
+    ("llava7b_b1", dict(L=2, H=64, N=90, T=2), CLUSTER),              # 64 heads
+    ("llava7b_b1", dict(L=2, H=72, D=64, N=90, T=2), CLUSTER),        # more heads than the row-split kernel takes
+    ("llava7b_b16", dict(B=40, L=32, H=2, D=64, N=24, T=2), PAIR),    # 1280 segments
+    ("llava7b_b16", dict(B=40, L=32, H=16, D=64, N=24, T=2), ROWS),   # the same with longer rows: two launches, of 25 layers and of seven
+    ("llava7b_b1", dict(L=270, H=72, D=64, N=24, T=2), TWO),
+    # a CTA to a (segment, head) pair
+    ("llava7b_b1", dict(L=20, H=32, N=100, T=3), PAIR),               # bf16, 256-byte head slices
+    ("tiny", dict(L=16, H=40, N=70, T=3), PAIR),                      # fp32, D = 64
+    ("tiny", dict(B=2, L=10, H=32, D=128, N=50, T=2), PAIR),          # fp32, D = 128: 512-byte slices, one row per warp step
+    ("llava7b_b1", dict(L=10, H=64, D=64, N=150, T=2), PAIR),         # bf16, D = 64: 128-byte slices, four rows per warp step
+    ("llava7b_b1", dict(L=20, H=32, N=700, T=2, budget_ratios=(1.0,)), PAIR),
+    ("llava7b_b1", dict(L=24, H=27, N=100, T=2), PAIR),               # odd head count
+    ("llava7b_b1", dict(L=24, H=40, D=64, N=100, T=2), PAIR),         # bf16, D = 64, 40 heads
+    ("llava7b_b1", dict(L=37, H=18, N=100, T=2), PAIR),
+    ("llava7b_b1", dict(B=4, L=32, H=8, N=60, T=2), PAIR),            # 128 segments (several samples)
+    # short pairs of several waves: the per-head kernel (whole softmax rows per CTA)
+    ("llava7b_b1", dict(L=32, H=48, N=80, T=3), HEADS),
+    ("tiny", dict(L=32, H=48, N=70, T=3), HEADS),
+    ("tiny", dict(B=2, L=16, H=48, D=128, N=50, T=2), HEADS),
+    ("llava7b_b1", dict(L=24, H=64, D=64, N=80, T=2), HEADS),
+    ("llava7b_b1", dict(L=57, H=27, N=60, T=2), HEADS),               # 1539 items over 148 CTAs: ten or eleven each
+    ("llava7b_b1", dict(B=4, L=32, H=12, N=60, T=2), HEADS),
 ])
-def test_decode_matches_oracle(api, name, kw):
+def test_decode_matches_oracle(api, name, kw, kernel):
     w = wl.scaled(wl.WORKLOADS[name], **kw)
     q, k, v = wl.make_prompt(w, "cuda")
     scale = wl.layer_scale(w)
     scores = np.stack([wl.synthetic_scores(w.L, w.N, seed=b + 7) for b in range(w.B)])
     budgets = [w.budget_rows()] * w.B
     s = _session(w.B, w.L, w.H, w.D, w.N, w.dtype, scale, decode_cap=w.T)
+    check_kernel(s, kernel)
     s.search(torch.tensor(budgets), scores=torch.from_numpy(scores).cuda())
     s.compact(k, v)
     ref_sel = oracle_select(scores, budgets)
@@ -327,11 +337,13 @@ def test_decode_full_budget_is_dense_attention(api):
         assert (out[0, l] - ref).abs().max() <= DECODE_TOL[w.dtype]
 
 
-@pytest.mark.parametrize("kw,step", [
-    (dict(L=4, H=4, N=80, T=2), 1),                 # a model calls one layer at a time (cluster kernel)
-    (dict(B=2, L=20, H=32, N=70, T=2), 10),         # two samples, ten layers per call: the per-head kernel on a sub-range
+@pytest.mark.parametrize("kw,step,kernel", [
+    (dict(L=4, H=4, N=80, T=2), 1, CLUSTER),        # a model calls one layer at a time
+    (dict(B=2, L=20, H=32, N=70, T=2), 10, PAIR),   # two samples, ten layers per call
+    (dict(B=2, L=32, H=48, N=70, T=2), 16, HEADS),
+    (dict(B=10, L=60, H=16, N=40, T=2), 30, ROWS),
 ])
-def test_decode_layer_range(api, kw, step):
+def test_decode_layer_range(api, kw, step, kernel):
     w = wl.scaled(wl.WORKLOADS["llava7b_b1"], **kw)
     q, k, v = wl.make_prompt(w, "cuda")
     scale = wl.layer_scale(w)
@@ -344,15 +356,16 @@ def test_decode_layer_range(api, kw, step):
     qd, kn, vn = wl.make_decode_inputs(w, 0, "cuda")
     full = a.decode(qd, kn, vn).float().clone()
     b.out.zero_()
+    check_kernel(b, kernel, layer_end=step)
     for l in range(0, w.L, step):
         b.decode(qd, kn, vn, layer_begin=l, layer_end=l + step)
     assert (full - b.out.float()).abs().max() <= DECODE_TOL[w.dtype]
     assert torch.equal(a.cache.len, b.cache.len)
 
 
-@pytest.mark.parametrize("kw", [dict(L=6, H=8, N=300, T=5),        # cluster kernel
-                                dict(L=20, H=32, N=100, T=5)])     # per-head kernel
-def test_decode_replayed_from_a_cuda_graph(api, kw):
+@pytest.mark.parametrize("kw,kernel", [(dict(L=6, H=8, N=300, T=5), CLUSTER), (dict(L=20, H=32, N=100, T=5), PAIR),
+                                       (dict(L=32, H=48, N=80, T=5), HEADS), (dict(L=260, H=16, N=40, T=5), ROWS)])
+def test_decode_replayed_from_a_cuda_graph(api, kw, kernel):
     """One decode call captured in a CUDA graph and replayed token after token gives, bit for bit,
     what separate calls give: nothing a call leaves behind (lengths, workspace flags) may depend
     on its being launched afresh."""
@@ -361,6 +374,7 @@ def test_decode_replayed_from_a_cuda_graph(api, kw):
     scale = wl.layer_scale(w)
     scores = torch.from_numpy(wl.synthetic_scores(w.L, w.N, 9)[None]).cuda()
     a, b, warm = (_session(w.B, w.L, w.H, w.D, w.N, w.dtype, scale, decode_cap=w.T) for _ in range(3))
+    check_kernel(a, kernel)
     for s in (a, b, warm):
         s.search(w.budget_rows(), scores=scores)
         s.compact(k, v)
@@ -381,12 +395,12 @@ def test_decode_replayed_from_a_cuda_graph(api, kw):
     assert int(b.status.max()) == 0
 
 
-@pytest.mark.parametrize("kw", [dict(L=6, H=8, N=300, T=2),        # cluster kernel
-                                dict(L=20, H=32, N=120, T=2)])     # per-head kernel (its flags live in the workspace)
+@pytest.mark.parametrize("kw,kernel", [(dict(L=6, H=8, N=300, T=2), CLUSTER), (dict(L=20, H=32, N=120, T=2), PAIR),
+                                       (dict(L=32, H=48, N=80, T=2), HEADS), (dict(L=260, H=16, N=40, T=2), ROWS)])
 @pytest.mark.parametrize("byte", [0x7f, 0xff, 0x00])
-def test_decode_with_stale_workspace(api, byte, kw):
+def test_decode_with_stale_workspace(api, byte, kw, kernel):
     """The decode workspace may hold anything (another shape's partials, an earlier call's plan):
-    results do not depend on it.  (The cluster and the per-head kernel keep their CTAs' flags there.)"""
+    results do not depend on it.  (Pair by pair, counts of a length's readers live there, in the per-head kernel its CTAs' flags.)"""
     w = wl.scaled(wl.WORKLOADS["llava7b_b1"], **kw)
     q, k, v = wl.make_prompt(w, "cuda")
     scale = wl.layer_scale(w)
@@ -396,6 +410,7 @@ def test_decode_with_stale_workspace(api, byte, kw):
     for s in (a, b):
         s.search(w.budget_rows(), scores=scores)
         s.compact(k, v)
+    check_kernel(a, kernel)
     b.ws_decode.fill_(byte)
     for t in range(w.T):
         qd, kn, vn = wl.make_decode_inputs(w, t, "cuda")
@@ -408,9 +423,9 @@ def test_decode_with_stale_workspace(api, byte, kw):
     assert a.status.cpu().tolist() == b.status.cpu().tolist() == [0]
 
 
-@pytest.mark.parametrize("kw", [dict(H=4), dict(H=72, D=64),       # cluster kernel, also above 64 heads
-                                dict(H=32, L=10)])                 # per-head kernel
-def test_decode_empty_segment_is_reported(api, kw):
+@pytest.mark.parametrize("kw,kernel", [(dict(H=4), CLUSTER), (dict(H=72, D=64), CLUSTER), (dict(H=32, L=10), PAIR),
+                                       (dict(H=48, L=16), HEADS), (dict(H=16, L=130, N=40), ROWS), (dict(H=72, D=64, L=135, N=24), TWO)])
+def test_decode_empty_segment_is_reported(api, kw, kernel):
     """A segment with no rows (never compacted) cannot be attended over: the sample's status says
     so, its output is zero, its length stays, and the other segments are unaffected."""
     w = wl.scaled(wl.WORKLOADS["llava7b_b16"], **{**dict(B=2, L=3, N=80, T=2), **kw})
@@ -422,6 +437,7 @@ def test_decode_empty_segment_is_reported(api, kw):
     for s in (a, b):
         s.search(w.budget_rows(), scores=torch.from_numpy(scores).cuda())
         s.compact(k, v)
+    check_kernel(b, kernel)
     empty = 1 * w.L + 2                              # sample 1, layer 2
     b.cache.len[empty] = 0
     qd, kn, vn = wl.make_decode_inputs(w, 0, "cuda")
@@ -437,12 +453,14 @@ def test_decode_empty_segment_is_reported(api, kw):
     assert torch.equal(b.cache.len[mask.flatten().cuda()], a.cache.len[mask.flatten().cuda()])
 
 
-@pytest.mark.parametrize("name,kw", [
-    ("tiny", {}),
-    ("llava7b_b1", dict(L=3, H=8, N=200, T=3)),
-    ("llava7b_b1", dict(L=20, H=32, N=90, T=3)),            # per-head kernel
+@pytest.mark.parametrize("name,kw,kernel", [
+    ("tiny", {}, CLUSTER),
+    ("llava7b_b1", dict(L=3, H=8, N=200, T=3), CLUSTER),
+    ("llava7b_b1", dict(L=20, H=32, N=90, T=3), PAIR),
+    ("llava7b_b1", dict(L=32, H=48, N=80, T=3), HEADS),
+    ("llava7b_b1", dict(L=260, H=16, N=40, T=3), ROWS),
 ])
-def test_decode_without_append(api, name, kw):
+def test_decode_without_append(api, name, kw, kernel):
     """k_new = v_new = NULL: the query attends over the rows already cached and nothing changes."""
     w = wl.scaled(wl.WORKLOADS[name], **kw)
     q, k, v = wl.make_prompt(w, "cuda")
@@ -454,6 +472,7 @@ def test_decode_without_append(api, name, kw):
     s.compact(k, v)
     qd, kn, vn = wl.make_decode_inputs(w, 0, "cuda")
     s.decode(qd, kn, vn)                           # one ordinary step first: the cache now ends in a decoded row
+    check_kernel(s, kernel, appends=False)
     len1 = s.cache.len.clone()
     ck, cv = s.cache.k.clone(), s.cache.v.clone()
     q2, _, _ = wl.make_decode_inputs(w, 1, "cuda")
