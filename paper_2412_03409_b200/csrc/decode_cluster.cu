@@ -66,46 +66,6 @@ struct ClusterArgs {
     uint32_t row_bytes;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t cluster_size()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-// Store into the first CTA of the cluster, at the place that `p` has in this CTA's shared memory.
-__device__ __forceinline__ void store_first_cta(float *p, float v)
-{
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"((uint32_t)__cvta_generic_to_shared(p)));
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
-}
-// Two fp32 operations in one instruction (same rounding as the scalar ones): half the issue slots.
-__device__ __forceinline__ float2 fma_pair(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("{\n\t.reg .b64 x, y, z, w;\n\t"
-        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
-        "fma.rn.f32x2 w, x, y, z;\n\tmov.b64 {%0, %1}, w;\n\t}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-__device__ __forceinline__ float2 mul_pair(float2 a, float2 b)
-{
-    float2 d;
-    asm("{\n\t.reg .b64 x, y, w;\n\t"
-        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
-        "mul.rn.f32x2 w, x, y;\n\tmov.b64 {%0, %1}, w;\n\t}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
-}
 __device__ __forceinline__ void copy16(void *dst, const unsigned char *src)
 {
     asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
@@ -256,7 +216,7 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
         float2 d = make_float2(0.f, 0.f);
         RowVec<T>::unpack(raw, x);
 #pragma unroll
-        for (int i = 0; i < VE; i += 2) d = fma_pair(make_float2(qf[i], qf[i + 1]), make_float2(x[i], x[i + 1]), d);
+        for (int i = 0; i < VE; i += 2) d = fma2(make_float2(qf[i], qf[i + 1]), make_float2(x[i], x[i + 1]), d);
         return d.x + d.y;
     };
     auto add = [&](float p, const uint4 &raw) {
@@ -264,7 +224,7 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
         RowVec<T>::unpack(raw, x);
         lsum += p;
 #pragma unroll
-        for (int i = 0; i < VE; i += 2) acc[i / 2] = fma_pair(make_float2(p, p), make_float2(x[i], x[i + 1]), acc[i / 2]);
+        for (int i = 0; i < VE; i += 2) acc[i / 2] = fma2(make_float2(p, p), make_float2(x[i], x[i + 1]), acc[i / 2]);
     };
     auto rescale = [&](float mx) {
 #pragma unroll
@@ -274,7 +234,7 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
         M = mx;
         lsum *= corr;
 #pragma unroll
-        for (int i = 0; i < VE / 2; ++i) acc[i] = mul_pair(acc[i], make_float2(corr, corr));
+        for (int i = 0; i < VE / 2; ++i) acc[i] = mul2(acc[i], make_float2(corr, corr));
     };
     int stage = 0;
     for (int base = rw.r0 + warp * STEP; base < rw.r1; base += kCWarps * STEP) {
@@ -357,10 +317,10 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
     }
     if (C > 1) {
         asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-        if (tid < D) store_first_cta(&c_acc[rank][tid], o);
+        if (tid < D) store_in_first_cta(&c_acc[rank][tid], o);
         if (tid == 0) {
-            store_first_cta(&c_ml[rank][0], m);
-            store_first_cta(&c_ml[rank][1], z);
+            store_in_first_cta(&c_ml[rank][0], m);
+            store_in_first_cta(&c_ml[rank][1], z);
         }
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         if (rank != 0) return;  // (only the first CTA's memory is written, and it waits for everyone)

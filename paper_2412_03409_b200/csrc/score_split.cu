@@ -157,14 +157,6 @@ __device__ __noinline__ float redo_colsum(const SplitArgs &a, int sh, int key, i
     return sum;
 }
 
-// Store into the first CTA of the cluster, at the place that `p` has in this CTA's shared memory.
-__device__ __forceinline__ void store_in_first(float *p, float v)
-{
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(saddr(p)));
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
-}
-
 // MODE 3: as MODE 1, and the item's logits are kept (64 KiB a tile, which mostly stay in the L2); once a query's
 // normaliser is known, the reader warp that has its row reads them back and adds up what the warp's queries give to every
 // key: the second pass without its products and splits.
@@ -187,8 +179,8 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
     __shared__ int s_abort;
     __shared__ int q_item[kQueue];
     __shared__ __align__(16) float s_lse[2][kReaders][TT];
-    __shared__ float s_col[MODE == 0 ? TT : 1], s_cols[MODE == 0 ? kMeanHeads : 1][TT];  // column sums; (first CTA) those of all heads
-    __shared__ int s_gave_up[kMeanHeads];
+    __shared__ float s_col[MODE == 0 ? TT : 1], s_cols[MODE == 0 ? kMeanHeads : 1][MODE == 0 ? TT : 1];  // column sums; (first CTA) those of all heads
+    __shared__ int s_gave_up[MODE == 0 ? kMeanHeads : 1];
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int nitems = a.nsh * a.tiles;
@@ -617,8 +609,8 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
     if (MODE == 0 && by_cluster) {
         const int seg = blockIdx.x / a.H, h = blockIdx.x - seg * a.H;
         asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-        if (tid < TT) store_in_first(&s_cols[h][tid], s_col[tid]);
-        if (tid == 0) store_in_first(reinterpret_cast<float *>(s_gave_up + h), __int_as_float(s_abort));
+        if (tid < TT) store_in_first_cta(&s_cols[h][tid], s_col[tid]);
+        if (tid == 0) store_in_first_cta(reinterpret_cast<float *>(s_gave_up + h), __int_as_float(s_abort));
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         if (h != 0) return;  // (only the first CTA's memory is written, and it waits for everyone)
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");

@@ -63,19 +63,7 @@ static size_t sort_smem_bytes(int threads, int ipt, bool split)
            std::max((size_t)kDigits * (threads / 32), split ? items : 0) * sizeof(uint32_t);
 }
 
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// Address, in CTA `rank` of the cluster, of what `p` is in this one; and loads from there.
-__device__ __forceinline__ uint32_t in_cta(const void *p, uint32_t rank)
-{
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return a;
-}
+// Loads from another CTA of the cluster (in_cta).
 __device__ __forceinline__ uint4 load_there16(uint32_t a)
 {
     uint4 v;
