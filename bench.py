@@ -70,9 +70,7 @@ def measured_peaks():
         return FALLBACK_HBM_GBS, FALLBACK_BF16_TFLOPS, "fallback"
 
 
-# Which kernel a decode call takes: the library's rules (launch_decode_cluster and launch_decode_heads)
-# restated for the workloads below (the cluster kernel's line for long segments of few pairs is far from them), for the
-# kernel's name, the launch count and the traffic figure.
+# The decode kernels of the workloads below, by what the library says a call takes: the kernel's name, where its source is, launches a call.
 DECODE_KERNELS = {
     "cluster": ("decode_cluster_kernel", "decode_cluster.cu", "decode_cluster_kernel(const ClusterArgs a)", 1),
     "heads": ("decode_heads_kernel", "decode_heads.cu", "decode_heads_kernel(const __grid_constant__ HeadMaps maps", 1),
@@ -80,24 +78,13 @@ DECODE_KERNELS = {
 }
 
 
-def decode_path(w, sms):
-    nact = w.B * w.L
-    pairs = nact * w.H
+def decode_path(w):
+    from paper_2412_03409_b200 import api
+    shape = api.make_shape(w.B, w.L, w.H, w.D, w.N, w.dtype)
     cap_rows = w.B * (min(w.budget_rows(), w.L * w.N) + w.L * w.T)       # as Session sizes the cache
-    rows = cap_rows // nact - w.T // 2
-    kb = rows * w.D * 2 * w.esize >> 10
-    if pairs < 4 * sms:
-        return "cluster"
-    if pairs < 10 * sms:
-        cluster = kb <= (448 if pairs <= 5 * sms else 256 if pairs <= 6 * sms else 320 if pairs <= 7 * sms else 448)
-    elif nact > 256:
-        cluster = rows >= (0 if w.H * w.D * w.esize <= 1024 else 112)
-    else:
-        cluster = rows >= (96 if pairs < 20 * sms else 80)
-    if cluster:
-        return "cluster"
-    heads = w.D in (64, 128) and nact <= 256 and cap_rows // nact <= 1024
-    return "heads" if heads else "stream"
+    kernel = api.prefixkv_decode_kernel(shape, api.CacheStruct(None, None, None, None, None, cap_rows, w.T, 0, None, None, None))
+    return {api.KERNEL_CLUSTER: "cluster", api.KERNEL_PAIR: "cluster", api.KERNEL_HEADS: "heads", api.KERNEL_HEADS_SHARED: "heads",
+            api.KERNEL_ROWS: "stream"}[kernel]
 
 
 # DRAM bytes (read + write) of one launch of the workload's decode kernel from an ncu capture (its
@@ -389,7 +376,7 @@ def measure_workload(w, steps, warmup, dev, rank, world, sampler=None, with_lse=
     return res
 
 
-def workload_summary(w, m, hbm_peak, tf_peak, sms):
+def workload_summary(w, m, hbm_peak, tf_peak):
     """The figures of one configuration that the targets are stated on."""
     st = m["stage_ms"]
     dec_gbs = m["dec_bytes"] / (st["decode"] * 1e-3) / 1e9
@@ -399,7 +386,7 @@ def workload_summary(w, m, hbm_peak, tf_peak, sms):
             "compress_ms_per_prompt": compress_ms / w.B, "stages_ms": st,
             "score_tensor_util_vs_burst": m["causal_flop"] * 2 / (st["score"] * 1e-3) / (tf_peak * 1e12),
             "tok_s": w.B * w.T / (sum(st.values()) * 1e-3), "prompts_interleaved": m["R"], "clocks": m["clocks"],
-            "decode_kernel": DECODE_KERNELS[decode_path(w, sms)][0]}
+            "decode_kernel": DECODE_KERNELS[decode_path(w)][0]}
 
 
 def run_ours(args):
@@ -446,16 +433,15 @@ def run_ours(args):
     # The other configurations, a few steps each (rank 0 of a one-GPU run only): the figures the
     # bandwidth and latency targets are stated on, measured in this same process.
     others = {}
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
     if world == 1 and not args.no_workloads and args.workload == "llava7b_b1":
-        others[w.name] = workload_summary(w, m, hbm_peak, tf_peak, sms)
+        others[w.name] = workload_summary(w, m, hbm_peak, tf_peak)
         for name in wl.ORDER:
             if name == w.name:
                 continue
             wo = wl.WORKLOADS[name]
             mo = measure_workload(wo, args.workload_steps, 3, dev, 0, 1, sampler)
             del mo["reps"], mo["pool"]
-            others[name] = workload_summary(wo, mo, hbm_peak, tf_peak, sms)
+            others[name] = workload_summary(wo, mo, hbm_peak, tf_peak)
             torch.cuda.empty_cache()
     clocks = m["clocks"]
     sampler.stop()
@@ -465,7 +451,7 @@ def run_ours(args):
             dist.destroy_process_group()
         return
     value = world * w.B * w.T / (step_ms_max * 1e-3)
-    path = decode_path(w, sms)
+    path = decode_path(w)
     line = {
         "metric": "tok/s", "value": value, "unit": "tok/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": step_ms_max, "higher_is_better": True,

@@ -388,27 +388,65 @@ int decode_cluster_ctas(const pkv_shape *s, const pkv_cache *c, int nact, int sm
     const int64_t pair_bytes = seg_rows * D * 2 * (int64_t)esize(s);
     const int wave = kCPerSm * sms;
     if (items >= 4 * (int64_t)sms) {
-        // A CTA for every pair.  Measured, the per-head (or row-split) kernel / this one, us a call, bf16, heads of 128, lengths alike and
-        // from 0.3 to 1.7 of the mean.  One wave: 640 pairs of 30 rows 7.5 / 4.9, 8.4 / 5.4, of 128 12.7 / 9.9, 13.4 / 10.7, of 820 48.8 / 45.8,
-        // 46.7 / 46.0.  Up to seven CTAs an SM, in one wave too: 888 x 64 12.2 / 9.1, 11.8 / 9.2, x 400 34.9 / 33.6, 36.7 / 35.6, x 600 47.3 / 46.7,
-        // 47.4 / 49.7; 1024 x 32 10.5 / 7.1, 10.3 / 7.2, x 128 16.6 / 14.8, 18.1 / 15.2, x 256 25.9 / 25.7, 31.9 / 27.3, x 400 38.8 / 38.1, 39.8 / 39.3,
-        // x 600 53.0 / 53.5, 54.7 / 55.8, x 820 69.3 / 71.2, 71.2 / 73.8.  More waves: CTAs that begin cost the first rows' latency,
-        // which is little against long rows, and is hidden where lengths differ, as they do after a search: 1280 x 32 11.9 / 10.8, 11.7 / 10.7,
-        // x 128 19.5 / 20.1, 21.5 / 18.4, x 256 31.9 / 32.3, 38.4 / 31.5; 1600 x 128 23.0 / 24.4, 24.3 / 23.3, x 820 104.5 / 106.4, 106.6 / 104.5;
-        // 2048 x 32 15.8 / 16.5, 15.5 / 16.3, x 128 27.8 / 28.8, 29.2 / 27.2, x 400 68.6 / 67.4, 77.0 / 69.3; 4096 x 32 27.0 / 29.0, 26.2 / 28.6, x 64 35.5 / 35.3,
-        // 35.9 / 34.4, x 256 87.3 / 84.3, 95.7 / 83.4; 8192 x 128 97.2 / 90.0, 99.0 / 88.5; against the row-split kernel 16384 x 64 97.8 / 118.2,
-        // 96.5 / 114.9, x 128 180 / 169, 174 / 168; with pruning 640 x 64 17.0 / 9.7, 2048 x 64 22.7 / 21.3, 4096 x 64 34.1 / 37.4, x 128 51.8 / 51.2,
-        // 8192 x 128 94.1 / 94.5, x 200 138.6 / 130.3.
-        // More than 256 segments, always the row-split kernel's otherwise: 288 x 16 heads of 64, 64 rows 28.9 / 29.5, 128 42.3 / 36.0, 256 69.8 / 53.5;
-        // 960 x 32, 32 rows 99 / 179, 128 318 / 313, 256 601 / 573, but rows of 1 KiB, which it splits badly, 288 x 8 of 64, 32 rows 18.6 / 14.3, 960 x 8,
-        // 64 rows 65.6 / 43.9.
+        // A CTA for every pair.  Measured, us a call replayed from a graph, the kernel that takes the call otherwise (per head, or split by rows
+        // with more than 256 segments or 1024 rows, or with pruning) / this one; lengths all alike, random (lognormal, sigma 0.5), as a
+        // search at a budget of 0.2 leaves them; bf16 heads of 128 (512 bytes a row) where nothing else is said:
+        //   pairs x rows          alike           random          searched
+        //   one wave, five CTAs an SM and fewer:
+        //    640 x 64          10.1 / 7.5       9.7 / 7.5      10.4 / 7.7
+        //    640 x 512         34.0 / 30.5     32.4 / 29.1     42.4 / 31.5
+        //    640 x 820         48.8 / 44.7     46.3 / 43.6     53.1 / 47.2
+        //    640 x 1000        59.4 / 53.4     54.2 / 51.6     58.2 / 56.6
+        //   six and seven CTAs an SM, in one wave too:
+        //    888 x 64          12.3 / 9.2      11.7 / 10.0     11.6 / 9.4
+        //    888 x 480         40.1 / 37.8     40.4 / 44.4     42.1 / 39.8
+        //    888 x 640         50.4 / 48.2     50.7 / 57.2     52.1 / 51.6
+        //   1024 x 32          10.5 / 7.0      10.3 / 7.7      10.6 / 7.4
+        //   1024 x 136         17.3 / 14.9     17.5 / 17.5     20.7 / 15.5
+        //   1024 x 256         26.1 / 24.8     27.5 / 29.5     32.8 / 25.4
+        //   1024 x 600         52.9 / 52.6     52.4 / 61.7     58.0 / 56.0
+        //   1024 x 820         69.3 / 69.6     67.8 / 83.0     73.2 / 73.9
+        //   more waves: CTAs that begin cost the first rows' latency, which is little against long rows:
+        //   1280 x 32          11.8 / 9.5      12.2 / 10.2     11.9 / 9.9
+        //   1280 x 410         47.6 / 44.8     47.3 / 49.7     50.7 / 46.7
+        //   1280 x 700         75.0 / 69.7     72.7 / 80.8     76.4 / 76.5
+        //   2048 x 64          20.0 / 19.2     18.9 / 19.5     21.5 / 19.0
+        //   2048 x 128         27.8 / 27.7     27.3 / 26.5     32.6 / 26.0
+        //   2048 x 820          131 / 125       127 / 121       143 / 130
+        //   4096 x 16          20.3 / 22.2     20.6 / 21.9     20.1 / 22.0
+        //   4096 x 64          35.5 / 33.6     34.3 / 34.0     35.8 / 31.7
+        //   4096 x 820          257 / 243       260 / 251       283 / 250
+        //   8192 x 128         97.1 / 89.6                      101 / 87.5
+        //   heads of 64:
+        //   2048 x 100         17.4 / 17.4     17.5 / 17.4
+        //   4096 x 32          20.4 / 22.1     20.6 / 22.6     20.3 / 22.3
+        //   4096 x 256         50.7 / 47.6     50.5 / 49.5     54.0 / 47.6
+        //   fp32:
+        //   2048 x 128         46.7 / 45.7     46.6 / 43.3     55.5 / 44.1
+        //   4096 x 100, of 64  42.1 / 40.2                     42.7 / 39.8
+        //   with pruning:
+        //    640 x 64          16.3 / 9.3                      18.5 / 9.5
+        //   2048 x 64          22.1 / 22.3                     22.8 / 21.2
+        //   2048 x 128         33.1 / 31.2                     33.3 / 28.5
+        //   4096 x 64          33.5 / 38.4                     34.8 / 36.1
+        //   4096 x 220         82.5 / 79.0                     80.8 / 74.2
+        //   8192 x 128         95.7 / 96.7                     95.2 / 92.4
+        //   more than 256 segments, 32 heads of 128, 16 of 64, eight of 64:
+        //   9216 x 64          60.2 / 65.4                     59.8 / 64.0
+        //   9216 x 128          106 / 98.7                      104 / 96.4
+        //   30720 x 128         320 / 304                       321 / 308
+        //   4608 x 128         42.6 / 34.6                     44.0 / 33.9
+        //   2304 x 16          13.4 / 13.0                     15.1 / 12.8
+        //   7680 x 64          65.7 / 40.5                     66.8 / 40.3
+        // One segment of a multiple of the mean (first or last of the call) sets the time of its CTAs, which the other kernels split up: 1024 x
+        // 136 five times the mean 19.6 / 24.2, twenty 33.2 / 75.5; 1024 x 512 ten 50 / 122, twenty 53 / 222; 4096 x 820 five 266 / 289, ten
+        // 266 / 345; 6400 x 410 ten 225 / 243.  A search of the repository's workloads leaves 2.7 times the mean at most.
         // By a pair's rows, and their bytes, halfway through the tokens that the cache has room for.
         const int64_t rows = seg_rows - c->decode_cap / 2, kb = rows * D * 2 * (int64_t)esize(s) >> 10;
         int64_t least = 0, most_kb = INT64_MAX;
         if (items <= wave) most_kb = 448;
         else if (items <= 6 * (int64_t)sms) most_kb = 256;
-        else if (items <= 7 * (int64_t)sms) most_kb = 320;
-        else if (items < 10 * (int64_t)sms) most_kb = 448;
+        else if (items < 10 * (int64_t)sms) most_kb = 320;
         else if (c->evict_distance > 0) least = items < 20 * (int64_t)sms ? 80 : 200;
         else if (nact > 256) least = (size_t)H * D * esize(s) <= 1024 ? 0 : 112;
         else least = items < 20 * (int64_t)sms ? 96 : 80;

@@ -142,7 +142,7 @@ def test_a_plan_changed_just_before_the_call(place):
     (9, 30, 64, 64, 40, 15, torch.bfloat16, 0, ROWS), (9, 32, 16, 128, 40, 12, torch.float32, 3, ROWS), (9, 32, 32, 128, 40, 12, torch.float32, 3, ROWS),
     (9, 30, 40, 128, 24, 8, torch.float32, 0, ROWS), (9, 32, 16, 64, 40, 12, torch.float32, 3, ROWS),
     (9, 32, 32, 64, 40, 12, torch.float32, 3, ROWS), (9, 30, 40, 64, 24, 9, torch.float32, 0, ROWS), (9, 30, 64, 64, 24, 9, torch.float32, 3, ROWS),
-    (1, 32, 32, 128, 1500, 700, torch.bfloat16, 0, SHARED), (2, 18, 25, 128, 900, 660, torch.bfloat16, 0, SHARED), (3, 32, 32, 64, 90, 40, torch.bfloat16, 0, HEADS),
+    (1, 32, 32, 128, 1500, 700, torch.bfloat16, 0, SHARED), (2, 18, 25, 128, 900, 660, torch.bfloat16, 0, SHARED), (2, 22, 30, 128, 800, 660, torch.bfloat16, 0, SHARED), (3, 32, 32, 64, 90, 40, torch.bfloat16, 0, HEADS),
     (2, 32, 32, 128, 90, 30, torch.float32, 0, HEADS),
 ])
 def test_what_goes_elsewhere(B, L, H, D, N, rows, dtype, d, kernel):
