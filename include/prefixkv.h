@@ -343,8 +343,8 @@ int prefixkv_gini(const pkv_shape *shape, const uint64_t *cum, double *gini, voi
  * waiting, finishes in bounds and reports.  This call runs that give-up path alone: one warp
  * waits, with a limit of a few thousand tries (milliseconds), on a barrier that nothing
  * completes, and dev_status[0] is raised to PKV_DEV_TIMEOUT.  Nothing faults or hangs.
- * which = 2: the wait of the decode kernels that write the lengths themselves for the flags of
- * their CTAs; one block plays both parts, some flags not coming before the limit and then late,
+ * which = 2: the wait of the per-head decode kernel, which writes the lengths itself, for the flags of
+ * its CTAs; one block plays both parts, some flags not coming before the limit and then late,
  * and raises the same code when every flag was left as a later call needs it.
  * which = 3: the wait of the scoring kernel for short bf16 prompts for its other product warp.
  * which = 4: the wait of the per-head decode kernel for parts of an item that other CTAs pass on, as which = 2.

@@ -27,7 +27,9 @@
 // lists what the producers issue, and at the end puts the cut item together, away from the consumers; whatever
 // happened, it puts the flags of the parts that it was owed back.  Where the lengths are short or alike already, items stay dealt.
 //
-// Measured on the 32-layer, 32-head, 128-rows-per-layer case (22.3 us per call with this design),
+// (Most calls go to the kernel with a CTA to a pair, decode_cluster.cu: what it leaves to this one stands at decode_heads_form.)
+//
+// Measured on the 32-layer, 32-head, 128-rows-per-layer case (22.3 us per call with this design; 14.8 in that kernel now),
 // each alone: one producer thread 24.1 us, five 22.9, ten 23.1; eight stages 22.4, twelve 21.9 (with
 // the prefetch below, against 21.95 for ten); two consumer warps per tile
 // (half the rows each) 22.4; an item's last, partial tile fetched in quarter-tile boxes 22.6 with

@@ -157,7 +157,7 @@ __device__ __noinline__ float redo_colsum(const SplitArgs &a, int sh, int key, i
     return sum;
 }
 
-// MODE 3: as MODE 1, and the item's logits are kept (64 KiB a tile, which mostly stay in the L2); once a query's
+// MODE 3: as MODE 1, and the item's logits are kept (64 KiB a tile, half of which go no further than the L2); once a query's
 // normaliser is known, the reader warp that has its row reads them back and adds up what the warp's queries give to every
 // key: the second pass without its products and splits.
 // MODE 1: stationary = Q tile t, streamed = K tiles 0..t (log-sum-exp).  MODE 2: stationary = K tile
