@@ -68,7 +68,6 @@ struct SplitArgs {
     int *next_item;       // work counter of this pass, zeroed before it; NULL: a CTA takes item blockIdx.x alone
     int clear_abort;      // this launch is the call's first and nothing has zeroed the abort word
     int L, H, N, tiles, nsh, group;
-    int seg0;             // the segment of the launch's first heads (mode 3)
 };
 
 // One float into its three bf16 parts, two elements at a time (packed low, high).  (Above the largest bf16,
@@ -122,7 +121,7 @@ template <int D> __device__ __forceinline__ float fma_logit(const float *x, cons
 }
 __device__ __forceinline__ const float *head_rows(const float *p, const pkv_strides &st, const SplitArgs &a, int sh)
 {
-    const int turn = sh / a.H, h = sh - turn * a.H, seg = a.seg0 + turn, b = seg / a.L, l = seg - b * a.L;
+    const int seg = sh / a.H, h = sh - seg * a.H, b = seg / a.L, l = seg - b * a.L;
     return p + b * st.b + l * st.l + h * st.h;
 }
 __device__ __forceinline__ void store8(float *p, const float *v)
@@ -262,7 +261,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
             }
             int sh, t;
             decode_item<PASS>(w, a.nsh, a.tiles, a.group, sh, t);
-            const int turn = sh / a.H, h = sh - turn * a.H, seg = a.seg0 + turn, b = seg / a.L, l = seg - b * a.L;
+            const int seg = sh / a.H, h = sh - seg * a.H, b = seg / a.L, l = seg - b * a.L;
             const float *qb = a.q + b * a.qs.b + l * a.qs.l + h * a.qs.h + c8 * 8;
             const float *kb = a.k + b * a.ks.b + l * a.ks.l + h * a.ks.h + c8 * 8;
             const int arow = t * TT + r0, brow = (PASS == 1 ? 0 : t) * TT + r0;
@@ -491,7 +490,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) score_split_kernel(const __g
             if (w < 0) break;
             int sh, t;
             decode_item<PASS>(w, a.nsh, a.tiles, a.group, sh, t);
-            const float sc = a.layer_scale[(a.seg0 + sh / a.H) % a.L] * kLog2eT;
+            const float sc = a.layer_scale[(sh / a.H) % a.L] * kLog2eT;
             const int grow = t * TT + row;  // query (pass 1) or key (pass 2) of this thread
             float *kept = MODE == 3 ? a.logits + ((size_t)blockIdx.x * a.tiles * TT + row) * TT : nullptr;
             float run_max = -INFINITY, run_sum = 0.f, col_sum = 0.f;
@@ -711,11 +710,12 @@ int launch_head_mean(const float *partial, int H, int N, size_t total, float *sc
 // Workspace: partial [rows][N], lse2 [rows][N], then two work counters and the abort word.  Short prompts: part sums of every
 // pair of tiles in the place of these, of as many segments at a time as kPartBytes hold, and the logits of a CTA's item, where the
 // workspace has room for them: one that was sized for a longer prompt, or for the caller's log-sum-exp, need not, and then
-// serves two passes.  (1024 tokens, us at once, in turns of 128 MiB, 64, 16: 6144 heads of 64, 432 MiB, 7626, 7742, 7796, 8424; 1024 heads
-// of 128, 72 MiB, 1525, 1526, 1589, 1770.)
+// serves two passes.  (1024 tokens, us at once, in turns of 128 MiB, 64, 16: 6144 heads of 64, 432 MiB, 7386, 7498, 7589, 8182; 1024 heads
+// of 128, 72 MiB, 1538, 1538, 1605, 1783.  A turn's first segment as an argument of the kernel instead of whole samples or layers of one:
+// 300 tokens x 16 17.2 -> 17.8.)
 struct SplitSpace {
     size_t partial, lse2, logits, words, bytes;
-    int turn;  // segments of a turn
+    int turn;  // segments of a turn: whole samples, or some of a sample's layers
 };
 static SplitSpace split_space(const pkv_shape *s, bool keep)
 {
@@ -724,8 +724,9 @@ static SplitSpace split_space(const pkv_shape *s, bool keep)
     SplitSpace w = {0, per, 0, 0, 0, 0};
     size_t end = 2 * per;
     if (keep) {
-        const size_t one = part_bytes(s->heads, tiles), most = kPartBytes / one, turns = (segs + most - 1) / most;
-        const size_t turn = (segs + turns - 1) / turns;
+        const size_t one = part_bytes(s->heads, tiles), most = kPartBytes / one, B = s->batch, L = s->layers;
+        auto evenly = [](size_t n, size_t at_once) { const size_t turns = (n + at_once - 1) / at_once; return (n + turns - 1) / turns; };
+        const size_t turn = most >= L ? evenly(B, most / L) * L : evenly(L, most);
         const size_t ctas = turn * s->heads * tiles < kKeepCtas ? turn * s->heads * tiles : kKeepCtas;
         w.turn = (int)turn;
         w.logits = round_up(turn * one, kWsAlign);
@@ -783,11 +784,15 @@ int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const
     } else if (keep) {
         const int ctas = sms < (int)kKeepCtas ? sms : (int)kKeepCtas, segs = B * L;
         a.next_item = counted ? words : nullptr;
-        for (a.seg0 = 0; a.seg0 < segs; a.seg0 += space.turn) {
-            const int now = segs - a.seg0 < space.turn ? segs - a.seg0 : space.turn;
+        for (int seg0 = 0, now; seg0 < segs; seg0 += now) {
+            const int b0 = seg0 / L, l0 = seg0 % L, end = space.turn < L ? (b0 + 1) * L : segs;
+            now = end - seg0 < space.turn ? end - seg0 : space.turn;
+            a.q = q + b0 * qs.b + l0 * qs.l;
+            a.k = k + b0 * ks.b + l0 * ks.l;
+            a.layer_scale = scale + l0;
             a.nsh = now * H;
             a.group = head_group(a.nsh, N, s->head_dim, 4);
-            cudaError_t e = a.seg0 > 0 ? cudaMemsetAsync(words, 0, sizeof(int), st) : cudaSuccess;
+            cudaError_t e = seg0 > 0 ? cudaMemsetAsync(words, 0, sizeof(int), st) : cudaSuccess;
             if (e != cudaSuccess) {
                 set_cuda_error(e, "cudaMemsetAsync(score work counter)");
                 return PKV_ERR_CUDA;
@@ -795,8 +800,8 @@ int launch_score_split(const pkv_shape *s, const float *q, pkv_strides qs, const
             rc = wide ? launch_split<3, 128>(a, ctas, st) : launch_split<3, 64>(a, ctas, st);
             if (rc != PKV_OK) return rc;
             e = launch_dependent(split_mean_kernel, dim3((unsigned)((size_t)now * ((N + 31) / 32))), dim3(256), 0, st, a.partial, H, N, a.tiles,
-                                 scores + (size_t)a.seg0 * N, a.abort_word);
-            if (e == cudaSuccess && now < segs && a.seg0 + now == segs)
+                                 scores + (size_t)seg0 * N, a.abort_word);
+            if (e == cudaSuccess && now < segs && seg0 + now == segs)
                 e = launch_dependent(split_abort_kernel, dim3((unsigned)sms), dim3(256), 0, st, scores, (size_t)segs * N, a.abort_word);
             if (e != cudaSuccess) {
                 set_cuda_error(e, "split_mean_kernel");
