@@ -27,8 +27,8 @@
 // 136 rows 16.7 -> 15.0.  (Partial sums of four rows reduced together, 12 shuffles for 17: no gain.)
 //
 // Measured, device time of calls replayed from a graph, one layer, bf16, D = 128, every call on another layer: 1 segment
-// x 32 heads x 128 rows 3.77 us (4.44 before all of this), 4 x 32 x 128 rows 5.23 (6.01), 16 x 32 x 128 9.84 (11.55),
-// 1 x 40 x 410 4.96 (5.65), 8 x 40 x 410 15.9 (18.8; 10.3 us of bytes); against the row-split kernel and its merge
+// x 32 heads x 128 rows 3.64 us (4.44 before all of this), 4 x 32 x 128 rows 5.30 (6.01), 16 x 32 x 128 9.87 (11.55),
+// 1 x 40 x 410 4.91 (5.65), 8 x 40 x 410 15.7 (18.8; 10.3 us of bytes); against the row-split kernel and its merge
 // kernel, before that: 1 x 32 x 128 rows 4.5 (10.0), 1024 rows 8.0 (26.4); 4 x 32 x 128 rows 6.1 (12.1);
 // 8 x 40 x 410 rows 17.4 (25.7); 8 x 64 x 900 rows 50 (51).  A second wave of CTAs costs as much as the
 // first's latency, 4-5 us (C = 8 for 4 x 32 x 128 rows: 8.9 us), hence the choice of C below.  Loads to
@@ -63,6 +63,7 @@ struct ClusterArgs {
     unsigned long long visit_tag;
     int32_t *dev_status;
     int H;
+    int guess_more;  // rows that a length read ahead may be short of
     uint32_t row_bytes;
 };
 
@@ -170,6 +171,7 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
     Rows rw{nullptr, nullptr, 0, 0, -1};
     if (guesses) {
         rw = rows_of(plan_of(a.p, guess_ln, guess_cp, guess_off, PruneState{0, 0, -1}));
+        if (rw.r1 > 0) rw.r1 += a.guess_more;
 #pragma unroll
         for (int i = 0; i < kCStages; ++i) request(rw, rw.r0 + (warp + i * kCWarps) * STEP, i);
     }
@@ -191,6 +193,7 @@ __global__ void __launch_bounds__(kCWarps * 32, P) decode_cluster_kernel(const C
     const SegPlan sp = s_plan;
     if (P != kCPerSm) last_one();
     const Rows now = rows_of(sp);
+    if (now.r1 + a.guess_more >= rw.r1 && now.r1 < rw.r1) rw.r1 = now.r1;
     if (now.r0 != rw.r0 || now.r1 != rw.r1 || now.skip != rw.skip || now.kb != rw.kb) {
         // (a row more or less at the end: the same bytes come to the same places again)
         if (now.r0 != rw.r0 || now.skip != rw.skip || now.kb != rw.kb) asm volatile("cp.async.wait_all;" ::: "memory");
@@ -493,6 +496,9 @@ int launch_decode_cluster(const pkv_shape *s, pkv_cache *c, const void *q, const
     a.visit_tag = visit_tag();
     a.dev_status = dev_status;
     a.H = H;
+    // A call of one wave is set up while the one in front, of the same cache maybe, has yet to write the lengths.  (24 x 16 heads of 64, 90
+    // rows, call after call: 5.9 us a call, 5.25 so.)  With clusters another length moves most CTAs' rows.
+    a.guess_more = kn != nullptr && c->evict_distance == 0 && C == 1 && items <= kCPerSm * (int64_t)sms ? 1 : 0;
     a.row_bytes = (uint32_t)((size_t)H * D * esize(s));
     if (C == 1 && items > kCPerSm * (int64_t)sms && items <= 6 * (int64_t)sms) return launch_shape<4, 6>(s, a, C, st);
     if (C == 1 && items > kCPerSm * (int64_t)sms && items <= 7 * (int64_t)sms) return launch_shape<3, 7>(s, a, C, st);

@@ -117,6 +117,29 @@ def test_a_segment_that_cannot_take_the_row_keeps_its_word(word, H):
     assert torch.equal(s.cache.k[o:], before[o:])
 
 
+@pytest.mark.parametrize("B,L,H,D,rows,dtype", [(1, 24, 16, 64, 90, torch.bfloat16), (1, 13, 57, 128, 33, torch.bfloat16), (3, 16, 8, 64, 31, torch.float32)])
+def test_lengths_off_by_more_than_a_row_ahead_of_the_call(B, L, H, D, rows, dtype):
+    """A CTA to a pair in one wave asks for a row more than the length read ahead has: right, a row short, and far off; to the last row of
+    the cache."""
+    T = 6
+    lens = [rows + i % 3 for i in range(B * L)]
+    s, tok = _session(B, L, H, D, lens, dtype, T)
+    full = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    for t, back in enumerate((0, 0, 3, 0, 1, 0)):      # (the rows taken back are overwritten)
+        if back:
+            s.cache.len.sub_(back)
+        n = [int(x) for x in (s.cache.len if t == 0 or back else last + 1).tolist()]
+        last = torch.tensor(n, dtype=torch.int32, device="cuda")
+        out = s.decode(*tok[t])
+        if back == 0 and t % 2:
+            continue                                   # (the next call right behind it)
+        torch.cuda.synchronize()
+        for i in (0, B * L // 2, B * L - 1):
+            ref = _attend(s, tok[t][0], i, n[i] + 1)
+            assert (out[i // L, i % L].double() - ref).abs().max().item() <= TOL[dtype], (t, i)
+    assert s.cache.len.tolist() == [n + T - 4 for n in full.tolist()] and s.status.tolist() == [0] * B
+
+
 @pytest.mark.parametrize("place", ["len", "row_offset"])
 def test_a_plan_changed_just_before_the_call(place):
     """The rows that count are those of the plan after the kernel in front, whatever was there while it ran."""
