@@ -1,6 +1,6 @@
 // Decode attention over the ragged cache (Sec. 3.1, Fig. 2a), (segment, head) pair by pair: calls with few pairs (a layer at
 // a time, or a few layers, of a small batch) by a cluster of CTAs to a pair, most others by a CTA to a pair
-// (launch_decode_cluster has the lines).
+// (decode_cluster_ctas has the lines).
 //
 // A call of few pairs moves a few megabytes, so what counts is the chain of latencies of one launch and that
 // every SM has a share.  A cluster of C CTAs takes one (segment, head); each CTA takes a C-th of its
